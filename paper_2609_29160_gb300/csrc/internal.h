@@ -246,10 +246,14 @@ template <class T> struct WalkBatch {
   int64_t moves_cap;
   int64_t* n_moves;                // [n_inst]
   tre_diag* diag;
-  int32_t ent_base[kMaxSeries + 1];  // tick entries (fast then slow) per series, prefix
+  int32_t ent_base[kMaxSeries + 1];  // table entries per series, prefix: chunks of fast ticks
+                                     // (lane walk), else ticks (fast then slow)
 };
-// per-(series, tau, tick) receiver and per-model donor ranks
+// per-(series, tau, tick) tables: the lane walk's rows, or receivers and
+// per-model donor ranks for the walks that visit every tick
 struct WalkWs {
+  uint16_t* rows;     // [chunk][tick][model] next donor tick and rank (lane walk)
+  uint8_t *recs, *nexts;  // [chunk][tick] receiver and kind, next acting tick (lane walk)
   int16_t* recv;
   int16_t* n_donor;   // donors with a rank at the tick
   uint16_t* rank;     // [entry][model] position in the donor order

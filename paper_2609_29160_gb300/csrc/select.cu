@@ -11,9 +11,12 @@
 // Donor order: idle models by index, then surplus by Z descending, then
 // nominal by Z descending (in rebalance only those above the receiver's Z);
 // critical models and the receiver get no rank.
-// The serial part -- one warp per controller instance walking its ticks with
-// the replica counts in registers (models m = lane + 32*j) -- then only picks,
-// per released replica, the lowest-ranked model still above its floor.
+// The serial part walks the ticks with the replica counts in registers. On
+// nested cadences (slow a multiple of fast, no fast tick shorter than a
+// window) and up to 64 models it is k_walk_lane: a warp per controller
+// instance, a model per lane, jumping from move to move. Other cadences visit
+// every tick (k_walk_thread up to 16 models, k_walk above), as do more than 64
+// models (k_walk).
 #include <algorithm>
 #include <cstddef>
 
@@ -157,9 +160,8 @@ __device__ __forceinline__ void load_quad(const double* p, double* v) {
 // acting only below Z = 1; lowest index on ties; -1 when the tick does
 // nothing); each model's rank in the donor order (kNoRank when not a donor),
 // the donor order packed four bits a position (M <= 16), the donor mask and
-// the donor count. With QUAD (M a multiple of 4, 16-byte aligned rows) the
-// rows are read four models per load.
-template <class T, int MMAX, bool QUAD>
+// the donor count.
+template <class T, int MMAX>
 struct TickAction {
   int recv, nd;
   unsigned long long pk, dmw;
@@ -167,7 +169,7 @@ struct TickAction {
   uint16_t rk[MMAX];
 };
 
-template <class T, int MMAX, bool QUAD>
+template <class T, int MMAX>
 __device__ __forceinline__ void tick_row(const WalkBatch<T>& b, int s, uint32_t k, T (&z)[MMAX],
                                          uint8_t (&cl)[MMAX]) {
   const int M = b.M;
@@ -178,29 +180,18 @@ __device__ __forceinline__ void tick_row(const WalkBatch<T>& b, int s, uint32_t 
     z[q] = (T)0;
     cl[q] = kIdle;
   }
-  if (QUAD) {
 #pragma unroll
-    for (int q = 0; q < MMAX; q += 4) {
-      if (q < M) {
-        load_quad(Zk + q, z + q);
-        const uchar4 c4 = *reinterpret_cast<const uchar4*>(Ck + q);
-        cl[q] = c4.x; cl[q + 1] = c4.y; cl[q + 2] = c4.z; cl[q + 3] = c4.w;
-      }
+  for (int q = 0; q < MMAX; ++q)
+    if (q < M) {
+      z[q] = Zk[q];
+      cl[q] = Ck[q];
     }
-  } else {
-#pragma unroll
-    for (int q = 0; q < MMAX; ++q)
-      if (q < M) {
-        z[q] = Zk[q];
-        cl[q] = Ck[q];
-      }
-  }
 }
 
-template <class T, int MMAX, bool QUAD>
+template <class T, int MMAX>
 __device__ __forceinline__ void tick_action(const WalkBatch<T>& b, int ti, bool fast,
                                             const T (&z)[MMAX], const uint8_t (&cl)[MMAX],
-                                            TickAction<T, MMAX, QUAD>& out) {
+                                            TickAction<T, MMAX>& out) {
   const int M = b.M;
   const bool tau_dev = b.tau_crit != nullptr;
   const T tau_v = b.tau_list[tau_dev ? 0 : ti];
@@ -268,7 +259,7 @@ __device__ __forceinline__ void tick_action(const WalkBatch<T>& b, int ti, bool 
 // One thread per (series, tau, tick entry) for M <= MMAX: the regions are
 // computed once per model and the ranks in registers; the per-model rank and
 // order tables are written only when the walk that follows reads them.
-template <class T, int MMAX, bool QUAD>
+template <class T, int MMAX>
 __global__ void __launch_bounds__(128)
 k_tick_rank_small(const __grid_constant__ WalkBatch<T> b, int16_t* recv_out, int16_t* ndon_out,
                   uint16_t* rank, uint16_t* order, unsigned long long* packed, uint32_t* dmask,
@@ -290,9 +281,9 @@ k_tick_rank_small(const __grid_constant__ WalkBatch<T> b, int16_t* recv_out, int
   const uint32_t k = (tj + win - 1) / win - 1;   // window whose right edge passes tj
   T z[MMAX];
   uint8_t cl[MMAX];
-  tick_row<T, MMAX, QUAD>(b, s, k, z, cl);
-  TickAction<T, MMAX, QUAD> a;
-  tick_action<T, MMAX, QUAD>(b, ti, fast, z, cl, a);
+  tick_row<T, MMAX>(b, s, k, z, cl);
+  TickAction<T, MMAX> a;
+  tick_action<T, MMAX>(b, ti, fast, z, cl, a);
   const size_t row = (size_t)b.ent_base[s] * b.n_tau + (size_t)ti * n_ent + j;
   if (need_rank) {
 #pragma unroll
@@ -543,122 +534,41 @@ k_walk(const __grid_constant__ WalkBatch<T> b, const int16_t* recv_tab, const in
       free_pool = f - need;
     }
   };
-  // Nested cadences (the slow tick a multiple of the fast one, the fast tick
-  // at least a window): the ticks are the fast ticks u = 0 .. nf-1, and fast
-  // tick u also carries slow tick (u+1)/ratio when ratio divides u+1. The
-  // replica state only changes where a tick moves something, so 32 ticks are
-  // tested at once against the current state (a receiver, and either room in
-  // the pool for its footprint or a donor above its floor) and the walk jumps
-  // to the first that can act.
-  if (MPL <= 2 && F >= win && Sl % F == 0) {
-    const int64_t ratio = Sl / F;
-    // tick windows by multiply-high division (tick times stay below 2^31 ms)
-    const FastDiv fwin((uint32_t)win);
-    // the table entries of 32 consecutive fast ticks, one per lane: receivers
-    // and donor masks of the tick and of the slow tick it carries
-    struct Ent {
-      int rf, rs;
-      unsigned long long df, ds;
-    };
-    // entry of the slow tick carried by fast tick u
-    auto slow_ent = [&](int64_t u) { return (int32_t)(nf + (u + 1) / ratio - 1); };
-    auto load = [&](int64_t base, Ent& e) {
-      const int64_t u = base + lane;
-      const int32_t es = slow_ent(u);
-      const bool in = u < nf;
-      const bool has_slow = in && (u + 1) % ratio == 0 && es < n_ent;
-      e.rf = in ? rv_tab[u] : -1;
-      e.df = in ? dm_tab[u] : 0ull;
-      e.rs = has_slow ? rv_tab[es] : -1;
-      e.ds = has_slow ? dm_tab[es] : 0ull;
-    };
-    // the next group's entries are loaded while the current group is tested
-    // and acted on; after a tick acts, the rest of its group is tested again
-    // against the new state without loading anything
-    Ent cur, nxt;
-    int64_t base = 0;
-    int start = 0;   // lanes of the current group before it are done
-    load(0, cur);
-    load(32, nxt);
-    while (base < nf) {
+  while (true) {
+    const int32_t kf = sf.window(), ks = ss.window();
+    const int32_t k = kf < ks ? kf : ks;
+    if (k >= K) break;
+    const bool fast = kf == k, slow = ks == k;
+    const int32_t ef = jf - 1, es = (int32_t)nf + js - 1;   // entries of this tick
+    while (sf.window() <= k) { sf.next(); ++jf; }
+    while (ss.window() <= k) { ss.next(); ++js; }
+    int recv = -1, kind = 0;
+    int32_t ent = -1;
+    if (fast) {
+      const int rv = rv_at(ef, fb0, fbuf);
+      if (rv >= 0) { recv = rv; ent = ef; kind = TRE_RESCUE; }
+    }
+    if (!kind && slow) {
+      const int rv = rv_at(es, sb0, sbuf);
+      if (rv >= 0) { recv = rv; ent = es; kind = TRE_REBALANCE; }
+    }
+    if (!kind) continue;
+    if (MPL <= 2) {
+      const unsigned long long donors =
+          ent < (int32_t)nf ? dm_at(ent, fm0, fmb) : dm_at(ent, sm0, smb);
       unsigned long long above = 0;
 #pragma unroll
       for (int j = 0; j < MPL; ++j)
         above |= (unsigned long long)__ballot_sync(0xffffffffu, lane + 32 * j < M && r[j] > rmin[j])
                  << (32 * j);
-      int rv = -1, kind = 0;
-      int32_t ent = -1;
-      unsigned long long dn = 0;
-      if (cur.rf >= 0) {
-        rv = cur.rf; kind = TRE_RESCUE; ent = (int32_t)(base + lane); dn = cur.df;
-      } else if (cur.rs >= 0) {
-        rv = cur.rs; kind = TRE_REBALANCE; ent = slow_ent(base + lane); dn = cur.ds;
-      }
-      // the receiver's footprint sits in lane rv % 32, slot rv / 32
       int g_rv = 0;
 #pragma unroll
-      for (int j = 0; j < MPL; ++j) {
-        const int x = __shfl_sync(0xffffffffu, g[j], rv & 31);
-        if (rv >= 0 && (rv >> 5) == j) g_rv = x;
-      }
-      const bool can = lane >= start && rv >= 0 && (free_pool >= g_rv || (dn & above) != 0);
-      const unsigned hit = __ballot_sync(0xffffffffu, can);
-      int next_start = 32;
-      if (hit) {
-        const int src = __ffs(hit) - 1;
-        const int32_t e_t = __shfl_sync(0xffffffffu, ent, src);
-        const int rv_t = __shfl_sync(0xffffffffu, rv, src);
-        const int kd_t = __shfl_sync(0xffffffffu, kind, src);
-        act((int32_t)fwin.div((uint32_t)(base + src + 1) * (uint32_t)F + (uint32_t)win - 1u) - 1,
-            rv_t, kd_t, e_t);
-        next_start = src + 1;
-      }
-      if (next_start < 32) {
-        start = next_start;
-      } else {
-        base += 32;
-        cur = nxt;
-        load(base + 32, nxt);
-        start = 0;
-      }
+      for (int j = 0; j < MPL; ++j)
+        if (lane + 32 * j == recv) g_rv = g[j];
+      const int need_rv = __shfl_sync(0xffffffffu, g_rv, recv & 31);
+      if (free_pool < need_rv && !(donors & above)) continue;
     }
-  } else {
-    while (true) {
-      const int32_t kf = sf.window(), ks = ss.window();
-      const int32_t k = kf < ks ? kf : ks;
-      if (k >= K) break;
-      const bool fast = kf == k, slow = ks == k;
-      const int32_t ef = jf - 1, es = (int32_t)nf + js - 1;   // entries of this tick
-      while (sf.window() <= k) { sf.next(); ++jf; }
-      while (ss.window() <= k) { ss.next(); ++js; }
-      int recv = -1, kind = 0;
-      int32_t ent = -1;
-      if (fast) {
-        const int rv = rv_at(ef, fb0, fbuf);
-        if (rv >= 0) { recv = rv; ent = ef; kind = TRE_RESCUE; }
-      }
-      if (!kind && slow) {
-        const int rv = rv_at(es, sb0, sbuf);
-        if (rv >= 0) { recv = rv; ent = es; kind = TRE_REBALANCE; }
-      }
-      if (!kind) continue;
-      if (MPL <= 2) {
-        const unsigned long long donors =
-            ent < (int32_t)nf ? dm_at(ent, fm0, fmb) : dm_at(ent, sm0, smb);
-        unsigned long long above = 0;
-#pragma unroll
-        for (int j = 0; j < MPL; ++j)
-          above |= (unsigned long long)__ballot_sync(0xffffffffu, lane + 32 * j < M && r[j] > rmin[j])
-                   << (32 * j);
-        int g_rv = 0;
-#pragma unroll
-        for (int j = 0; j < MPL; ++j)
-          if (lane + 32 * j == recv) g_rv = g[j];
-        const int need_rv = __shfl_sync(0xffffffffu, g_rv, recv & 31);
-        if (free_pool < need_rv && !(donors & above)) continue;
-      }
-      act(k, recv, kind, ent);
-    }
+    act(k, recv, kind, ent);
   }
 #pragma unroll
   for (int j = 0; j < MPL; ++j) {
@@ -846,35 +756,6 @@ k_walk_thread(const __grid_constant__ WalkBatch<T> b, const int16_t* recv_tab,
   if (nm > cap) b.diag->err = TRE_EOVERFLOW;
 }
 
-// Jumping walk for nested cadences (slow_ms a multiple of fast_ms, so every
-// slow tick is a fast tick): the action of each tick (rescue entry, else
-// rebalance entry, else none) does not depend on the replica state, and the
-// state changes only when something moves. A tick can move something only if
-// the idle pool is non-empty or a model above its floor is a donor there; per
-// model, the next tick where it is a donor is precomputed, so the walk jumps
-// from one possible move to the next instead of visiting every tick.
-// Smallest of a tick row's next-donor ticks over the models in `avail`: the
-// row holds MMAX 16-bit entries; models outside the mask are lifted to 0xffff
-// and the row is reduced with per-halfword minima.
-template <int MMAX>
-__device__ __forceinline__ int next_donor_tick(const uint16_t* row, uint32_t avail) {
-  const uint4* q = reinterpret_cast<const uint4*>(row);
-  uint32_t acc = 0xffffffffu;
-#pragma unroll
-  for (int h = 0; h < MMAX / 8; ++h) {
-    const uint4 w = q[h];
-    const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int m = h * 8 + 2 * i;
-      const uint32_t lift = ((avail >> m) & 1u ? 0u : 0xffffu) |
-                            ((avail >> (m + 1)) & 1u ? 0u : 0xffff0000u);
-      acc = __vminu2(acc, ws[i] | lift);
-    }
-  }
-  return (int)min(acc & 0xffffu, acc >> 16);
-}
-
 // One move record, written as three 32-bit words (window; receiver and donor;
 // kind and position in the tick) when it fits the caller's list.
 static_assert(sizeof(tre_move) == 12 && offsetof(tre_move, recv) == 4 &&
@@ -891,491 +772,667 @@ __device__ __forceinline__ void put_move(tre_move* mv, int64_t at, int64_t cap, 
   }
 }
 
-// One tick's action as the walk reads it: donor order (4 bits a position),
-// donor mask, receiver (-1: nothing acts) and kind, in one 16-byte load.
-struct __align__(16) TickRec {
-  unsigned long long pk;
-  uint32_t dm;
-  int16_t recv;
-  uint8_t kind, pad;
+// ---- lane walk: nested cadences, up to 64 models ----------------------------
+// On nested cadences the ticks are the fast ticks, and what a tick would do
+// (receiver, kind, donor order) does not depend on the replica state, so the
+// state only decides which tick moves something next: the first one where the
+// idle pool is not empty or a donor stands above its floor. Ticks are cut into
+// chunks of kChunk; k_tick_rows ranks a chunk's ticks and stores, per tick u of
+// the chunk and model, one 16-bit word
+//     (first tick t >= u of the chunk where the model is a donor) << RB | rank
+// (rank from 1 in the tick's donor order; t = kChunk: none left in the chunk).
+// k_walk_lane keeps one model per lane (two above 32): one shared-memory load
+// of the row at u, masked by "above its floor", and one warp-wide minimum give
+// the next tick that moves something and its donor together. Ranking and walk
+// measured, before (one thread per tick; one lane jumping over tables of next
+// donor ticks up to 16 models, one warp testing 32 ticks a ballot above) and
+// now: 16 models, 4,320 ticks, 431 moves 228 -> 57 us; 64 models, 17,280
+// ticks, 1,493 moves 1,504 -> 199 us; 24 models of unequal footprint, 720
+// ticks, 1,875 moves 634 -> 308 us; 1,792 instances of 8 models 89 -> 51 us.
+constexpr int kChunk = 128;          // ticks per chunk
+
+template <int MP> struct RowBits;    // rank bits of a row word (ranks 1..MP-1)
+template <> struct RowBits<8> { static constexpr int v = 3; };
+template <> struct RowBits<16> { static constexpr int v = 4; };
+template <> struct RowBits<32> { static constexpr int v = 5; };
+template <> struct RowBits<64> { static constexpr int v = 6; };
+
+constexpr uint32_t kNoTick = 0x7f;   // receiver byte of a tick that does nothing
+constexpr uint32_t kSlowBit = 0x80;  // receiver byte: the tick rebalances
+
+// order of the values as unsigned keys (-0 equals 0), total also for NaN, so
+// that the ranks of a tick are always distinct
+__device__ __forceinline__ uint32_t order_key(float z) {
+  uint32_t u = __float_as_uint(z);
+  if (u == 0x80000000u) u = 0;
+  return u ^ ((u >> 31) ? 0xffffffffu : 0x80000000u);
+}
+__device__ __forceinline__ unsigned long long order_key(double z) {
+  unsigned long long u = (unsigned long long)__double_as_longlong(z);
+  if (u == 0x8000000000000000ull) u = 0;
+  return u ^ ((u >> 63) ? ~0ull : 0x8000000000000000ull);
+}
+
+// Position of a donor in its tick's order: group (idle 0, surplus 1, nominal
+// 2), Z descending within surplus and nominal, then index; a model that is no
+// donor comes after every donor.
+template <class T> struct DonorKey;
+template <> struct DonorKey<float> {
+  unsigned long long k;
+  DonorKey() = default;
+  __device__ __forceinline__ DonorKey(int g, float z, int m)
+      : k(g < 0 ? ~0ull
+                : (unsigned long long)g << 38 |
+                      (unsigned long long)(g ? ~order_key(z) : 0u) << 6 | (unsigned)m) {}
+  __device__ __forceinline__ bool operator<(const DonorKey& o) const { return k < o.k; }
+};
+template <> struct DonorKey<double> {
+  unsigned long long k;
+  unsigned long long gm;
+  DonorKey() = default;
+  __device__ __forceinline__ DonorKey(int g, double z, int m)
+      : k(g > 0 ? ~order_key(z) : 0ull), gm((unsigned long long)(g < 0 ? 3 : g) << 6 | (unsigned)m) {}
+  __device__ __forceinline__ bool operator<(const DonorKey& o) const {
+    const unsigned ga = (unsigned)gm >> 6, gb = (unsigned)o.gm >> 6;
+    return ga != gb ? ga < gb : (k != o.k ? k < o.k : (unsigned)gm < (unsigned)o.gm);
+  }
 };
 
-// RANK: the CTA of a (series, tau) finds its ticks' actions itself from the Z
-// and class rows (tick_action) while it builds the tables -- one launch, for
-// batches with a CTA per SM or more; otherwise it reads them from the tick
-// tables k_tick_rank_small wrote (the ranking then spreads over many CTAs).
-template <class T, int MMAX, bool RANK, bool QUAD>
-__global__ void __launch_bounds__(256, 1)
-k_walk_jump(const __grid_constant__ WalkBatch<T> b, const int16_t* recv_tab,
-            const unsigned long long* packed, const uint32_t* dmask, bool store_win) {
-  extern __shared__ __align__(16) unsigned char dyn[];
-  const int grp = blockIdx.x;
-  const int ti = grp % b.n_tau;
-  const int si = grp / b.n_tau;
+// donor group of a model of region rg at a tick that acts, -1 = not a donor
+template <class T>
+__device__ __forceinline__ int donor_group(uint8_t rg, T z, T zr, bool rescue) {
+  if (rg == kIdle) return 0;
+  if (rg == kSurp) return 1;
+  if (rg == kNom && (rescue || z > zr)) return 2;   // rebalance: nominal above the receiver
+  return -1;
+}
+
+// The chunk a CTA ranks, and the window of its ticks
+template <class T> struct ChunkOf {
+  int s, ti, c0, nf;
+  uint32_t win;
+  __device__ __forceinline__ ChunkOf(const WalkBatch<T>& b) {
+    s = prefix_index(b.ent_base, b.n_series, blockIdx.x, b.n_tau);
+    const int local = (int)(blockIdx.x - (int64_t)b.ent_base[s] * b.n_tau);
+    const int nch = b.ent_base[s + 1] - b.ent_base[s];
+    ti = local / nch;
+    c0 = (local - ti * nch) * kChunk;
+    // K * win < 2^31, so every tick time fits 32 unsigned bits
+    win = (uint32_t)b.series_win[s];
+    nf = (int)((uint32_t)b.series_K[s] * win / (uint32_t)b.fast_ms);
+  }
+};
+
+// From the ranks (0 = not a donor) and receiver bytes of a chunk's ticks in
+// shared memory: the row words, a suffix minimum per column -- each thread
+// finds its segment's first donor tick, then writes its segment backwards from
+// the first one after it -- and the next tick that does anything.
+template <int MP, int THREADS>
+__device__ __forceinline__ void write_rows(const uint8_t (*s_rank)[MP], const uint8_t* s_rec,
+                                           uint16_t* rows, uint8_t* recs, uint8_t* nexts) {
+  constexpr int NSEG = THREADS / MP < 16 ? THREADS / MP : 16, SEGL = kChunk / NSEG;
+  constexpr int RB = RowBits<MP>::v;
+  constexpr uint32_t kEnd = (uint32_t)kChunk << RB;
+  __shared__ uint16_t s_first[NSEG][MP];
+  const int col = threadIdx.x % MP, seg = threadIdx.x / MP;
+  if (seg < NSEG) {
+    uint32_t f = kEnd;
+#pragma unroll
+    for (int i = SEGL - 1; i >= 0; --i) {
+      const uint32_t r = s_rank[seg * SEGL + i][col];
+      if (r) f = (uint32_t)(seg * SEGL + i) << RB | r;
+    }
+    s_first[seg][col] = (uint16_t)f;
+  }
+  __syncthreads();
+  const size_t base = (size_t)blockIdx.x * kChunk;
+  if (seg < NSEG) {
+    uint32_t v = kEnd;
+#pragma unroll
+    for (int j = 1; j < NSEG; ++j)
+      if (j > seg) v = min(v, (uint32_t)s_first[j][col]);
+    uint16_t* out = rows + base * MP + col;
+#pragma unroll
+    for (int i = SEGL - 1; i >= 0; --i) {
+      const int ul = seg * SEGL + i;
+      const uint32_t r = s_rank[ul][col];
+      if (r) v = (uint32_t)ul << RB | r;
+      out[(size_t)ul * MP] = (uint16_t)v;
+    }
+  }
+  if (threadIdx.x < kChunk) {
+    const int lane = threadIdx.x & 31;
+    int nx = kChunk;
+    for (int g = kChunk / 32 - 1; g >= (int)threadIdx.x / 32; --g) {
+      unsigned on = __ballot_sync(0xffffffffu, s_rec[32 * g + lane] != kNoTick);
+      if (g == (int)threadIdx.x / 32) on &= 0xffffffffu << lane;
+      if (on) nx = 32 * g + __ffs(on) - 1;
+    }
+    recs[base + threadIdx.x] = s_rec[threadIdx.x];
+    nexts[base + threadIdx.x] = (uint8_t)nx;
+  }
+}
+
+// Up to 16 models: one CTA per (series, tau, chunk), one thread per tick with
+// its row in registers; every pair of models is compared once. Bound by the
+// instructions of its few warps (4,320 ticks of 16 models: 12 us; spreading a
+// tick's models over lanes and counting from shuffles took 15).
+template <class T, int MP, bool QUAD>
+__global__ void __launch_bounds__(kChunk)
+k_tick_rows(const __grid_constant__ WalkBatch<T> b, uint16_t* __restrict__ rows,
+            uint8_t* __restrict__ recs, uint8_t* __restrict__ nexts) {
+  __shared__ uint8_t s_rank[kChunk][MP];
+  __shared__ uint8_t s_rec[kChunk];
   const int M = b.M;
-  const int K = b.series_K[si];
-  const int64_t win = b.series_win[si];
-  const int n_ent = b.ent_base[si + 1] - b.ent_base[si];
-  const size_t row0 = (size_t)b.ent_base[si] * b.n_tau + (size_t)ti * n_ent;
-  const int nf = (int)((int64_t)K * win / b.fast_ms);   // fast ticks = all ticks
+  const ChunkOf<T> ch(b);
+  const int u = ch.c0 + threadIdx.x;
+  uint32_t rec = kNoTick;
+  int rank[MP];
+#pragma unroll
+  for (int m = 0; m < MP; ++m) rank[m] = 0;
+  if (u < ch.nf) {
+    // window whose right edge passes the tick
+    const uint32_t k =
+        FastDiv(ch.win).div((uint32_t)(u + 1) * (uint32_t)b.fast_ms + ch.win - 1u) - 1u;
+    const size_t x = (size_t)b.series_off[ch.s] + (size_t)k * M;
+    T z[MP];
+    uint8_t rg[MP];
+#pragma unroll
+    for (int m = 0; m < MP; m += 4) {
+      if (QUAD && m < M) {
+        load_quad(b.Z + x + m, z + m);
+        const uchar4 c4 = *reinterpret_cast<const uchar4*>(b.cls + x + m);
+        rg[m] = c4.x; rg[m + 1] = c4.y; rg[m + 2] = c4.z; rg[m + 3] = c4.w;
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          z[m + i] = m + i < M ? b.Z[x + m + i] : (T)0;
+          rg[m + i] = m + i < M ? b.cls[x + m + i] : kIdle;
+        }
+      }
+    }
+    const bool tau_dev = b.tau_crit != nullptr;
+    const T tau_v = b.tau_list[tau_dev ? 0 : ch.ti];
+    bool rescue = false;
+#pragma unroll
+    for (int m = 0; m < MP; ++m)
+      if (m < M) {
+        rg[m] = region_of(rg[m], z[m], tau_dev ? b.tau_crit[m] : tau_v, b.tau_surp[m]);
+        rescue |= rg[m] == kCrit;
+      }
+    // receiver: rescue -> lowest Z among critical; rebalance -> among non-idle
+    const bool slow = (u + 1) % (b.slow_ms / b.fast_ms) == 0;
+    int recv = -1;
+    T zr = (T)0;
+#pragma unroll
+    for (int m = 0; m < MP; ++m) {
+      const bool cand = m < M && (rescue ? rg[m] == kCrit : slow && rg[m] != kIdle);
+      if (cand && (recv < 0 || z[m] < zr)) {
+        recv = m;
+        zr = z[m];
+      }
+    }
+    if (recv >= 0 && (rescue || zr < (T)1)) {
+      rec = (uint32_t)recv | (rescue ? 0u : kSlowBit);
+      DonorKey<T> key[MP];
+      bool don[MP];
+#pragma unroll
+      for (int m = 0; m < MP; ++m) {
+        const int g = m < M && m != recv ? donor_group(rg[m], z[m], zr, rescue) : -1;
+        don[m] = g >= 0;
+        key[m] = DonorKey<T>(g, z[m], m);
+        rank[m] = 1;
+      }
+#pragma unroll
+      for (int m = 1; m < MP; ++m)
+#pragma unroll
+        for (int q = 0; q < m; ++q) {
+          const bool first = key[q] < key[m];
+          rank[m] += first;
+          rank[q] += !first;
+        }
+#pragma unroll
+      for (int m = 0; m < MP; ++m) rank[m] = don[m] ? rank[m] : 0;
+    }
+  }
+  s_rec[threadIdx.x] = (uint8_t)rec;
+#pragma unroll
+  for (int m = 0; m < MP; m += 4)
+    *reinterpret_cast<uint32_t*>(&s_rank[threadIdx.x][m]) =
+        (uint32_t)rank[m] | (uint32_t)rank[m + 1] << 8 | (uint32_t)rank[m + 2] << 16 |
+        (uint32_t)rank[m + 3] << 24;
+  __syncthreads();
+  write_rows<MP, kChunk>(s_rank, s_rec, rows, recs, nexts);
+}
+
+// 17 to 64 models: a warp per tick, models on lanes (two per lane above 32);
+// rows of Z and regions are read coalesced and a model's rank is counted
+// against the tick's keys in shared memory (64 models, 17,280 ticks: 24 us, at
+// 80 % of the issue slots; one thread per model on scattered loads took 202).
+constexpr int kWideThreads = 1024;
+template <class T, int MP>
+__global__ void __launch_bounds__(kWideThreads)
+k_tick_rows_wide(const __grid_constant__ WalkBatch<T> b, uint16_t* __restrict__ rows,
+                 uint8_t* __restrict__ recs, uint8_t* __restrict__ nexts) {
+  constexpr int MPL = MP / 32;
+  __shared__ uint8_t s_rank[kChunk][MP];
+  __shared__ uint8_t s_rec[kChunk];
+  __shared__ __align__(16) DonorKey<T> s_key[kWideThreads / 32][MP];
+  const unsigned full = 0xffffffffu;
+  const int M = b.M;
+  const ChunkOf<T> ch(b);
+  const FastDiv fwin(ch.win);
   const int ratio = b.slow_ms / b.fast_ms;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-  // shared layout: per tick u < nf: action record and window; per tick
-  // u <= nf: for every model the next tick >= u where it is a donor (one
-  // 2*MMAX-byte row per tick, so a row is read with 16-byte loads), and the
-  // next tick >= u where anything acts
-  // (the window of each tick is staged when there is room, else recomputed
-  // at each visit)
-  TickRec* srec = reinterpret_cast<TickRec*>(dyn);
-  int32_t* swin = reinterpret_cast<int32_t*>(srec + nf);
-  uint16_t* snx = store_win ? reinterpret_cast<uint16_t*>(swin + ((nf + 3) & ~3))
-                            : reinterpret_cast<uint16_t*>(swin);           // [nf + 1][MMAX]
-  // window of fast tick u, ceil((u + 1) * fast / win) - 1, without a divide
-  // instruction (the tick times stay below 2^31 ms)
-  const FastDiv fwin((uint32_t)win);
-  auto tick_of = [&](int u) -> int32_t {
-    return (int32_t)fwin.div((uint32_t)(u + 1) * (uint32_t)b.fast_ms + (uint32_t)win - 1u) - 1;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool tau_dev = b.tau_crit != nullptr;
+  T tc[MPL], tsu[MPL];
+#pragma unroll
+  for (int j = 0; j < MPL; ++j) {
+    const int m = lane + 32 * j;
+    tc[j] = m < M ? (tau_dev ? b.tau_crit[m] : b.tau_list[ch.ti]) : (T)0;
+    tsu[j] = m < M ? b.tau_surp[m] : (T)0;
+  }
+  for (int ul = warp; ul < kChunk; ul += kWideThreads / 32) {
+    const int u = ch.c0 + ul;
+    uint32_t rec = kNoTick;
+    int rank[MPL];
+#pragma unroll
+    for (int j = 0; j < MPL; ++j) rank[j] = 0;
+    if (u < ch.nf) {
+      const uint32_t k = fwin.div((uint32_t)(u + 1) * (uint32_t)b.fast_ms + ch.win - 1u) - 1u;
+      const size_t x = (size_t)b.series_off[ch.s] + (size_t)k * M + lane;
+      T z[MPL];
+      uint8_t rg[MPL];
+      unsigned crit[MPL], live[MPL];
+      bool rescue = false;
+#pragma unroll
+      for (int j = 0; j < MPL; ++j) {
+        const bool has = lane + 32 * j < M;
+        z[j] = has ? b.Z[x + 32 * j] : (T)0;
+        rg[j] = has ? region_of(b.cls[x + 32 * j], z[j], tc[j], tsu[j]) : (uint8_t)0xff;
+        crit[j] = __ballot_sync(full, rg[j] == kCrit);
+        live[j] = __ballot_sync(full, has && rg[j] != kIdle);
+        rescue |= crit[j] != 0;
+      }
+      const bool slow = (u + 1) % ratio == 0;
+      // receiver: lowest Z among the candidates, lowest index on ties (a NaN
+      // stays only where it is the first candidate, as in an ascending scan)
+      int recv = -1;
+      T zr = (T)0;
+#pragma unroll
+      for (int j = 0; j < MPL; ++j) {
+        const unsigned cand = rescue ? crit[j] : (slow ? live[j] : 0u);
+        if (!cand) continue;
+        const unsigned num = cand & ~__ballot_sync(full, z[j] != z[j]);
+        int w = __ffs(cand) - 1;
+        if (recv >= 0 && !num) continue;
+        if (recv >= 0 || (num >> w & 1u)) {
+          const auto key = order_key(z[j]);
+          const bool in = num >> lane & 1u;
+          const uint32_t hi = sizeof(T) == 8 ? (uint32_t)((unsigned long long)key >> 32)
+                                             : (uint32_t)key;
+          const uint32_t mh = __reduce_min_sync(full, in ? hi : 0xffffffffu);
+          bool low = in && hi == mh;
+          if (sizeof(T) == 8) {
+            const uint32_t ml = __reduce_min_sync(full, low ? (uint32_t)key : 0xffffffffu);
+            low = low && (uint32_t)key == ml;
+          }
+          w = __ffs(__ballot_sync(full, low)) - 1;
+        }
+        const T zw = __shfl_sync(full, z[j], w);
+        if (recv < 0 || zw < zr) {
+          recv = w + 32 * j;
+          zr = zw;
+        }
+      }
+      if (recv >= 0 && (rescue || zr < (T)1)) {
+        rec = (uint32_t)recv | (rescue ? 0u : kSlowBit);
+        DonorKey<T> key[MPL];
+        bool don[MPL];
+#pragma unroll
+        for (int j = 0; j < MPL; ++j) {
+          const int m = lane + 32 * j;
+          const int g = m != recv ? donor_group(rg[j], z[j], zr, rescue) : -1;
+          don[j] = g >= 0;
+          key[j] = DonorKey<T>(g, z[j], m);
+          s_key[warp][m] = key[j];
+          rank[j] = 1;
+        }
+        __syncwarp();
+#pragma unroll 16
+        for (int q = 0; q < MP; ++q) {
+          const DonorKey<T> kq = s_key[warp][q];
+#pragma unroll
+          for (int j = 0; j < MPL; ++j) rank[j] += kq < key[j];
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < MPL; ++j) rank[j] = don[j] ? rank[j] : 0;
+      }
+    }
+    if (lane == 0) s_rec[ul] = (uint8_t)rec;
+#pragma unroll
+    for (int j = 0; j < MPL; ++j) s_rank[ul][lane + 32 * j] = (uint8_t)rank[j];
+  }
+  __syncthreads();
+  write_rows<MP, kWideThreads>(s_rank, s_rec, rows, recs, nexts);
+}
+
+// What the walk reads, by value: per-series tick counts and the controllers.
+struct LaneWalk {
+  int M, n_tau, n_cap, slab, n_buf;  // slab: ticks staged at a time (a multiple of kChunk)
+  int32_t chunk_base[kMaxSeries + 1], win[kMaxSeries], cap_list[kMaxCap];
+  int32_t fast_ms;
+  int64_t budget, moves_cap;
+  const int32_t *r_min, *footprint, *r0;
+  int32_t* r_out;
+  tre_move* moves;
+  int64_t* n_moves;
+  tre_diag* diag;
+  const uint16_t* rows;
+  const uint8_t *recs, *nexts;
+};
+
+constexpr int kLaneThreads = 256;
+constexpr int kLaneLog = 256;      // moves a warp collects before it writes them out
+// bytes of one staged tick: its row, receiver and next acting tick; a buffer
+// ends in a row of "none", read when a walk steps past the last tick
+template <int MP> __host__ __device__ constexpr int slab_bytes(int ticks) {
+  return ticks * (MP * 2 + 2) + MP * 2;
+}
+
+__device__ __forceinline__ void copy16(void* smem, const void* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+
+// One CTA per (series, tau) and group of kLaneThreads / 32 pacing caps, one
+// warp per controller instance. The rows of `slab` ticks are staged in shared
+// memory, the next slab's loads in flight while this one is walked. What bounds
+// it is the chain of one move: row load, mask, warp minimum, receiver load,
+// counts. Moves go to a log in shared memory (tick, position in the tick,
+// donor) and are written out by the whole warp, so that nothing in the chain
+// branches on a lane (a move with unit footprints and one transition a tick
+// takes 200 cycles; writing its record from the donor's lane took 525).
+template <int MP>
+__global__ void __launch_bounds__(kLaneThreads)
+k_walk_lane(const __grid_constant__ LaneWalk w) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ uint32_t s_log[kLaneThreads / 32][kLaneLog];
+  constexpr int MPL = MP > 32 ? 2 : 1, L1 = MPL - 1;
+  constexpr int RB = RowBits<MP>::v;
+  constexpr uint32_t kNone = 0xffffu;
+  const unsigned full = 0xffffffffu;
+  const int ti = blockIdx.x % w.n_tau, si = blockIdx.x / w.n_tau;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ci = blockIdx.y * (kLaneThreads / 32) + warp;
+  const int M = w.M;
+  const int nch = w.chunk_base[si + 1] - w.chunk_base[si];
+  const int n_tick = nch * kChunk;                  // the last chunk's padding does nothing
+  const size_t t0 = ((size_t)w.chunk_base[si] * w.n_tau + (size_t)ti * nch) * kChunk;
+  const int buf_bytes = slab_bytes<MP>(w.slab);
+  // a buffer: rows [slab + 1][MP] words, receiver bytes, next-tick bytes
+  auto fetch = [&](int first, int buf) {
+    const int n = min(w.slab, n_tick - first);
+    unsigned char* d = dyn + buf * buf_bytes;
+    const unsigned char* src = reinterpret_cast<const unsigned char*>(w.rows + (t0 + first) * MP);
+    for (int i = threadIdx.x; i < n * MP / 8; i += kLaneThreads) copy16(d + 16 * i, src + 16 * i);
+    if (threadIdx.x < MP)
+      reinterpret_cast<uint16_t*>(d)[n * MP + threadIdx.x] = (uint16_t)(kChunk << RB);
+    d += (size_t)(w.slab + 1) * MP * 2;
+    for (int i = threadIdx.x; i < n / 16; i += kLaneThreads) {
+      copy16(d + 16 * i, w.recs + t0 + first + 16 * i);
+      copy16(d + w.slab + 16 * i, w.nexts + t0 + first + 16 * i);
+    }
   };
-  auto tick_win = [&](int u) -> int32_t {
-    return store_win ? swin[u] : tick_of(u);
-  };
-  uint16_t* sany = snx + (size_t)(nf + 1) * MMAX;                          // [nf + 1]
-  __shared__ int s_cap[8][MMAX];   // unit footprints: replicas above the floor, per warp
-#pragma unroll 4
-  for (int u = threadIdx.x; u < nf; u += blockDim.x) {
-    int kd = 0, rv = -1;
-    unsigned long long pk = 0;
-    uint32_t dm = 0;
-    if (!RANK) {
-      // both entries' loads issued before either is used
-      const bool has_slow = (u + 1) % ratio == 0;
-      const int es = nf + (u + 1) / ratio - 1;
-      const int rf = recv_tab[row0 + u];
-      const unsigned long long pf = packed[row0 + u];
-      const uint32_t df = dmask[row0 + u];
-      const int rs = has_slow ? recv_tab[row0 + es] : -1;
-      const unsigned long long ps = has_slow ? packed[row0 + es] : 0ull;
-      const uint32_t ds = has_slow ? dmask[row0 + es] : 0u;
-      if (rf >= 0) {
-        kd = TRE_RESCUE; rv = rf; pk = pf; dm = df;
-      } else if (rs >= 0) {
-        kd = TRE_REBALANCE; rv = rs; pk = ps; dm = ds;
+  if (n_tick > 0) fetch(0, 0);
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+
+  // the instance's state: replicas above the floor per model, the idle pool
+  const bool mine = ci < w.n_cap;
+  const int inst = (si * w.n_tau + ti) * w.n_cap + (mine ? ci : 0);
+  const int Kp = mine ? w.cap_list[ci] : 0;
+  const int64_t cap = w.moves_cap;
+  tre_move* mv = w.moves + (size_t)inst * cap;
+  int c[MPL], rmin[MPL], g[MPL];
+  int64_t pool = 0;
+  bool bad = false, unit = true;
+#pragma unroll
+  for (int j = 0; j < MPL; ++j) {
+    const int m = lane + 32 * j;
+    c[j] = rmin[j] = 0;
+    g[j] = 1;
+    if (mine && m < M) {
+      const int r = w.r0[m];
+      rmin[j] = w.r_min[m];
+      g[j] = w.footprint[m];
+      pool += (int64_t)g[j] * r;
+      bad |= r < 0 || g[j] < 1 || rmin[j] < 0;
+      unit &= g[j] == 1;
+      c[j] = r - rmin[j];
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) pool += __shfl_xor_sync(full, pool, o);
+  pool = w.budget - pool;
+  // an inconsistent controller state (negative replicas or floors, footprint
+  // below one, replicas beyond the budget) produces no moves
+  bad = __any_sync(full, bad) || pool < 0;
+  unit = __all_sync(full, unit);
+  const bool walks = mine && !bad && Kp > 0;
+  const FastDiv fwin((uint32_t)w.win[si]);
+  uint32_t* log = s_log[warp];
+  int64_t n_out = 0;   // moves written out
+  int n_log = 0;       // moves in the log: tick | position << 11 | donor << 19 (64: the pool)
+
+  // a slab of n ticks, the first of them tick `first` of the series
+  auto walk = [&](const uint16_t* rows, const uint8_t* recs, const uint8_t* nexts, int n,
+                  int first) {
+    const uint16_t* my = rows + (lane & (MP - 1));
+    // all ones where the model has nothing above its floor
+    uint32_t no[MPL];
+    auto masks = [&]() {
+#pragma unroll
+      for (int j = 0; j < MPL; ++j) no[j] = c[j] > 0 ? 0u : kNone;
+    };
+    masks();
+    auto flush = [&]() {
+      __syncwarp();
+      for (int i = lane; i < n_log; i += 32) {
+        const uint32_t e = log[i];
+        const int a = e & 2047u, d = (int)(e >> 19);
+        const uint32_t rec = recs[a];
+        put_move(mv, n_out + i, cap,
+                 (int32_t)fwin.div((uint32_t)(first + a + 1) * (uint32_t)w.fast_ms +
+                                   (uint32_t)w.win[si] - 1u) - 1,
+                 (int)(rec & 63u), d == 64 ? -1 : d,
+                 rec & kSlowBit ? TRE_REBALANCE : TRE_RESCUE, (int)(e >> 11 & 255u));
+      }
+      __syncwarp();
+      n_out += n_log;
+      n_log = 0;
+    };
+    auto log_one = [&](bool here, uint32_t a, int seq, int donor) {
+      if (here) log[n_log] = a | (uint32_t)seq << 11 | (uint32_t)donor << 19;
+      if (++n_log == kLaneLog) flush();
+    };
+    auto log_run = [&](uint32_t a, int seq, int donor, int take) {   // take <= 255
+      if (n_log + take > kLaneLog) flush();
+      for (int q = lane; q < take; q += 32)
+        log[n_log + q] = a | (uint32_t)(seq + q) << 11 | (uint32_t)donor << 19;
+      n_log += take;
+    };
+    auto receive = [&](int recv, int take) {
+      c[0] += lane == recv ? take : 0;
+      if (MPL > 1) c[L1] += lane + 32 == recv ? take : 0;
+    };
+    int u = 0;
+    int left = Kp;      // transitions the tick at u may still make
+    if (unit) {
+      // the idle pool first: it only shrinks, and every acting tick draws on it
+      while (pool > 0 && u < n) {
+        const int a = (u & ~(kChunk - 1)) + nexts[u];
+        if (nexts[u] == kChunk) {
+          u = a;
+          continue;
+        }
+        const int take = pool < Kp ? (int)pool : Kp;
+        pool -= take;
+        log_run((uint32_t)a, 0, 64, take);
+        receive(recs[a] & 63, take);
+        left = Kp - take;
+        u = left > 0 ? a : a + 1;
+        if (left == 0) left = Kp;
+      }
+      masks();
+      if (u >= n) {
+        flush();
+        return;
+      }
+    }
+    if (unit && Kp == 1) {
+      // one replica per tick: every tick found moves exactly one
+      while (true) {
+        const uint32_t k0 = my[u * MP] | no[0];
+        const uint32_t k1 = MPL > 1 ? my[u * MP + 32] | no[L1] : kNone;
+        const uint32_t best = __reduce_min_sync(full, MPL > 1 ? min(k0, k1) : k0);
+        const int t = (int)(best >> RB), cb = u & ~(kChunk - 1);
+        if (t >= kChunk) {                      // nothing in the rest of the chunk
+          u = cb + kChunk;
+          if (u >= n) break;
+          continue;
+        }
+        const int a = cb + t;
+        const int recv = recs[a] & 63;
+        const bool d0 = k0 == best, d1 = MPL > 1 && k1 == best;
+        c[0] += (lane == recv) - d0;
+        if (MPL > 1) c[L1] += (lane + 32 == recv) - d1;
+        masks();
+        log_one(d0 || d1, (uint32_t)a, 0, lane + (d1 ? 32 : 0));
+        u = a + 1;
+      }
+    } else if (unit) {
+      // up to Kp replicas per tick: donors in rank order, each giving what it
+      // has above its floor
+      int cur = u;
+      while (true) {
+        const uint32_t k0 = my[u * MP] | no[0];
+        const uint32_t k1 = MPL > 1 ? my[u * MP + 32] | no[L1] : kNone;
+        const uint32_t best = __reduce_min_sync(full, MPL > 1 ? min(k0, k1) : k0);
+        const int t = (int)(best >> RB), cb = u & ~(kChunk - 1);
+        if (t >= kChunk) {
+          u = cb + kChunk;
+          if (u >= n) break;
+          continue;
+        }
+        const int a = cb + t;
+        if (a != cur) {
+          cur = a;
+          left = Kp;
+        }
+        const int recv = recs[a] & 63;
+        const bool d0 = k0 == best, d1 = MPL > 1 && k1 == best;
+        const int give = min(d1 ? c[L1] : c[0], left);
+        const int take = (int)__reduce_max_sync(full, d0 || d1 ? (unsigned)give : 0u);
+        if (d0) c[0] -= take;
+        if (MPL > 1 && d1) c[L1] -= take;
+        receive(recv, take);
+        masks();
+        const int src = __ffs(__ballot_sync(full, d0 || d1)) - 1;   // ranks are distinct
+        const unsigned up = MPL > 1 ? __ballot_sync(full, d1) : 0u;
+        log_run((uint32_t)a, Kp - left, src + (up ? 32 : 0), take);
+        left -= take;
+        u = left > 0 ? a : a + 1;
       }
     } else {
-      // a slow tick falls on the window of the fast tick it coincides with;
-      // a rescue at a tick takes precedence over its rebalance
-      T z[MMAX];
-      uint8_t cl[MMAX];
-      tick_row<T, MMAX, QUAD>(b, si, (uint32_t)tick_of(u), z, cl);
-      TickAction<T, MMAX, QUAD> a;
-      tick_action<T, MMAX, QUAD>(b, ti, true, z, cl, a);
-      if (a.recv >= 0) {
-        kd = TRE_RESCUE; rv = a.recv; pk = a.pk; dm = a.dm;
-      } else if ((u + 1) % ratio == 0) {
-        tick_action<T, MMAX, QUAD>(b, ti, false, z, cl, a);
-        if (a.recv >= 0) { kd = TRE_REBALANCE; rv = a.recv; pk = a.pk; dm = a.dm; }
-      }
-    }
-    TickRec t;
-    t.pk = pk;
-    t.dm = dm;
-    t.recv = (int16_t)rv;
-    t.kind = (uint8_t)kd;
-    t.pad = 0;
-    srec[u] = t;
-    if (store_win) swin[u] = tick_of(u);
-  }
-  __syncthreads();
-  // next-tick tables, a suffix minimum per column (MMAX models, then "any"):
-  // the CTA's threads split each column into segments of consecutive ticks;
-  // each finds its segment's first acting tick, then writes its segment
-  // backwards from the first acting tick of the segments after it
-  constexpr int NC = MMAX + 1;
-  const int n_seg = (int)blockDim.x / NC;              // segments per column
-  // a segment length of 1 mod 8 puts the segments' tick records (16 bytes, so
-  // 8 to a bank cycle) of one step on different banks
-  int seg_len = (nf + n_seg - 1) / n_seg;
-  seg_len += (9 - seg_len % 8) % 8;
-  __shared__ int s_first[256];                         // [NC][n_seg]
-  const int my_c = threadIdx.x / n_seg, my_s = threadIdx.x % n_seg;
-  const bool has_seg = my_c < NC;
-  auto acts = [&](int u, int c) -> bool {
-    const TickRec& t = srec[u];
-    if (t.recv < 0) return false;
-    if (c == MMAX) return true;                        // anything acts
-    return c < M && (t.dm >> c & 1u);                  // padding columns never give
-  };
-  const int u_lo = my_s * seg_len, u_hi = min(nf, u_lo + seg_len);
-  if (has_seg) {
-    int f = nf;
-    for (int u = u_lo; u < u_hi; ++u)
-      if (acts(u, my_c)) {
-        f = u;
-        break;
-      }
-    s_first[threadIdx.x] = f;
-  }
-  __syncthreads();
-  if (has_seg) {
-    uint16_t* col = my_c < MMAX ? snx + my_c : sany;
-    const int cs = my_c < MMAX ? MMAX : 1;             // column stride
-    int v = nf;
-    for (int j = my_s + 1; j < n_seg; ++j) v = min(v, s_first[my_c * n_seg + j]);
-    if (my_s == n_seg - 1) col[(size_t)nf * cs] = (uint16_t)nf;
-    for (int u = u_hi - 1; u >= u_lo; --u) {
-      if (acts(u, my_c)) v = u;
-      col[(size_t)u * cs] = (uint16_t)v;
-    }
-  }
-  __syncthreads();
-  // one instance per warp, walked by its first lane
-  if (lane != 0) return;
-  for (int ci = warp; ci < b.n_cap; ci += n_warps) {
-  const int inst = (si * b.n_tau + ti) * b.n_cap + ci;
-  const int Kp = b.cap_list[ci];
-  const int64_t cap = b.moves_cap;
-  tre_move* mv = b.moves + (size_t)inst * cap;
-  int r[MMAX], rmin[MMAX], g[MMAX];
-  int64_t used = 0;
-  bool bad = false, unit = true;
-  uint32_t avail = 0;
-#pragma unroll
-  for (int m = 0; m < MMAX; ++m) {
-    r[m] = 0;
-    rmin[m] = 0;
-    g[m] = 1;
-    if (m < M) {
-      r[m] = b.r0[m];
-      rmin[m] = b.r_min[m];
-      g[m] = b.footprint[m];
-      used += (int64_t)g[m] * r[m];
-      if (r[m] < 0 || rmin[m] < 0 || g[m] < 1) bad = true;
-      if (g[m] != 1) unit = false;
-      if (r[m] > rmin[m]) avail |= 1u << m;
-    }
-  }
-  int64_t free_pool = b.budget - used;
-  if (bad || free_pool < 0) {
-    for (int m = 0; m < M && m < MMAX; ++m) b.r_out[(size_t)inst * M + m] = sel<T, MMAX>(r, m);
-    b.n_moves[inst] = 0;
-    b.diag->err = TRE_EINVAL;
-    continue;
-  }
-  auto emit = [&](int64_t at, int32_t k, int recv, int donor, int kind, int sq) {
-    if (at < cap) mv[at] = tre_move{k, (int16_t)recv, (int16_t)donor, (uint8_t)kind, (uint8_t)sq, 0};
-  };
-  int64_t nm = 0;
-  int u = 0;
-  if (unit) {
-    // unit footprints: a transition is one replica, so a tick moves up to
-    // K_p replicas from the pool, then from donors in order
-    int* scap = s_cap[warp];
-    for (int m = 0; m < M && m < MMAX; ++m) scap[m] = sel<T, MMAX>(r, m) - sel<T, MMAX>(rmin, m);
-    // next-donor rows are masked by `avail` with these halfword lifts, rebuilt
-    // only when `avail` changes
-    uint32_t lw[MMAX / 2];
-    uint32_t lw_for = ~avail;
-    auto next_tick = [&](int uu) -> int {
-      if (free_pool > 0) return sany[uu];
-      if (lw_for != avail) {
-#pragma unroll
-        for (int i = 0; i < MMAX / 2; ++i)
-          lw[i] = ((avail >> (2 * i)) & 1u ? 0u : 0xffffu) |
-                  ((avail >> (2 * i + 1)) & 1u ? 0u : 0xffff0000u);
-        lw_for = avail;
-      }
-      const uint4* q = reinterpret_cast<const uint4*>(snx + (size_t)uu * MMAX);
-      uint32_t acc = 0xffffffffu;
-#pragma unroll
-      for (int h = 0; h < MMAX / 8; ++h) {
-        const uint4 w = q[h];
-        acc = __vminu2(acc, w.x | lw[4 * h]);
-        acc = __vminu2(acc, w.y | lw[4 * h + 1]);
-        acc = __vminu2(acc, w.z | lw[4 * h + 2]);
-        acc = __vminu2(acc, w.w | lw[4 * h + 3]);
-      }
-      return (int)min(acc & 0xffffu, acc >> 16);
-    };
-    if (Kp == 1 && MMAX == 8 && b.budget <= 255) {
-      // as below, with the replicas above the floor packed one byte per model
-      // in a register (a model never holds more than the budget)
-      unsigned long long cp = 0;
-      for (int m = 0; m < M; ++m) cp |= (unsigned long long)scap[m] << (8 * m);
-      int32_t nm1 = 0;
+      // footprints differ: per transition the pool if it covers the receiver's
+      // footprint, else donor replicas until it is covered; an uncoverable
+      // transition releases nothing and ends the tick
       while (true) {
-        const int nxt = next_tick(u);
-        if (nxt >= nf) break;
-        u = nxt + 1;
-        const TickRec tr = srec[nxt];
-        const int32_t k = tick_win(nxt);
-        const int recv = tr.recv;
-        int donor = -1;
-        if (free_pool > 0) {
-          --free_pool;
-        } else {
-          const uint32_t left = avail & tr.dm;
-          const uint32_t tl = ((left & 0xFu) * 0x00204081u) & 0x01010101u;
-          const uint32_t th = (((left >> 4) & 0xFu) * 0x00204081u) & 0x01010101u;
-          const uint32_t pl = (uint32_t)tr.pk;
-          const int nd = __popc(tr.dm);
-          uint32_t f0 = __byte_perm(tl, th, pl & 0xFFFFu);
-          uint32_t f1 = __byte_perm(tl, th, pl >> 16);
-          if (nd < 4) f0 &= (1u << (8 * nd)) - 1u;
-          if (nd < 8) f1 &= nd <= 4 ? 0u : (1u << (8 * (nd - 4))) - 1u;
-          const int j = f0 ? (__ffs(f0) - 1) >> 3 : 4 + ((__ffs(f1) - 1) >> 3);
-          donor = (int)((pl >> (4 * j)) & 15u);
-          cp -= 1ull << (8 * donor);
-          if (((cp >> (8 * donor)) & 0xFFull) == 0) avail &= ~(1u << donor);
+        uint32_t k = my[u * MP] | no[0];
+        if (MPL > 1) k = min(k, my[u * MP + 32] | no[L1]);
+        const int cb = u & ~(kChunk - 1);
+        int t = (int)(__reduce_min_sync(full, k) >> RB);
+        if (pool > 0 && u < n) t = min(t, (int)nexts[u]);
+        if (t >= kChunk) {
+          u = cb + kChunk;
+          if (u >= n) break;
+          continue;
         }
-        put_move(mv, nm1, cap, k, recv, donor, tr.kind, 0);
-        ++nm1;
-        cp += 1ull << (8 * recv);
-        avail |= 1u << recv;
-      }
-      for (int m = 0; m < M; ++m) scap[m] = (int)((cp >> (8 * m)) & 0xFFull);
-      nm = nm1;
-      u = nf;
-    }
-    if (Kp == 1 && MMAX == 16 && b.budget <= 255) {
-      // as above for up to 16 models: the replicas above the floor packed a
-      // byte per model in two registers, and the donor the first model of
-      // the tick's order that can still give (the jump only lands on ticks
-      // that have one when the pool is empty)
-      unsigned long long c0 = 0ull, c1 = 0ull;
-      for (int m = 0; m < M; ++m) {
-        const unsigned long long v = (unsigned long long)scap[m] << (8 * (m & 7));
-        if (m < 8) c0 |= v; else c1 |= v;
-      }
-      int32_t nm1 = 0;
-      while (true) {
-        const int nxt = next_tick(u);
-        if (nxt >= nf) break;
-        u = nxt + 1;
-        const TickRec tr = srec[nxt];
-        const int32_t k = tick_win(nxt);
-        const int recv = tr.recv;
-        int donor = -1;
-        if (free_pool > 0) {
-          --free_pool;
-        } else {
-          const uint32_t left = avail & tr.dm;
-          unsigned long long pk = tr.pk;
-          int d = (int)(pk & 15u);
-          for (int p = 1; p < MMAX && !((left >> d) & 1u); ++p) {
-            pk >>= 4;
-            d = (int)(pk & 15u);
+        const int a = cb + t;
+        const int recv = recs[a] & 63;
+        const int need = __shfl_sync(full, MPL > 1 && recv >= 32 ? g[L1] : g[0], recv & 31);
+        // the donors of this very tick: words of the row at the tick itself
+        const uint32_t r0 = my[a * MP], r1 = MPL > 1 ? my[a * MP + 32] : kNone;
+        const bool don0 = (int)(r0 >> RB) == t, don1 = MPL > 1 && (int)(r1 >> RB) == t;
+        for (int seq = 0; seq < Kp; ++seq) {
+          if (pool >= need) {
+            pool -= need;
+            log_one(lane == 0, (uint32_t)a, seq, 64);
+            receive(recv, 1);
+            continue;
           }
-          donor = d;
-          const int sh = 8 * (d & 7);
-          const unsigned long long c = (d < 8 ? c0 : c1) - (1ull << sh);
-          if (d < 8) c0 = c; else c1 = c;
-          if (((c >> sh) & 0xFFull) == 0) avail &= ~(1u << d);
-        }
-        put_move(mv, nm1, cap, k, recv, donor, tr.kind, 0);
-        ++nm1;
-        if (recv < 8) c0 += 1ull << (8 * recv);
-        else c1 += 1ull << (8 * (recv - 8));
-        avail |= 1u << recv;
-      }
-      for (int m = 0; m < M; ++m)
-        scap[m] = (int)(((m < 8 ? c0 : c1) >> (8 * (m & 7))) & 0xFFull);
-      nm = nm1;
-      u = nf;
-    }
-    if (Kp == 1 && MMAX == 8 && u < nf) {
-      // one transition per tick: every tick the jump lands on moves exactly
-      // one replica (it has a receiver, and a usable donor when the pool is
-      // empty), so the visit is straight-line code
-      int32_t nm1 = 0;
-      while (true) {
-        const int nxt = next_tick(u);
-        if (nxt >= nf) break;
-        u = nxt + 1;
-        const TickRec tr = srec[nxt];
-        const int32_t k = tick_win(nxt);
-        const int recv = tr.recv;
-        int donor = -1;
-        if (free_pool > 0) {
-          --free_pool;
-        } else {
-          const uint32_t left = avail & tr.dm;
-          const uint32_t tl = ((left & 0xFu) * 0x00204081u) & 0x01010101u;
-          const uint32_t th = (((left >> 4) & 0xFu) * 0x00204081u) & 0x01010101u;
-          const uint32_t pl = (uint32_t)tr.pk;
-          const int nd = __popc(tr.dm);
-          uint32_t f0 = __byte_perm(tl, th, pl & 0xFFFFu);
-          uint32_t f1 = __byte_perm(tl, th, pl >> 16);
-          if (nd < 4) f0 &= (1u << (8 * nd)) - 1u;
-          if (nd < 8) f1 &= nd <= 4 ? 0u : (1u << (8 * (nd - 4))) - 1u;
-          const int j = f0 ? (__ffs(f0) - 1) >> 3 : 4 + ((__ffs(f1) - 1) >> 3);
-          donor = (int)((pl >> (4 * j)) & 15u);
-          const int c = scap[donor] - 1;
-          scap[donor] = c;
-          if (c == 0) avail &= ~(1u << donor);
-        }
-        put_move(mv, nm1, cap, k, recv, donor, tr.kind, 0);
-        ++nm1;
-        scap[recv] += 1;
-        avail |= 1u << recv;
-      }
-      nm = nm1;
-      u = nf;
-    }
-    while (u < nf) {
-      const int nxt = next_tick(u);
-      if (nxt >= nf) break;
-      u = nxt;
-      const TickRec tr = srec[u];
-      const int32_t k = tick_win(u);
-      ++u;
-      const int recv = tr.recv;
-      if (recv < 0) continue;
-      uint32_t left = avail & tr.dm;
-      if (free_pool <= 0 && !left) continue;
-      const int kind = tr.kind;
-      const int n_pool = free_pool < Kp ? (int)free_pool : Kp;
-      for (int q = 0; q < n_pool; ++q) put_move(mv, nm + q, cap, k, recv, -1, kind, q);
-      int sq = n_pool;
-      unsigned long long pk = tr.pk;
-      if (MMAX == 8) {
-        // usable donors by position in the order, one flag byte per position:
-        // spread the usable bits to bytes, then gather them by the order's
-        // model nibbles; positions past the tick's donor count are masked
-        const uint32_t tl = ((left & 0xFu) * 0x00204081u) & 0x01010101u;
-        const uint32_t th = (((left >> 4) & 0xFu) * 0x00204081u) & 0x01010101u;
-        const uint32_t pl = (uint32_t)pk;
-        const int nd = __popc(tr.dm);
-        uint32_t f0 = __byte_perm(tl, th, pl & 0xFFFFu);
-        uint32_t f1 = __byte_perm(tl, th, pl >> 16);
-        if (nd < 4) f0 &= (1u << (8 * nd)) - 1u;
-        if (nd < 8) f1 &= nd <= 4 ? 0u : (1u << (8 * (nd - 4))) - 1u;
-        while (sq < Kp && (f0 | f1)) {
-          int j;
-          if (f0) {
-            j = (__ffs(f0) - 1) >> 3;
-            f0 &= ~(0xFFu << (8 * j));
-          } else {
-            const int j1 = (__ffs(f1) - 1) >> 3;
-            f1 &= ~(0xFFu << (8 * j1));
-            j = 4 + j1;
+          int64_t f = pool;
+          const int64_t n0 = n_out + n_log;
+          int h[MPL];
+#pragma unroll
+          for (int j = 0; j < MPL; ++j) h[j] = c[j];
+          while (f < need) {
+            const uint32_t e0 = don0 && h[0] > 0 ? r0 : kNone;
+            const uint32_t e1 = don1 && h[L1] > 0 ? r1 : kNone;
+            const uint32_t best = __reduce_min_sync(full, MPL > 1 ? min(e0, e1) : e0);
+            if (best == kNone) break;
+            const bool d0 = e0 == best, d1 = MPL > 1 && e1 == best;
+            const unsigned gd = d0 ? (unsigned)g[0] : d1 ? (unsigned)g[L1] : 0u;
+            f += __reduce_max_sync(full, gd);
+            h[0] -= d0;
+            if (MPL > 1) h[L1] -= d1;
+            log_one(d0 || d1, (uint32_t)a, seq, lane + (d1 ? 32 : 0));
           }
-          const int m = (int)((pl >> (4 * j)) & 15u);
-          const int c = scap[m];
-          const int take = min(c, Kp - sq);
-          scap[m] = c - take;
-          if (take == c) avail &= ~(1u << m);
-          for (int i = 0; i < take; ++i, ++sq) put_move(mv, nm + sq, cap, k, recv, m, kind, sq);
-        }
-      } else {
-        while (sq < Kp && left) {
-          const int m = (int)(pk & 15);
-          pk >>= 4;
-          if (!(left >> m & 1)) continue;
-          left &= ~(1u << m);
-          const int c = scap[m];
-          const int take = min(c, Kp - sq);
-          scap[m] = c - take;
-          if (take == c) avail &= ~(1u << m);
-          for (int i = 0; i < take; ++i, ++sq) put_move(mv, nm + sq, cap, k, recv, m, kind, sq);
-        }
-      }
-      const int cr = scap[recv] + sq;
-      scap[recv] = cr;
-      if (cr > 0) avail |= 1u << recv;
-      free_pool -= n_pool;
-      nm += sq;
-    }
-    for (int m = 0; m < M && m < MMAX; ++m)
-      b.r_out[(size_t)inst * M + m] = scap[m] + sel<T, MMAX>(rmin, m);
-    b.n_moves[inst] = nm;
-    if (nm > cap) b.diag->err = TRE_EOVERFLOW;
-    continue;
-  }
-  while (u < nf) {
-    // the next tick where something may move
-    int nxt;
-    if (free_pool > 0) nxt = sany[u];
-    else nxt = next_donor_tick<MMAX>(snx + (size_t)u * MMAX, avail);
-    if (nxt >= nf) break;
-    u = nxt;
-    const TickRec tr = srec[u];
-    const int recv = tr.recv;
-    const int kind = tr.kind;
-    const int32_t k = tick_win(u);
-    ++u;
-    if (recv < 0) continue;
-    const uint32_t usable = avail & tr.dm;
-    const int need = unit ? 1 : sel<T, MMAX>(g, recv);
-    if (free_pool < need && !usable) continue;
-    unsigned long long pk = tr.pk;
-    if (unit) {
-      const int n_pool = (int)(free_pool < Kp ? free_pool : Kp);
-      for (int q = 0; q < n_pool; ++q) emit(nm + q, k, recv, -1, kind, q);
-      int sq = n_pool;
-      uint32_t left = usable;
-      while (sq < Kp && left) {
-        const int m = (int)(pk & 15);
-        pk >>= 4;
-        if (!(left >> m & 1)) continue;
-        left &= ~(1u << m);
-        const int c = sel<T, MMAX>(r, m) - sel<T, MMAX>(rmin, m);
-        const int take = min(c, Kp - sq);
-        add_at<T, MMAX>(r, m, -take);
-        if (take == c) avail &= ~(1u << m);
-        for (int i = 0; i < take; ++i, ++sq) emit(nm + sq, k, recv, m, kind, sq);
-      }
-      add_at<T, MMAX>(r, recv, sq);
-      if (sel<T, MMAX>(r, recv) > sel<T, MMAX>(rmin, recv)) avail |= 1u << recv;
-      free_pool -= n_pool;
-      nm += sq;
-      continue;
-    }
-    for (int sq = 0; sq < Kp; ++sq) {
-      if (free_pool >= need) {
-        free_pool -= need;
-        add_at<T, MMAX>(r, recv, 1);
-        if (sel<T, MMAX>(r, recv) > sel<T, MMAX>(rmin, recv)) avail |= 1u << recv;
-        emit(nm++, k, recv, -1, kind, sq);
-        continue;
-      }
-      int64_t f = free_pool;
-      const int64_t nm0 = nm;
-      int taken[MMAX];
+          if (f < need) {                       // take the tentative releases back
+            if (n0 < n_out) {
+              n_out = n0;
+              n_log = 0;
+            } else {
+              n_log = (int)(n0 - n_out);
+            }
+            break;
+          }
 #pragma unroll
-      for (int m = 0; m < MMAX; ++m) taken[m] = 0;
-      unsigned long long order = pk;
-      uint32_t left = avail & tr.dm;
-      while (f < need && left) {
-        const int m = (int)(order & 15);
-        order >>= 4;
-        if (!(left >> m & 1)) continue;
-        left &= ~(1u << m);
-        int c = sel<T, MMAX>(r, m) - sel<T, MMAX>(rmin, m);
-        const int gm = sel<T, MMAX>(g, m);
-        while (f < need && c > 0) {
-          add_at<T, MMAX>(taken, m, 1);
-          --c;
-          f += gm;
-          emit(nm++, k, recv, m, kind, sq);
+          for (int j = 0; j < MPL; ++j) c[j] = h[j];
+          pool = f - need;
+          receive(recv, 1);
         }
+        masks();
+        u = a + 1;
       }
-      if (f < need) {
-        nm = nm0;
-        break;
-      }
-#pragma unroll
-      for (int m = 0; m < MMAX; ++m) {
-        r[m] -= taken[m];
-        if (m < M && !(r[m] > rmin[m])) avail &= ~(1u << m);
-      }
-      add_at<T, MMAX>(r, recv, 1);
-      if (sel<T, MMAX>(r, recv) > sel<T, MMAX>(rmin, recv)) avail |= 1u << recv;
-      free_pool = f - need;
     }
+    flush();
+  };
+
+  int buf = 0;
+  for (int first = 0; first < n_tick; first += w.slab, buf ^= w.n_buf - 1) {
+    const int more = first + w.slab;
+    if (more < n_tick) fetch(more, buf ^ 1);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    __syncthreads();
+    const unsigned char* d = dyn + buf * buf_bytes;
+    const uint8_t* recs = d + (size_t)(w.slab + 1) * MP * 2;
+    if (walks)
+      walk(reinterpret_cast<const uint16_t*>(d), recs, recs + w.slab, min(w.slab, n_tick - first),
+           first);
+    __syncthreads();
   }
-  for (int m = 0; m < M && m < MMAX; ++m) b.r_out[(size_t)inst * M + m] = sel<T, MMAX>(r, m);
-  b.n_moves[inst] = nm;
-  if (nm > cap) b.diag->err = TRE_EOVERFLOW;
+  if (!mine) return;
+#pragma unroll
+  for (int j = 0; j < MPL; ++j) {
+    const int m = lane + 32 * j;
+    if (m < M) w.r_out[(size_t)inst * M + m] = c[j] + rmin[j];
+  }
+  if (lane == 0) {
+    w.n_moves[inst] = n_out;
+    if (bad) w.diag->err = TRE_EINVAL;
+    else if (n_out > cap) w.diag->err = TRE_EOVERFLOW;
   }
 }
 
@@ -1400,73 +1457,75 @@ cudaError_t walk_launch(const WalkBatch<T>& b, WalkWs& w, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-}  // namespace
-
-template <class T> void walk_ws_layout(Arena& a, WalkBatch<T>& b, WalkWs& w) {
-  int64_t total = 0;
-  for (int s = 0; s < b.n_series; ++s) {
-    b.ent_base[s] = (int32_t)total;
-    const int64_t span = (int64_t)b.series_K[s] * b.series_win[s];
-    total += span / b.fast_ms + span / b.slow_ms;
-  }
-  b.ent_base[b.n_series] = (int32_t)total;
-  w.recv = a.take<int16_t>((size_t)std::max<int64_t>(total * b.n_tau, 1));
-  w.n_donor = a.take<int16_t>((size_t)std::max<int64_t>(total * b.n_tau, 1));
-  w.rank = a.take<uint16_t>((size_t)std::max<int64_t>(total * b.n_tau * b.M, 1));
-  w.order = a.take<uint16_t>((size_t)std::max<int64_t>(total * b.n_tau * b.M, 1));
-  w.packed = a.take<unsigned long long>((size_t)std::max<int64_t>(total * b.n_tau, 1));
-  w.dmask = a.take<uint32_t>((size_t)std::max<int64_t>(total * b.n_tau, 1));
-  w.dm64 = a.take<unsigned long long>((size_t)std::max<int64_t>(total * b.n_tau, 1));
+// The lane walk takes nested cadences (every slow tick a fast tick, no fast
+// tick shorter than a window, so a window ends at most one tick) and up to 64
+// models (two per lane; a row word has six rank bits). Elsewhere ticks are
+// visited one by one.
+template <class T> bool lane_walk(const WalkBatch<T>& b) {
+  if (b.M > 64 || b.slow_ms % b.fast_ms != 0) return false;
+  for (int s = 0; s < b.n_series; ++s)
+    if (b.fast_ms < b.series_win[s]) return false;
+  return true;
 }
 
-// unit footprints and few models: thread-per-instance walk with staged tables
-// Whether the jump walk applies (nested cadences, a fast tick not shorter
-// than a window, tick tables within the opt-in shared-memory limit) and its
-// shared memory: the tables, with or without the staged tick windows.
-struct JumpPlan {
-  bool ok, store_win;
-  size_t smem, lim;
-};
-template <class T, int MMAX> JumpPlan jump_plan(const WalkBatch<T>& b) {
-  JumpPlan p{false, false, 0, 0};
-  if (b.slow_ms % b.fast_ms != 0 || b.fast_ms < b.series_win[0]) return p;
-  bool ok = true;
-  size_t jsmem = 0, wsmem = 0;
+int row_models(int M) { return M <= 8 ? 8 : M <= 16 ? 16 : M <= 32 ? 32 : 64; }
+
+template <class T, int MP>
+cudaError_t lane_launch(const WalkBatch<T>& b, const WalkWs& w, cudaStream_t s, int* launches) {
+  const int64_t chunks = (int64_t)b.ent_base[b.n_series] * b.n_tau;
+  if (chunks > 0) {
+    if constexpr (MP <= 16) {
+      // rows start on 16-byte boundaries when M is a multiple of 4 (series
+      // offsets are multiples of M) and both arrays are 16-byte aligned
+      if (b.M % 4 == 0 && (((uintptr_t)b.Z | (uintptr_t)b.cls) & 15) == 0)
+        k_tick_rows<T, MP, true><<<(unsigned)chunks, kChunk, 0, s>>>(b, w.rows, w.recs, w.nexts);
+      else
+        k_tick_rows<T, MP, false><<<(unsigned)chunks, kChunk, 0, s>>>(b, w.rows, w.recs, w.nexts);
+    } else {
+      k_tick_rows_wide<T, MP><<<(unsigned)chunks, kWideThreads, 0, s>>>(b, w.rows, w.recs,
+                                                                        w.nexts);
+    }
+    if (launches) ++*launches;
+  }
+  LaneWalk v;
+  v.M = b.M;
+  v.n_tau = b.n_tau;
+  v.n_cap = b.n_cap;
+  int longest = 0;
   for (int i = 0; i < b.n_series; ++i) {
-    if (b.fast_ms < b.series_win[i]) ok = false;
-    const int64_t nf = (int64_t)b.series_K[i] * b.series_win[i] / b.fast_ms;
-    if (nf >= 32767) ok = false;
-    const size_t need = (size_t)nf * sizeof(TickRec) + (size_t)(nf + 1) * MMAX * 2 +
-                        (size_t)(nf + 1) * 2;
-    jsmem = std::max(jsmem, need);
-    wsmem = std::max(wsmem, (size_t)((nf + 3) & ~3) * 4);
+    v.chunk_base[i] = b.ent_base[i];
+    v.win[i] = b.series_win[i];
+    longest = std::max(longest, (b.ent_base[i + 1] - b.ent_base[i]) * kChunk);
   }
-  // the largest dynamic shared memory a block may opt into, beside the
-  // kernel's static per-warp counts
-  int dev = 0, optin = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
-          cudaSuccess || optin <= 4096) {
-    cudaGetLastError();
-    return p;
-  }
-  p.lim = (size_t)optin - 2048;
-  p.store_win = jsmem + wsmem <= p.lim;
-  p.smem = p.store_win ? jsmem + wsmem : jsmem;
-  p.ok = ok && p.smem <= p.lim;
-  return p;
-}
-
-// The jump walk; RANK: it ranks its own ticks (one launch for the selection).
-template <class T, int MMAX, bool RANK, bool QUAD>
-cudaError_t jump_launch(const WalkBatch<T>& b, const WalkWs& w, const JumpPlan& p,
-                        cudaStream_t s) {
-  cudaError_t e =
-      func_smem_once((const void*)k_walk_jump<T, MMAX, RANK, QUAD>, (int)p.lim, false);
+  v.chunk_base[b.n_series] = b.ent_base[b.n_series];
+  for (int i = 0; i < b.n_cap; ++i) v.cap_list[i] = b.cap_list[i];
+  v.fast_ms = b.fast_ms;
+  v.budget = b.budget;
+  v.moves_cap = b.moves_cap;
+  v.r_min = b.r_min;
+  v.footprint = b.footprint;
+  v.r0 = b.r0;
+  v.r_out = b.r_out;
+  v.moves = b.moves;
+  v.n_moves = b.n_moves;
+  v.diag = b.diag;
+  v.rows = w.rows;
+  v.recs = w.recs;
+  v.nexts = w.nexts;
+  // short series are staged whole; longer ones in two buffers, the next
+  // slab's load behind the walk of this one
+  constexpr int kSlab = MP == 64 ? 768 : 1024;
+  constexpr int kSmem = 2 * slab_bytes<MP>(kSlab);
+  static_assert(kSmem <= 200 * 1024, "two slabs and the logs fit a block's shared memory");
+  static_assert(kSlab < 2048, "a logged tick has 11 bits");
+  v.slab = longest <= kSlab ? std::max(longest, kChunk) : kSlab;
+  v.n_buf = longest <= kSlab ? 1 : 2;
+  cudaError_t e = func_smem_once((const void*)k_walk_lane<MP>, kSmem, false);
   if (e) return e;
-  // eight warps build the tables; the first n_cap of them walk
-  k_walk_jump<T, MMAX, RANK, QUAD><<<b.n_series * b.n_tau, 256, p.smem, s>>>(
-      b, w.recv, w.packed, w.dmask, p.store_win);
+  const dim3 grid((unsigned)(b.n_series * b.n_tau),
+                  (unsigned)((b.n_cap + kLaneThreads / 32 - 1) / (kLaneThreads / 32)));
+  k_walk_lane<MP><<<grid, kLaneThreads, (size_t)slab_bytes<MP>(v.slab) * v.n_buf, s>>>(v);
+  if (launches) ++*launches;
   return cudaGetLastError();
 }
 
@@ -1478,10 +1537,49 @@ cudaError_t walk_thread_launch(const WalkBatch<T>& b, WalkWs& w, size_t smem, cu
   return cudaGetLastError();
 }
 
+}  // namespace
+
+template <class T> void walk_ws_layout(Arena& a, WalkBatch<T>& b, WalkWs& w) {
+  w = WalkWs{};
+  const bool lanes = lane_walk(b);
+  // entries per series: chunks of fast ticks (lane walk), else its fast and
+  // its slow ticks
+  int64_t total = 0;
+  for (int s = 0; s < b.n_series; ++s) {
+    b.ent_base[s] = (int32_t)total;
+    const int64_t span = (int64_t)b.series_K[s] * b.series_win[s];
+    total += lanes ? (span / b.fast_ms + kChunk - 1) / kChunk
+                   : span / b.fast_ms + span / b.slow_ms;
+  }
+  b.ent_base[b.n_series] = (int32_t)total;
+  const size_t ents = (size_t)std::max<int64_t>(total * b.n_tau, 1);
+  if (lanes) {
+    w.rows = a.take<uint16_t>(ents * kChunk * row_models(b.M));
+    w.recs = a.take<uint8_t>(ents * kChunk);
+    w.nexts = a.take<uint8_t>(ents * kChunk);
+    return;
+  }
+  w.recv = a.take<int16_t>(ents);
+  w.n_donor = a.take<int16_t>(ents);
+  w.rank = a.take<uint16_t>(ents * b.M);
+  w.order = a.take<uint16_t>(ents * b.M);
+  w.packed = a.take<unsigned long long>(ents);
+  w.dmask = a.take<uint32_t>(ents);
+  w.dm64 = a.take<unsigned long long>(ents);
+}
+
 template <class T>
 cudaError_t launch_walk(const WalkBatch<T>& b, WalkWs& w, cudaStream_t s, int* launches) {
   if (launches) *launches = 0;
   if (b.n_inst == 0) return cudaSuccess;
+  if (lane_walk(b)) {
+    switch (row_models(b.M)) {
+      case 8: return lane_launch<T, 8>(b, w, s, launches);
+      case 16: return lane_launch<T, 16>(b, w, s, launches);
+      case 32: return lane_launch<T, 32>(b, w, s, launches);
+      default: return lane_launch<T, 64>(b, w, s, launches);
+    }
+  }
   const int64_t ents = (int64_t)b.ent_base[b.n_series] * b.n_tau;
   // which walk runs decides whether the per-model rank tables are needed
   int max_ent = 0;
@@ -1489,45 +1587,25 @@ cudaError_t launch_walk(const WalkBatch<T>& b, WalkWs& w, cudaStream_t s, int* l
     max_ent = std::max(max_ent, b.ent_base[i + 1] - b.ent_base[i]);
   const size_t thread_smem = (size_t)max_ent * (8 + 4 + 2) + 16;
   const bool thread_walk = b.M <= 16 && b.n_cap <= 32 && thread_smem <= kStageMax;
-  // rows start on 16-byte boundaries when M is a multiple of 4 (series
-  // offsets are multiples of M) and both arrays are 16-byte aligned
-  const bool quad = b.M % 4 == 0 && (((uintptr_t)b.Z | (uintptr_t)b.cls) & 15) == 0;
-  JumpPlan jp{false, false, 0, 0};
-  if (thread_walk && ents > 0) jp = b.M <= 8 ? jump_plan<T, 8>(b) : jump_plan<T, 16>(b);
-  // with a CTA per SM or more, the jump walk ranks its own ticks: one launch
-  if (jp.ok && b.n_series * b.n_tau >= device_sm_count()) {
-    if (launches) *launches = 1;
-    if (b.M <= 8)
-      return quad ? jump_launch<T, 8, true, true>(b, w, jp, s)
-                  : jump_launch<T, 8, true, false>(b, w, jp, s);
-    return quad ? jump_launch<T, 16, true, true>(b, w, jp, s)
-                : jump_launch<T, 16, true, false>(b, w, jp, s);
-  }
   // the tick ranking, then the walk
   if (launches) *launches = (ents > 0 ? 1 : 0) + 1;
   if (ents > 0) {
     const unsigned g = (unsigned)((ents + 127) / 128);
-    if (b.M <= 8 && quad) {
-      k_tick_rank_small<T, 8, true><<<g, 128, 0, s>>>(b, w.recv, w.n_donor, w.rank, w.order,
-                                                      w.packed, w.dmask, !thread_walk, w.dm64);
-    } else if (b.M <= 8) {
-      k_tick_rank_small<T, 8, false><<<g, 128, 0, s>>>(b, w.recv, w.n_donor, w.rank, w.order,
-                                                       w.packed, w.dmask, !thread_walk, w.dm64);
+    if (b.M <= 8) {
+      k_tick_rank_small<T, 8><<<g, 128, 0, s>>>(b, w.recv, w.n_donor, w.rank, w.order, w.packed,
+                                                w.dmask, !thread_walk, w.dm64);
     } else if (b.M <= 16) {
-      k_tick_rank_small<T, 16, false><<<g, 128, 0, s>>>(b, w.recv, w.n_donor, w.rank, w.order,
-                                                        w.packed, w.dmask, !thread_walk, w.dm64);
+      k_tick_rank_small<T, 16><<<g, 128, 0, s>>>(b, w.recv, w.n_donor, w.rank, w.order,
+                                                 w.packed, w.dmask, !thread_walk, w.dm64);
     } else if (b.M <= 32) {
-      k_tick_rank_small<T, 32, false><<<g, 128, 0, s>>>(b, w.recv, w.n_donor, w.rank, w.order,
-                                                        w.packed, w.dmask, true, w.dm64);
+      k_tick_rank_small<T, 32><<<g, 128, 0, s>>>(b, w.recv, w.n_donor, w.rank, w.order,
+                                                 w.packed, w.dmask, true, w.dm64);
     } else {
       const int64_t th = ents * b.M;
       k_tick_rank<T><<<(unsigned)((th + 255) / 256), 256, 0, s>>>(b, w.recv, w.n_donor, w.rank,
                                                                    w.order, w.dm64);
     }
   }
-  if (jp.ok)
-    return b.M <= 8 ? jump_launch<T, 8, false, false>(b, w, jp, s)
-                    : jump_launch<T, 16, false, false>(b, w, jp, s);
   if (thread_walk)
     return b.M <= 8 ? walk_thread_launch<T, 8>(b, w, thread_smem, s)
                     : walk_thread_launch<T, 16>(b, w, thread_smem, s);

@@ -1,10 +1,9 @@
 """GPU parity of move selection (Sec. IV-B rescue / rebalance, Eq. 3, Sec. IV-C
 bounded transfer) on every walk variant of the library, against the oracle's
-walk, bit for bit: the warp walk for more than 16 models (shared-memory staged
-tick tables and, for long series or many models, tables read from global
-memory), the per-tick ranking for 17-32 models and beyond, the thread walk
-that visits every tick (cadences that are not nested, or a fast tick shorter
-than a window), and pacing caps above 32 on few models."""
+walk, bit for bit: the lane walk (nested cadences, up to 64 models) at the
+edges of its tick chunks and staged slabs, the warp walk beyond 64 models, the
+walks that visit every tick (cadences that are not nested, or a fast tick
+shorter than a window), and pacing caps above 32 on few models."""
 import numpy as np
 import pytest
 
@@ -62,10 +61,8 @@ def _check(tre, Z, cls, g, r0, budget, r_min, win, cap, fast_ms=5000, slow_ms=10
     return n
 
 
-# 17-32 models: one model per lane, per-tick ranking of up to 32 models;
-# 33-64: two models per lane; 100: four. K = 3000 one-second windows keeps the
-# tick tables in shared memory for up to ~40 models, above that they are read
-# from global memory.
+# 17-32 models: one model per lane; 33-64: two; 100: the warp walk, four per
+# lane, on rank tables in shared memory.
 @pytest.mark.parametrize("M", [17, 24, 32, 33, 40, 48, 64, 100])
 @pytest.mark.parametrize("cap", [1, 3])
 def test_warp_walk_many_models(tre, M, cap):
@@ -182,3 +179,21 @@ def test_warp_walk_cadences(tre, M, fast_ms, slow_ms, win):
     Z, cls, g, r0, budget, r_min = _case(900 + M + fast_ms, 3000, M)
     for cap in (1, 3):
         _check(tre, Z, cls, g, r0, budget, r_min, win, cap, fast_ms, slow_ms)
+
+
+# One tick per window. Ticks are ranked in chunks of 128 and staged 1024 (768
+# for more than 32 models) at a time; row words hold 3 to 6 rank bits for 8,
+# 16, 32 and 64 models. Infinite Z and zeros of both signs (equal, so the lower
+# index goes first) sit among the ties.
+@pytest.mark.parametrize("hetero,cap", [(False, 1), (False, 5), (True, 3)])
+@pytest.mark.parametrize("M,ticks", [(2, 129), (8, 127), (8, 128), (8, 1025), (9, 2200),
+                                     (16, 1024), (17, 129), (32, 1153), (33, 769), (64, 768),
+                                     (64, 1700)])
+def test_lane_walk_chunk_and_slab_edges(tre, M, ticks, hetero, cap):
+    dtype = np.float64 if ticks % 2 else np.float32
+    Z, cls, g, r0, budget, r_min = _case(40 + M + ticks, ticks, M, hetero=hetero, dtype=dtype)
+    rng = np.random.default_rng(M)
+    for v in (np.inf, 0.0, -0.0):
+        Z[rng.random(Z.shape) < 0.04] = v
+    budget += 2
+    _check(tre, Z, cls, g, r0, budget, r_min, 1000, cap, 1000, 2000)
