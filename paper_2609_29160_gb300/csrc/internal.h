@@ -287,19 +287,15 @@ template <class T> struct ReplayBatch {
   const int32_t* slo_ms;           // device [M] or null
   const int32_t* guard_ms;         // device [M] or null: latency guard per model
   // scratch
-  const int32_t* list;             // valid request indices grouped by model
-  const int4* grp;                 // per grouped request: (t_arr, d_first, d_total, index),
-                                   // (L_in, L_out, -, -)
+  const int4* grp;                 // per request, grouped by model in input order: (t_arr,
+                                   // d_first, d_total, index), (L_in, L_out, -, -)
   const int32_t* base;             // [M + 1]
   const int32_t* arr_cnt;          // [K][M] arrivals
   uint32_t* acc;                   // per instance: P, D, ends, late first tokens, [K + 1][M] each
-  long long* gheap;                // per instance [M][hcap] when the heaps are global
+  uint32_t* gsrv;                  // per instance [M][hcap] free times when not in shared memory
   int hcap;
-  int warps_per_cta;
-  int warp_bytes, heap_off;        // shared memory per warp, heap offset in it
-  int act_off, acap;               // decoding-request lists: offset, entries per model
-  int ring_off;                    // per-model window rings and pending far windows
-  int q_off;                       // per-model staged requests
+  int ring_off, srv_off;           // shared memory: window rings, free times
+  int smem_bytes;
   // outputs
   int32_t *o_ts, *o_tf, *o_te;     // [n_inst][n] or null
   T* Z;                            // [n_inst][K][M] or null (with cls)
@@ -313,12 +309,10 @@ template <class T> struct ReplayBatch {
 };
 struct ReplayWs {
   int8_t* vm;
-  int32_t *arr_cnt, *n_valid, *base, *list;
+  int32_t *arr_cnt, *blk_cnt, *base;
   int4* grp;
   uint32_t* acc;
-  long long* gheap;
-  bool shared_heaps;
-  int warps_per_cta;
+  int n_blk;
 };
 // lays out the scratch and fills the batch's shared-memory plan
 template <class T> void replay_ws_layout(Arena& a, ReplayBatch<T>& b, ReplayWs& w);

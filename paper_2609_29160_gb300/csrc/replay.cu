@@ -22,13 +22,22 @@
 //  * a request not started by the end of the grid reports K*win for its
 //    times; an invalid latent record reports -1 and is not served.
 //
-// GPU layout: one warp per controller instance (a rescue threshold and a
-// pacing cap), one lane per model (two for more than 32 models). A lane keeps
-// its model's request cursor, gauge counters and smoothing state in
-// registers and its servers as a binary min-heap of free times (shared memory
-// when the instance's heaps fit, else the workspace). Tokens are attributed to
-// future windows in per-instance accumulators; lane 0 runs the controller on
-// control ticks from the window's Z and regions staged in shared memory.
+// GPU layout: one CTA per controller instance (a rescue threshold and a pacing
+// cap). The servers only change on control ticks, so between two ticks the
+// models are independent of each other: each warp takes a model's windows up to
+// the next tick (at most 32 of them, one per lane) and
+//   1. starts its requests in order. Only this is serial: a start takes the
+//      server that frees first, a warp-wide minimum over free times held one
+//      per lane (two or four for more servers);
+//   2. attributes the started requests, one per lane, to the windows of a ring
+//      in shared memory (windows beyond it in the workspace);
+//   3. scores the windows, one per lane, with the smoothing chain passed from
+//      lane to lane.
+// On a tick one warp runs the controller with the models on its lanes. What
+// bounds a replay is the start chain of its busiest model, some 250 cycles a
+// start. 160,000 requests of 8 models over 600 windows, 64 instances: 7.7 ms; a
+// warp per instance with a lane per model (heaps of free times, attribution
+// inside the start loop) took 78.3, 2,700 cycles a start.
 #include <algorithm>
 
 #include "common.cuh"
@@ -37,76 +46,88 @@
 namespace tre {
 namespace {
 
-constexpr int kFillThreads = 1024;
+constexpr unsigned kFull = 0xffffffffu;
 
 // ---- latent records grouped by model, input order kept ----------------------
-// valid model id per record (-1 when the record is not served) and arrivals
-// per (window, model)
-__global__ void k_rp_valid(ReplayLatent lat, int M, int win, int K, int8_t* __restrict__ vm,
-                           int32_t* __restrict__ arr_cnt, int32_t* __restrict__ n_valid) {
-  const int64_t span = (int64_t)K * win;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < lat.n;
-       i += (int64_t)gridDim.x * blockDim.x) {
+// One CTA per kGroupBlock records: valid model id per record (-1 when the record
+// is not served), arrivals per (window, model), valid records per (block, model).
+constexpr int kGroupBlock = 1024;
+__global__ void __launch_bounds__(kGroupBlock)
+k_rp_valid(ReplayLatent lat, int M, FastDiv fwin, int64_t span, int8_t* __restrict__ vm,
+           int32_t* __restrict__ arr_cnt, int32_t* __restrict__ blk_cnt) {
+  __shared__ int32_t cnt[64];
+  if (threadIdx.x < M) cnt[threadIdx.x] = 0;
+  __syncthreads();
+  const int64_t i = (int64_t)blockIdx.x * kGroupBlock + threadIdx.x;
+  if (i < lat.n) {
     const int m = lat.model[i];
-    const int64_t ta = lat.t_arr[i];
-    bool ok = m >= 0 && m < M && ta >= 0 && ta < span;
-    ok = ok && lat.d_first[i] >= 0 && lat.d_total[i] >= lat.d_first[i] && lat.L_in[i] >= 0 &&
-         lat.L_out[i] >= 1;
+    const int ta = lat.t_arr[i], df = lat.d_first[i];
+    const bool ok = m >= 0 && m < M && ta >= 0 && ta < span && df >= 0 && lat.d_total[i] >= df &&
+                    lat.L_in[i] >= 0 && lat.L_out[i] >= 1;
     vm[i] = ok ? (int8_t)m : (int8_t)-1;
     if (ok) {
-      atomicAdd(&arr_cnt[(ta / win) * M + m], 1);
-      atomicAdd(&n_valid[m], 1);
+      atomicAdd(&arr_cnt[(size_t)fwin.div((uint32_t)ta) * M + m], 1);
+      atomicAdd(&cnt[m], 1);
     }
-  }
-}
-
-// one CTA per model: the model's record indices in input order
-__global__ void __launch_bounds__(kFillThreads)
-k_rp_fill(int64_t n, int M, const int8_t* __restrict__ vm, const int32_t* __restrict__ n_valid,
-          int32_t* __restrict__ list, int32_t* __restrict__ base_out) {
-  __shared__ int32_t wcnt[kFillThreads / 32];
-  __shared__ int32_t s_base;
-  const int m = blockIdx.x;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (threadIdx.x == 0) {
-    int32_t b = 0;
-    for (int j = 0; j < m; ++j) b += n_valid[j];
-    s_base = b;
-    base_out[m] = b;
-    if (m == M - 1) base_out[M] = b + n_valid[m];
   }
   __syncthreads();
-  int32_t base = s_base;
-  for (int64_t i0 = 0; i0 < n; i0 += kFillThreads) {
-    const int64_t i = i0 + threadIdx.x;
-    const bool f = i < n && vm[i] == m;
-    const unsigned b = __ballot_sync(0xffffffffu, f);
-    if (lane == 0) wcnt[wid] = __popc(b);
-    __syncthreads();
-    int32_t before = 0, total = 0;
-    for (int w = 0; w < kFillThreads / 32; ++w) {
-      const int32_t c = wcnt[w];
-      before += w < wid ? c : 0;
-      total += c;
+  if (threadIdx.x < M) blk_cnt[(size_t)blockIdx.x * M + threadIdx.x] = cnt[threadIdx.x];
+}
+
+// one warp per model (warp w takes models w, w + 32, ...): exclusive prefix of
+// its block counts, then the models' offsets in the grouped order
+__global__ void __launch_bounds__(1024)
+k_rp_offsets(int M, int n_blk, int32_t* __restrict__ blk_cnt, int32_t* __restrict__ base) {
+  __shared__ int32_t total[64];
+  const int lane = threadIdx.x & 31;
+  for (int m = threadIdx.x >> 5; m < M; m += 32) {
+    int32_t run = 0;
+    for (int b0 = 0; b0 < n_blk; b0 += 32) {
+      const int b = b0 + lane;
+      const int32_t v = b < n_blk ? blk_cnt[(size_t)b * M + m] : 0;
+      int32_t inc = v;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int32_t x = __shfl_up_sync(kFull, inc, o);
+        if (lane >= o) inc += x;
+      }
+      if (b < n_blk) blk_cnt[(size_t)b * M + m] = run + inc - v;
+      run += __shfl_sync(kFull, inc, 31);
     }
-    if (f) list[base + before + __popc(b & ((1u << lane) - 1u))] = (int32_t)i;
-    base += total;
-    __syncthreads();
+    if (lane == 0) total[m] = run;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int32_t b = 0;
+    for (int m = 0; m < M; ++m) {
+      base[m] = b;
+      b += total[m];
+    }
+    base[M] = b;
   }
 }
 
 // the model-grouped columns a lane walks: arrival, time to first and last
-// token, prompt and output lengths, in the grouped order
-__global__ void k_rp_gather(int64_t n_valid_total, ReplayLatent lat,
-                            const int32_t* __restrict__ list, const int32_t* __restrict__ base,
-                            int M, int4* __restrict__ g) {
-  const int64_t n = base[M];
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
-       p += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t i = list[p];
-    g[2 * p] = make_int4(lat.t_arr[i], lat.d_first[i], lat.d_total[i], i);
-    g[2 * p + 1] = make_int4(lat.L_in[i], lat.L_out[i], 0, 0);
-  }
+// token, index; prompt and output lengths. A record's place among its model's
+// records of the block is counted within the warp and over the warps before it.
+__global__ void __launch_bounds__(kGroupBlock)
+k_rp_group(ReplayLatent lat, int M, const int8_t* __restrict__ vm,
+           const int32_t* __restrict__ blk_off, const int32_t* __restrict__ base,
+           int4* __restrict__ g) {
+  __shared__ int32_t wcnt[kGroupBlock / 32][64];
+  const int64_t i = (int64_t)blockIdx.x * kGroupBlock + threadIdx.x;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int c = threadIdx.x; c < (kGroupBlock / 32) * 64; c += kGroupBlock) wcnt[c >> 6][c & 63] = 0;
+  __syncthreads();
+  const int m = i < lat.n ? vm[i] : -1;
+  const unsigned same = __match_any_sync(kFull, m);
+  const int before = __popc(same & ((1u << lane) - 1u));
+  if (m >= 0 && before == 0) wcnt[wid][m] = __popc(same);
+  __syncthreads();
+  if (m < 0) return;
+  int32_t p = base[m] + blk_off[(size_t)blockIdx.x * M + m] + before;
+  for (int w = 0; w < wid; ++w) p += wcnt[w][m];
+  g[2 * (size_t)p] = make_int4(lat.t_arr[i], lat.d_first[i], lat.d_total[i], (int32_t)i);
+  g[2 * (size_t)p + 1] = make_int4(lat.L_in[i], lat.L_out[i], 0, 0);
 }
 
 // served records start as "not started" (K*win) or "not served" (-1)
@@ -122,436 +143,493 @@ __global__ void k_rp_init_records(int64_t n, int n_inst, int32_t span, const int
   }
 }
 
-// ---- per-model server heaps -----------------------------------------------
-struct Heap {
-  long long* h;
+// ---- the replay ------------------------------------------------------------
+// Per-model window ring (power of two) and the counts a window collects. A
+// segment is at most 32 windows, so a ring of 64 holds every window a request
+// started in the segment can reach within 32 windows of its end.
+constexpr int kRing = 64;
+enum { kP = 0, kD = 1, kEnd = 2, kLate = 3, kStart = 4, kCounts = 5 };
+constexpr int kFarCounts = 4;        // a start is never beyond its own segment
+constexpr int kMaxWarps = 16;        // models of an instance take turns beyond this
+// a server's free time as an unsigned 32-bit millisecond; later ones (wake and
+// sleep delays near 2^31) are kept at kNever, past the end of every grid
+constexpr uint32_t kNever = 0xfffffffeu, kNoServer = 0xffffffffu;
+
+__device__ __forceinline__ uint32_t free_at(long long t) {
+  return t < (long long)kNever ? (uint32_t)t : kNever;
+}
+
+// first window at or after k that ends a tick of cadence c (a multiple of c
+// falls in (k*win, (k+1)*win]): the window of the next multiple above k*win
+__device__ __forceinline__ int next_tick(int k, uint32_t win, uint32_t c) {
+  const unsigned long long t = ((unsigned long long)k * win / c + 1) * c;
+  const unsigned long long w = (t + win - 1) / win - 1;
+  return w < 0x7fffffffull ? (int)w : 0x7fffffff;
+}
+
+__device__ __forceinline__ uint32_t key_order(float z) {
+  const uint32_t u = __float_as_uint(z);
+  return u == 0x80000000u ? 0x80000000u : u ^ ((u >> 31) ? 0xffffffffu : 0x80000000u);
+}
+__device__ __forceinline__ unsigned long long key_order(double z) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(z);
+  return u == 0x8000000000000000ull ? u : u ^ ((u >> 63) ? ~0ull : 0x8000000000000000ull);
+}
+
+// Lowest (MAX: highest) value among the lanes of `elig`, -1 when there is none,
+// as an ascending scan finds it: the first lane of equal ones; a NaN only when
+// it is the first eligible one.
+template <bool MAX, class T>
+__device__ __forceinline__ int best_lane(unsigned elig, T z) {
+  if (!elig) return -1;
+  const unsigned num = elig & ~__ballot_sync(kFull, z != z);
+  const int first = __ffs(elig) - 1;
+  if (!(num >> first & 1u)) return first;
+  const int lane = threadIdx.x & 31;
+  const auto key = MAX ? ~key_order(z) : key_order(z);
+  bool in = num >> lane & 1u;
+  if (sizeof(T) == 8) {
+    const uint32_t hi = (uint32_t)((unsigned long long)key >> 32);
+    const uint32_t mh = __reduce_min_sync(kFull, in ? hi : 0xffffffffu);
+    in = in && hi == mh;
+  }
+  const uint32_t lo = (uint32_t)key;
+  const uint32_t ml = __reduce_min_sync(kFull, in ? lo : 0xffffffffu);
+  return __ffs(__ballot_sync(kFull, in && lo == ml)) - 1;
+}
+
+// The same over up to 64 models, two per lane (z[0] models 0-31, z[1] 32-63)
+template <bool MAX, class T>
+__device__ __forceinline__ int best_model(const unsigned (&elig)[2], const T (&z)[2]) {
+  const int a = best_lane<MAX>(elig[0], z[0]);
+  const int c = best_lane<MAX>(elig[1], z[1]);
+  if (a < 0) return c < 0 ? -1 : 32 + c;
+  if (c < 0) return a;
+  const T za = __shfl_sync(kFull, z[0], a), zc = __shfl_sync(kFull, z[1], c);
+  // a NaN first in the upper half stays out when the lower half has a model
+  if (zc == zc) return (MAX ? zc > za : zc < za) ? 32 + c : a;
+  const unsigned num = elig[1] & ~__ballot_sync(kFull, z[1] != z[1]);
+  const int c2 = best_lane<MAX>(num, z[1]);
+  if (c2 < 0) return a;
+  const T z2 = __shfl_sync(kFull, z[1], c2);
+  return (MAX ? z2 > za : z2 < za) ? 32 + c2 : a;
+}
+
+// A model's servers in shared memory (or the workspace), unordered; the warp
+// finds the one that frees first.
+struct Servers {
+  uint32_t* v;
   int n;
-  __device__ void sift_down(int i) {
-    const long long v = h[i];
-    for (;;) {
-      int c = 2 * i + 1;
-      if (c >= n) break;
-      if (c + 1 < n && h[c + 1] < h[c]) ++c;
-      if (h[c] >= v) break;
-      h[i] = h[c];
-      i = c;
-    }
-    h[i] = v;
-  }
-  __device__ void replace_top(long long v) {
-    h[0] = v;
-    sift_down(0);
-  }
-  __device__ void pop() {
-    --n;
-    if (n > 0) {
-      h[0] = h[n];
-      sift_down(0);
-    }
-  }
-  __device__ void push(long long v) {
-    int i = n++;
-    while (i > 0) {
-      const int p = (i - 1) >> 1;
-      if (h[p] <= v) break;
-      h[i] = h[p];
-      i = p;
-    }
-    h[i] = v;
+  __device__ __forceinline__ uint32_t first(int& at) const {
+    const int lane = threadIdx.x & 31;
+    uint32_t best = kNoServer;
+    int i = -1;
+    for (int q = lane; q < n; q += 32)
+      if (v[q] < best) {
+        best = v[q];
+        i = q;
+      }
+    const uint32_t f = __reduce_min_sync(kFull, best);
+    const int src = __ffs(__ballot_sync(kFull, best == f)) - 1;
+    at = __shfl_sync(kFull, i, src);
+    return f;
   }
 };
 
-// tokens emitted strictly before tick t by a request with first token at tf,
-// last at te and L output tokens (token j at tf + floor(j*(te-tf)/(L-1)))
-__device__ __forceinline__ long long tokens_before(long long t, long long tf, long long te,
-                                                   long long L) {
-  if (t <= tf) return 0;
-  if (t > te) return L;
-  if (L == 1) return 1;
-  const unsigned long long num = (unsigned long long)(t - tf) * (unsigned long long)(L - 1);
-  const unsigned long long dur = (unsigned long long)(te - tf);
-  const unsigned long long y = num + dur - 1;
-  if ((y >> 32) == 0) return (long long)((uint32_t)y / (uint32_t)dur);   // 32-bit divide
-  return (long long)(y / dur);
+// what a model carries from segment to segment
+template <class T> struct ModelState {
+  int32_t head, end;
+  uint32_t arrived, started, ended;   // running totals (differences are exact modulo 2^32)
+  int32_t far_hi;                     // last window with counts in the workspace
+  int32_t init;
+  unsigned long long met;
+  T S;
+};
+
+// Starts a model's requests in order until one cannot start before t_end, its
+// free times in registers, R per lane. Calls `done(st, c0, c1)` with the lanes'
+// started requests, up to 32 at a time (st = kNoServer: none).
+template <int R, class F>
+__device__ __forceinline__ void start_requests(uint32_t* sv, int n, const int4* __restrict__ grp,
+                                               int& head, int end, uint32_t t_end, F&& done) {
+  const int lane = threadIdx.x & 31;
+  uint32_t s[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) s[r] = lane + 32 * r < n ? sv[lane + 32 * r] : kNoServer;
+  auto fetch = [&](int p, int4& a, int4& c) {
+    if (p < end) {
+      a = __ldg(&grp[2 * (size_t)p]);
+      c = __ldg(&grp[2 * (size_t)p + 1]);
+    }
+  };
+  int4 c0 = make_int4(0, 0, 0, 0), c1 = c0, n0 = c0, n1 = c0;
+  fetch(head + lane, c0, c1);
+  bool more = head < end;
+  while (more) {
+    fetch(head + 32 + lane, n0, n1);               // the next 32, behind this batch's chain
+    const int cnt = min(32, end - head);
+    uint32_t mine = kNoServer;
+    int j = 0;
+    for (; j < cnt; ++j) {
+      const uint32_t ta = (uint32_t)__shfl_sync(kFull, c0.x, j);
+      const uint32_t dt = (uint32_t)__shfl_sync(kFull, c0.z, j);
+      uint32_t low = s[0];
+#pragma unroll
+      for (int r = 1; r < R; ++r) low = min(low, s[r]);
+      const uint32_t f = __reduce_min_sync(kFull, low);
+      const uint32_t st = max(ta, f);
+      if (st >= t_end) break;
+      const int src = __ffs(__ballot_sync(kFull, low == f)) - 1;
+      if (lane == src) {
+        bool put = false;
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          if (!put && s[r] == f) {
+            s[r] = min(st + dt, kNever);
+            put = true;
+          }
+      }
+      if (lane == j) mine = st;
+    }
+    head += j;
+    if (j > 0) done(mine, c0, c1);
+    more = j == 32 && head < end;
+    c0 = n0;
+    c1 = n1;
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+    if (lane + 32 * r < n) sv[lane + 32 * r] = s[r];
 }
 
-// A request still emitting decode tokens after its first-token window: the
-// window from which it contributes, its last window (within the grid), its
-// last token time, output length and tokens counted so far. With
-// y = (T - tf)(L - 1) + dur - 1 the tokens before T are floor(y / dur) while
-// T <= te; moving T one window on adds win * (L - 1) = qd * dur + rd to y, so
-// the count is carried as a quotient and remainder without dividing.
-struct Decoding {
-  int32_t k_from, k_last, te, L, done;
-  int32_t q, r;            // floor and remainder of y / dur at T = k_from * win
-  int32_t qd, rd, dur;
-};
-// per-model window ring (power of two) and pending far-window list sizes; the
-// four counts a window collects
-constexpr int kRing = 64, kFar = 32, kQ = 32;
-enum { kP = 0, kD = 1, kEnd = 2, kLate = 3 };
-
-// window k ends a tick of cadence c when a multiple of c falls in (k*win, (k+1)*win]
-__device__ __forceinline__ bool ends_tick(long long k, int win, int c) {
-  return ((k + 1) * (long long)win) / c > (k * (long long)win) / c;
+// the same with the free times left in memory, for more servers than four per lane
+template <class F>
+__device__ __forceinline__ void start_requests_mem(uint32_t* sv, int n,
+                                                   const int4* __restrict__ grp, int& head,
+                                                   int end, uint32_t t_end, F&& done) {
+  const int lane = threadIdx.x & 31;
+  bool more = head < end;
+  while (more) {
+    int4 c0 = make_int4(0, 0, 0, 0), c1 = c0;
+    if (head + lane < end) {
+      c0 = __ldg(&grp[2 * (size_t)(head + lane)]);
+      c1 = __ldg(&grp[2 * (size_t)(head + lane) + 1]);
+    }
+    const int cnt = min(32, end - head);
+    uint32_t mine = kNoServer;
+    int j = 0;
+    for (; j < cnt; ++j) {
+      const uint32_t ta = (uint32_t)__shfl_sync(kFull, c0.x, j);
+      const uint32_t dt = (uint32_t)__shfl_sync(kFull, c0.z, j);
+      int at;
+      const uint32_t st = max(ta, Servers{sv, n}.first(at));
+      if (st >= t_end) break;
+      __syncwarp();
+      if (lane == 0) sv[at] = min(st + dt, kNever);
+      __syncwarp();
+      if (lane == j) mine = st;
+    }
+    head += j;
+    if (j > 0) done(mine, c0, c1);
+    more = j == 32 && head < end;
+  }
 }
 
-template <class T> struct Ctl {
-  const ReplayBatch<T>& b;
-  const T* z;
-  const uint8_t* c;
-  const uint8_t* flag;   // bit 0: latency guard breached in the window; bit 1: lost capacity
-  int32_t* r;
-  T tc;            // the instance's rescue threshold (NaN: per model from the profile)
-  __device__ T tcrit(int m) const { return tc == tc ? tc : b.tau_crit[m]; }
-  __device__ uint8_t region(int m) const {
-    if (c[m] == TRE_IDLE) return TRE_IDLE;
-    if (z[m] < tcrit(m)) return TRE_CRIT;
-    if (z[m] > b.tau_surp[m]) return TRE_SURP;
-    return TRE_NOM;
+__device__ __forceinline__ uint32_t warp_scan(uint32_t v) {
+  const int lane = threadIdx.x & 31;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t x = __shfl_up_sync(kFull, v, o);
+    if (lane >= o) v += x;
   }
-  __device__ bool held(int m) const { return flag[m] & 1; }
-  // donor preference: idle models (lowest index), then surplus by Z
-  // descending, then nominal by Z descending (with nom_above only above the
-  // receiver's Z); never critical, never the receiver, never below the floor,
-  // never a donor whose latency guard is breached (its release is deferred)
-  __device__ int pick(const int32_t* rr, int recv, bool nom_above) const {
-    const int M = b.M;
-    for (int m = 0; m < M; ++m)
-      if (m != recv && region(m) == TRE_IDLE && rr[m] > b.r_min[m] && !held(m)) return m;
-    int best = -1;
-    for (int m = 0; m < M; ++m)
-      if (m != recv && region(m) == TRE_SURP && rr[m] > b.r_min[m] && !held(m) &&
-          (best < 0 || z[m] > z[best]))
-        best = m;
-    if (best >= 0) return best;
-    for (int m = 0; m < M; ++m) {
-      if (m == recv || region(m) != TRE_NOM || rr[m] <= b.r_min[m] || held(m)) continue;
-      if (nom_above && !(z[m] > z[recv])) continue;
-      if (best < 0 || z[m] > z[best]) best = m;
-    }
-    return best;
-  }
-};
+  return v;
+}
 
-template <class T, int MPL, bool SHEAP>
-__global__ void __launch_bounds__(256, 1)
+template <class T>
+__global__ void __launch_bounds__(32 * kMaxWarps)
 k_replay(const __grid_constant__ ReplayBatch<T> b) {
-  extern __shared__ unsigned long long rsm[];
+  extern __shared__ __align__(16) unsigned char rsm[];
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int inst = blockIdx.x * b.warps_per_cta + wid;
-  if (inst >= b.n_inst) return;                 // whole warps only
-  const int M = b.M, win = b.win, K = b.K;
-  const long long span = (long long)K * win;
-  // this warp's shared region: Z row, class row, replicas, dry-run replicas,
-  // heap sizes, then (shared heaps) the heaps
-  char* base = reinterpret_cast<char*>(rsm) + (size_t)wid * b.warp_bytes;
-  T* zrow = reinterpret_cast<T*>(base);
-  int32_t* r = reinterpret_cast<int32_t*>(zrow + M);
-  int32_t* rr = r + M;
-  int32_t* hs = rr + M;
-  uint8_t* crow = reinterpret_cast<uint8_t*>(hs + M);
-  uint8_t* frow = crow + M;                     // guard / lost-capacity flags
-  long long* heaps = SHEAP ? reinterpret_cast<long long*>(base + b.heap_off)
-                           : b.gheap + (size_t)inst * M * b.hcap;
-  // per model, the requests still decoding past their first-token window
-  Decoding* act = reinterpret_cast<Decoding*>(base + b.act_off);
+  const int n_warps = blockDim.x >> 5;
+  const int inst = blockIdx.x;
+  const int M = b.M, K = b.K;
+  const uint32_t win = (uint32_t)b.win;
+  const FastDiv fwin(win);
+  const uint32_t span = (uint32_t)K * win;
+  // shared memory: model states, Z row, replicas, server counts, class and flag
+  // rows, rings, free times (when they fit)
+  ModelState<T>* st_m = reinterpret_cast<ModelState<T>*>(rsm);
+  T* zrow = reinterpret_cast<T*>(st_m + M);
+  int32_t* rep = reinterpret_cast<int32_t*>(zrow + M);
+  int32_t* n_srv = rep + M;
+  uint8_t* crow = reinterpret_cast<uint8_t*>(n_srv + M);
+  uint8_t* frow = crow + M;                     // bit 0: guard breached; bit 1: lost capacity
+  uint32_t* ring = reinterpret_cast<uint32_t*>(rsm + b.ring_off);    // [kCounts][M][kRing]
+  uint32_t* srv = b.gsrv ? b.gsrv + (size_t)inst * M * b.hcap
+                         : reinterpret_cast<uint32_t*>(rsm + b.srv_off);   // [M][hcap]
   const int ti = inst / b.n_cap, ci = inst % b.n_cap;
   const int pacing = b.cap_list[ci];
-  const T tc = b.n_tau > 0 ? b.tau_list[ti] : (T)NAN;
-  // per-window prompt tokens, decode tokens, running-span ends and late first
-  // tokens beyond the ring, [4][K + 1][M]
-  uint32_t* Gacc = b.acc + (size_t)inst * 4 * (K + 1) * M;
-  uint32_t* ring = reinterpret_cast<uint32_t*>(base + b.ring_off);   // [4][M][kRing]
-  int32_t* farl = reinterpret_cast<int32_t*>(ring + (size_t)4 * M * kRing);  // [M][kFar]
-  // each model's next requests, staged from the grouped columns: grouped
-  // positions [qend - kQ, qend) sit in slot position % kQ; qhead mirrors the
-  // owning lane's cursor for the refill
-  int4* qbuf = reinterpret_cast<int4*>(base + b.q_off);              // [M][kQ][2]
-  int32_t* qhead = reinterpret_cast<int32_t*>(qbuf + (size_t)M * kQ * 2);
-  int32_t* qend = qhead + M;
-  for (int c = lane; c < 4 * M * kRing; c += 32) ring[c] = 0;
-  // initial replicas: one server free at t = 0 per replica
+  // later windows' prompt tokens, decode tokens, running-span ends and late
+  // first tokens, [4][K + 1][M]
+  uint32_t* far = b.acc + (size_t)inst * kFarCounts * (K + 1) * M;
+  const size_t far_arr = (size_t)(K + 1) * M;
+  for (int c = threadIdx.x; c < kCounts * M * kRing; c += blockDim.x) ring[c] = 0;
+  for (int m = threadIdx.x; m < M; m += blockDim.x) {
+    ModelState<T>& s = st_m[m];
+    s.head = b.base[m];
+    s.end = b.base[m + 1];
+    s.arrived = s.started = s.ended = 0;
+    s.far_hi = -1;
+    s.init = 0;
+    s.met = 0;
+    s.S = (T)0;
+    rep[m] = b.r0[m];
+    n_srv[m] = max(b.r0[m], 0);
+  }
+  // initial replicas; every warp forms the sum itself
   long long used = 0;
   bool bad = false;
-  for (int j = 0; j < MPL; ++j) {
-    const int m = lane + 32 * j;
-    if (m >= M) continue;
+  for (int m = lane; m < M; m += 32) {
     const int32_t r0 = b.r0[m], g = b.footprint[m];
     bad |= r0 < 0 || g < 1 || b.r_min[m] < 0;
     used += (long long)g * r0;
-    r[m] = r0;
-    hs[m] = r0;
   }
-  for (int o = 16; o > 0; o >>= 1) used += __shfl_xor_sync(0xffffffffu, used, o);
-  bad = __any_sync(0xffffffffu, bad) || used > b.budget;
-  if (bad) {
-    if (lane == 0) {
+  for (int o = 16; o > 0; o >>= 1) used += __shfl_xor_sync(kFull, used, o);
+  if (__any_sync(kFull, bad) || used > b.budget) {
+    if (threadIdx.x == 0) {
       b.diag->err = TRE_EINVAL;
       b.n_moves[inst] = 0;
     }
     return;
   }
-  for (int j = 0; j < MPL; ++j) {
-    const int m = lane + 32 * j;
-    if (m >= M) continue;
-    for (int q = 0; q < r[m]; ++q) heaps[(size_t)m * b.hcap + q] = 0;
-  }
-  // per-model state of this lane
-  int32_t head[MPL], end[MPL], n_act[MPL], n_far[MPL];
-  bool far_all[MPL];
-  uint32_t arr_next[MPL];
-  T pw[MPL], pq[MPL], pa[MPL], pth[MPL], ptc[MPL], pts[MPL];   // the profile, per model
-  long long cum_arr[MPL], cum_start[MPL], cum_end[MPL], met[MPL];
-  T S[MPL];
-  bool init[MPL];
-  const T dt = (T)win / (T)1000;
-  for (int j = 0; j < MPL; ++j) {
-    const int m = lane + 32 * j;
-    head[j] = m < M ? b.base[m] : 0;
-    end[j] = m < M ? b.base[m + 1] : 0;
-    n_act[j] = 0;
-    n_far[j] = 0;
-    far_all[j] = false;
-    arr_next[j] = m < M && K > 0 ? (uint32_t)b.arr_cnt[m] : 0u;
-    if (m < M) {
-      pw[j] = b.w_p[m];
-      pq[j] = b.w_q[m];
-      pa[j] = b.alpha[m];
-      pth[j] = b.theta[m];
-      ptc[j] = tc == tc ? tc : b.tau_crit[m];
-      pts[j] = b.tau_surp[m];
-    }
-    if (m < M) {
-      qhead[m] = head[j];
-      qend[m] = head[j];
-    }
-    cum_arr[j] = cum_start[j] = cum_end[j] = met[j] = 0;
-    S[j] = (T)0;
-    init[j] = false;
-  }
-  long long free_pool = b.budget - used;        // lane 0's copy is the live one
-  long long reb_until = 0;                      // a rebalance transfer serves from here on
+  __syncthreads();
+  // one server free at t = 0 per replica
+  for (int m = wid; m < M; m += n_warps)
+    for (int q = lane; q < n_srv[m]; q += 32) srv[(size_t)m * b.hcap + q] = 0;
+  // the controller's state (the first warp's copy is the live one)
+  long long pool = b.budget - used, reb_until = 0;
   int64_t nm = 0;
-  __syncwarp();
-  for (int k = 0; k < K; ++k) {
-    const long long Tk = (long long)(k + 1) * win;
-    // top up the staged requests of every model that has used half of them:
-    // the warp loads up to kQ of a model's next requests at once
-    for (int j = 0; j < MPL; ++j) {
-      const int m = lane + 32 * j;
-      const bool want = m < M && qend[m] < end[j] && qend[m] - head[j] < kQ / 2 &&
-                        head[j] < end[j];
-      unsigned need = __ballot_sync(0xffffffffu, want);
-      while (need) {
-        const int l = __ffs(need) - 1;
-        need &= need - 1;
-        const int mm = l + 32 * j;
-        const int h = __shfl_sync(0xffffffffu, head[j], l);
-        const int ne = __shfl_sync(0xffffffffu, end[j], l);
-        const int e = max(qend[mm], h);          // the owner may have read past them
-        const int upto = min(h + kQ, ne);
-        const int p = e + lane;
-        if (p < upto) {
-          int4* slot = qbuf + ((size_t)mm * kQ + (p & (kQ - 1))) * 2;
-          slot[0] = b.grp[2 * (size_t)p];
-          slot[1] = b.grp[2 * (size_t)p + 1];
+  const T dt = div_rn(from_i32<T>(b.win), (T)1000);
+  __syncthreads();
+
+  for (int k0 = 0; k0 < K;) {
+    // the segment: windows k0 .. k1, up to the next tick, at most 32
+    const int tick = min(next_tick(k0, win, (uint32_t)b.fast_ms),
+                         next_tick(k0, win, (uint32_t)b.slow_ms));
+    const int k1 = min(min(tick, k0 + 31), K - 1);
+    const int n_win = k1 - k0 + 1;
+    const uint32_t t_end = (uint32_t)(k1 + 1) * win;
+    for (int m = wid; m < M; m += n_warps) {
+      ModelState<T>& s = st_m[m];
+      uint32_t* my_ring = ring + (size_t)m * kRing;
+      const int n = n_srv[m];
+      int head = s.head;
+      const int end = s.end, head0 = head;
+      int far_hi = -1;
+      unsigned met = 0;
+      int k_now = k0;                           // the window the last start was processed in
+      const long long slo = b.slo_ms ? (long long)b.slo_ms[m] : -1;
+      const long long guard = b.guard_ms ? (long long)b.guard_ms[m] : 0;
+      auto add = [&](int arr, int kt, uint32_t v) {
+        if (kt - k0 < kRing) {
+          atomicAdd(&my_ring[(size_t)arr * M * kRing + (kt & (kRing - 1))], v);
+        } else {
+          atomicAdd(&far[arr * far_arr + (size_t)kt * M + m], v);
+          far_hi = max(far_hi, kt);
         }
-        __syncwarp();
-        if (lane == 0) qend[mm] = upto;
-        __syncwarp();
-      }
-    }
-    for (int j = 0; j < MPL; ++j) {
-      const int m = lane + 32 * j;
-      if (m >= M) continue;
-      Heap hp{heaps + (size_t)m * b.hcap, hs[m]};
-      Decoding* am = act + (size_t)m * b.acap;
-      int32_t* fl = farl + (size_t)m * kFar;
-      // per-window counts of this model: windows k .. k+kRing-1 in the shared
-      // ring, later ones in the instance's global accumulators (their windows
-      // listed, or every row reads them once the list has overflowed)
-      auto add = [&](int arr, long long kt, uint32_t v) {
-        if (kt - k < kRing) {
-          ring[((size_t)arr * M + m) * kRing + (kt & (kRing - 1))] += v;
-          return;
-        }
-        Gacc[(size_t)arr * (K + 1) * M + kt * M + m] += v;
-        if (far_all[j]) return;
-        for (int q = 0; q < n_far[j]; ++q)
-          if (fl[q] == (int32_t)kt) return;
-        if (n_far[j] < kFar) fl[n_far[j]++] = (int32_t)kt;
-        else far_all[j] = true;
       };
-      // start every request of the model that can start before T, in order
-      const int staged_end = qend[m];
-      while (head[j] < end[j] && hp.n > 0) {
-        int4 c0, c1;
-        if (head[j] < staged_end) {
-          const int4* slot = qbuf + ((size_t)m * kQ + (head[j] & (kQ - 1))) * 2;
-          c0 = slot[0];
-          c1 = slot[1];
-        } else {                                 // beyond the staged ones
-          c0 = b.grp[2 * (size_t)head[j]];
-          c1 = b.grp[2 * (size_t)head[j] + 1];
+      auto done = [&](uint32_t st, const int4& c0, const int4& c1) {
+        // a request is processed in the window of its start, or in that of the
+        // one before it where arrivals are out of order; what it would add to
+        // windows already scored is not seen
+        const bool on = st != kNoServer;
+        int kp = on ? (int)fwin.div(st) : 0;
+        for (int o = 1; o < 32; o <<= 1) {
+          const int x = __shfl_up_sync(kFull, kp, o);
+          if (lane >= o) kp = max(kp, x);
         }
-        const long long ta = c0.x;
-        const long long st = max(ta, hp.h[0]);
-        if (st >= Tk) break;
-        const long long dtot = c0.z;
-        const long long tf = min(st + (long long)c0.y, 2147483647ll);
-        const long long te = min(st + dtot, 2147483647ll);
-        const int32_t i = c0.w, L_in = c1.x, L_out = c1.y;
-        hp.replace_top(st + dtot);
-        ++head[j];
-        ++cum_start[j];
+        kp = max(kp, k_now);
+        k_now = __shfl_sync(kFull, kp, 31);
+        if (!on) return;
+        const uint32_t ta = (uint32_t)c0.x;
+        const uint32_t tf = min(st + (uint32_t)c0.y, 2147483647u);
+        const uint32_t te = min(st + (uint32_t)c0.z, 2147483647u);
+        const uint32_t L = (uint32_t)c1.y;
         if (b.o_ts) {
-          const size_t x = (size_t)inst * b.lat.n + i;
+          const size_t x = (size_t)inst * b.lat.n + c0.w;
           b.o_ts[x] = (int32_t)st;
           b.o_tf[x] = (int32_t)tf;
           b.o_te[x] = (int32_t)te;
         }
-        if (b.slo_ms && tf - ta <= (long long)b.slo_ms[m]) ++met[j];
-        bool ends_via_list = false;
+        const long long ttft = (long long)tf - (long long)ta;
+        met += b.slo_ms && ttft <= slo;
+        add(kStart, kp, 1u);
+        const int ke = (int)fwin.div(te);
         if (tf < span) {
-          // times fit 31 bits: 32-bit divisions
-          const long long kf = (uint32_t)tf / (uint32_t)win;
-          const long long ke = min((long long)((uint32_t)te / (uint32_t)win), (long long)K - 1);
-          if (b.guard_ms && tf - ta > (long long)b.guard_ms[m]) add(kLate, kf, 1u);
-          add(kP, kf, (uint32_t)L_in);
-          const long long first = tokens_before((kf + 1) * win, tf, te, L_out);
-          if (first) add(kD, kf, (uint32_t)first);
-          if (ke > kf && L_out >= 2) {
-            if (n_act[j] < b.acap) {             // later windows: counted window by window
-              // here te >= (kf + 1) * win > tf and L_out >= 2 (else every token
-              // of the request falls in window kf)
-              const unsigned long long dur = (unsigned long long)(te - tf);
-              const unsigned long long y = (unsigned long long)((kf + 1) * win - tf) *
-                                               (unsigned long long)(L_out - 1) + dur - 1;
-              const unsigned long long step = (unsigned long long)win * (L_out - 1);
-              Decoding d;
-              d.k_from = (int32_t)kf + 1;
-              d.k_last = (int32_t)ke;
-              d.te = (int32_t)te;
-              d.L = L_out;
-              d.done = (int32_t)first;
-              d.q = (int32_t)(y / dur);
-              d.r = (int32_t)(y - (unsigned long long)d.q * dur);
-              // a step of more than L tokens ends the request in the next
-              // window, where the count is L: the clamp never shows
-              const unsigned long long qd = step / dur;
-              d.qd = (int32_t)min(qd, (unsigned long long)L_out + 1);
-              d.rd = (int32_t)(step - qd * dur);
-              d.dur = (int32_t)dur;
-              am[n_act[j]++] = d;
-              ends_via_list = true;
-            } else {                             // no room: add them all now
-              long long prev = first;
-              for (long long kk = kf + 1; kk <= ke; ++kk) {
-                const long long nxt = tokens_before((kk + 1) * win, tf, te, L_out);
-                if (nxt != prev) add(kD, kk, (uint32_t)(nxt - prev));
-                prev = nxt;
-              }
+          const int kf = (int)fwin.div(tf);
+          // tokens of the first-token window, then a window at a time without
+          // dividing: one window on adds win * (L - 1) = Q * dur + R
+          uint32_t tok = L, rem = 0, Q = 0, R = 0;
+          const uint32_t dur = te - tf;
+          const bool later = L > 1 && ke > kf;
+          if (later) {
+            unsigned long long q, r;
+            divmod((unsigned long long)((uint32_t)(kf + 1) * win - tf) * (L - 1), dur, q, r);
+            tok = (uint32_t)q + (r != 0);
+            rem = r ? (uint32_t)r - 1 : dur - 1;
+            if (ke > kf + 1) {                  // dur > win here
+              divmod((unsigned long long)win * (L - 1), dur, q, r);
+              Q = (uint32_t)q;
+              R = (uint32_t)r;
             }
           }
+          if (kf >= kp) {
+            if (b.guard_ms && ttft > guard) add(kLate, kf, 1u);
+            if (c1.x) add(kP, kf, (uint32_t)c1.x);
+            if (tok) add(kD, kf, tok);
+          }
+          if (later) {
+            const int k_full = min(ke - 1, K - 1);
+            for (int k = kf + 1; k <= k_full; ++k) {
+              const uint32_t t = rem + R, c = t >= dur ? 1u : 0u;
+              rem = t - (c ? dur : 0u);
+              const uint32_t d = Q + c;
+              tok += d;
+              if (d && k >= kp) add(kD, k, d);
+            }
+            if (ke < K && L != tok && ke >= kp) add(kD, ke, L - tok);
+          }
         }
-        // the running span ends in window te / win (never read when te is
-        // past the grid); a listed request counts its end when it retires
-        if (!ends_via_list && te < span) add(kEnd, (uint32_t)te / (uint32_t)win, 1u);
+        // the running span ends in window te / win (never read past the grid)
+        if (te < span && ke >= kp) add(kEnd, ke, 1u);
+      };
+      uint32_t* sv = srv + (size_t)m * b.hcap;
+      if (n > 0 && head < end) {
+        if (n <= 32) start_requests<1>(sv, n, b.grp, head, end, t_end, done);
+        else if (n <= 64) start_requests<2>(sv, n, b.grp, head, end, t_end, done);
+        else if (n <= 128) start_requests<4>(sv, n, b.grp, head, end, t_end, done);
+        else start_requests_mem(sv, n, b.grp, head, end, t_end, done);
       }
-      qhead[m] = head[j];
-      // decode tokens of the requests still decoding, for window k, and the
-      // ends of those that retire in it
-      uint32_t d_live = 0, e_live = 0;
-      for (int q = 0; q < n_act[j];) {
-        Decoding& e = am[q];
-        if (e.k_from > k) {
-          ++q;
-          continue;
-        }
-        // y at the end of window k
-        e.q += e.qd;
-        e.r += e.rd;
-        if (e.r >= e.dur) {
-          e.r -= e.dur;
-          e.q += 1;
-        }
-        const int32_t nxt = (long long)(k + 1) * win > (long long)e.te ? e.L : e.q;
-        d_live += (uint32_t)(nxt - e.done);
-        e.done = nxt;
-        if (e.k_last <= k) {
-          if ((long long)e.te < span) ++e_live;
-          am[q] = am[--n_act[j]];
-        } else {
-          ++q;
-        }
-      }
-      // window k's counts: the ring slot (cleared for window k + kRing) plus
-      // any later-window contributions made before the ring reached it
-      uint32_t v[4];
-      bool far = far_all[j];
-      for (int q = 0; q < n_far[j]; ++q)
-        if (fl[q] == k) {
-          far = true;
-          fl[q] = fl[--n_far[j]];
-          break;
-        }
+      __syncwarp();
+      // the segment's windows, one per lane
+      const int k = k0 + lane;
+      const bool in = lane < n_win;
+      uint32_t v[kCounts] = {0, 0, 0, 0, 0};
+      const int fh = max(s.far_hi, (int)__reduce_max_sync(kFull, far_hi));
+      if (fh > s.far_hi) __threadfence();       // far counts are read segments later
+      if (in) {
 #pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        uint32_t* slot = &ring[((size_t)a * M + m) * kRing + (k & (kRing - 1))];
-        v[a] = *slot;
-        *slot = 0;
-        if (far) v[a] += Gacc[(size_t)a * (K + 1) * M + (size_t)k * M + m];
-      }
-      const size_t x = (size_t)k * M + m;
-      cum_arr[j] += arr_next[j];
-      if (k + 1 < K) arr_next[j] = b.arr_cnt[x + M];   // the next window's arrivals, early
-      cum_end[j] += v[kEnd] + e_live;
-      const int32_t P = (int32_t)v[kP], D = (int32_t)(v[kD] + d_live);
-      const int32_t A = (int32_t)(cum_start[j] - cum_end[j]);
-      const int32_t W = (int32_t)(cum_arr[j] - cum_start[j]);
-      const bool idle = P == 0 && D == 0 && A == 0 && W == 0;
-      if (!idle) {
-        const T r_pre = (T)P / dt;
-        const T r_dec = (T)D / dt;
-        const T svc = pw[j] * r_pre;
-        const T num = svc + r_dec;
-        const T qw = pq[j] * (T)W;
-        T den = (T)A + qw;
-        if (den < (T)1) den = (T)1;
-        const T raw = num / den;
-        if (!init[j]) {
-          S[j] = raw;
-          init[j] = true;
-        } else {
-          const T x1 = pa[j] * raw;
-          const T x2 = ((T)1 - pa[j]) * S[j];
-          S[j] = x1 + x2;
+        for (int a = 0; a < kCounts; ++a) {
+          uint32_t* slot = &my_ring[(size_t)a * M * kRing + (k & (kRing - 1))];
+          v[a] = *slot;
+          *slot = 0;
+        }
+        if (k <= s.far_hi) {
+#pragma unroll
+          for (int a = 0; a < kFarCounts; ++a) v[a] += __ldcg(&far[a * far_arr + (size_t)k * M + m]);
         }
       }
-      const T Z = S[j] / pth[j];
+      const uint32_t arr = warp_scan(in ? (uint32_t)b.arr_cnt[(size_t)k * M + m] : 0u) + s.arrived;
+      const uint32_t started = warp_scan(v[kStart]) + s.started;
+      const uint32_t ended = warp_scan(v[kEnd]) + s.ended;
+      const int32_t P = (int32_t)v[kP], D = (int32_t)v[kD];
+      const int32_t A = (int32_t)(started - ended), W = (int32_t)(arr - started);
+      const bool idle = !in || (P == 0 && D == 0 && A == 0 && W == 0);
+      T raw = (T)0;
+      if (!idle) {
+        const T num = add_rn(mul_rn(b.w_p[m], div_rn(from_i32<T>(P), dt)),
+                             div_rn(from_i32<T>(D), dt));
+        T den = add_rn(from_i32<T>(A), mul_rn(b.w_q[m], from_i32<T>(W)));
+        if (den < (T)1) den = (T)1;
+        raw = div_rn(num, den);
+      }
+      const unsigned live = __ballot_sync(kFull, !idle);
+      const T al = b.alpha[m], be = (T)1 - al;
+      const T ar = mul_rn(al, raw);
+      T S = s.S, mine = (T)0;
+      int init = s.init;
+      for (int w = 0; w < n_win; ++w) {
+        const T x1 = __shfl_sync(kFull, ar, w), r1 = __shfl_sync(kFull, raw, w);
+        if (live >> w & 1u) {
+          S = init ? add_rn(x1, mul_rn(be, S)) : r1;
+          init = 1;
+        }
+        if (lane == w) mine = S;
+      }
+      const T Z = div_rn(mine, b.theta[m]);
       uint8_t cl;
-      if (idle) cl = TRE_IDLE;
-      else if (Z < ptc[j]) cl = TRE_CRIT;
-      else if (Z > pts[j]) cl = TRE_SURP;
-      else cl = TRE_NOM;
-      zrow[m] = Z;
-      crow[m] = cl;
-      // latency guard breached in the window; requests waiting with no
-      // routable replica (lost capacity)
-      frow[m] = (uint8_t)((b.guard_ms && v[kLate] ? 1 : 0) | (r[m] == 0 && W > 0 ? 2 : 0));
-      if (b.Z) {
-        const size_t y = (size_t)inst * K * M + x;
+      if (idle) cl = kIdle;
+      else if (Z < (b.n_tau > 0 ? b.tau_list[ti] : b.tau_crit[m])) cl = kCrit;
+      else if (Z > b.tau_surp[m]) cl = kSurp;
+      else cl = kNom;
+      if (in && b.Z) {
+        const size_t y = ((size_t)inst * K + k) * M + m;
         b.Z[y] = Z;
         b.cls[y] = cl;
       }
+      if (lane == n_win - 1) {
+        zrow[m] = Z;
+        crow[m] = cl;
+        // latency guard breached in the window; requests waiting with no
+        // routable replica (lost capacity)
+        frow[m] = (uint8_t)((b.guard_ms && v[kLate] ? 1 : 0) | (rep[m] == 0 && W > 0 ? 2 : 0));
+      }
+      const uint32_t a1 = __shfl_sync(kFull, arr, n_win - 1);
+      const uint32_t s1 = __shfl_sync(kFull, started, n_win - 1);
+      const uint32_t e1 = __shfl_sync(kFull, ended, n_win - 1);
+      const unsigned mt = b.slo_ms && head > head0 ? __reduce_add_sync(kFull, met) : 0u;
+      if (lane == 0) {
+        s.head = head;
+        s.arrived = a1;
+        s.started = s1;
+        s.ended = e1;
+        s.far_hi = fh;
+        s.met += mt;
+        s.S = S;
+        s.init = init;
+      }
+      __syncwarp();
     }
-    const bool fast = ends_tick(k, win, b.fast_ms), slow = ends_tick(k, win, b.slow_ms);
-    if (!fast && !slow) continue;
-    __threadfence_block();
-    __syncwarp();
-    if (lane == 0) {
-      Ctl<T> ctl{b, zrow, crow, frow, r, tc};
+    const int k = k1;
+    k0 = k1 + 1;
+    if (k != tick) continue;                    // no tick in the segment's last window
+    __syncthreads();
+    if (wid == 0) {
+      const long long Tk = (long long)t_end;
+      const bool fast = next_tick(k, win, (uint32_t)b.fast_ms) == k;
+      const bool slow = next_tick(k, win, (uint32_t)b.slow_ms) == k;
+      // models on lanes, two per lane
+      T z[2];
+      uint8_t rg[2];
+      bool held[2];
+      int32_t r[2], rmin[2], fp[2];
+      unsigned idle_m[2], surp_m[2], nom_m[2], crit_m[2], breach[2], lost[2];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int m = lane + 32 * j;
+        const bool has = m < M;
+        z[j] = has ? zrow[m] : (T)0;
+        const uint8_t c = has ? crow[m] : kIdle, f = has ? frow[m] : (uint8_t)0;
+        held[j] = f & 1;
+        r[j] = has ? rep[m] : 0;
+        rmin[j] = has ? b.r_min[m] : 0;
+        fp[j] = has ? b.footprint[m] : 0;
+        rg[j] = !has ? (uint8_t)0xff
+                : c == kIdle ? kIdle
+                : z[j] < (b.n_tau > 0 ? b.tau_list[ti] : b.tau_crit[m]) ? kCrit
+                : z[j] > b.tau_surp[m] ? kSurp : kNom;
+        idle_m[j] = __ballot_sync(kFull, rg[j] == kIdle);
+        surp_m[j] = __ballot_sync(kFull, rg[j] == kSurp);
+        nom_m[j] = __ballot_sync(kFull, rg[j] == kNom);
+        crit_m[j] = __ballot_sync(kFull, rg[j] == kCrit);
+        breach[j] = __ballot_sync(kFull, f & 1);
+        lost[j] = __ballot_sync(kFull, (f & 2) != 0);
+      }
+      auto value = [&](const T (&a)[2], int m) -> T {
+        return __shfl_sync(kFull, m < 32 ? a[0] : a[1], m & 31);
+      };
+      auto count = [&](const int32_t (&a)[2], int m) -> int32_t {
+        return __shfl_sync(kFull, m < 32 ? a[0] : a[1], m & 31);
+      };
       int recv = -1, kind = 0;
       bool nom_above = false, deferred = false;
       if (fast) {
@@ -560,208 +638,203 @@ k_replay(const __grid_constant__ ReplayBatch<T> b) {
         // models and models that lost their routable capacity. A rebalance
         // transfer in progress defers a rescue without a breach; the pending
         // rescue keeps the slow loop out of the tick.
-        bool hard = false;
-        for (int m = 0; m < M; ++m)
-          if ((frow[m] & 1) && (recv < 0 || zrow[m] < zrow[recv])) recv = m;
-        if (recv >= 0) {
-          hard = true;
-        } else {
-          for (int m = 0; m < M; ++m)
-            if ((ctl.region(m) == TRE_CRIT || (frow[m] & 2)) && (recv < 0 || zrow[m] < zrow[recv]))
-              recv = m;
-        }
+        const bool hard = (breach[0] | breach[1]) != 0;
+        const unsigned want[2] = {hard ? breach[0] : crit_m[0] | lost[0],
+                                  hard ? breach[1] : crit_m[1] | lost[1]};
+        recv = best_model<false>(want, z);
         if (recv >= 0) {
           if (Tk < reb_until && !hard) deferred = true;
           else kind = TRE_RESCUE;
         }
       }
       if (kind == 0 && recv < 0 && slow) {       // rebalance: Eq. 3 over non-idle models
-        for (int m = 0; m < M; ++m)
-          if (ctl.region(m) != TRE_IDLE && (recv < 0 || zrow[m] < zrow[recv])) recv = m;
-        if (recv >= 0 && zrow[recv] < (T)1) {
+        const unsigned want[2] = {surp_m[0] | nom_m[0] | crit_m[0],
+                                  surp_m[1] | nom_m[1] | crit_m[1]};
+        recv = best_model<false>(want, z);
+        if (recv >= 0 && value(z, recv) < (T)1) {
           kind = TRE_REBALANCE;
           nom_above = true;
         }
       }
-      auto emit = [&](int recv_m, int donor, int seq) {
-        if (nm < b.moves_cap) {
-          tre_move mv;
-          mv.window = k;
-          mv.recv = (int16_t)recv_m;
-          mv.donor = (int16_t)donor;
-          mv.kind = (uint8_t)kind;
-          mv.seq = (uint8_t)seq;
-          mv.reserved = 0;
-          b.moves[(size_t)inst * b.moves_cap + nm] = mv;
-        }
-        ++nm;
-      };
       if (deferred) kind = 0;
-      for (int seq = 0; kind && seq < pacing; ++seq) {
-        const long long need = b.footprint[recv];
-        Heap hr{heaps + (size_t)recv * b.hcap, hs[recv]};
-        if (free_pool >= need) {                 // idle capacity first
-          free_pool -= need;
-          r[recv] += 1;
-          emit(recv, -1, seq);
-          hr.push(Tk + b.wake_ms);
-          hs[recv] = hr.n;
-          if (kind == TRE_REBALANCE) reb_until = max(reb_until, Tk + (long long)b.wake_ms);
-          continue;
-        }
-        // dry run: can the eligible donors cover the receiver's footprint?
-        for (int m = 0; m < M; ++m) rr[m] = r[m];
-        long long f = free_pool;
-        bool ok = true;
-        while (f < need) {
-          const int d = ctl.pick(rr, recv, nom_above);
-          if (d < 0) {
-            ok = false;
-            break;
+      if (kind) {
+        const T zr = value(z, recv);
+        unsigned above[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          above[j] = nom_above ? __ballot_sync(kFull, z[j] > zr) : kFull;
+        // donor preference: idle models (lowest index), then surplus by Z
+        // descending, then nominal by Z descending (with nom_above only above
+        // the receiver's Z); never critical, never the receiver, never below
+        // the floor, never a donor whose latency guard is breached
+        auto pick = [&](const int32_t (&rr)[2]) -> int {
+          unsigned can[2];
+#pragma unroll
+          for (int j = 0; j < 2; ++j)
+            can[j] = __ballot_sync(kFull, lane + 32 * j != recv && rr[j] > rmin[j] && !held[j]);
+          if (can[0] & idle_m[0]) return __ffs(can[0] & idle_m[0]) - 1;
+          if (can[1] & idle_m[1]) return 32 + __ffs(can[1] & idle_m[1]) - 1;
+          const unsigned su[2] = {can[0] & surp_m[0], can[1] & surp_m[1]};
+          const int d = best_model<true>(su, z);
+          if (d >= 0) return d;
+          const unsigned no[2] = {can[0] & nom_m[0] & above[0], can[1] & nom_m[1] & above[1]};
+          return best_model<true>(no, z);
+        };
+        auto emit = [&](int donor, int seq) {
+          if (lane == 0 && nm < b.moves_cap) {
+            tre_move mv;
+            mv.window = k;
+            mv.recv = (int16_t)recv;
+            mv.donor = (int16_t)donor;
+            mv.kind = (uint8_t)kind;
+            mv.seq = (uint8_t)seq;
+            mv.reserved = 0;
+            b.moves[(size_t)inst * b.moves_cap + nm] = mv;
           }
-          rr[d] -= 1;
-          f += b.footprint[d];
+          ++nm;
+        };
+        auto give = [&](int m, int d) {
+          if (m == lane) r[0] += d;
+          if (m == lane + 32) r[1] += d;
+        };
+        auto push = [&](int m, long long t) {
+          if (lane == 0) {
+            srv[(size_t)m * b.hcap + n_srv[m]] = free_at(t);
+            n_srv[m] += 1;
+          }
+          __syncwarp();
+        };
+        const long long need = count(fp, recv);
+        for (int seq = 0; seq < pacing; ++seq) {
+          long long gpu_free = Tk;
+          if (pool >= need) {                    // idle capacity first
+            pool -= need;
+            emit(-1, seq);
+          } else {
+            // dry run: can the eligible donors cover the receiver's footprint?
+            int32_t rr[2] = {r[0], r[1]};
+            long long f = pool;
+            bool ok = true;
+            while (f < need) {
+              const int d = pick(rr);
+              if (d < 0) {
+                ok = false;
+                break;
+              }
+              if (d == lane) rr[0] -= 1;
+              if (d == lane + 32) rr[1] -= 1;
+              f += count(fp, d);
+            }
+            if (!ok) break;
+            // commit: the same releases, each the donor's server that frees first
+            f = pool;
+            while (f < need) {
+              const int d = pick(r);
+              give(d, -1);
+              f += count(fp, d);
+              emit(d, seq);
+              uint32_t* sv = srv + (size_t)d * b.hcap;
+              const int n = n_srv[d];
+              int at;
+              const long long fr = Servers{sv, n}.first(at);
+              const long long drained = max(fr, Tk);
+              __syncwarp();
+              if (lane == 0) {
+                sv[at] = sv[n - 1];
+                n_srv[d] = n - 1;
+              }
+              __syncwarp();
+              gpu_free = max(gpu_free, drained + b.sleep_ms);
+            }
+            pool = f - need;
+          }
+          give(recv, 1);
+          push(recv, gpu_free + b.wake_ms);
+          if (kind == TRE_REBALANCE) reb_until = max(reb_until, gpu_free + (long long)b.wake_ms);
         }
-        if (!ok) break;
-        // commit: the same releases, each the donor's server that frees first
-        f = free_pool;
-        long long gpu_free = Tk;
-        while (f < need) {
-          const int d = ctl.pick(r, recv, nom_above);
-          r[d] -= 1;
-          f += b.footprint[d];
-          emit(recv, d, seq);
-          Heap hd{heaps + (size_t)d * b.hcap, hs[d]};
-          const long long drained = max(hd.h[0], Tk);
-          hd.pop();
-          hs[d] = hd.n;
-          gpu_free = max(gpu_free, drained + b.sleep_ms);
-        }
-        free_pool = f - need;
-        r[recv] += 1;
-        hr.push(gpu_free + b.wake_ms);
-        hs[recv] = hr.n;
-        if (kind == TRE_REBALANCE) reb_until = max(reb_until, gpu_free + (long long)b.wake_ms);
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          if (lane + 32 * j < M) rep[lane + 32 * j] = r[j];
       }
     }
-    __threadfence_block();
-    __syncwarp();
+    __syncthreads();
   }
+  __syncthreads();
   // requests never started count against the SLO with their first token at
   // the end of the grid
-  for (int j = 0; j < MPL; ++j) {
-    const int m = lane + 32 * j;
-    if (m >= M) continue;
+  for (int m = wid; m < M; m += n_warps) {
+    const ModelState<T>& s = st_m[m];
+    unsigned met = 0;
     if (b.slo_ms) {
-      for (int32_t q = head[j]; q < end[j]; ++q)
-        if (span - (long long)b.grp[2 * q].x <= (long long)b.slo_ms[m]) ++met[j];
-      if (b.slo_met) b.slo_met[(size_t)inst * M + m] = met[j];
+      for (int q = s.head + lane; q < s.end; q += 32)
+        met += (long long)span - (long long)b.grp[2 * (size_t)q].x <= (long long)b.slo_ms[m];
+      met = __reduce_add_sync(kFull, met);
     }
-    if (b.served) b.served[(size_t)inst * M + m] = cum_start[j];
-    b.r_final[(size_t)inst * M + m] = r[m];
+    if (lane == 0) {
+      if (b.slo_ms && b.slo_met) b.slo_met[(size_t)inst * M + m] = (int64_t)(s.met + met);
+      if (b.served) b.served[(size_t)inst * M + m] = (int64_t)(s.head - b.base[m]);
+      b.r_final[(size_t)inst * M + m] = rep[m];
+    }
   }
-  if (lane == 0) {
+  if (threadIdx.x == 0) {
     b.n_moves[inst] = nm;
     if (nm > b.moves_cap) b.diag->err = TRE_EOVERFLOW;
   }
 }
 
-constexpr size_t kReplaySmemMax = 160 * 1024;
-
-template <class T> int warp_base_bytes(int M) {
-  size_t o = ((size_t)M * sizeof(T) + 15) & ~(size_t)15;   // Z row
-  o += (size_t)M * 4 * 3;                                   // r, dry-run r, heap sizes
-  o += (size_t)M * 2;                                       // class and flag rows
-  return (int)((o + 15) & ~(size_t)15);
-}
+// what a block may opt into, less the reserve of the system
+constexpr size_t kReplaySmemMax = 224 * 1024;
 
 }  // namespace
 
 template <class T> void replay_ws_layout(Arena& a, ReplayBatch<T>& b, ReplayWs& w) {
   const int M = b.M, K = b.K;
-  w.vm = a.take<int8_t>((size_t)std::max<int64_t>(b.lat.n, 1));
+  const size_t n = (size_t)std::max<int64_t>(b.lat.n, 1);
+  w.n_blk = (int)((b.lat.n + kGroupBlock - 1) / kGroupBlock);
+  w.vm = a.take<int8_t>(n);
   w.arr_cnt = a.take<int32_t>((size_t)K * M + 1);
-  w.n_valid = a.take<int32_t>((size_t)M);
+  w.blk_cnt = a.take<int32_t>((size_t)std::max(w.n_blk, 1) * M);
   w.base = a.take<int32_t>((size_t)M + 1);
-  w.list = a.take<int32_t>((size_t)std::max<int64_t>(b.lat.n, 1));
-  w.acc = a.take<uint32_t>((size_t)b.n_inst * 4 * (K + 1) * M);
-  w.grp = a.take<int4>((size_t)std::max<int64_t>(b.lat.n, 1) * 2);
-  // warps per CTA: spread the instances over the SMs first
-  const int sms = device_sm_count();
-  int W = (int)std::min<int64_t>(8, std::max<int64_t>(1, (b.n_inst + sms - 1) / sms));
+  w.acc = a.take<uint32_t>((size_t)b.n_inst * kFarCounts * (K + 1) * M);
+  w.grp = a.take<int4>(n * 2);
   auto a16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
-  const size_t wb = (size_t)warp_base_bytes<T>(M);
-  const size_t hb = a16((size_t)M * b.hcap * 8);
-  const size_t ring_bytes = a16((size_t)M * (4 * kRing + kFar) * 4);
-  const size_t q_bytes = a16((size_t)M * kQ * 32 + (size_t)M * 8);
-  // decoding requests per model: room for as many as the budget has replicas
-  // (more are added straight to the accumulators), at least 8
-  int acap = std::max(8, std::min(b.hcap, 256));
-  auto act_bytes = [&](int c) { return a16((size_t)M * c * sizeof(Decoding)); };
-  w.shared_heaps = false;
-  for (int tw = W; tw >= 1; tw >>= 1) {
-    if ((wb + hb + q_bytes + ring_bytes + act_bytes(8)) * tw <= kReplaySmemMax) {
-      w.shared_heaps = true;
-      W = tw;
-      break;
-    }
-  }
-  const size_t fixed = wb + (w.shared_heaps ? hb : 0) + q_bytes + ring_bytes;
-  if (!w.shared_heaps) W = 1;
-  while (acap > 8 && (fixed + act_bytes(acap)) * W > kReplaySmemMax) acap >>= 1;
-  w.warps_per_cta = W;
-  b.warps_per_cta = W;
-  // per warp: base rows | heaps (when shared) | staged requests | rings | lists
-  b.heap_off = (int)wb;
-  b.q_off = (int)(wb + (w.shared_heaps ? hb : 0));
-  b.ring_off = (int)(b.q_off + q_bytes);
-  b.act_off = (int)(b.ring_off + ring_bytes);
-  b.acap = acap;
-  b.warp_bytes = (int)(fixed + act_bytes(acap));
-  w.gheap = w.shared_heaps ? nullptr
-                           : a.take<long long>((size_t)b.n_inst * M * b.hcap);
-  b.list = w.list;
+  const size_t rows = a16((size_t)M * (sizeof(ModelState<T>) + sizeof(T) + 4 + 4 + 1 + 1));
+  const size_t rings = (size_t)kCounts * M * kRing * 4;
+  const size_t srv = (size_t)M * b.hcap * 4;
+  const bool fits = rows + rings + srv <= kReplaySmemMax;
+  b.ring_off = (int)rows;
+  b.srv_off = (int)(rows + rings);
+  b.smem_bytes = (int)(rows + rings + (fits ? srv : 0));
+  b.gsrv = nullptr;
+  uint32_t* g = fits ? nullptr : a.take<uint32_t>((size_t)b.n_inst * M * b.hcap);
+  b.gsrv = g;
   b.grp = w.grp;
   b.base = w.base;
   b.arr_cnt = w.arr_cnt;
   b.acc = w.acc;
-  b.gheap = w.gheap;
 }
 
 template <class T> cudaError_t launch_replay(ReplayBatch<T>& b, ReplayWs& w, cudaStream_t s) {
   const int M = b.M, K = b.K;
   cudaError_t e = cudaMemsetAsync(w.arr_cnt, 0, ((size_t)K * M + 1) * sizeof(int32_t), s);
-  if (!e) e = cudaMemsetAsync(w.n_valid, 0, (size_t)M * sizeof(int32_t), s);
-  if (!e) e = cudaMemsetAsync(w.acc, 0, (size_t)b.n_inst * 4 * (K + 1) * M * sizeof(uint32_t), s);
+  if (!e)
+    e = cudaMemsetAsync(w.acc, 0, (size_t)b.n_inst * kFarCounts * (K + 1) * M * sizeof(uint32_t), s);
   if (e) return e;
-  const int sms = device_sm_count();
-  const unsigned g1 = (unsigned)std::max<int64_t>(
-      1, std::min<int64_t>((b.lat.n + 255) / 256, (int64_t)sms * 8));
-  if (b.lat.n > 0) k_rp_valid<<<g1, 256, 0, s>>>(b.lat, M, b.win, K, w.vm, w.arr_cnt, w.n_valid);
-  k_rp_fill<<<M, kFillThreads, 0, s>>>(b.lat.n, M, w.vm, w.n_valid, w.list, w.base);
-  if (b.lat.n > 0) k_rp_gather<<<g1, 256, 0, s>>>(b.lat.n, b.lat, w.list, w.base, M, w.grp);
+  const FastDiv fwin((uint32_t)b.win);
+  if (w.n_blk > 0)
+    k_rp_valid<<<w.n_blk, kGroupBlock, 0, s>>>(b.lat, M, fwin, (int64_t)K * b.win, w.vm, w.arr_cnt,
+                                               w.blk_cnt);
+  k_rp_offsets<<<1, 1024, 0, s>>>(M, w.n_blk, w.blk_cnt, w.base);
+  if (w.n_blk > 0)
+    k_rp_group<<<w.n_blk, kGroupBlock, 0, s>>>(b.lat, M, w.vm, w.blk_cnt, w.base, w.grp);
   if ((e = cudaGetLastError())) return e;
   if (b.o_ts && b.lat.n > 0) {
-    k_rp_init_records<<<(unsigned)sms * 8, 256, 0, s>>>(b.lat.n, b.n_inst, (int32_t)(K * b.win),
-                                                        w.vm, b.o_ts, b.o_tf, b.o_te);
+    k_rp_init_records<<<(unsigned)device_sm_count() * 8, 256, 0, s>>>(
+        b.lat.n, b.n_inst, (int32_t)(K * b.win), w.vm, b.o_ts, b.o_tf, b.o_te);
     if ((e = cudaGetLastError())) return e;
   }
-  const int W = w.warps_per_cta;
-  const unsigned grid = (unsigned)((b.n_inst + W - 1) / W);
-  const size_t smem = (size_t)b.warp_bytes * W;
-  const void* fn;
-  if (M <= 32)
-    fn = w.shared_heaps ? (const void*)k_replay<T, 1, true> : (const void*)k_replay<T, 1, false>;
-  else
-    fn = w.shared_heaps ? (const void*)k_replay<T, 2, true> : (const void*)k_replay<T, 2, false>;
-  if ((e = func_smem_once(fn, (int)kReplaySmemMax, false))) return e;
-  if (M <= 32) {
-    if (w.shared_heaps) k_replay<T, 1, true><<<grid, 32 * W, smem, s>>>(b);
-    else k_replay<T, 1, false><<<grid, 32 * W, smem, s>>>(b);
-  } else {
-    if (w.shared_heaps) k_replay<T, 2, true><<<grid, 32 * W, smem, s>>>(b);
-    else k_replay<T, 2, false><<<grid, 32 * W, smem, s>>>(b);
-  }
+  if ((e = func_smem_once((const void*)k_replay<T>, (int)kReplaySmemMax, false))) return e;
+  k_replay<T><<<(unsigned)b.n_inst, 32 * std::min(M, kMaxWarps), (size_t)b.smem_bytes, s>>>(b);
   return cudaGetLastError();
 }
 

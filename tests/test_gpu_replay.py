@@ -144,9 +144,9 @@ def test_replay_heterogeneous_footprints_and_pool(tre):
            wake=500, sleep=700)
 
 
-def test_replay_sixty_four_models_global_heaps(tre):
-    """64 models (two per lane) with a 512-replica budget: the server heaps
-    do not fit in shared memory and live in the workspace."""
+def test_replay_sixty_four_models(tre):
+    """64 models (four to a warp, two to a lane of the controller) with a
+    512-replica budget."""
     spec = tracegen.spec_stream(scale=0.05, seed=11, duration_s=1800.0)
     lat = tracegen.gen_latent(spec)
     M = spec.n_models
@@ -154,6 +154,28 @@ def test_replay_sixty_four_models_global_heaps(tre):
     _check(tre, lat, M, 100, 18000, prof, int(spec.budget), lat["r0"], np.ones(M, np.int32),
            np.ones(M, np.int32), "f32", [(0.8, 1), (0.8, 2)], wake=1310, sleep=1870,
            guard=np.full(M, 6000, np.int32))
+
+
+# A model's free times sit one, two or four to a lane, in shared memory above
+# 128 servers, in the workspace when a budget's do not fit there. Arrivals out of
+# order: a request waits for the one before it in the input, and what it would
+# add to windows already scored is not seen.
+@pytest.mark.parametrize("shuffled", [False, True])
+@pytest.mark.parametrize("servers,budget", [((33, 5, 64), 120), ((65, 128, 1), 200),
+                                            ((129, 2, 300), 440), ((20, 30, 40), 30000)])
+def test_replay_server_counts_and_input_order(tre, servers, budget, shuffled):
+    rng = np.random.default_rng(budget + shuffled)
+    n, M, span = 3000, 3, 300000
+    t = rng.integers(0, span, n)
+    t = t if shuffled else np.sort(t)
+    total = rng.integers(0, 30000, n)
+    lat = {"model": rng.integers(0, M, n), "t_arr_ms": t,
+           "d_first_ms": (total * rng.random(n)).astype(np.int64), "d_total_ms": total,
+           "L_in": rng.integers(0, 500, n), "L_out": rng.integers(1, 300, n)}
+    lat = {k: v.astype(np.int32) for k, v in lat.items()}
+    _check(tre, lat, M, 1000, span // 1000, _prof(M, theta=20.0), budget,
+           np.array(servers, np.int32), np.ones(M, np.int32), np.ones(M, np.int32), "f32",
+           [(0.8, 2)], wake=1310, sleep=1870, guard=np.full(M, 3000, np.int32))
 
 
 def test_replay_invalid_records_are_not_served(tre):
