@@ -9,15 +9,14 @@
 //
 // Instead of sorting, each (series, model) packs its (S, healthy) pairs into
 // unsigned keys (the bit pattern of a positive float orders like the float)
-// and one CTA finds theta by a descent over the key range: the current range
-// is split linearly into buckets; a histogram gives per bucket the count, the
-// healthy count and the smallest key; per bucket, in parallel, the exact test
-// at its smallest value (everything at or above it included) and an upper
-// bound for any value inside it (only its healthy windows added). The lowest
-// bucket that passes either gives theta directly (its smallest value
-// qualifies and nothing below did) or is refined; a refinement that finds
-// nothing resumes with the buckets above it. Counts are exact integers and the
-// final test is the definition's double expression, so theta is exact.
+// and one CTA finds theta from a histogram over the key range: per bucket, in
+// parallel, the exact test at its smallest value (everything at or above it
+// included) and an upper bound for any value inside it (only its healthy
+// windows added). Values of buckets below the lowest one that passes, but whose
+// bound does, are tested one by one. When too many would have to be, a descent
+// over the key range refines one bucket after another. Counts are exact
+// integers and the tests give the definition's double comparison, so theta is
+// exact.
 #include <algorithm>
 
 #include "common.cuh"
@@ -45,6 +44,26 @@ __device__ __forceinline__ double value_of(unsigned long long k) {
   return __longlong_as_double((long long)k);
 }
 
+// (double)h >= rate * (double)c. Decided in float where the two sides are
+// further apart than the float conversions and the product can be off (a few
+// 2^-24 of either side); only near ties take the double expression (the FP64
+// pipe has two lanes an SM: testing all 4096 buckets in double took 8 us).
+__device__ __forceinline__ bool at_least(uint32_t h, uint32_t c, double rate, float rate_f) {
+  const float x = (float)h, t = rate_f * (float)c;
+  const float margin = 1.f + (x + fabsf(t)) * 0x1p-20f;
+  if (x >= t + margin) return true;
+  if (x <= t - margin) return false;
+  return (double)h >= rate * (double)c;
+}
+
+// smallest integer n with (double)n >= ok_frac * (double)a
+__device__ __forceinline__ int32_t healthy_from(double ok_frac, int a) {
+  const double v = ok_frac * (double)a;
+  if (!(v <= 2147483647.0)) return 0x7fffffff;        // unreachable (or NaN)
+  if (v <= -2147483647.0) return -0x7fffffff;
+  return (int32_t)ceil(v);
+}
+
 // thr[a] = smallest integer n with (double)n >= ok_frac * (double)a; also
 // resets the per-(series, model) candidate key ranges filled by k_pack
 template <class U>
@@ -56,12 +75,7 @@ __global__ void k_thr(double ok_frac, int32_t* thr, int n_sm, U* kmin, U* kmax, 
     ncand[a] = 0;
   }
   if (a >= kThrTable) return;
-  const double v = ok_frac * (double)a;
-  int32_t t;
-  if (!(v <= 2147483647.0)) t = 0x7fffffff;           // unreachable (or NaN)
-  else if (v <= -2147483647.0) t = -0x7fffffff;
-  else t = (int32_t)ceil(v);
-  thr[a] = t;
+  thr[a] = healthy_from(ok_frac, a);
 }
 
 __device__ __forceinline__ bool healthy(uint32_t n_arr, uint32_t n_met, const int32_t* thr,
@@ -274,275 +288,291 @@ k_pack(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ PackP
   }
 }
 
-// exclusive suffix sums over the block: out = sum of v over threads > tid
-__device__ __forceinline__ int64_t block_suffix(int64_t v, int64_t* red) {
+// exclusive suffix sums of two values over the block (sums over threads > tid)
+__device__ __forceinline__ int2 block_suffix(int a, int b, int2* red) {
+  const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, wid = threadIdx.x / 32;
-  // inclusive suffix within the warp (lanes above)
-  int64_t inc = v;
+  int ia = a, ib = b;               // inclusive suffix within the warp
   for (int o = 1; o < 32; o <<= 1) {
-    const int64_t x = __shfl_down_sync(0xffffffffu, inc, o);
-    if (lane + o < 32) inc += x;
+    const int xa = __shfl_down_sync(full, ia, o), xb = __shfl_down_sync(full, ib, o);
+    if (lane + o < 32) {
+      ia += xa;
+      ib += xb;
+    }
   }
-  if (lane == 0) red[wid] = inc;
+  if (lane == 0) red[wid] = make_int2(ia, ib);
   __syncthreads();
-  int64_t above = 0;
-  for (int w = wid + 1; w < kWarps; ++w) above += red[w];
+  const int2 w = red[lane];
+  const int above_a = __reduce_add_sync(full, lane > wid ? w.x : 0);
+  const int above_b = __reduce_add_sync(full, lane > wid ? w.y : 0);
   __syncthreads();
-  return inc - v + above;
+  return make_int2(ia - a + above_a, ib - b + above_b);
 }
 
 __device__ __forceinline__ int block_min(int v, int* red) {
+  const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, wid = threadIdx.x / 32;
-  v = __reduce_min_sync(0xffffffffu, v);
+  v = __reduce_min_sync(full, v);
   if (lane == 0) red[wid] = v;
   __syncthreads();
-  int r = 0x7fffffff;
-  for (int w = 0; w < kWarps; ++w) r = min(r, red[w]);
+  v = __reduce_min_sync(full, red[lane]);
   __syncthreads();
-  return r;
+  return v;
 }
+static_assert(kWarps == 32, "one block-wide value per lane");
 
 constexpr int kFine = 4096;     // buckets of the first histogram
 constexpr int kUnroll = 8;      // keys per thread whose loads are issued together
-constexpr int kCap = 2048;      // most keys the exact pass sorts in shared memory
+constexpr int kCap = 2048;      // most keys the exact pass tests one by one
+constexpr int kDirectK = kUnroll * kNB;       // longest series searched without packing
+constexpr int64_t kDirectCells = 1 << 18;     // and largest table: a CTA reads one column of
+                                              // the rows, 4 to 8 bytes of each 32-byte sector
 
 template <class T> size_t search_smem_bytes() {
   using U = typename KeyOf<T>::U;
-  const size_t fast = (size_t)kFine * (5 * 4) + (size_t)kCap * (sizeof(U) + 4);
+  const size_t fast = (size_t)kFine * (5 * 4) + (size_t)kCap * sizeof(U);
   const size_t descent = (size_t)KeyOf<T>::kLevels * kNB * (4 + 4 + sizeof(U));
   return fast > descent ? fast : descent;
 }
 
-template <class T>
-__global__ void __launch_bounds__(kNB)
-k_search(const __grid_constant__ SeriesTable<T> tab, const typename KeyOf<T>::U* __restrict__ keys,
+// One CTA per (series, model). DIRECT: the keys are made here, from the
+// model's column of S, classes and counts, and stay in registers (series of up
+// to kDirectK windows): one launch where packing, its threshold table and the
+// search were three. Otherwise they come from the packing pass, and are read
+// again for the gather. What bounds a search is its chain of block-wide steps.
+// 8 models, 3,600 windows: 15.4 us in one launch (25.3 in three, with a bitonic
+// sort of the gathered keys and every test in double); 16 models, 43,200
+// windows: 21.6 us (30.5); the sweep's 224 searches: 24.5 us (33.3).
+template <class T, bool DIRECT>
+__global__ void __launch_bounds__(kNB, !DIRECT && sizeof(T) == 4 ? 2 : 1)
+k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __restrict__ keys,
          const typename KeyOf<T>::U* kmin_g, const typename KeyOf<T>::U* kmax_g,
-         const uint32_t* ncand_g, double reliability, T* theta, tre_diag* diag) {
+         const uint32_t* ncand_g, const T* __restrict__ S, const uint8_t* __restrict__ cls,
+         const unsigned long long* __restrict__ slo, double ok_frac, double reliability, T* theta,
+         tre_diag* diag) {
   using U = typename KeyOf<T>::U;
   constexpr int NL = KeyOf<T>::kLevels;
+  constexpr int kThrDirect = 256;
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ U lo_s[NL], hi_s[NL];
   __shared__ int shift_s[NL], pos_s[NL];
-  __shared__ int64_t cab_s[NL], hab_s[NL];
-  __shared__ int64_t red64[kWarps];
+  __shared__ int cab_s[NL], hab_s[NL];
+  __shared__ int2 red2[kWarps];
   __shared__ int red32[kWarps];
-  __shared__ int nsel_s;
-  __shared__ U bfmin_s;
+  __shared__ U redU[2][kWarps];
+  __shared__ int thr_s[kThrDirect];
+  __shared__ U bfmin_s, best_s;
   const int M = tab.M;
   const int s = blockIdx.x / M, m = blockIdx.x % M;
   const int K = tab.K[s];
-  const U* mk = keys + (size_t)tab.off[s] + (size_t)m * K;
+  U* mk = keys + (size_t)tab.off[s] + (size_t)m * K;
   const int tid = threadIdx.x, lane = tid & 31;
   const size_t out = (size_t)s * M + m;
+  const float rel_f = (float)reliability;
+  int32_t* fcnt = reinterpret_cast<int32_t*>(dyn);
+  int32_t* fhl = fcnt + kFine;
+  int32_t* fst = fhl + kFine;                   // where a selected bucket's keys start, -1 if not
+  int32_t* fca = fst + kFine;                   // windows in buckets above
+  int32_t* fha = fca + kFine;                   // healthy windows in buckets above
+  U* list = reinterpret_cast<U*>(fha + kFine);
+  for (int b = tid; b < kFine; b += kNB) {
+    fcnt[b] = 0;
+    fhl[b] = 0;
+  }
+  if (tid == 0) {
+    bfmin_s = ~(U)0;
+    best_s = ~(U)0;
+  }
 
-  // ---- range of candidate keys (from the packing pass) ---------------------
-  if (ncand_g[out] == 0) {
+  // ---- candidate keys: their range and number -------------------------------
+  U pv[kUnroll];
+  U kmin, kmax;
+  uint32_t ncand;
+  if (DIRECT) {
+    if (tid < kThrDirect) thr_s[tid] = healthy_from(ok_frac, tid);
+    T sv[kUnroll];
+    uint8_t iv[kUnroll];
+    unsigned long long cv[kUnroll];
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) {
+      const int k = u * kNB + tid;
+      const size_t x = (size_t)tab.off[s] + (size_t)k * M + m;
+      const bool in = k < K;
+      sv[u] = in ? S[x] : (T)0;
+      iv[u] = in ? cls[x] : kIdle;
+      cv[u] = in ? slo[x] : 0ull;
+    }
+    __syncthreads();
+    const float ok_f = (float)ok_frac;
+    U lo = ~(U)0, hi = 0;
+    int n = 0;
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) {
+      const uint32_t n_arr = (uint32_t)cv[u], n_met = (uint32_t)(cv[u] >> 32);
+      pv[u] = 0;
+      if (iv[u] != kIdle && n_arr >= 1 && sv[u] > (T)0) {
+        const bool h = n_arr < (uint32_t)kThrDirect ? (int64_t)n_met >= (int64_t)thr_s[n_arr]
+                                                    : at_least(n_met, n_arr, ok_frac, ok_f);
+        const U key = (U)key_of(sv[u]);
+        pv[u] = (key << 1) | (U)(h ? 1 : 0);
+        lo = key < lo ? key : lo;
+        hi = key > hi ? key : hi;
+        ++n;
+      }
+    }
+    lo = warp_min(lo);
+    hi = warp_max(hi);
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (lane == 0) {
+      redU[0][tid / 32] = lo;
+      redU[1][tid / 32] = hi;
+      red32[tid / 32] = n;
+    }
+    __syncthreads();
+    kmin = warp_min(redU[0][lane]);
+    kmax = warp_max(redU[1][lane]);
+    ncand = (uint32_t)__reduce_add_sync(0xffffffffu, red32[lane]);
+  } else {
+    ncand = ncand_g[out];
+    kmin = kmin_g[out];
+    kmax = kmax_g[out];
+  }
+  if (ncand == 0) {
     if (tid == 0) {
       theta[out] = (T)1;
       atomicAdd(&diag->degenerate_calib, 1ull);
     }
     return;
   }
-  const U kmin = kmin_g[out], kmax = kmax_g[out];
 
   // ---- fast path -----------------------------------------------------------
   // A fine histogram over [kmin, kmax]; per bucket the exact test at its
   // smallest value ("found") and the bound for values inside it ("maybe").
   // With bf the lowest found bucket, theta is either a value inside a maybe
   // bucket below bf or the smallest value of bf. Those maybe buckets' keys are
-  // gathered, sorted and tested one distinct value at a time.
+  // gathered bucket by bucket, and each is tested with the counts of the keys
+  // not below it in its own bucket: no order within a bucket is needed.
   {
-    int32_t* fcnt = reinterpret_cast<int32_t*>(dyn);
-    int32_t* fhl = fcnt + kFine;
-    int32_t* fst = fhl + kFine;                 // run start of a selected bucket, -1 if not
-    int32_t* fca = fst + kFine;                 // windows in buckets above
-    int32_t* fha = fca + kFine;                 // healthy windows in buckets above
-    U* list = reinterpret_cast<U*>(fha + kFine);
-    int32_t* hpre = reinterpret_cast<int32_t*>(list + kCap);
     int sh = 0;
     while (sh < 63 && ((kmax - kmin) >> sh) >= (U)kFine) ++sh;
-    for (int b = tid; b < kFine; b += kNB) {
-      fcnt[b] = 0;
-      fhl[b] = 0;
-    }
-    if (tid == 0) bfmin_s = ~(U)0;
     __syncthreads();
     // with fewer than 2^16 candidates, a bucket's count and healthy count
     // share one 32-bit word (one atomic per key)
-    const bool packed = ncand_g[out] < 65536u;
+    const bool packed = ncand < 65536u;
     uint32_t* fpk = reinterpret_cast<uint32_t*>(fcnt);
-    for (int i0 = 0; i0 < K; i0 += kNB * kUnroll) {
-      U pv[kUnroll];
+    auto each_key = [&](auto&& f) {
+      if (DIRECT) {
 #pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        const int i = i0 + u * kNB + tid;
-        pv[u] = i < K ? mk[i] : (U)0;
-      }
+        for (int u = 0; u < kUnroll; ++u)
+          if (pv[u]) f(pv[u], (int)(((pv[u] >> 1) - kmin) >> sh));
+      } else {
+        for (int i0 = 0; i0 < K; i0 += kNB * kUnroll) {
 #pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        const U p = pv[u];
-        if (!p) continue;
-        const int b = (int)(((p >> 1) - kmin) >> sh);
-        if (packed) {
-          atomicAdd(&fpk[b], 1u + ((uint32_t)(p & 1) << 16));
-        } else {
-          atomicAdd(&fcnt[b], 1);
-          if (p & 1) atomicAdd(&fhl[b], 1);
+          for (int u = 0; u < kUnroll; ++u) {
+            const int i = i0 + u * kNB + tid;
+            pv[u] = i < K ? mk[i] : (U)0;
+          }
+#pragma unroll
+          for (int u = 0; u < kUnroll; ++u)
+            if (pv[u]) f(pv[u], (int)(((pv[u] >> 1) - kmin) >> sh));
         }
       }
-    }
+    };
+    each_key([&](U p, int b) {
+      if (packed) {
+        atomicAdd(&fpk[b], 1u + ((uint32_t)(p & 1) << 16));
+      } else {
+        atomicAdd(&fcnt[b], 1);
+        if (p & 1) atomicAdd(&fhl[b], 1);
+      }
+    });
     __syncthreads();
     constexpr int PER = kFine / kNB;            // consecutive buckets per thread
     const int b0 = tid * PER;
-    if (packed) {
-      for (int j = 0; j < PER; ++j) {
-        const uint32_t v = fpk[b0 + j];
-        fcnt[b0 + j] = (int32_t)(v & 0xffffu);
-        fhl[b0 + j] = (int32_t)(v >> 16);
-      }
-    }
-    int64_t tc = 0, th = 0;
+    int cb[PER], hb[PER], tc = 0, th = 0;
+#pragma unroll
     for (int j = 0; j < PER; ++j) {
-      tc += fcnt[b0 + j];
-      th += fhl[b0 + j];
+      const uint32_t v = fpk[b0 + j];
+      cb[j] = packed ? (int)(v & 0xffffu) : (int)v;
+      hb[j] = packed ? (int)(v >> 16) : fhl[b0 + j];
+      tc += cb[j];
+      th += hb[j];
     }
-    int64_t c_above = block_suffix(tc, red64), h_above = block_suffix(th, red64);
-    int my_found = 0x7fffffff;
+    const int2 above = block_suffix(tc, th, red2);
+    int ca[PER], ha[PER], my_found = 0x7fffffff;
     uint32_t maybe_bits = 0;
-    for (int j = PER - 1; j >= 0; --j) {
-      const int b = b0 + j;
-      const int32_t c = fcnt[b], h = fhl[b];
-      fca[b] = (int32_t)c_above;
-      fha[b] = (int32_t)h_above;
-      if (c > 0) {
-        if ((double)(h_above + h) >= reliability * (double)(c_above + c)) {
-          my_found = b;
-        } else if ((double)(h_above + h + 1) >= reliability * (double)(c_above + h)) {
-          // a value inside adds at most the bucket's healthy windows to those
-          // above; one window of slack keeps the bound valid under rounding
-          maybe_bits |= 1u << j;
+    {
+      int c = above.x, h = above.y;
+#pragma unroll
+      for (int j = PER - 1; j >= 0; --j) {
+        ca[j] = c;
+        ha[j] = h;
+        if (cb[j] > 0) {
+          if (at_least(h + hb[j], c + cb[j], reliability, rel_f)) {
+            my_found = b0 + j;
+          } else if (at_least(h + hb[j] + 1, c + hb[j], reliability, rel_f)) {
+            // a value inside adds at most the bucket's healthy windows to those
+            // above; one window of slack keeps the bound valid under rounding
+            maybe_bits |= 1u << j;
+          }
         }
+        c += cb[j];
+        h += hb[j];
       }
-      c_above += c;
-      h_above += h;
     }
     const int bf = block_min(my_found, red32);
-    int64_t my_sel = 0;
-    for (int j = 0; j < PER; ++j)
-      if ((maybe_bits >> j & 1) && b0 + j < bf) my_sel += fcnt[b0 + j];
-    const int64_t sel_above = block_suffix(my_sel, red64);
-    if (tid == 0) nsel_s = 0;
+    int my_sel = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      if (b0 + j >= bf) maybe_bits &= ~(1u << j);
+      my_sel += maybe_bits >> j & 1u ? cb[j] : 0;
+    }
+    const int sel_above = block_suffix(my_sel, 0, red2).x;
+    if (tid == 0) red32[0] = sel_above + my_sel;
     __syncthreads();
-    if (my_sel) atomicAdd(&nsel_s, (int)my_sel);
-    __syncthreads();
-    const int nsel = nsel_s;
-    // smallest key of the found bucket bf, by a pass over the keys (the gather
-    // pass below does it on the way when there are keys to gather)
-    auto bucket_min_pass = [&]() {
-      U lm = ~(U)0;
-      for (int i = tid; i < K; i += kNB) {
-        const U p = mk[i];
-        if (p && (int)(((p >> 1) - kmin) >> sh) == bf && (p >> 1) < lm) lm = p >> 1;
-      }
-      if (lm != ~(U)0) atomicMin(&bfmin_s, lm);
-      __syncthreads();
-    };
+    const int nsel = red32[0];
     if (nsel <= kCap) {
-      if (nsel == 0) {
-        if (bf != 0x7fffffff) bucket_min_pass();
-        if (tid == 0) {
-          if (bf != 0x7fffffff) {
-            theta[out] = value_of(bfmin_s);
-          } else {
-            theta[out] = value_of(kmax);
-            atomicAdd(&diag->degenerate_calib, 1ull);
-          }
-        }
-        return;
-      }
-      // where each selected bucket's keys start in ascending order
-      int64_t run = nsel - sel_above - my_sel;
+      int run = sel_above;
+#pragma unroll
       for (int j = 0; j < PER; ++j) {
-        const int b = b0 + j;
-        if ((maybe_bits >> j & 1) && b < bf) {
-          fst[b] = (int32_t)run;
-          run += fcnt[b];
-        } else {
-          fst[b] = -1;
-        }
+        const bool on = maybe_bits >> j & 1u;
+        fst[b0 + j] = on ? run : -1;
+        fca[b0 + j] = ca[j];
+        fha[b0 + j] = ha[j];
+        fcnt[b0 + j] = cb[j];
+        fhl[b0 + j] = 0;                        // from here on: keys of the bucket listed
+        run += on ? cb[j] : 0;
       }
-      if (tid == 0) nsel_s = 0;
       __syncthreads();
-      U lmin = ~(U)0;
-      for (int i0 = 0; i0 < K; i0 += kNB * kUnroll) {
-        U pv[kUnroll];
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-          const int i = i0 + u * kNB + tid;
-          pv[u] = i < K ? mk[i] : (U)0;
-        }
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-          const U p = pv[u];
-          if (!p) continue;
-          const int b = (int)(((p >> 1) - kmin) >> sh);
-          if (fst[b] >= 0) list[atomicAdd(&nsel_s, 1)] = p;
+      if (nsel > 0 || bf != 0x7fffffff) {
+        U lmin = ~(U)0;
+        each_key([&](U p, int b) {
+          const int st = fst[b];
+          if (st >= 0) list[st + atomicAdd(&fhl[b], 1)] = p;
           if (b == bf && (p >> 1) < lmin) lmin = p >> 1;
-        }
-      }
-      if (lmin != ~(U)0) atomicMin(&bfmin_s, lmin);
-      int n2 = 32;
-      while (n2 < nsel) n2 <<= 1;
-      for (int i = nsel + tid; i < n2; i += kNB) list[i] = ~(U)0;
-      __syncthreads();
-      for (int k2 = 2; k2 <= n2; k2 <<= 1) {       // bitonic sort, ascending
-        for (int j2 = k2 >> 1; j2 > 0; j2 >>= 1) {
-          for (int i = tid; i < n2; i += kNB) {
-            const int ixj = i ^ j2;
-            if (ixj > i) {
-              const U a = list[i], c = list[ixj];
-              if ((a > c) == ((i & k2) == 0)) {
-                list[i] = c;
-                list[ixj] = a;
-              }
-            }
+        });
+        if (lmin != ~(U)0) atomicMin(&bfmin_s, lmin);
+        __syncthreads();
+        U best = ~(U)0;
+        for (int i = tid; i < nsel; i += kNB) {
+          const U key = list[i] >> 1;
+          const int b = (int)((key - kmin) >> sh);
+          const int st = fst[b], e = st + fcnt[b];
+          int C = fca[b], H = fha[b];
+          for (int j = st; j < e; ++j) {
+            const U o = list[j];
+            const bool ge = (o >> 1) >= key;
+            C += ge;
+            H += ge && (o & 1);
           }
-          __syncthreads();
+          if (key < best && at_least(H, C, reliability, rel_f)) best = key;
         }
+        if (best != ~(U)0) atomicMin(&best_s, best);
+        __syncthreads();
       }
-      // inclusive healthy prefix over the sorted keys
-      constexpr int PERC = kCap / kNB;
-      int hs = 0;
-      for (int j = 0; j < PERC; ++j) {
-        const int i = tid * PERC + j;
-        if (i < nsel) hs += (int)(list[i] & 1);
-      }
-      const int64_t h_after = block_suffix(hs, red64);
-      if (tid == 0) red64[0] = h_after + hs;       // total
-      __syncthreads();
-      int64_t hp = red64[0] - (h_after + hs);
-      __syncthreads();
-      for (int j = 0; j < PERC; ++j) {
-        const int i = tid * PERC + j;
-        if (i < nsel) hp += (int64_t)(list[i] & 1);
-        hpre[i] = (int32_t)hp;
-      }
-      __syncthreads();
-      // exact test at the first position of every distinct value
-      int best = 0x7fffffff;
-      for (int i = tid; i < nsel; i += kNB) {
-        const U key = list[i] >> 1;
-        if (i > 0 && (list[i - 1] >> 1) == key) continue;
-        const int b = (int)((key - kmin) >> sh);
-        const int end = fst[b] + fcnt[b];
-        const int64_t C = (int64_t)fca[b] + (end - i);
-        const int64_t H = (int64_t)fha[b] + hpre[end - 1] - (i > 0 ? hpre[i - 1] : 0);
-        if ((double)H >= reliability * (double)C) best = min(best, i);
-      }
-      best = block_min(best, red32);
       if (tid == 0) {
-        if (best != 0x7fffffff) {
-          theta[out] = value_of(list[best] >> 1);
+        if (best_s != ~(U)0) {
+          theta[out] = value_of(best_s);
         } else if (bf != 0x7fffffff) {
           theta[out] = value_of(bfmin_s);
         } else {
@@ -552,6 +582,12 @@ k_search(const __grid_constant__ SeriesTable<T> tab, const typename KeyOf<T>::U*
       }
       return;
     }
+  }
+  if (DIRECT) {
+    // the descent reads the keys from memory
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u)
+      if (u * kNB + tid < K) mk[u * kNB + tid] = pv[u];
   }
   __syncthreads();
 
@@ -585,7 +621,7 @@ k_search(const __grid_constant__ SeriesTable<T> tab, const typename KeyOf<T>::U*
     }
     __syncthreads();
   };
-  auto set_range = [&](int l, U lo, U hi, int64_t ca, int64_t ha) {
+  auto set_range = [&](int l, U lo, U hi, int ca, int ha) {
     int sh = 0;
     while (sh < 63 && ((hi - lo) >> sh) >= (U)kNB) ++sh;
     lo_s[l] = lo;
@@ -600,8 +636,8 @@ k_search(const __grid_constant__ SeriesTable<T> tab, const typename KeyOf<T>::U*
   build(0);
   int l = 0;
   while (true) {
-    const int64_t c_above = block_suffix(cnt[l][tid], red64) + cab_s[l];
-    const int64_t h_above = block_suffix(hl[l][tid], red64) + hab_s[l];
+    const int2 up = block_suffix(cnt[l][tid], hl[l][tid], red2);
+    const int c_above = up.x + cab_s[l], h_above = up.y + hab_s[l];
     const int32_t c = cnt[l][tid], h = hl[l][tid];
     int cand = 0x7fffffff;
     int kind = 0;   // 1 = its smallest value qualifies, 2 = may contain one
@@ -668,6 +704,20 @@ cudaError_t launch_calibrate(const SeriesTable<T>& tab, const T* S, const uint8_
   if (n_sm > w.n_sm) return cudaErrorInvalidValue;
   U* kmin = static_cast<U*>(w.kmin);
   U* kmax = static_cast<U*>(w.kmax);
+  const size_t smem = search_smem_bytes<T>();
+  bool direct = true;
+  int64_t cells = 0;
+  for (int i = 0; i < tab.n; ++i) {
+    direct = direct && tab.K[i] <= kDirectK;
+    cells += (int64_t)tab.K[i] * tab.M;
+  }
+  if (direct && cells <= kDirectCells) {
+    cudaError_t e = func_smem_once((const void*)k_search<T, true>, (int)smem, true);
+    if (e) return e;
+    k_search<T, true><<<n_sm, kNB, smem, s>>>(tab, static_cast<U*>(w.keys), kmin, kmax, w.ncand, S,
+                                              cls, slo, ok_frac, reliability, theta, diag);
+    return cudaGetLastError();
+  }
   const int thr_n = std::max(kThrTable, n_sm);
   k_thr<U><<<(thr_n + 255) / 256, 256, 0, s>>>(ok_frac, w.thr, n_sm, kmin, kmax, w.ncand);
   PackPlan pp;
@@ -692,12 +742,11 @@ cudaError_t launch_calibrate(const SeriesTable<T>& tab, const T* S, const uint8_
   else if (tiles > 0)
     k_pack<T><<<tiles, kPackThreads, 0, s>>>(tab, pp, S, cls, slo, w.thr, ok_frac,
                                              static_cast<U*>(w.keys), kmin, kmax, w.ncand);
-  const size_t smem = search_smem_bytes<T>();
   // the largest carveout lets two searches share an SM where their tables fit
-  cudaError_t e = func_smem_once((const void*)k_search<T>, (int)smem, true);
+  cudaError_t e = func_smem_once((const void*)k_search<T, false>, (int)smem, true);
   if (e) return e;
-  k_search<T><<<tab.n * tab.M, kNB, smem, s>>>(tab, static_cast<const U*>(w.keys), kmin, kmax,
-                                               w.ncand, reliability, theta, diag);
+  k_search<T, false><<<n_sm, kNB, smem, s>>>(tab, static_cast<U*>(w.keys), kmin, kmax, w.ncand, S,
+                                             cls, slo, ok_frac, reliability, theta, diag);
   return cudaGetLastError();
 }
 

@@ -800,6 +800,51 @@ def test_reduce_requests_1024_models(tre, where):
     assert [d["dropped_range"], d["dropped_model"], d["dropped_order"]] == drops.tolist()
 
 
+# Series of up to 8192 windows (and tables of up to 2^18 cells) are searched
+# without packing their keys. With reliability near the healthy share the
+# running shares hover around it: many buckets may hold the boundary, up to the
+# descent over the key range; few levels of S put many equal keys in a bucket.
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("levels", [0, 40])
+@pytest.mark.parametrize("K,M", [(1, 1), (63, 3), (1024, 2), (8192, 2), (8193, 2), (7000, 37),
+                                 (7100, 37)])
+def test_calibrate_search_edges(tre, dtype, levels, K, M):
+    rng = np.random.default_rng(K + M + levels)
+    npdt = np.float32 if dtype == "f32" else np.float64
+    win = 1000
+    cnt = {k: np.zeros((K, M), np.int32) for k in "PDAW"}
+    cnt["D"] = (rng.integers(1, levels + 1, (K, M)) if levels
+                else rng.integers(1, 1 << 24, (K, M))).astype(np.int32)
+    cnt["D"][rng.random((K, M)) < 0.05] = 0
+    cnt["A"][:] = cnt["D"] > 0
+    prof = {"w_p": 0.25, "w_q": 2.0, "alpha": 1.0, "theta": 1.0, "tau_crit": 0.8,
+            "tau_surplus": 1.2}
+    n = 300 if M == 1 else 2 * K * M
+    model, w = rng.integers(0, M, n), np.sort(rng.integers(0, K, n))
+    if K == 63:
+        w[:] = w // 8 * 8                       # more than 256 arrivals in a window
+        model[:] = 0
+        model, w = np.repeat(model, 20), np.repeat(w, 20)
+        n = len(w)
+    ok = rng.random(n) < 0.97
+    ta = w * win
+    req = {"model": model, "t_arr_ms": ta, "t_start_ms": ta,
+           "t_first_ms": ta + np.where(ok, 100, 5000), "L_in": np.ones(n), "L_out": np.ones(n)}
+    req["t_end_ms"] = req["t_first_ms"]
+    req = {k: req[k].astype(np.int32) for k in REQ_KEYS}
+    slo = np.full(M, 1000, np.int32)
+    S, _, cls, _ = oracle.score(cnt["P"], cnt["D"], cnt["A"], cnt["W"], prof, win, npdt)
+    n_arr, n_met = oracle.slo_counts_requests(req, M, win, K, slo)
+    share = float((n_met >= 0.95 * n_arr)[n_arr > 0].mean())
+    for rho in (share, 0.5, 1.0, 0.95, float("nan"), -1.0):
+        theta, deg = oracle.calibrate(S, cls, n_arr, n_met, 0.95, rho)
+        diag = tre.new_diag()
+        th = tre.tss_calibrate(_cuda(cnt), prof, win, slo, requests=_cuda(req), dtype=dtype,
+                               reliability=rho, diag=diag)
+        np.testing.assert_array_equal(_np(th), theta, err_msg=f"rho {rho}")
+        assert tre.read_diag(diag)["degenerate_calib"] == deg
+
+
 def test_calibrate_1024_models(tre):
     import torch
     rng = np.random.default_rng(4)
