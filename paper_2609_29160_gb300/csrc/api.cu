@@ -177,17 +177,13 @@ tre_status score_typed(const tre_grid* g, const tre_counts* in, const tre_profil
   if (st != TRE_OK || query) return st;
   cudaError_t e;
   {
-    Scope sc(kScore, score_launches(tab), s);
+    Scope sc(kScore, score_launches(tab, true), s);
     e = launch_score<T>(tab, in->P, in->D, in->A, in->W, static_cast<const T*>(p->w_p),
                         static_cast<const T*>(p->w_q), static_cast<const T*>(p->alpha),
                         static_cast<const T*>(p->theta), static_cast<const T*>(p->tau_crit),
                         static_cast<const T*>(p->tau_surplus), static_cast<T*>(S_carry),
-                        init_carry, static_cast<T*>(S_out), static_cast<T*>(Z_out), cls_out, w,
-                        diag, s, in->A_ms, in->W_ms);
-  }
-  if (!e && recv_out) {
-    Scope sc(kReceiver, 1, s);
-    e = launch_receiver<T>(M, K, static_cast<const T*>(Z_out), cls_out, recv_out, s);
+                        init_carry, static_cast<T*>(S_out), static_cast<T*>(Z_out), cls_out,
+                        recv_out, w, diag, s, in->A_ms, in->W_ms);
   }
   return cuda_status(e);
 }
@@ -222,10 +218,10 @@ tre_status calibrate_typed(const tre_grid* g, const tre_requests* req, const tre
             : launch_slo_events(cols_of(ev), M, g->window_ms, K, slo, slo_ms, s);
   }
   if (!e) {
-    Scope sc(kScore, score_launches(tab), s);
+    Scope sc(kScore, score_launches(tab, false), s);
     e = launch_score<T>(tab, in->P, in->D, in->A, in->W, static_cast<const T*>(p->w_p),
                         static_cast<const T*>(p->w_q), static_cast<const T*>(p->alpha), nullptr,
-                        nullptr, nullptr, nullptr, nullptr, S, nullptr, cls, sw, diag, s,
+                        nullptr, nullptr, nullptr, nullptr, S, nullptr, cls, nullptr, sw, diag, s,
                         in->A_ms, in->W_ms);
   }
   if (!e) {
@@ -485,10 +481,10 @@ tre_status sweep_typed(const tre_sweep_spec* sp, const SweepPlan& pl, const tre_
     }
   }
   if (!e) {
-    Scope sc(kScore, score_launches(tab), s);
+    Scope sc(kScore, score_launches(tab, false), s);
     e = launch_score<T>(tab, P, D, A, W, static_cast<const T*>(sp->w_p),
                         static_cast<const T*>(sp->w_q), nullptr, nullptr, nullptr, nullptr,
-                        nullptr, nullptr, S, nullptr, idle, sw, diag, s);
+                        nullptr, nullptr, S, nullptr, idle, nullptr, sw, diag, s);
   }
   if (!e) {
     Scope sc(kCalibrate, 3, s);
@@ -497,7 +493,7 @@ tre_status sweep_typed(const tre_sweep_spec* sp, const SweepPlan& pl, const tre_
   if (!e) {
     Scope sc(kNormalize, 1, s);
     e = launch_normalize<T>(tab, S, idle, theta, nullptr, to_t<T>(sp->tau_crit[0]),
-                            static_cast<const T*>(sp->tau_surplus), Z, out->cls, s);
+                            static_cast<const T*>(sp->tau_surplus), Z, out->cls, nullptr, s);
   }
   if (e) return TRE_ECUDA;
   Scope sc(kSelect, 2, s);
@@ -549,9 +545,9 @@ tre_status stage_calibrate_typed(const tre_grid* g, const tre_requests* req, con
   if (!e) e = launch_fill<T>(ones, M, (T)1, s);
   // prefill: (P/dt) / max(A_prefill + w_q W, 1), calibrated on TTFT
   if (!e) {
-    Scope sc(kScore, score_launches(tab), s);
+    Scope sc(kScore, score_launches(tab, false), s);
     e = launch_score<T>(tab, in->P, zero, A_pre, in->W, ones, w_q, alpha, nullptr, nullptr,
-                        nullptr, nullptr, nullptr, S, nullptr, cls, sw, diag, s);
+                        nullptr, nullptr, nullptr, S, nullptr, cls, nullptr, sw, diag, s);
   }
   if (!e) {
     Scope sc(kCalibrate, 3, s);
@@ -559,9 +555,9 @@ tre_status stage_calibrate_typed(const tre_grid* g, const tre_requests* req, con
   }
   // decode: (D/dt) / max(A_decode, 1), calibrated on TPOT
   if (!e) {
-    Scope sc(kScore, score_launches(tab), s);
+    Scope sc(kScore, score_launches(tab, false), s);
     e = launch_score<T>(tab, zero, in->D, A_dec, zero, w_p, w_q, alpha, nullptr, nullptr,
-                        nullptr, nullptr, nullptr, S, nullptr, cls, sw, diag, s);
+                        nullptr, nullptr, nullptr, S, nullptr, cls, nullptr, sw, diag, s);
   }
   if (!e) {
     Scope sc(kCalibrate, 3, s);
@@ -594,16 +590,16 @@ tre_status stage_score_typed(const tre_grid* g, const tre_counts* in, const int3
   cudaError_t e = cudaMemsetAsync(zero, 0, cells * sizeof(int32_t), s);
   if (!e) e = launch_fill<T>(ones, M, (T)1, s);
   if (!e) {
-    Scope sc(kScore, score_launches(tab), s);
+    Scope sc(kScore, score_launches(tab, true), s);
     e = launch_score<T>(tab, in->P, zero, A_pre, in->W, ones, w_q, alpha,
                         static_cast<const T*>(th_pre), tc, tsu, nullptr, nullptr,
-                        static_cast<T*>(S_pre), static_cast<T*>(Z_pre), cls_pre, sw, diag, s);
+                        static_cast<T*>(S_pre), static_cast<T*>(Z_pre), cls_pre, nullptr, sw, diag, s);
   }
   if (!e) {
-    Scope sc(kScore, score_launches(tab), s);
+    Scope sc(kScore, score_launches(tab, true), s);
     e = launch_score<T>(tab, zero, in->D, A_dec, zero, static_cast<const T*>(p->w_p), w_q,
                         alpha, static_cast<const T*>(th_dec), tc, tsu, nullptr, nullptr,
-                        static_cast<T*>(S_dec), static_cast<T*>(Z_dec), cls_dec, sw, diag, s);
+                        static_cast<T*>(S_dec), static_cast<T*>(Z_dec), cls_dec, nullptr, sw, diag, s);
   }
   return cuda_status(e);
 }
@@ -802,38 +798,24 @@ tre_status tss_normalize(const tre_grid* grid, const tre_profile* prof, const vo
   if (!grid_ok(grid) || !prof_ok(prof, true)) return TRE_EINVAL;
   if (grid->n_windows > 0 && (!S || !idle_cls || !Z_out || !cls_out)) return TRE_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const int M = grid->n_models, K = grid->n_windows;
-  if (K == 0) return TRE_OK;
+  if (grid->n_windows == 0) return TRE_OK;
   cudaError_t e;
   if (prof->dtype == TRE_F32) {
     const SeriesTable<float> tab = single_series<float>(grid);
-    {
-      Scope sc(kNormalize, 1, s);
-      e = launch_normalize<float>(tab, static_cast<const float*>(S), idle_cls,
-                                  static_cast<const float*>(prof->theta),
-                                  static_cast<const float*>(prof->tau_crit), 0.f,
-                                  static_cast<const float*>(prof->tau_surplus),
-                                  static_cast<float*>(Z_out), cls_out, s);
-    }
-    if (!e && recv_out) {
-      Scope sc(kReceiver, 1, s);
-      e = launch_receiver<float>(M, K, static_cast<const float*>(Z_out), cls_out, recv_out, s);
-    }
+    Scope sc(kNormalize, 1, s);
+    e = launch_normalize<float>(tab, static_cast<const float*>(S), idle_cls,
+                             static_cast<const float*>(prof->theta),
+                             static_cast<const float*>(prof->tau_crit), 0.f,
+                             static_cast<const float*>(prof->tau_surplus),
+                             static_cast<float*>(Z_out), cls_out, recv_out, s);
   } else {
     const SeriesTable<double> tab = single_series<double>(grid);
-    {
-      Scope sc(kNormalize, 1, s);
-      e = launch_normalize<double>(tab, static_cast<const double*>(S), idle_cls,
-                                   static_cast<const double*>(prof->theta),
-                                   static_cast<const double*>(prof->tau_crit), 0.0,
-                                   static_cast<const double*>(prof->tau_surplus),
-                                   static_cast<double*>(Z_out), cls_out, s);
-    }
-    if (!e && recv_out) {
-      Scope sc(kReceiver, 1, s);
-      e = launch_receiver<double>(M, K, static_cast<const double*>(Z_out), cls_out, recv_out,
-                                  s);
-    }
+    Scope sc(kNormalize, 1, s);
+    e = launch_normalize<double>(tab, static_cast<const double*>(S), idle_cls,
+                             static_cast<const double*>(prof->theta),
+                             static_cast<const double*>(prof->tau_crit), 0.0,
+                             static_cast<const double*>(prof->tau_surplus),
+                             static_cast<double*>(Z_out), cls_out, recv_out, s);
   }
   return cuda_status(e);
 }

@@ -186,28 +186,26 @@ template <class T> void score_ws_layout(Arena& a, int M, int64_t elems, int n_se
 // table's per-series value is used); theta null = S only (cls = IDLE / NOM).
 // The carries (device [M], may be null) apply to a one-series table.
 // kernels one launch_score call issues (for the phase trace)
-template <class T> int score_launches(const SeriesTable<T>& tab);
+template <class T> int score_launches(const SeriesTable<T>& tab, bool with_z);
 template <class T>
 cudaError_t launch_score(const SeriesTable<T>& tab, const int32_t* P, const int32_t* D,
                          const int32_t* A, const int32_t* W, const T* w_p, const T* w_q,
                          const T* alpha, const T* theta, const T* tau_crit, const T* tau_surp,
                          T* S_carry, uint8_t* init_carry, T* S, T* Z, uint8_t* cls,
-                         ScoreWs<T>& w, tre_diag* diag, cudaStream_t s,
+                         int32_t* recv, ScoreWs<T>& w, tre_diag* diag, cudaStream_t s,
                          const int64_t* A_ms = nullptr, const int64_t* W_ms = nullptr);
 // Z = S / theta[series][m] and regions for every series (tau_crit device [M] or
-// one value for all)
+// one value for all); with recv (a one-series table, tau_crit per model) also
+// the Eq. 3 receiver of every window
 template <class T>
 cudaError_t launch_normalize(const SeriesTable<T>& tab, const T* S, const uint8_t* idle_cls,
                              const T* theta, const T* tau_crit, T tau_crit_v, const T* tau_surp,
-                             T* Z, uint8_t* cls, cudaStream_t s);
+                             T* Z, uint8_t* cls, int32_t* recv, cudaStream_t s);
 // donors listed per window by tss_rank
 constexpr int kRankDonors = 8;
 template <class T>
 cudaError_t launch_rank(int M, int K, const T* Z, const uint8_t* cls, int32_t* recv,
                         int32_t* donors, cudaStream_t s);
-template <class T>
-cudaError_t launch_receiver(int M, int K, const T* Z, const uint8_t* cls, int32_t* recv,
-                            cudaStream_t s);
 
 // ---- calibrate.cu ---------------------------------------------------------
 template <class T> struct CalibWs {

@@ -75,17 +75,13 @@ tre_status run(const tre_grid* g, const tre_counts* in, const tre_profile* p, vo
   score_ws_layout<T>(a, M, elems, n_seg, w);
   cudaError_t e;
   {
-    Scope sc(kScore, score_launches(tab), s);
+    Scope sc(kScore, score_launches(tab, true), s);
     e = launch_score<T>(tab, in->P, in->D, in->A, in->W, static_cast<const T*>(p->w_p),
                         static_cast<const T*>(p->w_q), static_cast<const T*>(p->alpha),
                         static_cast<const T*>(p->theta), static_cast<const T*>(p->tau_crit),
                         static_cast<const T*>(p->tau_surplus), static_cast<T*>(S_carry),
-                        init_carry, static_cast<T*>(S_out), static_cast<T*>(Z_out), cls_out, w,
-                        diag, s, in->A_ms, in->W_ms);
-  }
-  if (!e && recv_out) {
-    Scope sc(kReceiver, 1, s);
-    e = launch_receiver<T>(M, K, static_cast<const T*>(Z_out), cls_out, recv_out, s);
+                        init_carry, static_cast<T*>(S_out), static_cast<T*>(Z_out), cls_out,
+                        recv_out, w, diag, s, in->A_ms, in->W_ms);
   }
   return e == cudaSuccess ? TRE_OK : TRE_ECUDA;
 }

@@ -11,7 +11,7 @@
 //      so a start error shrinks by e^-c before the chunk: c = 28 for float, 45
 //      for double), records the state
 //      it reached, then runs its chunk from that state and stores the result;
-//   2. one thread per model walks the chunk boundaries in order: a chunk whose
+//   2. one CTA per (series, model) checks the chunk boundaries: a chunk whose
 //      recorded burn-in state equals its predecessor's exact end state (bit
 //      for bit, with the same started/not-started flag) is exact, because
 //      every step depends only on the previous state; any other chunk is run
@@ -60,19 +60,15 @@ template <class T> __device__ __forceinline__ int series_of_seg(const SeriesTabl
 }
 
 template <class T> struct ModelParams {
-  T a, b, th, tc, ts;
+  T a, b;
 };
 
 template <class T>
 __device__ __forceinline__ ModelParams<T> load_params(const SeriesTable<T>& t, int s, int m,
-                                                      const T* alpha, const T* theta,
-                                                      const T* tau_crit, const T* tau_surp) {
+                                                      const T* alpha) {
   ModelParams<T> p;
   p.a = alpha ? alpha[m] : t.alpha[s];
   p.b = sub_rn<T>((T)1, p.a);
-  p.th = theta ? theta[m] : (T)1;
-  p.tc = tau_crit ? tau_crit[m] : (T)0;
-  p.ts = tau_surp ? tau_surp[m] : (T)0;
   return p;
 }
 
@@ -88,12 +84,17 @@ __device__ __forceinline__ bool is_idle_raw(double r) {
 }
 
 // ---- pass 0: Eq. 1 for every (window, model) of every series ---------------
-// Element-wise passes run over tiles of kTile consecutive elements of one
-// series; a thread takes four consecutive elements, with 16-byte loads and
+// Element-wise passes run over tiles of consecutive elements of one series. On
+// large tables a thread takes four consecutive elements, with 16-byte loads and
 // stores when they are aligned (scalar ones otherwise), so that enough bytes
-// are in flight to cover memory latency.
+// are in flight to cover memory latency. Below kSmallCells a thread takes one
+// element and a CTA has four warps, one per scheduler: the divisions of an
+// element are its latency (64 cycles an operation in double), and a small table
+// leaves the SMs idle anyway (3 models, 600 windows in double: Eq. 1 14.3 us on
+// two CTAs).
 constexpr int kEwThreads = 256;
-constexpr int kTile = 4 * kEwThreads;
+constexpr int kSmallThreads = 128;
+constexpr int64_t kSmallCells = 1 << 18;
 struct TilePlan {
   int tile_base[kMaxSeries + 1];   // prefix of tiles per series
 };
@@ -124,7 +125,7 @@ __device__ __forceinline__ T raw_tss_mean(int32_t p, int32_t d, long long a_ms, 
   return div_rn(num, den);
 }
 
-template <class T, bool MEAN>
+template <class T, bool MEAN, int EPT>
 __global__ void __launch_bounds__(kEwThreads)
 k_raw(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ TilePlan tp, FastDiv fm,
       bool vec, Counts c, const T* __restrict__ w_p, const T* __restrict__ w_q,
@@ -132,14 +133,14 @@ k_raw(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ TilePl
   const int s = prefix_index(tp.tile_base, tab.n, blockIdx.x);
   const int M = tab.M;
   const int64_t n = (int64_t)tab.K[s] * M;
-  const int64_t l0 = (int64_t)(blockIdx.x - tp.tile_base[s]) * kTile + 4 * threadIdx.x;
+  const int64_t l0 = ((int64_t)(blockIdx.x - tp.tile_base[s]) * blockDim.x + threadIdx.x) * EPT;
   if (l0 >= n) return;
   const size_t x0 = (size_t)(tab.off[s] + l0);
   const T dt = div_rn((T)tab.win[s], (T)1000);      // window length in seconds
-  int32_t p[4], d[4], a[4], w[4];
-  long long am[4], wm[4];
-  const bool v4 = vec && l0 + 4 <= n;
-  if (v4) {
+  int32_t p[EPT], d[EPT], a[EPT], w[EPT];
+  long long am[EPT], wm[EPT];
+  const bool v4 = EPT == 4 && vec && l0 + 4 <= n;
+  if constexpr (EPT == 4) if (v4) {
     const int4 P4 = *reinterpret_cast<const int4*>(c.P + x0);
     const int4 D4 = *reinterpret_cast<const int4*>(c.D + x0);
     p[0] = P4.x; p[1] = P4.y; p[2] = P4.z; p[3] = P4.w;
@@ -158,9 +159,10 @@ k_raw(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ TilePl
       a[0] = A4.x; a[1] = A4.y; a[2] = A4.z; a[3] = A4.w;
       w[0] = W4.x; w[1] = W4.y; w[2] = W4.z; w[3] = W4.w;
     }
-  } else {
+  }
+  if (!v4) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < EPT; ++i) {
       const bool in = l0 + i < n;
       p[i] = in ? c.P[x0 + i] : 0;
       d[i] = in ? c.D[x0 + i] : 0;
@@ -175,10 +177,10 @@ k_raw(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ TilePl
   }
   int m = l0 <= 0xffffffffll ? (int)((uint32_t)l0 - fm.div((uint32_t)l0) * (uint32_t)M)
                              : (int)(l0 % M);
-  T rv[4];
-  uint8_t cv[4];
+  T rv[EPT];
+  uint8_t cv[EPT];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < EPT; ++i) {
     bool idle;
     if (MEAN) {
       idle = (p[i] | d[i]) == 0 && (am[i] | wm[i]) == 0;
@@ -191,17 +193,15 @@ k_raw(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ TilePl
     cv[i] = idle ? kIdle : kNom;
     if (++m == M) m = 0;
   }
-  if (v4) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) raw[x0 + i] = rv[i];
-    *reinterpret_cast<uchar4*>(cls + x0) = make_uchar4(cv[0], cv[1], cv[2], cv[3]);
-  } else {
+  for (int i = 0; i < EPT; ++i)
+    if (v4 || l0 + i < n) raw[x0 + i] = rv[i];
+  if constexpr (EPT == 4)
+    if (v4) *reinterpret_cast<uchar4*>(cls + x0) = make_uchar4(cv[0], cv[1], cv[2], cv[3]);
+  if (!v4) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (l0 + i < n) {
-        raw[x0 + i] = rv[i];
-        cls[x0 + i] = cv[i];
-      }
+    for (int i = 0; i < EPT; ++i)
+      if (l0 + i < n) cls[x0 + i] = cv[i];
   }
 }
 
@@ -231,16 +231,15 @@ __device__ __forceinline__ void load_batch(const T* __restrict__ raw, const uint
   }
 }
 
-// Run windows [k0, k1) of model m exactly from (S, init), writing S and, with
-// `with_z`, Z and the region (idle windows keep their class). With `verify`,
-// stop at the first window whose new S equals the stored one with the same
-// init state: from there the stored trajectory is the one this start produces.
-// Returns true if it stopped early.
+// Run windows [k0, k1) of model m exactly from (S, init), writing S. With
+// `verify`, stop at the first window whose new S equals the stored one with the
+// same init state: from there the stored trajectory is the one this start
+// produces. Returns true if it stopped early.
 template <class T, bool WRITE = true>
 __device__ __forceinline__ bool run_segment(size_t base, int M, int64_t k0, int64_t k1,
                                             const T* __restrict__ raw, const ModelParams<T>& q,
                                             T& S, int& init, bool verify, int stored_init,
-                                            T* S_out, T* Z_out, uint8_t* cls, bool with_z) {
+                                            T* S_out, const uint8_t* __restrict__ cls) {
   T r[kBatch], rn[kBatch];
   uint8_t c[kBatch], cn[kBatch];
   load_batch(raw, cls, base, M, k0, k1, r, c);
@@ -256,8 +255,7 @@ __device__ __forceinline__ bool run_segment(size_t base, int M, int64_t k0, int6
 #pragma unroll
     for (int j = 0; j < kBatch; ++j) {
       if (k + j >= k1) break;
-      const bool active = c[j] != kIdle;
-      if (active) {
+      if (c[j] != kIdle) {
         if (!init) {
           S = r[j];
           init = 1;
@@ -268,14 +266,7 @@ __device__ __forceinline__ bool run_segment(size_t base, int M, int64_t k0, int6
       }
       if (verify && init == stored_init && same_bits(S, old[j])) return true;
       if (!WRITE) continue;
-      const size_t x = base + (size_t)(k + j) * M;
-      const T Sv = init ? S : (T)0;
-      S_out[x] = Sv;
-      if (with_z) {
-        const T Z = div_rn(Sv, q.th);
-        Z_out[x] = Z;
-        if (active) cls[x] = Z < q.tc ? kCrit : (Z > q.ts ? kSurp : kNom);
-      }
+      S_out[base + (size_t)(k + j) * M] = init ? S : (T)0;
     }
 #pragma unroll
     for (int j = 0; j < kBatch; ++j) {
@@ -331,99 +322,126 @@ k_active(const __grid_constant__ SeriesTable<T> tab, FastDiv fm, const uint8_t* 
     active[(size_t)seg * M + m] = rows - s_idle[m];
 }
 
-// ---- pass 1: burn-in and chunk run, one thread per (chunk, model) ----------
-// Each thread streams its model's windows through its own slots of a shared
-// memory ring with asynchronous copies (cp.async, kStages groups of kBlk
-// windows in flight), so the dependent chain reads shared memory while the
-// next windows are on their way.
-constexpr int kEmaThreads = 32;    // few chains in all: spread them over every SM
-constexpr int kBlk = 16;           // windows per copy group
-constexpr int kStages = 8;         // copy groups in flight
-constexpr int kRingStride = 64;    // chunk and burn-in lengths are multiples of this
+// ---- pass 1: burn-in and chunk run, one lane per (chunk, model) -------------
+// A CTA runs 32 chains, one per lane, in groups of kGroup windows. Three warps
+// load the groups in turn and lay them in shared memory, one stage each; one runs
+// the recurrences and writes S to shared memory; one stores S. They meet at named
+// barriers, a pair per stage, so that none waits for another's whole group. The
+// dependent chain is what bounds it (a product and a sum a window: 8.6 cycles in
+// float, 128 in double, whose products and sums take 64 cycles each on this part
+// and do not overlap within a warp), so its warp does little else: it moves four
+// (in double two) windows with one 16-byte shared-memory access (a 4-byte store a
+// window cost as much as the chain), and in double the product with alpha is the
+// loaders' (warps 1 to 3 sit on other schedulers, with FP64 units of their own).
+// One warp that copied, ran and stored took 37 cycles a window in float, 270 in
+// double: 3 models, 600 windows in double 69 us, now 30.5; 8 models, 36,000
+// windows in float 10.5, now 8.1; 64 models, 864,000 windows 204, now 149.
+constexpr int kChains = 32;        // chains per CTA
+constexpr int kLoaders = 3;
+constexpr int kEmaThreads = 32 * (kLoaders + 2);
+constexpr int kGroup = 32;         // windows per group
 constexpr int kMaxBurn = 16384;    // burn-in cap (tiny alpha: the in-order pass repairs)
 constexpr int64_t kActiveMinCells = 1 << 22;   // series cells from which burn-ins skip idle chunks
 constexpr int64_t kEmaChains = 32768;         // (chunk, model) chains a long table is cut into
+constexpr int64_t kShortChains = 16384;       // most chains a table is cut into by short chunks
+// chunk and burn-in lengths are multiples of the group; short chunks are one
+// group in double, two in float, where a chain's start costs as much as a group
+template <class T> constexpr int short_chunk() { return sizeof(T) == 8 ? kGroup : 2 * kGroup; }
 
-template <int BYTES>
-__device__ __forceinline__ void cp_async(void* smem, const void* gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(sa), "l"(gmem), "n"(BYTES)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-template <int N> __device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
+// The chain's input for one window: raw, or in double alpha * raw
+template <class T> constexpr bool kPremul = sizeof(T) == 8;
 
-// One group of kBlk windows of the chain, read from its ring stage. FULL: all
-// kBlk windows exist; STARTED: the chain has seen a non-idle window already
-// (then the step is branch-free); STORE: write S (and Z, regions with WITHZ).
-template <class T, bool FULL, bool STARTED, bool STORE, bool WITHZ>
-__device__ __forceinline__ void ema_group(const T* src, int n, const ModelParams<T>& q, T& S,
-                                          int& init, T*& sp, int M, T* S_out, T* Z_out,
-                                          uint8_t* cls) {
-  T r[kBlk];
+// Consecutive windows of one chain, moved together; a stage holds [kGroup / V]
+// rows of one such quad (pair) per chain.
+template <class T> struct __align__(16) Windows {
+  static constexpr int V = 16 / sizeof(T);
+  T x[V];
+};
+
+// One group of windows of the chains; idle windows (and the padding of a lane's
+// missing groups) carry the marker and leave S as it is. x: the chain's input,
+// raw: the Eq. 1 values. STARTED: every lane has seen a non-idle window; STORE:
+// write S.
+template <class T, bool STARTED, bool STORE>
+__device__ __forceinline__ void ema_group(const Windows<T>* x, const Windows<T>* raw,
+                                          Windows<T>* dst, const ModelParams<T>& q, T& S,
+                                          int& init) {
+  constexpr int V = Windows<T>::V, N = kGroup / V;
+  Windows<T> v[N];
 #pragma unroll
-  for (int j = 0; j < kBlk; ++j) r[j] = src[j * kEmaThreads];
+  for (int h = 0; h < N; ++h) v[h] = x[h * kChains];
 #pragma unroll
-  for (int j = 0; j < kBlk; ++j) {
-    if (!FULL && j >= n) break;
-    const bool idle = is_idle_raw(r[j]);
-    if (STARTED) {
-      const T nxt = add_rn(mul_rn(q.a, r[j]), mul_rn(q.b, S));
-      S = idle ? S : nxt;
-    } else if (!idle) {
-      S = init ? add_rn(mul_rn(q.a, r[j]), mul_rn(q.b, S)) : r[j];
-      init = 1;
-    }
-    if (STORE) {
-      const T Sv = (STARTED || init) ? S : (T)0;
-      *sp = Sv;
-      if (WITHZ) {
-        const size_t x = (size_t)(sp - S_out);
-        const T Z = div_rn(Sv, q.th);
-        Z_out[x] = Z;
-        if (!idle) cls[x] = Z < q.tc ? kCrit : (Z > q.ts ? kSurp : kNom);
+  for (int h = 0; h < N; ++h) {
+    Windows<T> o;
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+      const T in = v[h].x[j];
+      const bool idle = is_idle_raw(in);
+      const T nxt = add_rn(kPremul<T> ? in : mul_rn(q.a, in), mul_rn(q.b, S));
+      if (STARTED) {
+        S = idle ? S : nxt;
+      } else if (!idle) {
+        S = init ? nxt : raw[h * kChains].x[j];
+        init = 1;
       }
-      sp += M;
+      o.x[j] = S;                              // 0 until the chain starts
     }
+    if (STORE) dst[h * kChains] = o;
   }
 }
 
-template <class T, bool WITHZ>
+// Named barriers between one warp that fills (or empties) a stage and one that
+// waits for it.
+__device__ __forceinline__ void pair_wait(int id) {
+  asm volatile("bar.sync %0, 64;\n" ::"r"(id) : "memory");
+}
+__device__ __forceinline__ void pair_arrive(int id) {
+  asm volatile("bar.arrive %0, 64;\n" ::"r"(id) : "memory");
+}
+constexpr int kFullBar = 1, kEmptyBar = kFullBar + kLoaders;      // input stages
+constexpr int kOutFullBar = kEmptyBar + kLoaders, kOutEmptyBar = kOutFullBar + 2;
+static_assert(kOutEmptyBar + 2 <= 16, "named barriers of a CTA");
+
+// stages of a buffer: the chain's inputs and, in double, the raw values too
+template <class T> constexpr int ema_smem_bytes() {
+  return (kLoaders * (kPremul<T> ? 2 : 1) + 2) * kGroup * kChains * (int)sizeof(T);
+}
+
+template <class T>
 __global__ void __launch_bounds__(kEmaThreads)
 k_ema(const __grid_constant__ SeriesTable<T> tab, const T* __restrict__ raw, const T* alpha,
-      const T* theta, const T* tau_crit, const T* tau_surp, const T* S_carry,
-      const uint8_t* init_carry, const int32_t* __restrict__ active, T* __restrict__ b_S,
-      int32_t* __restrict__ b_init, T* __restrict__ e_S, int32_t* __restrict__ e_init,
-      T* __restrict__ S_out, T* __restrict__ Z_out, uint8_t* __restrict__ cls) {
-  __shared__ T ring[kStages * kBlk * kEmaThreads];
+      const T* S_carry, const uint8_t* init_carry, const int32_t* __restrict__ active,
+      T* __restrict__ b_S, int32_t* __restrict__ b_init, T* __restrict__ e_S,
+      int32_t* __restrict__ e_init, T* __restrict__ S_out) {
+  extern __shared__ __align__(16) unsigned char ema_smem[];
+  constexpr int V = Windows<T>::V, kStage = kGroup / V * kChains;
+  Windows<T>* inb = reinterpret_cast<Windows<T>*>(ema_smem);    // [kLoaders] stages of inputs
+  Windows<T>* rawb = kPremul<T> ? inb + kLoaders * kStage : inb;   // raw values
+  Windows<T>* outb = rawb + kLoaders * kStage;                  // [2] stages of S
   const int M = tab.M;
-  const int lane = threadIdx.x;
-  const int64_t t = (int64_t)blockIdx.x * kEmaThreads + lane;
-  if (t >= (int64_t)tab.seg_base[tab.n] * M) return;
-  const int m = (int)(t % M);
-  const int seg = (int)(t / M);
+  const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
+  const int64_t t = (int64_t)blockIdx.x * kChains + lane;
+  const bool has = t < (int64_t)tab.seg_base[tab.n] * M;  // a last CTA's spare lanes stay idle
+  const int m = has ? (int)(t % M) : 0;
+  const int seg = has ? (int)(t / M) : 0;
   const int s = series_of_seg(tab, seg);
-  const ModelParams<T> q = load_params(tab, s, m, alpha, theta, tau_crit, tau_surp);
+  const ModelParams<T> q = load_params(tab, s, m, alpha);
   const int L = tab.seg_len[s];
   const int64_t k0 = (int64_t)(seg - tab.seg_base[s]) * L, k1 = min64(k0 + L, tab.K[s]);
   // burn-in length, in updates (non-idle windows): (1 - alpha)^B <= e^-c, in
-  // whole ring strides, with c well past the point where a start error falls
+  // whole groups, with c well past the point where a start error falls
   // below the type's last bit, so that the rounded trajectories have met
   // (c = 28 for float's 6e-8 = e^-16.6, 45 for double's 1.1e-16 = e^-36.7)
   int B = kMaxBurn;
   {
     const float a = (float)q.a;
     const float c = sizeof(T) == 4 ? 28.f : 45.f;
-    if (a >= 1.f) B = kRingStride;
+    if (a >= 1.f) B = kGroup;
     else if (a > 0.f) {
       const float x = c / -log1pf(-a);
       if (x < (float)kMaxBurn) B = (int)x + 1;
     }
-    B = (B + kRingStride - 1) / kRingStride * kRingStride;
+    B = (B + kGroup - 1) / kGroup * kGroup;
   }
   // The burn-in runs over spans of windows [sp_lo, sp_hi), ascending. Without
   // activity counts it is the one span [k0 - B, k0). With them (non-idle
@@ -461,7 +479,7 @@ k_ema(const __grid_constant__ SeriesTable<T> tab, const T* __restrict__ raw, con
       const int64_t hi = (int64_t)(cb + 1) * L;   // chunks before this one are whole
       int64_t lo = (int64_t)cb * L;
       if (na == L && acc + L > B)
-        lo = hi - (B - acc + kRingStride - 1) / kRingStride * kRingStride;
+        lo = hi - (B - acc + kGroup - 1) / kGroup * kGroup;
       acc += na == L ? hi - lo : na;
       if (nsp > 0 && sp_lo[nsp - 1] == hi) {
         sp_lo[nsp - 1] = lo;
@@ -481,96 +499,166 @@ k_ema(const __grid_constant__ SeriesTable<T> tab, const T* __restrict__ raw, con
       sp_hi[nsp - 1 - i] = h;
     }
   }
-  T S = (T)0;
-  int init = 0;
-  if (from_start) {   // begin from the true state
-    init = (init_carry && init_carry[m]) ? 1 : 0;
-    S = init ? S_carry[m] : (T)0;
-  }
   const size_t base = (size_t)tab.off[s] + m;
-  int burn_grp = 0;
-  for (int i = 0; i < nsp; ++i) burn_grp += (int)((sp_hi[i] - sp_lo[i]) / kBlk);
-  const int n_grp = burn_grp + (int)((k1 - k0 + kBlk - 1) / kBlk);
-  // groups are issued in order: the spans of the burn-in, then the chunk; a
-  // group never straddles two spans (span lengths are multiples of kBlk)
-  int cur = 0;
-  int64_t cur_k = nsp > 0 ? sp_lo[0] : k0, cur_end = nsp > 0 ? sp_hi[0] : k1;
-  const size_t step = (size_t)M;
-  auto issue = [&](int g) {
-    if (g < n_grp) {
-      T* dst = ring + (size_t)(g % kStages) * kBlk * kEmaThreads + lane;
-      const T* src = raw + base + (size_t)cur_k * M;
-      const int64_t left = cur_end - cur_k;
-      if (left >= kBlk) {
+  int burn = 0;                                     // groups of the burn-in
+  for (int i = 0; i < nsp; ++i) burn += (int)((sp_hi[i] - sp_lo[i]) / kGroup);
+  int own = (int)((k1 - k0 + kGroup - 1) / kGroup);  // groups of the chunk
+  if (!has) burn = own = nsp = 0;
+  // the lanes' chunks start together: a lane with a shorter burn-in waits
+  const int lead = (int)__reduce_max_sync(0xffffffffu, (unsigned)burn);
+  const int n_it = lead + (int)__reduce_max_sync(0xffffffffu, (unsigned)own);
+
+  if (role == 0) {
+    // the recurrences
+    T S = (T)0;
+    int init = has ? 0 : 1;                         // spare lanes do not hold the others up
+    if (has && from_start) {                        // begin from the true state
+      init = (init_carry && init_carry[m]) ? 1 : 0;
+      S = init ? S_carry[m] : (T)0;
+    }
+    int stage = 0;
+    for (int i = 0; i < n_it; ++i) {
+      if (i == lead && has) {
+        b_S[t] = S;
+        b_init[t] = init;
+      }
+      const bool started = __all_sync(0xffffffffu, init);
+      const int at = stage * kStage + lane;
+      pair_wait(kFullBar + stage);
+      if (i < lead) {
+        if (started) ema_group<T, true, false>(inb + at, rawb + at, nullptr, q, S, init);
+        else ema_group<T, false, false>(inb + at, rawb + at, nullptr, q, S, init);
+      } else {
+        const int o = (i - lead) & 1;
+        Windows<T>* dst = outb + o * kStage + lane;
+        if (i - lead >= 2) pair_wait(kOutEmptyBar + o);
+        if (started) ema_group<T, true, true>(inb + at, rawb + at, dst, q, S, init);
+        else ema_group<T, false, true>(inb + at, rawb + at, dst, q, S, init);
+        pair_arrive(kOutFullBar + o);
+      }
+      if (i + kLoaders < n_it) pair_arrive(kEmptyBar + stage);
+      stage = stage + 1 == kLoaders ? 0 : stage + 1;
+    }
+    if (has) {
+      e_S[t] = S;
+      e_init[t] = init;
+    }
+  } else if (role <= kLoaders) {
+    // loader w fills stage w with groups w, w + 3, ...; the next kAhead of them
+    // are on their way in registers
+    constexpr int kAhead = sizeof(T) == 4 ? 2 : 1;
+    T buf[kAhead][kGroup];
+    auto load = [&](int gi, T (&v)[kGroup]) {
+      int64_t k = k0, left = 0;
+      int li = gi - (lead - burn);
+      if (gi >= lead) {
+        k = k0 + (int64_t)(gi - lead) * kGroup;
+        left = gi < lead + own ? k1 - k : 0;
+      } else if (li >= 0) {
+        for (int i = 0; i < nsp; ++i) {             // span lengths are multiples of kGroup
+          const int ng = (int)((sp_hi[i] - sp_lo[i]) / kGroup);
+          if (li < ng) {
+            k = sp_lo[i] + (int64_t)li * kGroup;
+            left = kGroup;
+            break;
+          }
+          li -= ng;
+        }
+      }
+      const T* src = raw + base + (size_t)k * M;
+      if (left >= kGroup) {
 #pragma unroll
-        for (int j = 0; j < kBlk; ++j) cp_async<sizeof(T)>(dst + j * kEmaThreads, src + j * step);
+        for (int j = 0; j < kGroup; ++j) v[j] = __ldg(src + (size_t)j * M);
       } else {
 #pragma unroll
-        for (int j = 0; j < kBlk; ++j)
-          if (j < left) cp_async<sizeof(T)>(dst + j * kEmaThreads, src + j * step);
+        for (int j = 0; j < kGroup; ++j) v[j] = j < left ? __ldg(src + (size_t)j * M) : idle_raw((T)0);
       }
-      cur_k += left < kBlk ? left : kBlk;
-      if (cur_k >= cur_end && cur < nsp) {
-        ++cur;
-        cur_k = cur < nsp ? sp_lo[cur] : k0;
-        cur_end = cur < nsp ? sp_hi[cur] : k1;
+    };
+    const int w = role - 1, at = w * kStage + lane;
+#pragma unroll
+    for (int h = 0; h < kAhead; ++h)
+      if (w + h * kLoaders < n_it) load(w + h * kLoaders, buf[h]);
+    for (int g0 = w; g0 < n_it; g0 += kAhead * kLoaders) {
+#pragma unroll
+      for (int h = 0; h < kAhead; ++h) {
+        const int gi = g0 + h * kLoaders;
+        if (gi < n_it) {
+          if (gi >= kLoaders) pair_wait(kEmptyBar + w);
+#pragma unroll
+          for (int j = 0; j < kGroup; j += V) {
+            Windows<T> r, x;
+#pragma unroll
+            for (int u = 0; u < V; ++u) {
+              r.x[u] = buf[h][j + u];
+              x.x[u] = is_idle_raw(r.x[u]) ? r.x[u] : mul_rn(q.a, r.x[u]);
+            }
+            rawb[at + j / V * kChains] = r;
+            if (kPremul<T>) inb[at + j / V * kChains] = x;
+          }
+          pair_arrive(kFullBar + w);
+          if (gi + kAhead * kLoaders < n_it) load(gi + kAhead * kLoaders, buf[h]);
+        }
       }
     }
-    cp_async_commit();
-  };
+  } else {
+    // stores
+    T* out = S_out + base + (size_t)k0 * M;
+    for (int gi = 0; gi < n_it - lead; ++gi) {
+      const int o = gi & 1;
+      pair_wait(kOutFullBar + o);
+      const Windows<T>* src = outb + o * kStage + lane;
+      const int64_t n = gi < own ? k1 - k0 - (int64_t)gi * kGroup : 0;
+      T* d = out + (size_t)gi * kGroup * M;
 #pragma unroll
-  for (int g = 0; g < kStages - 1; ++g) issue(g);
-  T* sp = S_out + base + (size_t)k0 * M;
-  auto stage_of = [&](int g) { return ring + (size_t)(g % kStages) * kBlk * kEmaThreads + lane; };
-  int g = 0;
-  // burn-in: full groups, nothing stored
-  for (; g < burn_grp; ++g) {
-    issue(g + kStages - 1);
-    cp_async_wait<kStages - 1>();
-    if (init) ema_group<T, true, true, false, WITHZ>(stage_of(g), kBlk, q, S, init, sp, M, S_out, Z_out, cls);
-    else ema_group<T, true, false, false, WITHZ>(stage_of(g), kBlk, q, S, init, sp, M, S_out, Z_out, cls);
+      for (int j = 0; j < kGroup; j += V) {
+        const Windows<T> v = src[j / V * kChains];
+#pragma unroll
+        for (int u = 0; u < V; ++u)
+          if (j + u < n) d[(size_t)(j + u) * M] = v.x[u];
+      }
+      if (gi + 2 < n_it - lead) pair_arrive(kOutEmptyBar + o);
+    }
   }
-  b_S[t] = S;
-  b_init[t] = init;
-  // the chunk: full groups, then the last (possibly partial) one
-  for (; g + 1 < n_grp; ++g) {
-    issue(g + kStages - 1);
-    cp_async_wait<kStages - 1>();
-    if (init) ema_group<T, true, true, true, WITHZ>(stage_of(g), kBlk, q, S, init, sp, M, S_out, Z_out, cls);
-    else ema_group<T, true, false, true, WITHZ>(stage_of(g), kBlk, q, S, init, sp, M, S_out, Z_out, cls);
-  }
-  cp_async_wait<0>();
-  {
-    const int n = (int)(k1 - (k0 + (int64_t)(g - burn_grp) * kBlk));
-    ema_group<T, false, false, true, WITHZ>(stage_of(g), n, q, S, init, sp, M, S_out, Z_out, cls);
-  }
-  e_S[t] = S;
-  e_init[t] = init;
 }
 
-// ---- pass 2: boundary check and repair, one warp per (series, model) -------
-// Lanes check 32 chunk boundaries at a time. A chunk whose burn-in state
-// differs from its predecessor's end state is run again from that end until its
-// new trajectory meets the stored one; first as a dry run, so that a chunk is
-// rewritten only when every chunk before it keeps its end state. A chunk whose
-// re-run never meets its stored trajectory changes its end state, and from the
-// next chunk on the boundaries are walked in order by one lane.
+// ---- pass 2: boundary check and repair, one CTA per (series, model) ---------
+// The CTA compares every chunk's burn-in state with its predecessor's end state
+// (one round of loads; a warp that took 32 boundaries at a time waited on
+// memory once per 32). Where none differs, as almost always, that is all. Else
+// one warp repairs: a chunk whose burn-in state differs is run again from its
+// predecessor's end until its new trajectory meets the stored one; first as a
+// dry run, so that a chunk is rewritten only when every chunk before it keeps
+// its end state. A chunk whose re-run never meets its stored trajectory changes
+// its end state, and from the next chunk on the boundaries are walked in order
+// by one lane.
+constexpr int kResolveThreads = 128;
 template <class T>
-__global__ void k_resolve(const __grid_constant__ SeriesTable<T> tab, const T* __restrict__ raw,
-                          const T* alpha, const T* theta, const T* tau_crit, const T* tau_surp,
-                          const T* start_S, const int32_t* start_init, T* end_S,
-                          int32_t* end_init, T* S_out, T* Z_out, uint8_t* cls,
-                          T* S_carry, uint8_t* init_carry, tre_diag* diag) {
+__global__ void __launch_bounds__(kResolveThreads)
+k_resolve(const __grid_constant__ SeriesTable<T> tab, const T* __restrict__ raw, const T* alpha,
+          const T* start_S, const int32_t* start_init, T* end_S, int32_t* end_init, T* S_out,
+          const uint8_t* __restrict__ cls, T* S_carry, uint8_t* init_carry, tre_diag* diag) {
   const int M = tab.M;
-  const int w = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  if (w >= tab.n * M) return;
   const int lane = threadIdx.x & 31;
-  const int s = w / M, m = w % M;
+  const int s = blockIdx.x / M, m = blockIdx.x % M;
   const int n_seg = tab.seg_base[s + 1] - tab.seg_base[s];
   if (n_seg == 0) return;
   const size_t g0 = (size_t)tab.seg_base[s] * M + m;
-  const ModelParams<T> q = load_params(tab, s, m, alpha, theta, tau_crit, tau_surp);
-  const bool with_z = theta != nullptr;
+  bool differs = false;
+#pragma unroll 4
+  for (int c = 1 + threadIdx.x; c < n_seg; c += kResolveThreads) {
+    const size_t x = g0 + (size_t)c * M;
+    differs |= start_init[x] != end_init[x - M] || !same_bits(start_S[x], end_S[x - M]);
+  }
+  if (!__syncthreads_or(differs)) {
+    if (S_carry && threadIdx.x == 0) {
+      const size_t last = g0 + (size_t)(n_seg - 1) * M;
+      S_carry[m] = end_S[last];
+      init_carry[m] = (uint8_t)end_init[last];
+    }
+    return;
+  }
+  if (threadIdx.x >= 32) return;
+  const ModelParams<T> q = load_params(tab, s, m, alpha);
   const int L = tab.seg_len[s];
   const size_t base = (size_t)tab.off[s] + m;
   int first_bad = n_seg;   // the in-order walk starts here
@@ -592,16 +680,14 @@ __global__ void k_resolve(const __grid_constant__ SeriesTable<T> tab, const T* _
     if (bad) {
       T S = pS;
       int init = pI;
-      moved = !run_segment<T, false>(base, M, k0, k1, raw, q, S, init, true, sI, S_out, Z_out,
-                                     cls, with_z);
+      moved = !run_segment<T, false>(base, M, k0, k1, raw, q, S, init, true, sI, S_out, cls);
     }
     const unsigned mv = __ballot_sync(0xffffffffu, moved);
     const int lim = mv ? c0 + __ffs(mv) - 1 : n_seg;   // predecessors final up to here
     if (bad && c <= lim) {
       T S = pS;
       int init = pI;
-      const bool met = run_segment<T>(base, M, k0, k1, raw, q, S, init, true, sI, S_out, Z_out,
-                                      cls, with_z);
+      const bool met = run_segment<T>(base, M, k0, k1, raw, q, S, init, true, sI, S_out, cls);
       if (!met) {
         end_S[g0 + (size_t)c * M] = S;
         end_init[g0 + (size_t)c * M] = init;
@@ -649,8 +735,7 @@ __global__ void k_resolve(const __grid_constant__ SeriesTable<T> tab, const T* _
         continue;
       }
       const int64_t k0 = (int64_t)qq * L, k1 = min64(k0 + L, tab.K[s]);
-      const bool met = run_segment<T>((size_t)tab.off[s] + m, M, k0, k1, raw, q, S, init, true,
-                                      bI[j], S_out, Z_out, cls, theta != nullptr);
+      const bool met = run_segment<T>(base, M, k0, k1, raw, q, S, init, true, bI[j], S_out, cls);
       if (met) {
         S = bE[j];
         init = bEI[j];
@@ -664,8 +749,15 @@ __global__ void k_resolve(const __grid_constant__ SeriesTable<T> tab, const T* _
   }
 }
 
-// ---- Z and regions from S for every series ---------------------------------
+// ---- Z and regions from S ----------------------------------------------------
 template <class T>
+__device__ __forceinline__ uint8_t region_of(uint8_t idle, T z, T tc, T ts) {
+  if (idle == kIdle) return kIdle;
+  return z < tc ? kCrit : (z > ts ? kSurp : kNom);
+}
+
+// for every series of a table, elements in tiles as above
+template <class T, int EPT>
 __global__ void __launch_bounds__(kEwThreads)
 k_normalize(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ TilePlan tp,
             FastDiv fm, bool vec, const T* S, const uint8_t* idle_cls, const T* theta,
@@ -673,53 +765,45 @@ k_normalize(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ 
   const int s = prefix_index(tp.tile_base, tab.n, blockIdx.x);
   const int M = tab.M;
   const int64_t n = (int64_t)tab.K[s] * M;
-  const int64_t l0 = (int64_t)(blockIdx.x - tp.tile_base[s]) * kTile + 4 * threadIdx.x;
+  const int64_t l0 =
+      ((int64_t)(blockIdx.x - tp.tile_base[s]) * blockDim.x + threadIdx.x) * EPT;
   if (l0 >= n) return;
   const size_t x0 = (size_t)(tab.off[s] + l0);
-  const bool v4 = vec && l0 + 4 <= n;
-  T sv[4];
-  uint8_t ic[4];
-  if (v4) {
+  const bool v4 = EPT == 4 && vec && l0 + 4 <= n;
+  T sv[EPT];
+  uint8_t ic[EPT];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) sv[i] = S[x0 + i];
-    const uchar4 c4 = *reinterpret_cast<const uchar4*>(idle_cls + x0);
-    ic[0] = c4.x; ic[1] = c4.y; ic[2] = c4.z; ic[3] = c4.w;
-  } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const bool in = l0 + i < n;
-      sv[i] = in ? S[x0 + i] : (T)0;
-      ic[i] = in ? idle_cls[x0 + i] : kIdle;
+  for (int i = 0; i < EPT; ++i) sv[i] = v4 || l0 + i < n ? S[x0 + i] : (T)0;
+  if constexpr (EPT == 4)
+    if (v4) {
+      const uchar4 c4 = *reinterpret_cast<const uchar4*>(idle_cls + x0);
+      ic[0] = c4.x; ic[1] = c4.y; ic[2] = c4.z; ic[3] = c4.w;
     }
+  if (!v4) {
+#pragma unroll
+    for (int i = 0; i < EPT; ++i) ic[i] = l0 + i < n ? idle_cls[x0 + i] : kIdle;
   }
   int m = l0 <= 0xffffffffll ? (int)((uint32_t)l0 - fm.div((uint32_t)l0) * (uint32_t)M)
                              : (int)(l0 % M);
-  T zv[4];
-  uint8_t cv[4];
+  T zv[EPT];
+  uint8_t cv[EPT];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const T z = div_rn(sv[i], theta[(size_t)s * M + m]);
-    zv[i] = z;
-    uint8_t c;
-    if (ic[i] == kIdle) c = kIdle;
-    else if (z < (tau_crit ? tau_crit[m] : tau_crit_v)) c = kCrit;
-    else if (z > tau_surp[m]) c = kSurp;
-    else c = kNom;
-    cv[i] = c;
+  for (int i = 0; i < EPT; ++i) {
+    zv[i] = div_rn(sv[i], theta[(size_t)s * M + m]);
+    cv[i] = region_of(ic[i], zv[i], tau_crit ? tau_crit[m] : tau_crit_v, tau_surp[m]);
     if (++m == M) m = 0;
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < EPT; ++i) {
     if (!v4 && l0 + i >= n) break;
     if (Z) Z[x0 + i] = zv[i];
     if (cls && !v4) cls[x0 + i] = cv[i];
   }
-  if (cls && v4) *reinterpret_cast<uchar4*>(cls + x0) = make_uchar4(cv[0], cv[1], cv[2], cv[3]);
+  if constexpr (EPT == 4)
+    if (cls && v4) *reinterpret_cast<uchar4*>(cls + x0) = make_uchar4(cv[0], cv[1], cv[2], cv[3]);
 }
 
-// ---- Eq. 3 receiver per window: warp per window ----------------------------
-template <class T>
-__device__ __forceinline__ void load_quad_z(const T* p, T (&v)[4]);
+template <class T> __device__ __forceinline__ void load_quad_z(const T* p, T (&v)[4]);
 template <> __device__ __forceinline__ void load_quad_z<float>(const float* p, float (&v)[4]) {
   const float4 q = *reinterpret_cast<const float4*>(p);
   v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
@@ -730,46 +814,68 @@ template <> __device__ __forceinline__ void load_quad_z<double>(const double* p,
   v[0] = a.x; v[1] = a.y; v[2] = c.x; v[3] = c.y;
 }
 
-// Eq. 3 receiver per window: argmin Z over non-idle models, lowest index on
-// ties (the first minimum in index order), -1 when every model is idle. One
-// thread per window; with QUAD (M a multiple of 4, 16-byte aligned rows) a
-// row is read four models per load, several loads in flight.
-template <class T, bool QUAD>
-__global__ void __launch_bounds__(256)
-k_receiver(int M, int K, const T* __restrict__ Z, const uint8_t* __restrict__ cls,
-           int32_t* __restrict__ recv) {
-  const int64_t k = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (k >= K) return;
-  const T* z = Z + (size_t)k * M;
-  const uint8_t* c = cls + (size_t)k * M;
-  int best = -1;
-  T bz = (T)0;
-  if (QUAD) {
-#pragma unroll 4
-    for (int m0 = 0; m0 < M; m0 += 4) {
-      T zv[4];
-      load_quad_z<T>(z + m0, zv);
-      const uchar4 c4 = *reinterpret_cast<const uchar4*>(c + m0);
-      const uint8_t cv[4] = {c4.x, c4.y, c4.z, c4.w};
+// One series with the Eq. 3 receiver per window: argmin Z over non-idle models,
+// lowest index on ties (the first minimum in index order), -1 when every model
+// is idle. A CTA takes wt whole windows; their Z stay in shared memory (padded
+// rows) for one thread per window to scan, where a kernel of its own read Z and
+// the regions again, one row per thread (64 models, 864,000 windows: 124 us for
+// Z and regions and 120 for the receivers).
+constexpr int kNormCells = 1024;
+template <class T>
+__global__ void __launch_bounds__(kEwThreads)
+k_norm_recv(int M, int K, int wt, FastDiv fm, bool vec, const T* __restrict__ S,
+            const uint8_t* idle_cls, const T* __restrict__ theta, const T* __restrict__ tau_crit,
+            const T* __restrict__ tau_surp, T* __restrict__ Z, uint8_t* cls,
+            int32_t* __restrict__ recv) {
+  __shared__ T zs[2 * kNormCells];                     // [wt][M + 1]
+  __shared__ uint8_t on[2 * kNormCells];               // not idle
+  const int k0 = (int)min64((int64_t)blockIdx.x * wt, K);
+  const int nw = min(wt, K - k0), n = nw * M;
+  const size_t x0 = (size_t)k0 * M;
+  auto one = [&](int c, T sv, uint8_t ic, T& z, uint8_t& cl) {
+    const int w = (int)fm.div((uint32_t)c), m = c - w * M;
+    z = div_rn(sv, theta[m]);
+    cl = region_of(ic, z, tau_crit[m], tau_surp[m]);
+    zs[w * (M + 1) + m] = z;
+    on[w * (M + 1) + m] = cl != kIdle;
+  };
+  if (vec) {                                           // wt * M is a multiple of 4
+    for (int c = 4 * threadIdx.x; c < n; c += 4 * blockDim.x) {
+      T sv[4], z[4];
+      load_quad_z<T>(S + x0 + c, sv);
+      const uchar4 c4 = *reinterpret_cast<const uchar4*>(idle_cls + x0 + c);
+      uint8_t cl[4];
+      one(c, sv[0], c4.x, z[0], cl[0]);
+      one(c + 1, sv[1], c4.y, z[1], cl[1]);
+      one(c + 2, sv[2], c4.z, z[2], cl[2]);
+      one(c + 3, sv[3], c4.w, z[3], cl[3]);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (cv[i] != kIdle && (best < 0 || zv[i] < bz)) {
-          best = m0 + i;
-          bz = zv[i];
-        }
+      for (int i = 0; i < 4; ++i) Z[x0 + c + i] = z[i];
+      *reinterpret_cast<uchar4*>(cls + x0 + c) = make_uchar4(cl[0], cl[1], cl[2], cl[3]);
     }
   } else {
-#pragma unroll 4
-    for (int m = 0; m < M; ++m) {
-      const uint8_t cv = c[m];
-      const T zv = z[m];
-      if (cv != kIdle && (best < 0 || zv < bz)) {
-        best = m;
-        bz = zv;
-      }
+    for (int c = threadIdx.x; c < n; c += blockDim.x) {
+      T z;
+      uint8_t cl;
+      one(c, S[x0 + c], idle_cls[x0 + c], z, cl);
+      Z[x0 + c] = z;
+      cls[x0 + c] = cl;
     }
   }
-  recv[k] = best;
+  __syncthreads();
+  for (int w = threadIdx.x; w < nw; w += blockDim.x) {
+    int best = -1;
+    T bz = (T)0;
+#pragma unroll 8
+    for (int m = 0; m < M; ++m) {
+      const T z = zs[w * (M + 1) + m];
+      if (on[w * (M + 1) + m] && (best < 0 || z < bz)) {
+        best = m;
+        bz = z;
+      }
+    }
+    recv[k0 + w] = best;
+  }
 }
 
 // ---- per-window donor preference order (Sec. IV-B), warp per window ---------
@@ -893,12 +999,12 @@ k_rank_small(int M, int K, const T* __restrict__ Z, const uint8_t* __restrict__ 
   }
 }
 
-template <class T> TilePlan tile_plan(const SeriesTable<T>& t, int& n_tiles) {
+template <class T> TilePlan tile_plan(const SeriesTable<T>& t, int tile, int& n_tiles) {
   TilePlan tp;
   n_tiles = 0;
   for (int s = 0; s < t.n; ++s) {
     tp.tile_base[s] = n_tiles;
-    n_tiles += (int)(((int64_t)t.K[s] * t.M + kTile - 1) / kTile);
+    n_tiles += (int)(((int64_t)t.K[s] * t.M + tile - 1) / tile);
   }
   tp.tile_base[t.n] = n_tiles;
   return tp;
@@ -926,15 +1032,18 @@ template <class T> int series_segments(SeriesTable<T>& t) {
   int total = 0;
   int64_t cells = 0;
   for (int s = 0; s < t.n; ++s) cells += (int64_t)t.K[s] * t.M;
+  const bool few = cells / short_chunk<T>() <= kShortChains;
   for (int s = 0; s < t.n; ++s) {
     const int K = t.K[s];
-    // chunks of 256 windows, longer for very long series (to bound the count)
-    // and for large tables: about kEmaChains chains keep the GPU busy, and
-    // longer chunks re-read fewer windows in their burn-ins; a multiple of the
-    // smoothing pass's ring stride
-    int L = 256;
+    // A chain takes its burn-in plus its chunk, one window after another: short
+    // chunks while the table gives few chains (three models, 600 windows in
+    // double: 512 dependent steps with chunks of 256, 256 with 32), else 256
+    // windows, longer for very long series (to bound the count) and for large
+    // tables: about kEmaChains chains keep the GPU busy, and longer chunks
+    // re-read fewer windows in their burn-ins. Multiples of the group.
+    int L = few ? short_chunk<T>() : 256;
     int64_t need = std::max<int64_t>((K + 2047) / 2048, cells / kEmaChains);
-    if (need > L) L = (int)((need + kRingStride - 1) / kRingStride * kRingStride);
+    if (need > L) L = (int)((need + 2 * kGroup - 1) / (2 * kGroup) * (2 * kGroup));
     t.seg_len[s] = L;
     t.seg_base[s] = total;
     total += (K + L - 1) / L;
@@ -954,8 +1063,8 @@ template <class T> void score_ws_layout(Arena& a, int M, int64_t elems, int n_se
   w.active = a.take<int32_t>(n);
 }
 
-template <class T> int score_launches(const SeriesTable<T>& tab) {
-  return (total_elems(tab) >= kActiveMinCells ? 1 : 0) + 3;
+template <class T> int score_launches(const SeriesTable<T>& tab, bool with_z) {
+  return (total_elems(tab) >= kActiveMinCells ? 1 : 0) + 3 + (with_z ? 1 : 0);
 }
 
 template <class T>
@@ -963,8 +1072,8 @@ cudaError_t launch_score(const SeriesTable<T>& tab, const int32_t* P, const int3
                          const int32_t* A, const int32_t* W, const T* w_p, const T* w_q,
                          const T* alpha, const T* theta, const T* tau_crit, const T* tau_surp,
                          T* S_carry, uint8_t* init_carry, T* S, T* Z, uint8_t* cls,
-                         ScoreWs<T>& w, tre_diag* diag, cudaStream_t s, const int64_t* A_ms,
-                         const int64_t* W_ms) {
+                         int32_t* recv, ScoreWs<T>& w, tre_diag* diag, cudaStream_t s,
+                         const int64_t* A_ms, const int64_t* W_ms) {
   const int M = tab.M;
   const int n_seg = tab.seg_base[tab.n];
   if (n_seg > w.cap_seg) return cudaErrorInvalidValue;
@@ -972,19 +1081,21 @@ cudaError_t launch_score(const SeriesTable<T>& tab, const int32_t* P, const int3
   const int64_t total = total_elems(tab);
   if (total == 0) return cudaSuccess;
   const Counts c{P, D, A, W, A_ms, W_ms};
+  const bool small = total <= kSmallCells;
+  const int th = small ? kSmallThreads : kEwThreads;
   int n_tiles = 0;
-  const TilePlan tp = tile_plan(tab, n_tiles);
+  const TilePlan tp = tile_plan(tab, small ? th : 4 * th, n_tiles);
   if (A_ms) {
     const bool vec = quad_aligned(tab, {P, D, A_ms, W_ms, w.raw, cls});
-    k_raw<T, true><<<n_tiles, kEwThreads, 0, s>>>(tab, tp, FastDiv(M), vec, c, w_p, w_q, w.raw,
-                                                  cls);
+    auto f = small ? k_raw<T, true, 1> : k_raw<T, true, 4>;
+    f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(M), vec, c, w_p, w_q, w.raw, cls);
   } else {
     const bool vec = quad_aligned(tab, {P, D, A, W, w.raw, cls});
-    k_raw<T, false><<<n_tiles, kEwThreads, 0, s>>>(tab, tp, FastDiv(M), vec, c, w_p, w_q, w.raw,
-                                                   cls);
+    auto f = small ? k_raw<T, false, 1> : k_raw<T, false, 4>;
+    f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(M), vec, c, w_p, w_q, w.raw, cls);
   }
   const int64_t segs = (int64_t)n_seg * M;
-  const unsigned g = (unsigned)((segs + kEmaThreads - 1) / kEmaThreads);
+  const unsigned g = (unsigned)((segs + kChains - 1) / kChains);
   // activity counts for the burn-ins where the series are long enough that
   // idle stretches would otherwise send chunks to the in-order pass, and the
   // extra pass over the classes is small beside the smoothing
@@ -993,44 +1104,45 @@ cudaError_t launch_score(const SeriesTable<T>& tab, const int32_t* P, const int3
     k_active<T><<<n_seg, 256, (size_t)M * sizeof(int32_t), s>>>(tab, FastDiv(M), cls, w.active);
     active = w.active;
   }
-  if (theta)
-    k_ema<T, true><<<g, kEmaThreads, 0, s>>>(tab, w.raw, alpha, theta, tau_crit, tau_surp,
-                                             S_carry, init_carry, active, w.start_S,
-                                             w.start_init, w.end_S, w.end_init, S, Z, cls);
-  else
-    k_ema<T, false><<<g, kEmaThreads, 0, s>>>(tab, w.raw, alpha, theta, tau_crit, tau_surp,
-                                              S_carry, init_carry, active, w.start_S,
-                                              w.start_init, w.end_S, w.end_init, S, Z, cls);
-  const int warps = tab.n * M;
-  k_resolve<T><<<(warps + 1) / 2, 64, 0, s>>>(tab, w.raw, alpha, theta, tau_crit, tau_surp,
-                                                w.start_S, w.start_init, w.end_S, w.end_init,
-                                                S, Z, cls, S_carry, init_carry, diag);
-  return cudaGetLastError();
+  cudaError_t e = func_smem_once((const void*)k_ema<T>, ema_smem_bytes<T>(), false);
+  if (e) return e;
+  k_ema<T><<<g, kEmaThreads, ema_smem_bytes<T>(), s>>>(tab, w.raw, alpha, S_carry, init_carry,
+                                                       active, w.start_S, w.start_init, w.end_S,
+                                                       w.end_init, S);
+  k_resolve<T><<<tab.n * M, kResolveThreads, 0, s>>>(tab, w.raw, alpha, w.start_S, w.start_init,
+                                                     w.end_S, w.end_init, S, cls, S_carry,
+                                                     init_carry, diag);
+  if ((e = cudaGetLastError())) return e;
+  // Z and regions in a pass of their own: the division in the chain's warp
+  // cost more than re-reading S (8 models, 60 windows in double: 33 us of
+  // smoothing with it; one hour of 100 ms windows in float: 42)
+  if (theta) return launch_normalize<T>(tab, S, cls, theta, tau_crit, (T)0, tau_surp, Z, cls, recv, s);
+  return cudaSuccess;
 }
 
 template <class T>
 cudaError_t launch_normalize(const SeriesTable<T>& tab, const T* S, const uint8_t* idle_cls,
                              const T* theta, const T* tau_crit, T tau_crit_v, const T* tau_surp,
-                             T* Z, uint8_t* cls, cudaStream_t s) {
+                             T* Z, uint8_t* cls, int32_t* recv, cudaStream_t s) {
   const int64_t total = total_elems(tab);
   if (total == 0) return cudaSuccess;
-  int n_tiles = 0;
-  const TilePlan tp = tile_plan(tab, n_tiles);
+  const bool small = total <= kSmallCells;
   const bool vec = quad_aligned(tab, {S, idle_cls, Z, cls});
-  k_normalize<T><<<n_tiles, kEwThreads, 0, s>>>(tab, tp, FastDiv(tab.M), vec, S, idle_cls, theta,
-                                                tau_crit, tau_crit_v, tau_surp, Z, cls);
-  return cudaGetLastError();
-}
-
-template <class T>
-cudaError_t launch_receiver(int M, int K, const T* Z, const uint8_t* cls, int32_t* recv,
-                            cudaStream_t s) {
-  if (K == 0) return cudaSuccess;
-  const unsigned g = (unsigned)((K + 255) / 256);
-  if (M % 4 == 0 && (((uintptr_t)Z | (uintptr_t)cls) & 15) == 0)
-    k_receiver<T, true><<<g, 256, 0, s>>>(M, K, Z, cls, recv);
-  else
-    k_receiver<T, false><<<g, 256, 0, s>>>(M, K, Z, cls, recv);
+  if (recv) {
+    if (tab.n != 1 || !tau_crit || !Z || !cls) return cudaErrorInvalidValue;
+    const int M = tab.M, K = tab.K[0], th = small ? kSmallThreads : kEwThreads;
+    const int wt = std::max(1, (small ? th : kNormCells) / M);
+    k_norm_recv<T><<<(unsigned)((K + wt - 1) / wt), th, 0, s>>>(
+        M, K, wt, FastDiv(M), vec && !small && M % 4 == 0, S, idle_cls, theta, tau_crit, tau_surp,
+        Z, cls, recv);
+    return cudaGetLastError();
+  }
+  int n_tiles = 0;
+  const int th = small ? kSmallThreads : kEwThreads;
+  const TilePlan tp = tile_plan(tab, small ? th : 4 * th, n_tiles);
+  auto f = small ? k_normalize<T, 1> : k_normalize<T, 4>;
+  f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(tab.M), vec, S, idle_cls, theta, tau_crit, tau_crit_v,
+                           tau_surp, Z, cls);
   return cudaGetLastError();
 }
 
@@ -1050,18 +1162,17 @@ cudaError_t launch_rank(int M, int K, const T* Z, const uint8_t* cls, int32_t* r
 
 #define TRE_INST(T)                                                                               \
   template int series_segments<T>(SeriesTable<T>&);                                               \
-  template int score_launches<T>(const SeriesTable<T>&);                                          \
+  template int score_launches<T>(const SeriesTable<T>&, bool);                                        \
   template void score_ws_layout<T>(Arena&, int, int64_t, int, ScoreWs<T>&);                       \
   template cudaError_t launch_score<T>(const SeriesTable<T>&, const int32_t*, const int32_t*,      \
                                        const int32_t*, const int32_t*, const T*, const T*,         \
                                        const T*, const T*, const T*, const T*, T*, uint8_t*, T*,   \
-                                       T*, uint8_t*, ScoreWs<T>&, tre_diag*, cudaStream_t,         \
+                                       T*, uint8_t*, int32_t*, ScoreWs<T>&, tre_diag*,             \
+                                       cudaStream_t,                                               \
                                        const int64_t*, const int64_t*);                            \
   template cudaError_t launch_normalize<T>(const SeriesTable<T>&, const T*, const uint8_t*,        \
                                            const T*, const T*, T, const T*, T*, uint8_t*,          \
-                                           cudaStream_t);                                          \
-  template cudaError_t launch_receiver<T>(int, int, const T*, const uint8_t*, int32_t*,            \
-                                          cudaStream_t);                                          \
+                                           int32_t*, cudaStream_t);                                \
   template cudaError_t launch_rank<T>(int, int, const T*, const uint8_t*, int32_t*, int32_t*,      \
                                       cudaStream_t);
 TRE_INST(float)

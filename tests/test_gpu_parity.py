@@ -241,6 +241,33 @@ def test_score_is_deterministic(tre):
         assert (a[k] == b[k]).all()
 
 
+# Chunks are 64 windows (32 in double) up to 16,384 chunks, else 256 and more;
+# windows go in groups of 32 for 32 (chunk, model) chains at a time. 1100 x 1024
+# crosses to long chunks; alpha 1, 0.9 and 0.01 give burn-ins of one group and of
+# more than the series.
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("K,M,alpha", [(1, 1, 0.2), (31, 3, 0.9), (32, 33, 0.2), (33, 5, 1.0),
+                                       (64, 32, 0.01), (65, 1, 0.2), (129, 7, 0.9),
+                                       (4101, 3, 0.01), (1100, 1024, 0.05)])
+def test_score_chunk_edges(tre, dtype, K, M, alpha):
+    import torch
+    rng = np.random.default_rng(K + M)
+    cnt = _score_inputs(rng, K, M)
+    npdt = np.float32 if dtype == "f32" else np.float64
+    prof = {"w_p": 0.2, "w_q": 2.0, "alpha": alpha, "theta": 10.0, "tau_crit": 0.8,
+            "tau_surplus": 1.2}
+    init = (np.arange(M) % 2).astype(np.uint8)          # half the models carried in
+    carry = {"S": np.linspace(1, 9, M).astype(npdt), "init": init}
+    dev = _cuda({k: v.copy() for k, v in carry.items()})
+    S, Z, cls, recv = oracle.score(cnt["P"], cnt["D"], cnt["A"], cnt["W"], prof, 1000, npdt,
+                                   carry=carry)
+    out = tre.tss_score(_cuda(cnt), prof, 1000, dtype=dtype, carry=dev)
+    for k, ref in (("S", S), ("Z", Z), ("cls", cls), ("recv", recv)):
+        np.testing.assert_array_equal(_np(out[k]), ref, err_msg=k)
+    for k in ("S", "init"):
+        np.testing.assert_array_equal(_np(dev[k]), carry[k], err_msg=f"carry {k}")
+
+
 @pytest.mark.parametrize("dtype", ["f32", "f64"])
 @pytest.mark.parametrize("name,scale", [("tiny", 1.0), ("mid", 0.05), ("hetero", 0.005)])
 def test_pipeline_requests(tre, dtype, name, scale):
