@@ -508,6 +508,21 @@ tre_status sweep_typed(const tre_sweep_spec* sp, const SweepPlan& pl, const tre_
 namespace {
 
 // ---- stage-aware signal (Sec. VIII) ----------------------------------------
+// The prefill and decode signals as two series of one table, so that each pass
+// over them is one launch (8 models, 36,000 windows: gauges, calibration and
+// scoring 388 us with a table a stage, now 339; the host's launches bound it).
+// The second starts on a 16-byte boundary.
+template <class T> SeriesTable<T> stage_series(const tre_grid* g) {
+  SeriesTable<T> t = single_series<T>(g);
+  t.n = 2;
+  t.off[1] = ((int64_t)g->n_windows * g->n_models + 15) & ~(int64_t)15;
+  t.K[1] = t.K[0];
+  t.win[1] = t.win[0];
+  t.alpha[1] = t.alpha[0];
+  series_segments(t);
+  return t;
+}
+
 template <class T>
 tre_status stage_calibrate_typed(const tre_grid* g, const tre_requests* req, const tre_counts* in,
                                  const int32_t* A_pre, const int32_t* A_dec,
@@ -517,51 +532,37 @@ tre_status stage_calibrate_typed(const tre_grid* g, const tre_requests* req, con
                                  tre_diag* diag, cudaStream_t s) {
   const int M = g->n_models, K = g->n_windows;
   const size_t cells = (size_t)K * M;
-  SeriesTable<T> tab = single_series<T>(g);
+  const SeriesTable<T> tab = stage_series<T>(g);
+  const size_t both = (size_t)tab.off[1] + cells;
   Arena a(ws);
-  unsigned long long* ttft = a.take<unsigned long long>(cells);
-  unsigned long long* tpot = a.take<unsigned long long>(cells);
-  int32_t* zero = a.take<int32_t>(cells);
-  T* ones = a.take<T>((size_t)M);
-  T* S = a.take<T>(cells);
-  uint8_t* cls = a.take<uint8_t>(cells);
+  unsigned long long* ttft = a.take<unsigned long long>(both);
+  T* S = a.take<T>(both);
+  uint8_t* cls = a.take<uint8_t>(both);
   ScoreWs<T> sw;
-  score_ws_layout<T>(a, M, (int64_t)cells, tab.seg_base[1], sw);
+  score_ws_layout<T>(a, M, (int64_t)both, tab.seg_base[2], sw);
   CalibWs<T> cw;
-  calib_ws_layout<T>(a, (int64_t)cells, M, cw);
+  calib_ws_layout<T>(a, (int64_t)both, 2 * M, cw);
   bool query;
   tre_status st = ws_check(a, ws, ws_bytes, query);
   if (st != TRE_OK || query) return st;
-  const T* w_p = static_cast<const T*>(p->w_p);
-  const T* w_q = static_cast<const T*>(p->w_q);
-  const T* alpha = static_cast<const T*>(p->alpha);
   cudaError_t e;
   {
     Scope sc(kSlo, 1, s);
-    e = launch_stage_requests(cols_of(req), M, g->window_ms, K, nullptr, nullptr, ttft, tpot,
-                              ttft_ms, tpot_ms, s);
+    e = launch_stage_requests(cols_of(req), M, g->window_ms, K, nullptr, nullptr, ttft,
+                              ttft + tab.off[1], ttft_ms, tpot_ms, s);
   }
-  if (!e) e = cudaMemsetAsync(zero, 0, cells * sizeof(int32_t), s);
-  if (!e) e = launch_fill<T>(ones, M, (T)1, s);
-  // prefill: (P/dt) / max(A_prefill + w_q W, 1), calibrated on TTFT
+  // prefill: (P/dt) / max(A_prefill + w_q W, 1), calibrated on TTFT; decode:
+  // (D/dt) / max(A_decode, 1), calibrated on TPOT
   if (!e) {
     Scope sc(kScore, score_launches(tab, false), s);
-    e = launch_score<T>(tab, in->P, zero, A_pre, in->W, ones, w_q, alpha, nullptr, nullptr,
-                        nullptr, nullptr, nullptr, S, nullptr, cls, nullptr, sw, diag, s);
+    e = launch_score_stages<T>(tab, in->P, in->D, in->W, A_pre, A_dec,
+                               static_cast<const T*>(p->w_p), static_cast<const T*>(p->w_q),
+                               static_cast<const T*>(p->alpha), S, cls, sw, diag, s);
   }
   if (!e) {
     Scope sc(kCalibrate, 3, s);
-    e = launch_calibrate<T>(tab, S, cls, ttft, ok_frac, rel, static_cast<T*>(th_pre), cw, diag, s);
-  }
-  // decode: (D/dt) / max(A_decode, 1), calibrated on TPOT
-  if (!e) {
-    Scope sc(kScore, score_launches(tab, false), s);
-    e = launch_score<T>(tab, zero, in->D, A_dec, zero, w_p, w_q, alpha, nullptr, nullptr,
-                        nullptr, nullptr, nullptr, S, nullptr, cls, nullptr, sw, diag, s);
-  }
-  if (!e) {
-    Scope sc(kCalibrate, 3, s);
-    e = launch_calibrate<T>(tab, S, cls, tpot, ok_frac, rel, static_cast<T*>(th_dec), cw, diag, s);
+    e = launch_calibrate<T>(tab, S, cls, ttft, ok_frac, rel, static_cast<T*>(th_pre), cw, diag, s,
+                            static_cast<T*>(th_dec));
   }
   return cuda_status(e);
 }
@@ -572,35 +573,29 @@ tre_status stage_score_typed(const tre_grid* g, const tre_counts* in, const int3
                              const void* th_dec, void* S_pre, void* Z_pre, uint8_t* cls_pre,
                              void* S_dec, void* Z_dec, uint8_t* cls_dec, void* ws,
                              size_t* ws_bytes, tre_diag* diag, cudaStream_t s) {
-  const int M = g->n_models, K = g->n_windows;
-  const size_t cells = (size_t)K * M;
-  SeriesTable<T> tab = single_series<T>(g);
+  const int M = g->n_models;
+  const SeriesTable<T> tab = stage_series<T>(g);
+  const size_t both = (size_t)tab.off[1] + (size_t)g->n_windows * M;
   Arena a(ws);
-  int32_t* zero = a.take<int32_t>(cells);
-  T* ones = a.take<T>((size_t)M);
+  T* S = a.take<T>(both);
+  uint8_t* cls = a.take<uint8_t>(both);
   ScoreWs<T> sw;
-  score_ws_layout<T>(a, M, (int64_t)cells, tab.seg_base[1], sw);
+  score_ws_layout<T>(a, M, (int64_t)both, tab.seg_base[2], sw);
   bool query;
   tre_status st = ws_check(a, ws, ws_bytes, query);
   if (st != TRE_OK || query) return st;
-  const T* w_q = static_cast<const T*>(p->w_q);
-  const T* alpha = static_cast<const T*>(p->alpha);
-  const T* tc = static_cast<const T*>(p->tau_crit);
-  const T* tsu = static_cast<const T*>(p->tau_surplus);
-  cudaError_t e = cudaMemsetAsync(zero, 0, cells * sizeof(int32_t), s);
-  if (!e) e = launch_fill<T>(ones, M, (T)1, s);
-  if (!e) {
-    Scope sc(kScore, score_launches(tab, true), s);
-    e = launch_score<T>(tab, in->P, zero, A_pre, in->W, ones, w_q, alpha,
-                        static_cast<const T*>(th_pre), tc, tsu, nullptr, nullptr,
-                        static_cast<T*>(S_pre), static_cast<T*>(Z_pre), cls_pre, nullptr, sw, diag, s);
-  }
-  if (!e) {
-    Scope sc(kScore, score_launches(tab, true), s);
-    e = launch_score<T>(tab, zero, in->D, A_dec, zero, static_cast<const T*>(p->w_p), w_q,
-                        alpha, static_cast<const T*>(th_dec), tc, tsu, nullptr, nullptr,
-                        static_cast<T*>(S_dec), static_cast<T*>(Z_dec), cls_dec, nullptr, sw, diag, s);
-  }
+  Scope sc(kScore, score_launches(tab, true), s);
+  cudaError_t e = launch_score_stages<T>(
+      tab, in->P, in->D, in->W, A_pre, A_dec, static_cast<const T*>(p->w_p),
+      static_cast<const T*>(p->w_q), static_cast<const T*>(p->alpha), S, cls, sw, diag, s);
+  if (!e)
+    e = launch_norm_stages<T>(
+        tab, S, cls, static_cast<const T*>(p->tau_crit), static_cast<const T*>(p->tau_surplus),
+        StageOut<T>{static_cast<const T*>(th_pre), static_cast<T*>(S_pre), static_cast<T*>(Z_pre),
+                    cls_pre},
+        StageOut<T>{static_cast<const T*>(th_dec), static_cast<T*>(S_dec), static_cast<T*>(Z_dec),
+                    cls_dec},
+        s);
   return cuda_status(e);
 }
 

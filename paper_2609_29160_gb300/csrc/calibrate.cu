@@ -349,7 +349,7 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
          const typename KeyOf<T>::U* kmin_g, const typename KeyOf<T>::U* kmax_g,
          const uint32_t* ncand_g, const T* __restrict__ S, const uint8_t* __restrict__ cls,
          const unsigned long long* __restrict__ slo, double ok_frac, double reliability, T* theta,
-         tre_diag* diag) {
+         T* theta1, tre_diag* diag) {
   using U = typename KeyOf<T>::U;
   constexpr int NL = KeyOf<T>::kLevels;
   constexpr int kThrDirect = 256;
@@ -368,6 +368,7 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
   U* mk = keys + (size_t)tab.off[s] + (size_t)m * K;
   const int tid = threadIdx.x, lane = tid & 31;
   const size_t out = (size_t)s * M + m;
+  T* const th_out = theta1 && s == 1 ? theta1 + m : theta + out;
   const float rel_f = (float)reliability;
   int32_t* fcnt = reinterpret_cast<int32_t*>(dyn);
   int32_t* fhl = fcnt + kFine;
@@ -439,7 +440,7 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
   }
   if (ncand == 0) {
     if (tid == 0) {
-      theta[out] = (T)1;
+      *th_out = (T)1;
       atomicAdd(&diag->degenerate_calib, 1ull);
     }
     return;
@@ -572,11 +573,11 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
       }
       if (tid == 0) {
         if (best_s != ~(U)0) {
-          theta[out] = value_of(best_s);
+          *th_out = value_of(best_s);
         } else if (bf != 0x7fffffff) {
-          theta[out] = value_of(bfmin_s);
+          *th_out = value_of(bfmin_s);
         } else {
-          theta[out] = value_of(kmax);
+          *th_out = value_of(kmax);
           atomicAdd(&diag->degenerate_calib, 1ull);
         }
       }
@@ -654,7 +655,7 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
     if (b == 0x7fffffff) {
       if (l == 0) {
         if (tid == 0) {
-          theta[out] = value_of(kmax);
+          *th_out = value_of(kmax);
           atomicAdd(&diag->degenerate_calib, 1ull);
         }
         return;
@@ -667,7 +668,7 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
     __syncthreads();
     const int kb = red32[0];
     if (kb == 1) {
-      if (tid == 0) theta[out] = value_of(mn[l][b]);
+      if (tid == 0) *th_out = value_of(mn[l][b]);
       return;
     }
     if (tid == b) {
@@ -698,7 +699,7 @@ template <class T> void calib_ws_layout(Arena& a, int64_t elems, int n_sm, Calib
 template <class T>
 cudaError_t launch_calibrate(const SeriesTable<T>& tab, const T* S, const uint8_t* cls,
                              const unsigned long long* slo, double ok_frac, double reliability,
-                             T* theta, CalibWs<T>& w, tre_diag* diag, cudaStream_t s) {
+                             T* theta, CalibWs<T>& w, tre_diag* diag, cudaStream_t s, T* theta1) {
   using U = typename KeyOf<T>::U;
   const int n_sm = tab.n * tab.M;
   if (n_sm > w.n_sm) return cudaErrorInvalidValue;
@@ -715,7 +716,7 @@ cudaError_t launch_calibrate(const SeriesTable<T>& tab, const T* S, const uint8_
     cudaError_t e = func_smem_once((const void*)k_search<T, true>, (int)smem, true);
     if (e) return e;
     k_search<T, true><<<n_sm, kNB, smem, s>>>(tab, static_cast<U*>(w.keys), kmin, kmax, w.ncand, S,
-                                              cls, slo, ok_frac, reliability, theta, diag);
+                                              cls, slo, ok_frac, reliability, theta, theta1, diag);
     return cudaGetLastError();
   }
   const int thr_n = std::max(kThrTable, n_sm);
@@ -746,7 +747,7 @@ cudaError_t launch_calibrate(const SeriesTable<T>& tab, const T* S, const uint8_
   cudaError_t e = func_smem_once((const void*)k_search<T, false>, (int)smem, true);
   if (e) return e;
   k_search<T, false><<<n_sm, kNB, smem, s>>>(tab, static_cast<U*>(w.keys), kmin, kmax, w.ncand, S,
-                                             cls, slo, ok_frac, reliability, theta, diag);
+                                             cls, slo, ok_frac, reliability, theta, theta1, diag);
   return cudaGetLastError();
 }
 
@@ -755,10 +756,10 @@ template void calib_ws_layout<double>(Arena&, int64_t, int, CalibWs<double>&);
 template cudaError_t launch_calibrate<float>(const SeriesTable<float>&, const float*,
                                              const uint8_t*, const unsigned long long*, double,
                                              double, float*, CalibWs<float>&, tre_diag*,
-                                             cudaStream_t);
+                                             cudaStream_t, float*);
 template cudaError_t launch_calibrate<double>(const SeriesTable<double>&, const double*,
                                               const uint8_t*, const unsigned long long*, double,
                                               double, double*, CalibWs<double>&, tre_diag*,
-                                              cudaStream_t);
+                                              cudaStream_t, double*);
 
 }  // namespace tre

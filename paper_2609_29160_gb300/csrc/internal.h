@@ -146,12 +146,11 @@ cudaError_t launch_aggregate(const AggPlan& plan, const int32_t* P, const int32_
 // [t_start, t_first) into dPre, decode [t_first, t_end) into dDec, each
 // [K+1][M], cleared here; both null = skipped) and the packed TTFT and TPOT
 // calibration counts at the arrival window (count + met << 32, [K][M], cleared
-// here; both null = skipped).
+// here, tpot after ttft in one block; both null = skipped).
 cudaError_t launch_stage_requests(const ReqCols& r, int M, int win, int K, int32_t* dPre,
                                   int32_t* dDec, unsigned long long* ttft,
                                   unsigned long long* tpot, const int32_t* ttft_ms,
                                   const int32_t* tpot_ms, cudaStream_t s);
-template <class T> cudaError_t launch_fill(T* p, int64_t n, T v, cudaStream_t s);
 
 // ---- series tables ----------------------------------------------------------
 // A batch of series (one per (trace, window length) in a sweep, one for the
@@ -194,6 +193,22 @@ cudaError_t launch_score(const SeriesTable<T>& tab, const int32_t* P, const int3
                          T* S_carry, uint8_t* init_carry, T* S, T* Z, uint8_t* cls,
                          int32_t* recv, ScoreWs<T>& w, tre_diag* diag, cudaStream_t s,
                          const int64_t* A_ms = nullptr, const int64_t* W_ms = nullptr);
+// The stage-aware signal (prefill, decode) as a table of two series, smoothed
+// together (S, idle classes at the series' offsets), and its Z and regions.
+template <class T> struct StageOut {
+  const T* theta;
+  T *S, *Z;
+  uint8_t* cls;
+};
+template <class T>
+cudaError_t launch_score_stages(const SeriesTable<T>& tab, const int32_t* P, const int32_t* D,
+                                const int32_t* W, const int32_t* A_pre, const int32_t* A_dec,
+                                const T* w_p, const T* w_q, const T* alpha, T* S, uint8_t* cls,
+                                ScoreWs<T>& w, tre_diag* diag, cudaStream_t s);
+template <class T>
+cudaError_t launch_norm_stages(const SeriesTable<T>& tab, const T* S, const uint8_t* idle_cls,
+                               const T* tau_crit, const T* tau_surp, const StageOut<T>& pre,
+                               const StageOut<T>& dec, cudaStream_t s);
 // Z = S / theta[series][m] and regions for every series (tau_crit device [M] or
 // one value for all); with recv (a one-series table, tau_crit per model) also
 // the Eq. 3 receiver of every window
@@ -216,11 +231,13 @@ template <class T> struct CalibWs {
   int n_sm;                    // (series, model) pairs the range arrays hold
 };
 template <class T> void calib_ws_layout(Arena& a, int64_t elems, int n_sm, CalibWs<T>& w);
-// theta[s*M + m] for every series of the table
+// theta[s*M + m] for every series of the table (theta1: where the second series'
+// boundaries go when not there)
 template <class T>
 cudaError_t launch_calibrate(const SeriesTable<T>& tab, const T* S, const uint8_t* cls,
                              const unsigned long long* slo, double ok_frac, double reliability,
-                             T* theta, CalibWs<T>& w, tre_diag* diag, cudaStream_t s);
+                             T* theta, CalibWs<T>& w, tre_diag* diag, cudaStream_t s,
+                             T* theta1 = nullptr);
 
 // ---- select.cu ------------------------------------------------------------
 // One controller instance per (series, tau, cap). The small per-series tables

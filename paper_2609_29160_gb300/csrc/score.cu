@@ -125,10 +125,14 @@ __device__ __forceinline__ T raw_tss_mean(int32_t p, int32_t d, long long a_ms, 
   return div_rn(num, den);
 }
 
-template <class T, bool MEAN, int EPT>
+// STAGES: the two series of the stage-aware signal, each from its own counts
+// (c0: prompt tokens over the prefill gauge and W with a token weight of one;
+// c1: decode tokens over the decode gauge), read at the series' own elements;
+// a null array counts as zeros.
+template <class T, bool MEAN, int EPT, bool STAGES>
 __global__ void __launch_bounds__(kEwThreads)
 k_raw(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ TilePlan tp, FastDiv fm,
-      bool vec, Counts c, const T* __restrict__ w_p, const T* __restrict__ w_q,
+      bool vec, Counts c0, Counts c1, const T* __restrict__ w_p, const T* __restrict__ w_q,
       T* __restrict__ raw, uint8_t* __restrict__ cls) {
   const int s = prefix_index(tp.tile_base, tab.n, blockIdx.x);
   const int M = tab.M;
@@ -136,42 +140,45 @@ k_raw(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ TilePl
   const int64_t l0 = ((int64_t)(blockIdx.x - tp.tile_base[s]) * blockDim.x + threadIdx.x) * EPT;
   if (l0 >= n) return;
   const size_t x0 = (size_t)(tab.off[s] + l0);
+  const Counts c = STAGES && s == 1 ? c1 : c0;
+  const size_t xi = STAGES ? (size_t)l0 : x0;
   const T dt = div_rn((T)tab.win[s], (T)1000);      // window length in seconds
   int32_t p[EPT], d[EPT], a[EPT], w[EPT];
   long long am[EPT], wm[EPT];
   const bool v4 = EPT == 4 && vec && l0 + 4 <= n;
   if constexpr (EPT == 4) if (v4) {
-    const int4 P4 = *reinterpret_cast<const int4*>(c.P + x0);
-    const int4 D4 = *reinterpret_cast<const int4*>(c.D + x0);
-    p[0] = P4.x; p[1] = P4.y; p[2] = P4.z; p[3] = P4.w;
-    d[0] = D4.x; d[1] = D4.y; d[2] = D4.z; d[3] = D4.w;
+    auto quad = [&](const int32_t* src, int32_t (&v)[EPT]) {
+      const int4 q = !STAGES || src ? *reinterpret_cast<const int4*>(src + xi)
+                                    : make_int4(0, 0, 0, 0);
+      v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+    };
+    quad(c.P, p);
+    quad(c.D, d);
     if (MEAN) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const longlong2 A2 = reinterpret_cast<const longlong2*>(c.A_ms + x0)[h];
-        const longlong2 W2 = reinterpret_cast<const longlong2*>(c.W_ms + x0)[h];
+        const longlong2 A2 = reinterpret_cast<const longlong2*>(c.A_ms + xi)[h];
+        const longlong2 W2 = reinterpret_cast<const longlong2*>(c.W_ms + xi)[h];
         am[2 * h] = A2.x; am[2 * h + 1] = A2.y;
         wm[2 * h] = W2.x; wm[2 * h + 1] = W2.y;
       }
     } else {
-      const int4 A4 = *reinterpret_cast<const int4*>(c.A + x0);
-      const int4 W4 = *reinterpret_cast<const int4*>(c.W + x0);
-      a[0] = A4.x; a[1] = A4.y; a[2] = A4.z; a[3] = A4.w;
-      w[0] = W4.x; w[1] = W4.y; w[2] = W4.z; w[3] = W4.w;
+      quad(c.A, a);
+      quad(c.W, w);
     }
   }
   if (!v4) {
 #pragma unroll
     for (int i = 0; i < EPT; ++i) {
       const bool in = l0 + i < n;
-      p[i] = in ? c.P[x0 + i] : 0;
-      d[i] = in ? c.D[x0 + i] : 0;
+      p[i] = in && (!STAGES || c.P) ? c.P[xi + i] : 0;
+      d[i] = in && (!STAGES || c.D) ? c.D[xi + i] : 0;
       if (MEAN) {
-        am[i] = in ? c.A_ms[x0 + i] : 0;
-        wm[i] = in ? c.W_ms[x0 + i] : 0;
+        am[i] = in ? c.A_ms[xi + i] : 0;
+        wm[i] = in ? c.W_ms[xi + i] : 0;
       } else {
-        a[i] = in ? c.A[x0 + i] : 0;
-        w[i] = in ? c.W[x0 + i] : 0;
+        a[i] = in ? c.A[xi + i] : 0;
+        w[i] = in && (!STAGES || c.W) ? c.W[xi + i] : 0;
       }
     }
   }
@@ -188,7 +195,9 @@ k_raw(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ TilePl
                    : raw_tss_mean<T>(p[i], d[i], am[i], wm[i], dt, (T)tab.win[s], w_p[m], w_q[m]);
     } else {
       idle = (p[i] | d[i] | a[i] | w[i]) == 0;
-      rv[i] = idle ? idle_raw((T)0) : raw_tss<T>(p[i], d[i], a[i], w[i], dt, w_p[m], w_q[m]);
+      rv[i] = idle ? idle_raw((T)0)
+                   : raw_tss<T>(p[i], d[i], a[i], w[i], dt, STAGES && s == 0 ? (T)1 : w_p[m],
+                                w_q[m]);
     }
     cv[i] = idle ? kIdle : kNom;
     if (++m == M) m = 0;
@@ -1067,40 +1076,21 @@ template <class T> int score_launches(const SeriesTable<T>& tab, bool with_z) {
   return (total_elems(tab) >= kActiveMinCells ? 1 : 0) + 3 + (with_z ? 1 : 0);
 }
 
+// the smoothing of Eq. 1 values and idle classes k_raw has written
 template <class T>
-cudaError_t launch_score(const SeriesTable<T>& tab, const int32_t* P, const int32_t* D,
-                         const int32_t* A, const int32_t* W, const T* w_p, const T* w_q,
-                         const T* alpha, const T* theta, const T* tau_crit, const T* tau_surp,
-                         T* S_carry, uint8_t* init_carry, T* S, T* Z, uint8_t* cls,
-                         int32_t* recv, ScoreWs<T>& w, tre_diag* diag, cudaStream_t s,
-                         const int64_t* A_ms, const int64_t* W_ms) {
+static cudaError_t smooth(const SeriesTable<T>& tab, const T* alpha, T* S_carry,
+                          uint8_t* init_carry, T* S, const uint8_t* cls, ScoreWs<T>& w,
+                          tre_diag* diag, cudaStream_t s) {
   const int M = tab.M;
   const int n_seg = tab.seg_base[tab.n];
   if (n_seg > w.cap_seg) return cudaErrorInvalidValue;
-  if ((A_ms == nullptr) != (W_ms == nullptr)) return cudaErrorInvalidValue;
-  const int64_t total = total_elems(tab);
-  if (total == 0) return cudaSuccess;
-  const Counts c{P, D, A, W, A_ms, W_ms};
-  const bool small = total <= kSmallCells;
-  const int th = small ? kSmallThreads : kEwThreads;
-  int n_tiles = 0;
-  const TilePlan tp = tile_plan(tab, small ? th : 4 * th, n_tiles);
-  if (A_ms) {
-    const bool vec = quad_aligned(tab, {P, D, A_ms, W_ms, w.raw, cls});
-    auto f = small ? k_raw<T, true, 1> : k_raw<T, true, 4>;
-    f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(M), vec, c, w_p, w_q, w.raw, cls);
-  } else {
-    const bool vec = quad_aligned(tab, {P, D, A, W, w.raw, cls});
-    auto f = small ? k_raw<T, false, 1> : k_raw<T, false, 4>;
-    f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(M), vec, c, w_p, w_q, w.raw, cls);
-  }
   const int64_t segs = (int64_t)n_seg * M;
   const unsigned g = (unsigned)((segs + kChains - 1) / kChains);
   // activity counts for the burn-ins where the series are long enough that
   // idle stretches would otherwise send chunks to the in-order pass, and the
   // extra pass over the classes is small beside the smoothing
   const int32_t* active = nullptr;
-  if (total >= kActiveMinCells) {
+  if (total_elems(tab) >= kActiveMinCells) {
     k_active<T><<<n_seg, 256, (size_t)M * sizeof(int32_t), s>>>(tab, FastDiv(M), cls, w.active);
     active = w.active;
   }
@@ -1112,12 +1102,95 @@ cudaError_t launch_score(const SeriesTable<T>& tab, const int32_t* P, const int3
   k_resolve<T><<<tab.n * M, kResolveThreads, 0, s>>>(tab, w.raw, alpha, w.start_S, w.start_init,
                                                      w.end_S, w.end_init, S, cls, S_carry,
                                                      init_carry, diag);
-  if ((e = cudaGetLastError())) return e;
+  return cudaGetLastError();
+}
+
+template <class T>
+cudaError_t launch_score(const SeriesTable<T>& tab, const int32_t* P, const int32_t* D,
+                         const int32_t* A, const int32_t* W, const T* w_p, const T* w_q,
+                         const T* alpha, const T* theta, const T* tau_crit, const T* tau_surp,
+                         T* S_carry, uint8_t* init_carry, T* S, T* Z, uint8_t* cls,
+                         int32_t* recv, ScoreWs<T>& w, tre_diag* diag, cudaStream_t s,
+                         const int64_t* A_ms, const int64_t* W_ms) {
+  const int M = tab.M;
+  if ((A_ms == nullptr) != (W_ms == nullptr)) return cudaErrorInvalidValue;
+  const int64_t total = total_elems(tab);
+  if (total == 0) return cudaSuccess;
+  const Counts c{P, D, A, W, A_ms, W_ms};
+  const bool small = total <= kSmallCells;
+  const int th = small ? kSmallThreads : kEwThreads;
+  int n_tiles = 0;
+  const TilePlan tp = tile_plan(tab, small ? th : 4 * th, n_tiles);
+  if (A_ms) {
+    const bool vec = quad_aligned(tab, {P, D, A_ms, W_ms, w.raw, cls});
+    auto f = small ? k_raw<T, true, 1, false> : k_raw<T, true, 4, false>;
+    f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(M), vec, c, c, w_p, w_q, w.raw, cls);
+  } else {
+    const bool vec = quad_aligned(tab, {P, D, A, W, w.raw, cls});
+    auto f = small ? k_raw<T, false, 1, false> : k_raw<T, false, 4, false>;
+    f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(M), vec, c, c, w_p, w_q, w.raw, cls);
+  }
+  const cudaError_t e = smooth<T>(tab, alpha, S_carry, init_carry, S, cls, w, diag, s);
+  if (e) return e;
   // Z and regions in a pass of their own: the division in the chain's warp
   // cost more than re-reading S (8 models, 60 windows in double: 33 us of
   // smoothing with it; one hour of 100 ms windows in float: 42)
   if (theta) return launch_normalize<T>(tab, S, cls, theta, tau_crit, (T)0, tau_surp, Z, cls, recv, s);
   return cudaSuccess;
+}
+
+// The stage-aware signal as a table of two series (prefill, decode): Eq. 1 of
+// each from its own counts, smoothed together; S, cls at the series' offsets.
+template <class T>
+cudaError_t launch_score_stages(const SeriesTable<T>& tab, const int32_t* P, const int32_t* D,
+                                const int32_t* W, const int32_t* A_pre, const int32_t* A_dec,
+                                const T* w_p, const T* w_q, const T* alpha, T* S, uint8_t* cls,
+                                ScoreWs<T>& w, tre_diag* diag, cudaStream_t s) {
+  const int64_t total = total_elems(tab);
+  if (total == 0) return cudaSuccess;
+  const bool small = total <= kSmallCells;
+  const int th = small ? kSmallThreads : kEwThreads;
+  int n_tiles = 0;
+  const TilePlan tp = tile_plan(tab, small ? th : 4 * th, n_tiles);
+  const Counts pre{P, nullptr, A_pre, W, nullptr, nullptr};
+  const Counts dec{nullptr, D, A_dec, nullptr, nullptr, nullptr};
+  const bool vec = quad_aligned(tab, {P, D, W, A_pre, A_dec, w.raw, cls});
+  auto f = small ? k_raw<T, false, 1, true> : k_raw<T, false, 4, true>;
+  f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(tab.M), vec, pre, dec, w_p, w_q, w.raw, cls);
+  return smooth<T>(tab, alpha, nullptr, nullptr, S, cls, w, diag, s);
+}
+
+// both stages' S, Z and regions into arrays of their own (blockIdx.y: stage)
+template <class T>
+__global__ void __launch_bounds__(kSmallThreads)
+k_norm_stages(const __grid_constant__ SeriesTable<T> tab, FastDiv fm, const T* __restrict__ S,
+              const uint8_t* __restrict__ idle_cls, const T* __restrict__ tau_crit,
+              const T* __restrict__ tau_surp, StageOut<T> o0, StageOut<T> o1) {
+  const StageOut<T> o = blockIdx.y ? o1 : o0;
+  const int M = tab.M;
+  const int64_t n = (int64_t)tab.K[0] * M, off = tab.off[blockIdx.y];
+  for (int64_t i = (int64_t)blockIdx.x * kSmallThreads + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * kSmallThreads) {
+    const int m = i <= 0xffffffffll ? (int)((uint32_t)i - fm.div((uint32_t)i) * (uint32_t)M)
+                                    : (int)(i % M);
+    const T v = S[off + i], z = div_rn(v, o.theta[m]);
+    o.S[i] = v;
+    o.Z[i] = z;
+    o.cls[i] = region_of(idle_cls[off + i], z, tau_crit[m], tau_surp[m]);
+  }
+}
+
+template <class T>
+cudaError_t launch_norm_stages(const SeriesTable<T>& tab, const T* S, const uint8_t* idle_cls,
+                               const T* tau_crit, const T* tau_surp, const StageOut<T>& pre,
+                               const StageOut<T>& dec, cudaStream_t s) {
+  const int64_t n = (int64_t)tab.K[0] * tab.M;
+  if (n == 0) return cudaSuccess;
+  const int64_t b = std::min<int64_t>((n + kSmallThreads - 1) / kSmallThreads,
+                                      (int64_t)device_sm_count() * 16);
+  k_norm_stages<T><<<dim3((unsigned)b, 2), kSmallThreads, 0, s>>>(
+      tab, FastDiv(tab.M), S, idle_cls, tau_crit, tau_surp, pre, dec);
+  return cudaGetLastError();
 }
 
 template <class T>
@@ -1161,6 +1234,13 @@ cudaError_t launch_rank(int M, int K, const T* Z, const uint8_t* cls, int32_t* r
 }
 
 #define TRE_INST(T)                                                                               \
+  template cudaError_t launch_score_stages<T>(const SeriesTable<T>&, const int32_t*,               \
+                                              const int32_t*, const int32_t*, const int32_t*,      \
+                                              const int32_t*, const T*, const T*, const T*, T*,    \
+                                              uint8_t*, ScoreWs<T>&, tre_diag*, cudaStream_t);     \
+  template cudaError_t launch_norm_stages<T>(const SeriesTable<T>&, const T*, const uint8_t*,      \
+                                             const T*, const T*, const StageOut<T>&,               \
+                                             const StageOut<T>&, cudaStream_t);                    \
   template int series_segments<T>(SeriesTable<T>&);                                               \
   template int score_launches<T>(const SeriesTable<T>&, bool);                                        \
   template void score_ws_layout<T>(Arena&, int, int64_t, int, ScoreWs<T>&);                       \

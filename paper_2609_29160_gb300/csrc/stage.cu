@@ -64,12 +64,6 @@ k_stage_requests(ReqCols r, int M, int win, FastDiv fd, int K, int32_t* __restri
   }
 }
 
-template <class T> __global__ void k_fill(T* p, int64_t n, T v) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    p[i] = v;
-}
-
 unsigned grid_of(int64_t n) {
   const int64_t b = (n + kThreads - 1) / kThreads;
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)device_sm_count() * 8));
@@ -88,23 +82,14 @@ cudaError_t launch_stage_requests(const ReqCols& r, int M, int win, int K, int32
     if ((e = cudaMemsetAsync(dDec, 0, cells1 * sizeof(int32_t), s))) return e;
   }
   if (ttft) {
-    if ((e = cudaMemsetAsync(ttft, 0, cells * sizeof(unsigned long long), s))) return e;
-    if ((e = cudaMemsetAsync(tpot, 0, cells * sizeof(unsigned long long), s))) return e;
+    // the block from the first count of ttft to the last of tpot
+    e = cudaMemsetAsync(ttft, 0, (size_t)(tpot - ttft + cells) * sizeof(unsigned long long), s);
+    if (e) return e;
   }
   if (r.n == 0) return cudaSuccess;
   k_stage_requests<<<grid_of(r.n), kThreads, 0, s>>>(r, M, win, FastDiv(win), K, dPre, dDec,
                                                       ttft, tpot, ttft_ms, tpot_ms);
   return cudaGetLastError();
 }
-
-template <class T> cudaError_t launch_fill(T* p, int64_t n, T v, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  k_fill<T><<<grid_of(n), kThreads, 0, s>>>(p, n, v);
-  return cudaGetLastError();
-}
-
-template cudaError_t launch_fill<float>(float*, int64_t, float, cudaStream_t);
-template cudaError_t launch_fill<double>(double*, int64_t, double, cudaStream_t);
-template cudaError_t launch_fill<int32_t>(int32_t*, int64_t, int32_t, cudaStream_t);
 
 }  // namespace tre

@@ -564,6 +564,27 @@ def test_stage_signal_adversarial(tre, seed, M, win, K):
             np.testing.assert_array_equal(_np(sd[k]), o["decode"][k], err_msg="decode " + k)
 
 
+# one cell; a second series off its own 16-byte boundary; a large table whose
+# last tile is ragged
+@pytest.mark.parametrize("M,win,K", [(1, 1000, 1), (3, 500, 301), (7, 100, 40001)])
+def test_stage_table_edges(tre, M, win, K):
+    rng = np.random.default_rng(K)
+    req = _adversarial(rng, 4 + K // 4, M, win, K)
+    tpot = rng.integers(1, 40, M).astype(np.int32)
+    slo = rng.integers(100, 3000, M).astype(np.int32)
+    prof = tracegen.default_profile(M, win)
+    o = oracle.stage_pipeline(req, M, win, K, prof, slo, tpot, np.float32)
+    rc = _cuda(req)
+    A_p, A_d = tre.tss_stage_gauges(M, win, K, rc)
+    c = tre.tss_window_reduce(M, win, K, requests=rc)
+    th = tre.tss_stage_calibrate(c, A_p, A_d, prof, win, slo, tpot, rc, dtype="f32")
+    out = tre.tss_stage_score(c, A_p, A_d, prof, win, *th, dtype="f32")
+    for stage, t, x in zip(("prefill", "decode"), th, out):
+        np.testing.assert_array_equal(_np(t), o[stage]["theta"], err_msg=stage)
+        for k in ("S", "Z", "cls"):
+            np.testing.assert_array_equal(_np(x[k]), o[stage][k], err_msg=stage + " " + k)
+
+
 def test_calibrate_events(tre):
     w = _events_case(6)
     ev, M, win, K = w["events"], w["M"], w["window_ms"], w["K"]
