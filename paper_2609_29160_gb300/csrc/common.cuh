@@ -68,6 +68,43 @@ struct FastDiv {
   }
 };
 
+// The same for dividends below 2^31 (non-negative milliseconds) and
+// 1 <= d < 2^31, in three instructions: with 2^(l-1) < d <= 2^l and
+// m = ceil(2^(31+l) / d), x * m / 2^(31+l) has the quotient as its floor.
+struct FastDiv31 {
+  uint32_t m, l;
+  FastDiv31() = default;
+  __host__ __device__ explicit FastDiv31(uint32_t d) : m(0), l(0) {
+    while ((1ull << l) < d) ++l;
+    m = (uint32_t)(((1ull << (31 + l)) + d - 1) / d);
+  }
+  __device__ __forceinline__ uint32_t div(uint32_t x) const { return __umulhi(x << 1, m) >> l; }
+};
+
+// floor and remainder of x / d with a quotient below 2^20 (q_lim: a bound known
+// to the caller), d < 2^30 and x < 2^32: an approximate float quotient is off by
+// less than one, so one correction either way makes it exact. Anything larger
+// divides in integers.
+__device__ __forceinline__ void divmod_near(unsigned long long x, uint32_t d, uint32_t q_lim,
+                                            uint32_t& q, uint32_t& r) {
+  if ((x >> 32) == 0 && q_lim < (1u << 20) && d < (1u << 30)) {
+    q = (uint32_t)__fdividef((float)(uint32_t)x, (float)d);
+    r = (uint32_t)x - q * d;
+    if ((int32_t)r < 0) {
+      --q;
+      r += d;
+    } else if (r >= d) {
+      ++q;
+      r -= d;
+    }
+  } else {
+    unsigned long long q64, r64;
+    divmod(x, d, q64, r64);
+    q = (uint32_t)q64;
+    r = (uint32_t)r64;
+  }
+}
+
 // Largest i in [0, n) with base[i] * scale <= v, for a non-decreasing table
 // (prefix sums of per-series counts) with base[0] * scale <= v: a binary
 // search, so a lookup in a 64-entry kernel-parameter table costs six steps.

@@ -41,7 +41,11 @@ __device__ __forceinline__ void stage_add(V* s, V* g, int64_t k, int64_t k_lo, i
 // --------------------------------------------------------------------------
 constexpr int kMaxTraces = 64;
 constexpr int kVec = 4;               // records per thread per pass
+constexpr size_t kSmemQuarter = 54 * 1024;   // of an SM's shared memory, for four CTAs on it
 constexpr int kMaxPerCta = 16384;     // bound that keeps the packed shared counters exact
+constexpr int kPass = kThreads * kVec;  // records per pass of a CTA
+// queue entries of a CTA of p records: whole passes of every warp
+constexpr __host__ __device__ int64_t queue_cap(int64_t p) { return (p + kPass - 1) / kPass * kPass; }
 constexpr int kFarScan = 1024;        // records that place a CTA's start-side rows
 struct ReqBatch {
   int n;
@@ -78,21 +82,29 @@ struct Stage {
 
 // Long decodes (beyond the window after the first-token window) are queued per
 // warp -- the record's index in the CTA, at most one entry per record -- and,
-// after the warp's last pass, walked one record per lane without a division
-// per window: with y the emitted-token bound shifted so that N(T) =
-// floor(y / dur), moving one window boundary adds win*(L-1) = Q*dur + R to y,
-// so a window gets Q or Q + 1 tokens.
+// after the warp's last pass, walked without a division per window: with y the
+// emitted-token bound shifted so that N(T) = floor(y / dur), moving one window
+// boundary adds win*(L-1) = Q*dur + R to y, so a window gets Q or Q + 1 tokens.
+// One record per lane walks its windows in turn; records of more than kLaneWalk
+// windows are taken by the whole warp, a window per lane (the s-th window on
+// gets Q + 1 tokens where (rem + s*R) mod dur < R), so that a lane's long record
+// does not hold the other 31 up.
+constexpr int kLaneWalk = 12;
 
-
+// What bounds the kernel is instructions (the sweep's seven traces of 1M records:
+// 96 M warp instructions, now 90 M, 131 us; 10M records of 16 models 120 us, now
+// 109; a third of it HBM time): windows by three-instruction division, token
+// quotients from a float estimate, record tests without branches, the staging
+// cleared 16 bytes a store.
 template <bool SLO, bool COPY>
 __global__ void __launch_bounds__(kThreads, 4)
-k_reduce_requests(const __grid_constant__ ReqBatch bt, int M, int lgMp, int win, FastDiv fd,
+k_reduce_requests(const __grid_constant__ ReqBatch bt, int M, int lgMp, int win, FastDiv31 fd,
                   int K, int near_rows, int lgF, int32_t* __restrict__ P0,
                   int32_t* __restrict__ D0, int32_t* __restrict__ dA0, int32_t* __restrict__ dW0,
                   unsigned long long* __restrict__ slo0, const int32_t* __restrict__ slo_ms,
                   tre_diag* diag) {
   extern __shared__ unsigned long long smem[];
-  unsigned long long n_range = 0, n_model = 0, n_order = 0;
+  uint32_t n_range = 0, n_model = 0, n_order = 0;
   // a CTA takes slices blockIdx.x, blockIdx.x + gridDim.x, ...: one slice when
   // the grid holds them all; a smaller grid leaves SMs to other streams' work
   // (records read over the host link keep fewer SMs busy just as well)
@@ -152,13 +164,14 @@ k_reduce_requests(const __grid_constant__ ReqBatch bt, int M, int lgMp, int win,
     st.slo_lim = st.far_lo + M;
     st.queue = reinterpret_cast<uint16_t*>((reinterpret_cast<uintptr_t>(st.slo_lim + M) + 15) &
                                            ~(uintptr_t)15) +
-               (size_t)(threadIdx.x >> 5) * (bt.per_cta[t] / (kThreads / 32));
-    const int ncell = used * Mp, fcell = M * F1;
-    for (int c = threadIdx.x; c < ncell; c += kThreads) {
-      st.aW[c] = 0;
-      if (SLO) st.aS[c] = 0;
-    }
-    for (int c = threadIdx.x; c < fcell; c += kThreads) { st.fP[c] = 0; st.fD[c] = 0; st.fAW[c] = 0; }
+               (size_t)(threadIdx.x >> 5) * (queue_cap(bt.per_cta[t]) / (kThreads / 32));
+    const int ncell = used * Mp;
+    // the staged arrays lie one behind the other, from a 16-byte boundary
+    const int n_stage = near_rows * Mp * (SLO ? 2 : 1) + 3 * M * F1;
+    int32_t* stage = st.aW;
+    for (int c = 4 * threadIdx.x; c + 4 <= n_stage; c += 4 * kThreads)
+      *reinterpret_cast<int4*>(stage + c) = make_int4(0, 0, 0, 0);
+    for (int c = (n_stage & ~3) + threadIdx.x; c < n_stage; c += kThreads) stage[c] = 0;
     for (int m = threadIdx.x; m < M; m += kThreads) {
       st.far_lo[m] = 0x7fffffff;
       if (SLO) st.slo_lim[m] = slo_ms[m];
@@ -246,40 +259,38 @@ k_reduce_requests(const __grid_constant__ ReqBatch bt, int M, int lgMp, int win,
       }
 #pragma unroll
       for (int u = 0; u < kVec; ++u) {
-        const bool present = b + u < n_loc;
         const int m = v[0][u], ta = v[1][u], ts = v[2][u], tf = v[3][u], te = v[4][u];
         const int L_in = v[5][u], L = v[6][u];
-        bool ok = false;
-        if (present) {
-          if (m < 0 || m >= M) ++n_model;
-          else if (ta < 0 || (uint32_t)ta >= span) ++n_range;
-          else if (!(ta <= ts && ts <= tf && tf <= te) || L_in < 0 || L < 1) ++n_order;
-          else ok = true;
-        }
+        const bool ok = (uint32_t)m < (uint32_t)M & (uint32_t)ta < span & ta <= ts & ts <= tf &
+                        tf <= te & L_in >= 0 & L >= 1;
         // decode windows after the first-token window go to the warp's queue
         bool lng = false;
-        int kf = 0;
-        if (ok) {
+        if (!ok) {
+          if (b + u < n_loc) {
+            if ((uint32_t)m >= (uint32_t)M) ++n_model;
+            else if ((uint32_t)ta >= span) ++n_range;
+            else ++n_order;
+          }
+        } else {
           const int lo = st.far_lo[m];
           const int ba = (int)fd.div((uint32_t)ta);
           const int bs = (int)min(fd.div((uint32_t)ts), (uint32_t)K);
+          const int kf = (int)fd.div((uint32_t)tf);
           const int be_raw = (int)fd.div((uint32_t)te);
           const int be = min(be_raw, K);
-          const bool tok = (uint32_t)tf < span;
-          kf = tok ? (int)fd.div((uint32_t)tf) : 0;
+          const bool tok = kf < K;                    // the first token falls inside the grid
           // decode tokens of the first-token window (d0) and, for a decode that
           // ends in the next window, of that window (d1); longer decodes leave
           // their later windows to the queue walk below
           int d0 = L, d1 = 0;
           if (tok && L != 1 && be_raw != kf) {
             // N(T) = tokens emitted before T = ceil((T - tf)(L-1)/dur)
-            unsigned long long qq, rr;
-            divmod((unsigned long long)((uint32_t)(kf + 1) * (uint32_t)win - (uint32_t)tf) *
-                       (uint32_t)(L - 1),
-                   (uint32_t)(te - tf), qq, rr);
-            const int n1 = (int)(qq + (rr != 0));
-            d0 = n1;
-            if (be_raw == kf + 1) d1 = L - n1;
+            uint32_t qq, rr;
+            divmod_near((unsigned long long)((uint32_t)(kf + 1) * (uint32_t)win - (uint32_t)tf) *
+                            (uint32_t)(L - 1),
+                        (uint32_t)(te - tf), (uint32_t)L, qq, rr);
+            d0 = (int)(qq + (rr != 0));
+            if (be_raw == kf + 1) d1 = L - d0;
             else lng = kf + 1 < K;   // windows kf+1 .. min(be, K-1)
           }
           const int wait = ba != bs ? 1 : 0, run = bs != be ? 1 : 0;
@@ -322,51 +333,75 @@ k_reduce_requests(const __grid_constant__ ReqBatch bt, int M, int lgMp, int win,
         qn += __popc(qb);
       }
     }
-    // walk the warp's long decodes, one record per lane
+    // walk the warp's long decodes
     __syncwarp();
-    for (int i = lane; i < qn; i += 32) {
-      const int j = st.queue[i];
-      const int m = colp[0][j], tf = colp[3][j], te = colp[4][j], L = colp[6][j];
-      const int kf = (int)fd.div((uint32_t)tf), be_raw = (int)fd.div((uint32_t)te);
-      const uint32_t dur = (uint32_t)(te - tf);
-      unsigned long long qq, rr;
-      divmod((unsigned long long)((uint32_t)(kf + 1) * (uint32_t)win - (uint32_t)tf) *
-                 (uint32_t)(L - 1),
-             dur, qq, rr);
-      const uint32_t q1 = (uint32_t)qq, r1 = (uint32_t)rr;
-      {
+    for (int i0 = 0; i0 < qn; i0 += 32) {
+      // one record per lane: its full windows kf+1 .. kf+nw, then the last one
+      int m = 0, lo = 0, kf = 0, be_raw = 0, nw = 0, L = 0;
+      uint32_t dur = 1, rem = 0, Q = 0, R = 0, n = 0;
+      if (i0 + lane < qn) {
+        const int j = st.queue[i0 + lane];
+        m = colp[0][j];
+        L = colp[6][j];
+        const int tf = colp[3][j], te = colp[4][j];
+        kf = (int)fd.div((uint32_t)tf);
+        be_raw = (int)fd.div((uint32_t)te);
+        dur = (uint32_t)(te - tf);
+        lo = st.far_lo[m];
+        uint32_t q1, r1;
+        divmod_near((unsigned long long)((uint32_t)(kf + 1) * (uint32_t)win - (uint32_t)tf) *
+                        (uint32_t)(L - 1),
+                    dur, (uint32_t)L, q1, r1);
         // y = x + dur - 1 at the end of window kf: N = floor(y / dur), rem = y mod dur
-        uint32_t n = q1 + (r1 != 0);
-        uint32_t rem = r1 ? r1 - 1 : dur - 1;
-        unsigned long long Q64, R64;
-        divmod((unsigned long long)(uint32_t)win * (uint32_t)(L - 1), dur, Q64, R64);
-        const uint32_t Q = (uint32_t)Q64, R = (uint32_t)R64;   // Q < L: dur > win here
-        const int lo = st.far_lo[m];
-        const int k_full = min(be_raw - 1, K - 1);   // windows ending at or before t_end
-        const int k_end = min(be_raw, K - 1);
-        if ((uint32_t)(k_end - lo) < (uint32_t)F && kf + 1 >= lo) {
-          int32_t* fd_row = st.fD + m * F1 - lo;
-          for (int k = kf + 1; k <= k_full; ++k) {
+        n = q1 + (r1 != 0);
+        rem = r1 ? r1 - 1 : dur - 1;
+        divmod_near((unsigned long long)(uint32_t)win * (uint32_t)(L - 1), dur, (uint32_t)L, Q, R);
+        nw = min(be_raw - 1, K - 1) - kf;             // windows ending at or before t_end
+      }
+      // the whole warp takes a long one while 32 * R fits 32 bits
+      const bool wide = nw > kLaneWalk && dur < (1u << 26);
+      if (nw > 0 && !wide) {
+        if ((uint32_t)(min(be_raw, K - 1) - lo) < (uint32_t)F && kf + 1 >= lo) {
+          int32_t* row = st.fD + m * F1 - lo + kf + 1;
+          for (int w = 0; w < nw; ++w) {
             const uint32_t t = rem + R;
             const uint32_t c = t >= dur ? 1u : 0u;
             rem = t - (c ? dur : 0u);
             const uint32_t d = Q + c;
             n += d;
-            if (d) atomicAdd(&fd_row[k], (int32_t)d);
+            if (d) atomicAdd(&row[w], (int32_t)d);
           }
-          if (be_raw <= K - 1 && (uint32_t)L != n) atomicAdd(&fd_row[be_raw], (int32_t)(L - n));
         } else {
-          for (int k = kf + 1; k <= k_full; ++k) {
+          for (int w = 0; w < nw; ++w) {
             const uint32_t t = rem + R;
             const uint32_t c = t >= dur ? 1u : 0u;
             rem = t - (c ? dur : 0u);
             const uint32_t d = Q + c;
             n += d;
-            if (d) add_tok(st.fD, D, k, m, lo, (int32_t)d);
+            if (d) add_tok(st.fD, D, kf + 1 + w, m, lo, (int32_t)d);
           }
-          if (be_raw <= K - 1 && (uint32_t)L != n) add_tok(st.fD, D, be_raw, m, lo, (int32_t)(L - n));
         }
       }
+      for (unsigned todo = __ballot_sync(full, wide); todo; todo &= todo - 1) {
+        const int src = __ffs(todo) - 1;
+        const int wm = __shfl_sync(full, m, src), wlo = __shfl_sync(full, lo, src);
+        const int wk = __shfl_sync(full, kf, src) + 1, ww = __shfl_sync(full, nw, src);
+        const uint32_t wd = __shfl_sync(full, dur, src), wQ = __shfl_sync(full, Q, src);
+        const uint32_t wR = __shfl_sync(full, R, src);
+        uint32_t wr = __shfl_sync(full, rem, src), wn = __shfl_sync(full, n, src);
+        for (int b0 = 0; b0 < ww; b0 += 32) {
+          uint32_t f, r;
+          divmod_near(wr + (uint32_t)(lane + 1) * wR, wd, 33u, f, r);
+          const uint32_t d = wQ + (r < wR ? 1u : 0u);
+          if (b0 + lane < ww && d) add_tok(st.fD, D, wk + b0 + lane, wm, wlo, (int32_t)d);
+          const int end = min(ww - b0, 32) - 1;
+          wn += (uint32_t)(end + 1) * wQ + __shfl_sync(full, f, end);
+          wr = __shfl_sync(full, r, end);
+        }
+        if (lane == src) n = wn;
+      }
+      if (nw > 0 && be_raw <= K - 1 && (uint32_t)L != n)
+        add_tok(st.fD, D, be_raw, m, lo, (int32_t)((uint32_t)L - n));
     }
     __syncthreads();
     for (int c = threadIdx.x; c < ncell; c += kThreads) {
@@ -1098,25 +1133,49 @@ cudaError_t launch_reduce_requests(const ReqCols* traces, int n_traces, int M, i
   int lgF = 3;
   while (lgF < 8 && (size_t)12 * M * ((2 << lgF) + 1) <= 16 * 1024) ++lgF;
   const int F = 1 << lgF;
-  // arrival-side rows (3x the mean arrival span of a CTA's records) and the
-  // shared memory a CTA of `p` records needs
+  // arrival-side rows (3x the mean arrival span of a CTA's records, less where
+  // that would keep four CTAs from sharing an SM) and the shared memory a CTA of
+  // `p` records needs
+  const size_t row_bytes = (size_t)Mp * (4 + (slo ? 4 : 0));
+  auto rest_for = [&](int64_t p) {
+    return (size_t)12 * M * (F + 1) + (size_t)M * 8 + 16 + (size_t)queue_cap(p) * sizeof(uint16_t);
+  };
   auto rows_for = [&](int64_t p) {
-    return (int)std::max<int64_t>(
-        1, std::min<int64_t>(near_cap, (int64_t)(3.0 * p / mean_n * K) + 34));
+    int64_t cap = near_cap;
+    if (rest_for(p) + 16 * 1024 <= kSmemQuarter)
+      cap = std::min<int64_t>(cap, (int64_t)((kSmemQuarter - rest_for(p)) / row_bytes));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(cap, (int64_t)(3.0 * p / mean_n * K) + 34));
   };
   auto smem_for = [&](int64_t p) {
-    const size_t stage = (size_t)rows_for(p) * Mp * (4 + (slo ? 4 : 0)) +
-                         (size_t)12 * M * (F + 1) + (size_t)M * 8 + 16 +
-                         (size_t)p * sizeof(uint16_t);
-    return stage + (copy_records ? (size_t)p * 7 * 4 : 0);
+    return (size_t)rows_for(p) * row_bytes + rest_for(p) + (copy_records ? (size_t)p * 7 * 4 : 0);
   };
   constexpr size_t kSmemMax = 200 * 1024;
-  // records per CTA sized on the whole batch so the grid fills the GPU, in
-  // whole passes of every warp; with copied records, fewer per CTA when many
-  // models leave less room beside the staging
-  int64_t per = per_cta_records(mean_n, 1024, copy_records ? 2048 : 8192, kThreads * kVec);
-  while (per > kThreads * kVec && smem_for(per) > kSmemMax) per -= kThreads * kVec;
-  static_assert(8192 <= kMaxPerCta, "packed shared counters need <= kMaxPerCta records per CTA");
+  // Records per CTA: whole waves of four CTAs an SM (10M records cut into 8192s
+  // were 1,221 CTAs, five more than two waves), but arrivals of no more than half
+  // the start side's windows, as starts and decodes past them go to global
+  // atomics. Copied records: fewer per CTA, and fewer still where many models
+  // leave less room beside the staging.
+  int64_t per;
+  if (copy_records) {
+    per = per_cta_records(mean_n, kPass, 2048, kPass);
+  } else {
+    static_assert(9 * kPass <= kMaxPerCta, "packed shared counters need <= kMaxPerCta records");
+    const int64_t cap = std::max<int64_t>(
+        2 * kPass, std::min<int64_t>(9 * kPass, (int64_t)(0.5 * F * mean_n / std::max(K, 1))));
+    const int64_t slots = (int64_t)num_sms() * 4;
+    const int64_t most =
+        slots * std::max<int64_t>(1, (total_n + slots * cap - 1) / (slots * cap));
+    per = std::max<int64_t>(kPass, (total_n + most - 1) / most);
+    const int64_t quantum = per <= 4 * kPass ? kPass : 32 * kVec;
+    auto ctas_of = [&](int64_t p) {
+      int64_t c = 0;
+      for (int t = 0; t < n_traces; ++t) c += (traces[t].n + p - 1) / p;
+      return c;
+    };
+    per = (per + quantum - 1) / quantum * quantum;
+    while (per + quantum <= cap && ctas_of(per) > most) per += quantum;
+  }
+  while (per > kPass && smem_for(per) > kSmemMax) per -= kPass;
   const int near_rows = rows_for(per);
   const size_t smem = smem_for(per);
   if (smem > kSmemMax) return cudaErrorInvalidValue;
@@ -1144,7 +1203,7 @@ cudaError_t launch_reduce_requests(const ReqCols* traces, int n_traces, int M, i
     cudaError_t e = func_smem_once(f, 200 * 1024, true);
     if (e) return e;
   }
-  const FastDiv fd(win);
+  const FastDiv31 fd(win);
   // Records read over the host link: one CTA per slice would hold every SM for
   // the length of the transfer. CTAs on two thirds of the SMs (two each) still
   // keep the link busy -- a CTA spends most of a slice copying it in -- and

@@ -176,6 +176,36 @@ def test_reduce_events_shuffled_and_corrupt(tre):
     assert [d["dropped_range"], d["dropped_model"], d["dropped_order"]] == drops.tolist()
 
 
+# Decodes over as many windows as one lane walks (12) and one more, over whole
+# and broken runs of 32; spans past 2^26 and 2^30 ms, outputs past 2^20 tokens and
+# products past 2^32 leave the float quotients and the warp's walk; window
+# lengths of 1 ms, a power of two and neither.
+@pytest.mark.parametrize("win,K", [(1, 5000), (64, 3000), (1000, 200), (997, 1_100_000)])
+def test_reduce_long_decode_edges(tre, win, K):
+    rng = np.random.default_rng(win)
+    M, n = 5, 700
+    nw = rng.choice([0, 1, 2, 11, 12, 13, 14, 31, 32, 33, 34, 63, 64, 65, 199, 1000], n)
+    tf = np.sort(rng.integers(0, K * win, n))
+    te = tf + nw * win + rng.integers(0, win + 1, n)
+    L = rng.choice([1, 2, 3, 50, 4000, 100_000], n)
+    if K > 1_000_000:
+        te[::9] = tf[::9] + (1 << 26) + rng.integers(-2, 3, len(te[::9]))
+        te[::70] = np.minimum(tf[::70] + (1 << 30) + 5, 2**31 - 2)
+        L[:3] = (1 << 20) - 1, 1 << 20, (1 << 20) + 1
+    te = np.minimum(te, 2**31 - 2)
+    te[L == 1] = tf[L == 1]
+    ta = np.maximum(tf - rng.integers(0, 3 * win + 1, n), 0)
+    req = {"model": rng.integers(0, M, n), "t_arr_ms": ta, "t_start_ms": (ta + tf) // 2,
+           "t_first_ms": tf, "t_end_ms": te, "L_in": rng.integers(0, 900, n), "L_out": L}
+    order = np.argsort(ta, kind="stable")
+    req = {k: v[order].astype(np.int32) for k, v in req.items()}
+    P, D, A, W, drops = oracle.reduce_requests(req, M, win, K)
+    c = tre.tss_window_reduce(M, win, K, requests=_cuda(req))
+    for k, ref in zip("PDAW", (P, D, A, W)):
+        np.testing.assert_array_equal(_np(c[k]), ref, err_msg=k)
+    assert drops.sum() == 0
+
+
 def _score_inputs(rng, K, M, idle_frac=0.2):
     cnt = {}
     for k, hi in (("P", 5000), ("D", 800), ("A", 30), ("W", 60)):
