@@ -472,7 +472,7 @@ tre_status sweep_typed(const tre_sweep_spec* sp, const SweepPlan& pl, const tre_
     }
   } else {
     if (!e) {
-      Scope sc(kScan, 3, s);
+      Scope sc(kScan, gauge_scan_launches(rw), s);
       e = launch_gauge_scan(M, pl.Kb, rw, Ab, Wb, s);
     }
     if (!e) {
@@ -721,14 +721,14 @@ tre_status tss_window_reduce(const tre_grid* grid, const tre_requests* req, cons
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   cudaError_t e;
   {
-    Scope sc(kReduce, req ? 2 : 3, s);   // clearing + reduction; or three event passes
+    Scope sc(kReduce, req ? 2 : 4, s);   // clearing + reduction; or clearing and three event passes
     const ReqCols rc = req ? cols_of(req) : ReqCols{};
     e = req ? launch_reduce_requests(&rc, 1, M, grid->window_ms, K, out.P, out.D, w, nullptr,
                                      nullptr, diag, s)
             : launch_reduce_events(cols_of(ev), M, grid->window_ms, K, out.P, out.D, w, diag, s);
   }
   if (!e) {
-    Scope sc(kScan, 3, s);
+    Scope sc(kScan, gauge_scan_launches(w), s);
     e = launch_gauge_scan(M, K, w, out.A, out.W, s);
   }
   if (!e && out.A_ms) {
@@ -870,7 +870,7 @@ tre_status tss_stage_gauges(const tre_grid* grid, const tre_requests* req, int32
                               nullptr, nullptr, s);
   }
   if (!e) {
-    Scope sc(kScan, 3, s);
+    Scope sc(kScan, gauge_scan_launches(w), s);
     e = launch_gauge_scan(M, K, w, A_prefill, A_decode, s);
   }
   return cuda_status(e);

@@ -80,6 +80,7 @@ struct ReduceWs {
   int32_t *partA, *partW;
   int64_t part_cap;            // partial entries per trace
   int n_traces;
+  bool chunks_summed;          // partA, partW hold the scan's chunk sums already (events)
 };
 constexpr int kGaugeMinBlk = 16;   // shortest row block of the fused gauge pass
 constexpr int kGaugeMaxWin = 8;    // most window lengths the fused gauge pass takes
@@ -100,6 +101,7 @@ cudaError_t launch_slo_requests(const ReqCols& r, int M, int win, int K,
 cudaError_t launch_slo_events(const EvCols& e, int M, int win, int K, unsigned long long* slo,
                               const int32_t* slo_ms, cudaStream_t s);
 // inclusive scan of the diff arrays over windows -> A, W (trace t at t*K*M)
+int gauge_scan_launches(const ReduceWs& w);
 cudaError_t launch_gauge_scan(int M, int K, ReduceWs& w, int32_t* A, int32_t* W, cudaStream_t s);
 // Time-averaged occupancy of one trace's request records: request-milliseconds
 // running and waiting per (window, model), int64 [K][M]; reuses the gauge

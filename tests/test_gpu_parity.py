@@ -206,6 +206,46 @@ def test_reduce_long_decode_edges(tre, win, K):
     assert drops.sum() == 0
 
 
+# Slices of 2048 events and more; an odd model count or misaligned columns take
+# single-cell flushes or scalar loads; more requests than table slots in a
+# slice; times past 2^21 s, denormals, both zeros, infinities and NaN.
+@pytest.mark.parametrize("M,n,n_req,win,K,shift", [
+    (1, 1, 1, 100, 50, 0), (2, 2047, 3, 100, 60, 0), (3, 2049, 5, 50, 400, 1),
+    (64, 20000, 3000, 100, 700, 0), (7, 40000, 40000, 1000, 90, 0),
+    (6, 9001, 40, 1_000_000, 2147, 0), (1024, 5000, 700, 500, 40, 2)])
+def test_reduce_events_edges(tre, M, n, n_req, win, K, shift):
+    import torch
+    rng = np.random.default_rng(n + M)
+    span = K * win / 1000.0
+    req_model = rng.integers(0, M, n_req).astype(np.int32)
+    if n_req >= 5:                              # requests of models that are not there
+        req_model[::5] = rng.choice([-2, -1, M, M + 3], len(req_model[::5]))
+    req = rng.integers(0, n_req, n).astype(np.int32)
+    t = np.sort(rng.random(n) * span).astype(np.float32)
+    odd = [np.float32(x) for x in (0.0, -0.0, 1e-40, -1e-40, np.inf, -np.inf, np.nan, 2097151.9,
+                                   2097152.0, 2147000.0, 0.001, 0.0009999999, span)]
+    at = rng.choice(n, min(n, len(odd)), replace=False)
+    if n > 1:
+        t[at] = odd[: len(at)]
+    model = req_model[req].copy()
+    model[::11] = rng.integers(0, M, len(model[::11]))       # not the request's
+    ev = {"model": model, "req": req, "t_s": t,
+          "phase": rng.integers(0, 2, n).astype(np.uint8), "req_model": req_model,
+          "req_t_arr_ms": np.zeros(n_req, np.int32), "req_ttft_ms": np.zeros(n_req, np.int32)}
+    dev = _cuda(ev)
+    for k in ("model", "req", "t_s", "phase"):          # columns off their alignment
+        pad = torch.empty(n + shift, dtype=dev[k].dtype, device="cuda")
+        pad[shift:] = dev[k]
+        dev[k] = pad[shift:]
+    P, D, A, W, drops = oracle.reduce_events(ev, M, win, K)
+    diag = tre.new_diag()
+    c = tre.tss_window_reduce(M, win, K, events=dev, diag=diag)
+    for k, ref in zip("PDAW", (P, D, A, W)):
+        np.testing.assert_array_equal(_np(c[k]), ref, err_msg=k)
+    d = tre.read_diag(diag)
+    assert [d["dropped_range"], d["dropped_model"], d["dropped_order"]] == drops.tolist()
+
+
 def _score_inputs(rng, K, M, idle_frac=0.2):
     cnt = {}
     for k, hi in (("P", 5000), ("D", 800), ("A", 30), ("W", 60)):
