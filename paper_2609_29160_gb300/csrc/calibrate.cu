@@ -17,6 +17,8 @@
 // over the key range refines one bucket after another. Counts are exact
 // integers and the tests give the definition's double comparison, so theta is
 // exact.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "common.cuh"
@@ -335,7 +337,7 @@ template <class T> size_t search_smem_bytes() {
   return fast > descent ? fast : descent;
 }
 
-// One CTA per (series, model). DIRECT: the keys are made here, from the
+// One CTA per (series, model), or a cluster of CL of them. DIRECT: the keys are made here, from the
 // model's column of S, classes and counts, and stay in registers (series of up
 // to kDirectK windows): one launch where packing, its threshold table and the
 // search were three. Otherwise they come from the packing pass, and are read
@@ -343,7 +345,12 @@ template <class T> size_t search_smem_bytes() {
 // 8 models, 3,600 windows: 15.4 us in one launch (25.3 in three, with a bitonic
 // sort of the gathered keys and every test in double); 16 models, 43,200
 // windows: 21.6 us (30.5); the sweep's 224 searches: 24.5 us (33.3).
-template <class T, bool DIRECT>
+//
+// With CL CTAs each reads its part of the keys: they count into their own
+// histograms, the first adds them up and chooses the buckets, all list the keys
+// of those buckets in the first one's memory, and the first tests them. Long
+// series leave SMs idle otherwise: 64 series of 864,000 windows took 250 us.
+template <class T, bool DIRECT, int CL>
 __global__ void __launch_bounds__(kNB, !DIRECT && sizeof(T) == 4 ? 2 : 1)
 k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __restrict__ keys,
          const typename KeyOf<T>::U* kmin_g, const typename KeyOf<T>::U* kmax_g,
@@ -362,9 +369,14 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
   __shared__ U redU[2][kWarps];
   __shared__ int thr_s[kThrDirect];
   __shared__ U bfmin_s, best_s;
+  __shared__ int plan_s[2];       // keys listed, lowest found bucket
+  namespace cg = cooperative_groups;
+  static_assert(!DIRECT || CL == 1, "short series need one CTA");
   const int M = tab.M;
-  const int s = blockIdx.x / M, m = blockIdx.x % M;
+  const int sm = blockIdx.x / CL, rank = blockIdx.x % CL;
+  const int s = sm / M, m = sm % M;
   const int K = tab.K[s];
+  const int part = (K + CL - 1) / CL, i_lo = rank * part, i_hi = min(K, i_lo + part);
   U* mk = keys + (size_t)tab.off[s] + (size_t)m * K;
   const int tid = threadIdx.x, lane = tid & 31;
   const size_t out = (size_t)s * M + m;
@@ -439,7 +451,7 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
     kmax = kmax_g[out];
   }
   if (ncand == 0) {
-    if (tid == 0) {
+    if (tid == 0 && rank == 0) {
       *th_out = (T)1;
       atomicAdd(&diag->degenerate_calib, 1ull);
     }
@@ -467,11 +479,11 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
         for (int u = 0; u < kUnroll; ++u)
           if (pv[u]) f(pv[u], (int)(((pv[u] >> 1) - kmin) >> sh));
       } else {
-        for (int i0 = 0; i0 < K; i0 += kNB * kUnroll) {
+        for (int i0 = i_lo; i0 < i_hi; i0 += kNB * kUnroll) {
 #pragma unroll
           for (int u = 0; u < kUnroll; ++u) {
             const int i = i0 + u * kNB + tid;
-            pv[u] = i < K ? mk[i] : (U)0;
+            pv[u] = i < i_hi ? mk[i] : (U)0;
           }
 #pragma unroll
           for (int u = 0; u < kUnroll; ++u)
@@ -488,7 +500,10 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
       }
     });
     __syncthreads();
+    if constexpr (CL > 1) cg::this_cluster().sync();
     constexpr int PER = kFine / kNB;            // consecutive buckets per thread
+    int bf = 0x7fffffff, nsel = 0;
+    if (rank == 0) {
     const int b0 = tid * PER;
     int cb[PER], hb[PER], tc = 0, th = 0;
 #pragma unroll
@@ -496,6 +511,16 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
       const uint32_t v = fpk[b0 + j];
       cb[j] = packed ? (int)(v & 0xffffu) : (int)v;
       hb[j] = packed ? (int)(v >> 16) : fhl[b0 + j];
+      if constexpr (CL > 1) {
+        // packed sums stay packed: fewer than 2^16 candidates in all
+        const cg::cluster_group cl = cg::this_cluster();
+#pragma unroll
+        for (int r = 1; r < CL; ++r) {
+          const uint32_t w = cl.map_shared_rank(fpk, r)[b0 + j];
+          cb[j] += packed ? (int)(w & 0xffffu) : (int)w;
+          hb[j] += packed ? (int)(w >> 16) : cl.map_shared_rank(fhl, r)[b0 + j];
+        }
+      }
       tc += cb[j];
       th += hb[j];
     }
@@ -521,7 +546,7 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
         h += hb[j];
       }
     }
-    const int bf = block_min(my_found, red32);
+    bf = block_min(my_found, red32);
     int my_sel = 0;
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
@@ -531,7 +556,7 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
     const int sel_above = block_suffix(my_sel, 0, red2).x;
     if (tid == 0) red32[0] = sel_above + my_sel;
     __syncthreads();
-    const int nsel = red32[0];
+    nsel = red32[0];
     if (nsel <= kCap) {
       int run = sel_above;
 #pragma unroll
@@ -544,15 +569,44 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
         fhl[b0 + j] = 0;                        // from here on: keys of the bucket listed
         run += on ? cb[j] : 0;
       }
-      __syncthreads();
+    }
+    if (tid == 0) {
+      plan_s[0] = nsel;
+      plan_s[1] = bf;
+    }
+    }
+    // where the buckets' keys go: this CTA's copy of the table, the first one's list
+    int32_t* place = fhl;
+    U* keep = list;
+    U* low = &bfmin_s;
+    if constexpr (CL > 1) {
+      const cg::cluster_group cl = cg::this_cluster();
+      cl.sync();
+      if (rank > 0) {
+        const int32_t* src = cl.map_shared_rank(fst, 0);
+        for (int q = tid; q < kFine; q += kNB) fst[q] = src[q];
+        nsel = cl.map_shared_rank(plan_s, 0)[0];
+        bf = cl.map_shared_rank(plan_s, 0)[1];
+        place = cl.map_shared_rank(fhl, 0);
+        keep = cl.map_shared_rank(list, 0);
+        low = cl.map_shared_rank(&bfmin_s, 0);
+      }
+      cl.sync();                    // the first CTA may end from here on unless keys are listed
+    }
+    __syncthreads();
+    if (nsel <= kCap) {
       if (nsel > 0 || bf != 0x7fffffff) {
         U lmin = ~(U)0;
         each_key([&](U p, int b) {
           const int st = fst[b];
-          if (st >= 0) list[st + atomicAdd(&fhl[b], 1)] = p;
+          if (st >= 0) keep[st + atomicAdd(&place[b], 1)] = p;
           if (b == bf && (p >> 1) < lmin) lmin = p >> 1;
         });
-        if (lmin != ~(U)0) atomicMin(&bfmin_s, lmin);
+        if (lmin != ~(U)0) atomicMin(low, lmin);
+        if constexpr (CL > 1) {
+          cg::this_cluster().sync();
+          if (rank > 0) return;
+        }
         __syncthreads();
         U best = ~(U)0;
         for (int i = tid; i < nsel; i += kNB) {
@@ -571,6 +625,7 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
         if (best != ~(U)0) atomicMin(&best_s, best);
         __syncthreads();
       }
+      if (rank > 0) return;
       if (tid == 0) {
         if (best_s != ~(U)0) {
           *th_out = value_of(best_s);
@@ -584,6 +639,7 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
       return;
     }
   }
+  if (rank > 0) return;             // the first CTA refines alone
   if (DIRECT) {
     // the descent reads the keys from memory
 #pragma unroll
@@ -713,9 +769,9 @@ cudaError_t launch_calibrate(const SeriesTable<T>& tab, const T* S, const uint8_
     cells += (int64_t)tab.K[i] * tab.M;
   }
   if (direct && cells <= kDirectCells) {
-    cudaError_t e = func_smem_once((const void*)k_search<T, true>, (int)smem, true);
+    cudaError_t e = func_smem_once((const void*)k_search<T, true, 1>, (int)smem, true);
     if (e) return e;
-    k_search<T, true><<<n_sm, kNB, smem, s>>>(tab, static_cast<U*>(w.keys), kmin, kmax, w.ncand, S,
+    k_search<T, true, 1><<<n_sm, kNB, smem, s>>>(tab, static_cast<U*>(w.keys), kmin, kmax, w.ncand, S,
                                               cls, slo, ok_frac, reliability, theta, theta1, diag);
     return cudaGetLastError();
   }
@@ -743,11 +799,32 @@ cudaError_t launch_calibrate(const SeriesTable<T>& tab, const T* S, const uint8_
   else if (tiles > 0)
     k_pack<T><<<tiles, kPackThreads, 0, s>>>(tab, pp, S, cls, slo, w.thr, ok_frac,
                                              static_cast<U*>(w.keys), kmin, kmax, w.ncand);
-  // the largest carveout lets two searches share an SM where their tables fit
-  cudaError_t e = func_smem_once((const void*)k_search<T, false>, (int)smem, true);
+  // clusters while the searches leave SMs idle (two share an SM where their
+  // tables fit) and a CTA's part still has eight windows a thread
+  int cl = 1;
+  int64_t longest = 0;
+  for (int i = 0; i < tab.n; ++i) longest = std::max<int64_t>(longest, tab.K[i]);
+  while (cl < 4 && n_sm * cl * 2 <= 2 * device_sm_count() && longest >= (int64_t)cl * 2 * kDirectK)
+    cl *= 2;
+  auto search = cl == 4 ? k_search<T, false, 4> : cl == 2 ? k_search<T, false, 2>
+                                                          : k_search<T, false, 1>;
+  cudaError_t e = func_smem_once((const void*)search, (int)smem, true);
   if (e) return e;
-  k_search<T, false><<<n_sm, kNB, smem, s>>>(tab, static_cast<U*>(w.keys), kmin, kmax, w.ncand, S,
-                                             cls, slo, ok_frac, reliability, theta, theta1, diag);
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3((unsigned)(n_sm * cl));
+  c.blockDim = dim3(kNB);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)cl;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  c.attrs = &at;
+  c.numAttrs = cl > 1 ? 1 : 0;
+  e = cudaLaunchKernelEx(&c, search, tab, static_cast<U*>(w.keys), static_cast<const U*>(kmin),
+                         static_cast<const U*>(kmax), static_cast<const uint32_t*>(w.ncand), S,
+                         cls, slo, ok_frac, reliability, theta, theta1, diag);
+  if (e) return e;
   return cudaGetLastError();
 }
 
