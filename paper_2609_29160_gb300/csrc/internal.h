@@ -269,7 +269,7 @@ template <class T> struct WalkBatch {
 // per-(series, tau, tick) tables: the lane walk's rows, or receivers and
 // per-model donor ranks for the walks that visit every tick
 struct WalkWs {
-  uint16_t* rows;     // [chunk][tick][model] next donor tick and rank (lane walk)
+  void* rows;     // [chunk][tick][model] next donor tick and rank (lane walk)
   uint8_t *recs, *nexts;  // [chunk][tick] receiver and kind, next acting tick (lane walk)
   int16_t* recv;
   int16_t* n_donor;   // donors with a rank at the tick

@@ -778,24 +778,33 @@ __device__ __forceinline__ void put_move(tre_move* mv, int64_t at, int64_t cap, 
 // state only decides which tick moves something next: the first one where the
 // idle pool is not empty or a donor stands above its floor. Ticks are cut into
 // chunks of kChunk; k_tick_rows ranks a chunk's ticks and stores, per tick u of
-// the chunk and model, one 16-bit word
-//     (first tick t >= u of the chunk where the model is a donor) << RB | rank
-// (rank from 1 in the tick's donor order; t = kChunk: none left in the chunk).
+// the chunk and model, one word (16 bits up to 16 models, else 32)
+//     first tick t >= u of the chunk where the model is a donor | rank | receiver
+// (rank from 1 in that tick's donor order; t = kChunk: none left in the chunk).
 // k_walk_lane keeps one model per lane (two above 32): one shared-memory load
 // of the row at u, masked by "above its floor", and one warp-wide minimum give
 // the next tick that moves something and its donor together. Ranking and walk
 // measured, before (one thread per tick; one lane jumping over tables of next
 // donor ticks up to 16 models, one warp testing 32 ticks a ballot above) and
 // now: 16 models, 4,320 ticks, 431 moves 228 -> 57 us; 64 models, 17,280
-// ticks, 1,493 moves 1,504 -> 199 us; 24 models of unequal footprint, 720
-// ticks, 1,875 moves 634 -> 308 us; 1,792 instances of 8 models 89 -> 51 us.
+// ticks, 1,493 moves 1,504 -> 202 us; 24 models of unequal footprint, 720
+// ticks, 1,875 moves 634 -> 320 us; 1,792 instances of 8 models 89 -> 50 us.
 constexpr int kChunk = 128;          // ticks per chunk
 
-template <int MP> struct RowBits;    // rank bits of a row word (ranks 1..MP-1)
-template <> struct RowBits<8> { static constexpr int v = 3; };
-template <> struct RowBits<16> { static constexpr int v = 4; };
-template <> struct RowBits<32> { static constexpr int v = 5; };
-template <> struct RowBits<64> { static constexpr int v = 6; };
+// A row word, from its low bits: receiver, rank (1..MP-1), tick. Words of
+// donors compare by tick, then by rank, which is distinct within a tick.
+template <class W, int RB> struct RowWordOf {
+  using Word = W;
+  static constexpr int kRank = RB, kTick = 2 * RB;
+  static constexpr uint32_t kRecv = (1u << RB) - 1, kEnd = (uint32_t)kChunk << kTick;
+  static constexpr uint32_t kNone = (W)~(W)0;
+  static_assert(kEnd < kNone, "the word holds a tick past the chunk");
+};
+template <int MP> struct RowWord;
+template <> struct RowWord<8> : RowWordOf<uint16_t, 3> {};
+template <> struct RowWord<16> : RowWordOf<uint16_t, 4> {};
+template <> struct RowWord<32> : RowWordOf<uint32_t, 5> {};
+template <> struct RowWord<64> : RowWordOf<uint32_t, 6> {};
 
 constexpr uint32_t kNoTick = 0x7f;   // receiver byte of a tick that does nothing
 constexpr uint32_t kSlowBit = 0x80;  // receiver byte: the tick rebalances
@@ -869,35 +878,38 @@ template <class T> struct ChunkOf {
 // the first one after it -- and the next tick that does anything.
 template <int MP, int THREADS>
 __device__ __forceinline__ void write_rows(const uint8_t (*s_rank)[MP], const uint8_t* s_rec,
-                                           uint16_t* rows, uint8_t* recs, uint8_t* nexts) {
+                                           void* row_words, uint8_t* recs, uint8_t* nexts) {
+  using R = RowWord<MP>;
+  using Word = typename R::Word;
   constexpr int NSEG = THREADS / MP < 16 ? THREADS / MP : 16, SEGL = kChunk / NSEG;
-  constexpr int RB = RowBits<MP>::v;
-  constexpr uint32_t kEnd = (uint32_t)kChunk << RB;
-  __shared__ uint16_t s_first[NSEG][MP];
+  __shared__ Word s_first[NSEG][MP];
+  auto word = [&](int u, uint32_t r) {
+    return (uint32_t)u << R::kTick | r << R::kRank | (s_rec[u] & R::kRecv);
+  };
   const int col = threadIdx.x % MP, seg = threadIdx.x / MP;
   if (seg < NSEG) {
-    uint32_t f = kEnd;
+    uint32_t f = R::kEnd;
 #pragma unroll
     for (int i = SEGL - 1; i >= 0; --i) {
       const uint32_t r = s_rank[seg * SEGL + i][col];
-      if (r) f = (uint32_t)(seg * SEGL + i) << RB | r;
+      if (r) f = word(seg * SEGL + i, r);
     }
-    s_first[seg][col] = (uint16_t)f;
+    s_first[seg][col] = (Word)f;
   }
   __syncthreads();
   const size_t base = (size_t)blockIdx.x * kChunk;
   if (seg < NSEG) {
-    uint32_t v = kEnd;
+    uint32_t v = R::kEnd;
 #pragma unroll
     for (int j = 1; j < NSEG; ++j)
       if (j > seg) v = min(v, (uint32_t)s_first[j][col]);
-    uint16_t* out = rows + base * MP + col;
+    Word* out = static_cast<Word*>(row_words) + base * MP + col;
 #pragma unroll
     for (int i = SEGL - 1; i >= 0; --i) {
       const int ul = seg * SEGL + i;
       const uint32_t r = s_rank[ul][col];
-      if (r) v = (uint32_t)ul << RB | r;
-      out[(size_t)ul * MP] = (uint16_t)v;
+      if (r) v = word(ul, r);
+      out[(size_t)ul * MP] = (Word)v;
     }
   }
   if (threadIdx.x < kChunk) {
@@ -919,7 +931,7 @@ __device__ __forceinline__ void write_rows(const uint8_t (*s_rank)[MP], const ui
 // tick's models over lanes and counting from shuffles took 15).
 template <class T, int MP, bool QUAD>
 __global__ void __launch_bounds__(kChunk)
-k_tick_rows(const __grid_constant__ WalkBatch<T> b, uint16_t* __restrict__ rows,
+k_tick_rows(const __grid_constant__ WalkBatch<T> b, void* __restrict__ rows,
             uint8_t* __restrict__ recs, uint8_t* __restrict__ nexts) {
   __shared__ uint8_t s_rank[kChunk][MP];
   __shared__ uint8_t s_rec[kChunk];
@@ -1012,7 +1024,7 @@ k_tick_rows(const __grid_constant__ WalkBatch<T> b, uint16_t* __restrict__ rows,
 constexpr int kWideThreads = 1024;
 template <class T, int MP>
 __global__ void __launch_bounds__(kWideThreads)
-k_tick_rows_wide(const __grid_constant__ WalkBatch<T> b, uint16_t* __restrict__ rows,
+k_tick_rows_wide(const __grid_constant__ WalkBatch<T> b, void* __restrict__ rows,
                  uint8_t* __restrict__ recs, uint8_t* __restrict__ nexts) {
   constexpr int MPL = MP / 32;
   __shared__ uint8_t s_rank[kChunk][MP];
@@ -1129,7 +1141,7 @@ struct LaneWalk {
   tre_move* moves;
   int64_t* n_moves;
   tre_diag* diag;
-  const uint16_t* rows;
+  const void* rows;
   const uint8_t *recs, *nexts;
 };
 
@@ -1138,7 +1150,8 @@ constexpr int kLaneLog = 256;      // moves a warp collects before it writes the
 // bytes of one staged tick: its row, receiver and next acting tick; a buffer
 // ends in a row of "none", read when a walk steps past the last tick
 template <int MP> __host__ __device__ constexpr int slab_bytes(int ticks) {
-  return ticks * (MP * 2 + 2) + MP * 2;
+  return ticks * (MP * (int)sizeof(typename RowWord<MP>::Word) + 2) +
+         MP * (int)sizeof(typename RowWord<MP>::Word);
 }
 
 __device__ __forceinline__ void copy16(void* smem, const void* gmem) {
@@ -1159,9 +1172,11 @@ __global__ void __launch_bounds__(kLaneThreads)
 k_walk_lane(const __grid_constant__ LaneWalk w) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ uint32_t s_log[kLaneThreads / 32][kLaneLog];
+  __shared__ int s_foot[64];
   constexpr int MPL = MP > 32 ? 2 : 1, L1 = MPL - 1;
-  constexpr int RB = RowBits<MP>::v;
-  constexpr uint32_t kNone = 0xffffu;
+  using R = RowWord<MP>;
+  using Word = typename R::Word;
+  constexpr uint32_t kNone = R::kNone;
   const unsigned full = 0xffffffffu;
   const int ti = blockIdx.x % w.n_tau, si = blockIdx.x / w.n_tau;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1175,11 +1190,12 @@ k_walk_lane(const __grid_constant__ LaneWalk w) {
   auto fetch = [&](int first, int buf) {
     const int n = min(w.slab, n_tick - first);
     unsigned char* d = dyn + buf * buf_bytes;
-    const unsigned char* src = reinterpret_cast<const unsigned char*>(w.rows + (t0 + first) * MP);
-    for (int i = threadIdx.x; i < n * MP / 8; i += kLaneThreads) copy16(d + 16 * i, src + 16 * i);
-    if (threadIdx.x < MP)
-      reinterpret_cast<uint16_t*>(d)[n * MP + threadIdx.x] = (uint16_t)(kChunk << RB);
-    d += (size_t)(w.slab + 1) * MP * 2;
+    const unsigned char* src =
+        reinterpret_cast<const unsigned char*>(static_cast<const Word*>(w.rows) + (t0 + first) * MP);
+    for (int i = threadIdx.x; i < n * MP * (int)sizeof(Word) / 16; i += kLaneThreads)
+      copy16(d + 16 * i, src + 16 * i);
+    if (threadIdx.x < MP) reinterpret_cast<Word*>(d)[n * MP + threadIdx.x] = (Word)R::kEnd;
+    d += (size_t)(w.slab + 1) * MP * sizeof(Word);
     for (int i = threadIdx.x; i < n / 16; i += kLaneThreads) {
       copy16(d + 16 * i, w.recs + t0 + first + 16 * i);
       copy16(d + w.slab + 16 * i, w.nexts + t0 + first + 16 * i);
@@ -1187,6 +1203,7 @@ k_walk_lane(const __grid_constant__ LaneWalk w) {
   };
   if (n_tick > 0) fetch(0, 0);
   asm volatile("cp.async.commit_group;\n" ::: "memory");
+  if (threadIdx.x < M) s_foot[threadIdx.x] = w.footprint[threadIdx.x];   // read past the slab's barrier
 
   // the instance's state: replicas above the floor per model, the idle pool
   const bool mine = ci < w.n_cap;
@@ -1225,9 +1242,9 @@ k_walk_lane(const __grid_constant__ LaneWalk w) {
   int n_log = 0;       // moves in the log: tick | position << 11 | donor << 19 (64: the pool)
 
   // a slab of n ticks, the first of them tick `first` of the series
-  auto walk = [&](const uint16_t* rows, const uint8_t* recs, const uint8_t* nexts, int n,
+  auto walk = [&](const Word* rows, const uint8_t* recs, const uint8_t* nexts, int n,
                   int first) {
-    const uint16_t* my = rows + (lane & (MP - 1));
+    const Word* my = rows + (lane & (MP - 1));
     // all ones where the model has nothing above its floor
     uint32_t no[MPL];
     auto masks = [&]() {
@@ -1295,14 +1312,14 @@ k_walk_lane(const __grid_constant__ LaneWalk w) {
         const uint32_t k0 = my[u * MP] | no[0];
         const uint32_t k1 = MPL > 1 ? my[u * MP + 32] | no[L1] : kNone;
         const uint32_t best = __reduce_min_sync(full, MPL > 1 ? min(k0, k1) : k0);
-        const int t = (int)(best >> RB), cb = u & ~(kChunk - 1);
+        const int t = (int)(best >> R::kTick), cb = u & ~(kChunk - 1);
         if (t >= kChunk) {                      // nothing in the rest of the chunk
           u = cb + kChunk;
           if (u >= n) break;
           continue;
         }
         const int a = cb + t;
-        const int recv = recs[a] & 63;
+        const int recv = (int)(best & R::kRecv);
         const bool d0 = k0 == best, d1 = MPL > 1 && k1 == best;
         c[0] += (lane == recv) - d0;
         if (MPL > 1) c[L1] += (lane + 32 == recv) - d1;
@@ -1318,7 +1335,7 @@ k_walk_lane(const __grid_constant__ LaneWalk w) {
         const uint32_t k0 = my[u * MP] | no[0];
         const uint32_t k1 = MPL > 1 ? my[u * MP + 32] | no[L1] : kNone;
         const uint32_t best = __reduce_min_sync(full, MPL > 1 ? min(k0, k1) : k0);
-        const int t = (int)(best >> RB), cb = u & ~(kChunk - 1);
+        const int t = (int)(best >> R::kTick), cb = u & ~(kChunk - 1);
         if (t >= kChunk) {
           u = cb + kChunk;
           if (u >= n) break;
@@ -1329,7 +1346,7 @@ k_walk_lane(const __grid_constant__ LaneWalk w) {
           cur = a;
           left = Kp;
         }
-        const int recv = recs[a] & 63;
+        const int recv = (int)(best & R::kRecv);
         const bool d0 = k0 == best, d1 = MPL > 1 && k1 == best;
         const int give = min(d1 ? c[L1] : c[0], left);
         const int take = (int)__reduce_max_sync(full, d0 || d1 ? (unsigned)give : 0u);
@@ -1350,20 +1367,31 @@ k_walk_lane(const __grid_constant__ LaneWalk w) {
       while (true) {
         uint32_t k = my[u * MP] | no[0];
         if (MPL > 1) k = min(k, my[u * MP + 32] | no[L1]);
+        const uint32_t next = __reduce_min_sync(full, k);
         const int cb = u & ~(kChunk - 1);
-        int t = (int)(__reduce_min_sync(full, k) >> RB);
-        if (pool > 0 && u < n) t = min(t, (int)nexts[u]);
+        int t = (int)(next >> R::kTick), recv = (int)(next & R::kRecv);
+        if (pool > 0 && u < n && (int)nexts[u] < t) {
+          t = nexts[u];
+          recv = recs[cb + t] & 63;
+        }
         if (t >= kChunk) {
           u = cb + kChunk;
           if (u >= n) break;
           continue;
         }
         const int a = cb + t;
-        const int recv = recs[a] & 63;
-        const int need = __shfl_sync(full, MPL > 1 && recv >= 32 ? g[L1] : g[0], recv & 31);
-        // the donors of this very tick: words of the row at the tick itself
-        const uint32_t r0 = my[a * MP], r1 = MPL > 1 ? my[a * MP + 32] : kNone;
-        const bool don0 = (int)(r0 >> RB) == t, don1 = MPL > 1 && (int)(r1 >> RB) == t;
+        const int need = s_foot[recv];
+        // the donors of this very tick, from the words of the row at the tick
+        // itself: rank above, footprint below (65,535 and more: looked up), so
+        // that one warp minimum finds the next donor and what it frees
+        uint32_t q[MPL];
+#pragma unroll
+        for (int j = 0; j < MPL; ++j) {
+          const uint32_t r = my[a * MP + 32 * j];
+          q[j] = (int)(r >> R::kTick) == t
+                     ? (r >> R::kRank & R::kRecv) << 16 | (uint32_t)min(g[j], 0xffff)
+                     : ~0u;
+        }
         for (int seq = 0; seq < Kp; ++seq) {
           if (pool >= need) {
             pool -= need;
@@ -1377,13 +1405,15 @@ k_walk_lane(const __grid_constant__ LaneWalk w) {
 #pragma unroll
           for (int j = 0; j < MPL; ++j) h[j] = c[j];
           while (f < need) {
-            const uint32_t e0 = don0 && h[0] > 0 ? r0 : kNone;
-            const uint32_t e1 = don1 && h[L1] > 0 ? r1 : kNone;
+            const uint32_t e0 = h[0] > 0 ? q[0] : ~0u;
+            const uint32_t e1 = MPL > 1 && h[L1] > 0 ? q[L1] : ~0u;
             const uint32_t best = __reduce_min_sync(full, MPL > 1 ? min(e0, e1) : e0);
-            if (best == kNone) break;
+            if (best == ~0u) break;
             const bool d0 = e0 == best, d1 = MPL > 1 && e1 == best;
-            const unsigned gd = d0 ? (unsigned)g[0] : d1 ? (unsigned)g[L1] : 0u;
-            f += __reduce_max_sync(full, gd);
+            uint32_t frees = best & 0xffffu;
+            if (frees == 0xffffu)
+              frees = __reduce_max_sync(full, d0 ? (unsigned)g[0] : d1 ? (unsigned)g[L1] : 0u);
+            f += frees;
             h[0] -= d0;
             if (MPL > 1) h[L1] -= d1;
             log_one(d0 || d1, (uint32_t)a, seq, lane + (d1 ? 32 : 0));
@@ -1417,9 +1447,9 @@ k_walk_lane(const __grid_constant__ LaneWalk w) {
     asm volatile("cp.async.wait_group 1;\n" ::: "memory");
     __syncthreads();
     const unsigned char* d = dyn + buf * buf_bytes;
-    const uint8_t* recs = d + (size_t)(w.slab + 1) * MP * 2;
+    const uint8_t* recs = d + (size_t)(w.slab + 1) * MP * sizeof(Word);
     if (walks)
-      walk(reinterpret_cast<const uint16_t*>(d), recs, recs + w.slab, min(w.slab, n_tick - first),
+      walk(reinterpret_cast<const Word*>(d), recs, recs + w.slab, min(w.slab, n_tick - first),
            first);
     __syncthreads();
   }
@@ -1514,7 +1544,7 @@ cudaError_t lane_launch(const WalkBatch<T>& b, const WalkWs& w, cudaStream_t s, 
   v.nexts = w.nexts;
   // short series are staged whole; longer ones in two buffers, the next
   // slab's load behind the walk of this one
-  constexpr int kSlab = MP == 64 ? 768 : 1024;
+  constexpr int kSlab = MP == 64 ? 384 : MP == 32 ? 768 : 1024;
   constexpr int kSmem = 2 * slab_bytes<MP>(kSlab);
   static_assert(kSmem <= 200 * 1024, "two slabs and the logs fit a block's shared memory");
   static_assert(kSlab < 2048, "a logged tick has 11 bits");
@@ -1554,7 +1584,8 @@ template <class T> void walk_ws_layout(Arena& a, WalkBatch<T>& b, WalkWs& w) {
   b.ent_base[b.n_series] = (int32_t)total;
   const size_t ents = (size_t)std::max<int64_t>(total * b.n_tau, 1);
   if (lanes) {
-    w.rows = a.take<uint16_t>(ents * kChunk * row_models(b.M));
+    const int words = row_models(b.M);
+    w.rows = a.take<uint32_t>(ents * kChunk * words / (words <= 16 ? 2 : 1));
     w.recs = a.take<uint8_t>(ents * kChunk);
     w.nexts = a.take<uint8_t>(ents * kChunk);
     return;
