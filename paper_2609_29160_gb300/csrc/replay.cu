@@ -34,10 +34,11 @@
 //   3. scores the windows, one per lane, with the smoothing chain passed from
 //      lane to lane.
 // On a tick one warp runs the controller with the models on its lanes. What
-// bounds a replay is the start chain of its busiest model, some 250 cycles a
-// start. 160,000 requests of 8 models over 600 windows, 64 instances: 7.7 ms; a
-// warp per instance with a lane per model (heaps of free times, attribution
-// inside the start loop) took 78.3, 2,700 cycles a start.
+// bounds a replay is the start chain of its busiest model and the attribution
+// behind it. 160,000 requests of 8 models over 600 windows, 64 instances: 4.9 ms
+// (7.7 when a start took two warp votes and a divergent write); a warp per
+// instance with a lane per model (heaps of free times, attribution inside the
+// start loop) took 78.3, 2,700 cycles a start.
 #include <algorithm>
 
 #include "common.cuh"
@@ -247,15 +248,35 @@ template <class T> struct ModelState {
 };
 
 // Starts a model's requests in order until one cannot start before t_end, its
-// free times in registers, R per lane. Calls `done(st, c0, c1)` with the lanes'
-// started requests, up to 32 at a time (st = kNoServer: none).
+// servers' free times in registers, R per lane. Calls `done(st, c0, c1)` with the
+// lanes' started requests, up to 32 at a time (st = kNoServer: none). A server is
+// a key: its free time since the earliest one, with its number in the low bits, so
+// that one warp minimum finds both the time and the server, and a start is a chain
+// of a minimum, a maximum, a sum and a select without a branch (two warp votes and
+// a divergent write of the server took 250 cycles a start). Times kLate and more
+// past the earliest one are all "late"; returns false, with nothing done, when
+// t_end itself lies past that (37 hours up to 32 servers, nine above 64).
 template <int R, class F>
-__device__ __forceinline__ void start_requests(uint32_t* sv, int n, const int4* __restrict__ grp,
+__device__ __forceinline__ bool start_requests(uint32_t* sv, int n, const int4* __restrict__ grp,
                                                int& head, int end, uint32_t t_end, F&& done) {
+  constexpr int kBits = R == 1 ? 5 : R == 2 ? 6 : 7;
+  constexpr uint32_t kLate = (1u << (32 - kBits)) - 2;
+  static_assert(R <= 4, "a server's number has seven bits");
   const int lane = threadIdx.x & 31;
-  uint32_t s[R];
+  uint32_t s[R], key[R], low = kNoServer;
 #pragma unroll
-  for (int r = 0; r < R; ++r) s[r] = lane + 32 * r < n ? sv[lane + 32 * r] : kNoServer;
+  for (int r = 0; r < R; ++r) {
+    s[r] = lane + 32 * r < n ? sv[lane + 32 * r] : kNoServer;
+    low = min(low, s[r]);
+  }
+  const uint32_t t0 = __reduce_min_sync(kFull, low);
+  if (t0 >= t_end) return true;
+  const uint32_t stop = t_end - t0;
+  if (stop > kLate) return false;
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+    key[r] = lane + 32 * r < n ? (min(s[r] - t0, kLate) << kBits) + (uint32_t)(lane + 32 * r)
+                               : kNoServer;
   auto fetch = [&](int p, int4& a, int4& c) {
     if (p < end) {
       a = __ldg(&grp[2 * (size_t)p]);
@@ -264,45 +285,48 @@ __device__ __forceinline__ void start_requests(uint32_t* sv, int n, const int4* 
   };
   int4 c0 = make_int4(0, 0, 0, 0), c1 = c0, n0 = c0, n1 = c0;
   fetch(head + lane, c0, c1);
-  bool more = head < end;
-  while (more) {
+  bool go = head < end;
+  while (go) {
     fetch(head + 32 + lane, n0, n1);               // the next 32, behind this batch's chain
-    const int cnt = min(32, end - head);
+    // past the last request: one that arrives too late
+    const uint32_t arr = head + lane < end
+                             ? min((uint32_t)c0.x > t0 ? (uint32_t)c0.x - t0 : 0u, kLate) : kLate;
     uint32_t mine = kNoServer;
-    int j = 0;
-    for (; j < cnt; ++j) {
-      const uint32_t ta = (uint32_t)__shfl_sync(kFull, c0.x, j);
-      const uint32_t dt = (uint32_t)__shfl_sync(kFull, c0.z, j);
-      uint32_t low = s[0];
+    for (int j8 = 0; j8 < 32 && go; j8 += 8) {
 #pragma unroll
-      for (int r = 1; r < R; ++r) low = min(low, s[r]);
-      const uint32_t f = __reduce_min_sync(kFull, low);
-      const uint32_t st = max(ta, f);
-      if (st >= t_end) break;
-      const int src = __ffs(__ballot_sync(kFull, low == f)) - 1;
-      if (lane == src) {
-        bool put = false;
+      for (int j = j8; j < j8 + 8; ++j) {
+        const uint32_t ta = __shfl_sync(kFull, arr, j);
+        const uint32_t dt = (uint32_t)__shfl_sync(kFull, c0.z, j);
+        uint32_t first = key[0];
+#pragma unroll
+        for (int r = 1; r < R; ++r) first = min(first, key[r]);
+        first = __reduce_min_sync(kFull, first);
+        const uint32_t st = max(first >> kBits, ta);
+        go = go && st < stop;
+        const uint32_t te = min(st + dt, kLate);
 #pragma unroll
         for (int r = 0; r < R; ++r)
-          if (!put && s[r] == f) {
-            s[r] = min(st + dt, kNever);
-            put = true;
+          if (go && key[r] == first) {
+            key[r] = (te << kBits) + (uint32_t)(lane + 32 * r);
+            s[r] = min(t0 + st + dt, kNever);
           }
+        if (go && lane == j) mine = t0 + st;
       }
-      if (lane == j) mine = st;
     }
-    head += j;
-    if (j > 0) done(mine, c0, c1);
-    more = j == 32 && head < end;
+    head += __popc(__ballot_sync(kFull, mine != kNoServer));
+    if (__any_sync(kFull, mine != kNoServer)) done(mine, c0, c1);
+    go = go && head < end;
     c0 = n0;
     c1 = n1;
   }
 #pragma unroll
   for (int r = 0; r < R; ++r)
     if (lane + 32 * r < n) sv[lane + 32 * r] = s[r];
+  return true;
 }
 
-// the same with the free times left in memory, for more servers than four per lane
+// the same with the free times left in memory, for more servers than four per
+// lane and for longer stretches of time
 template <class F>
 __device__ __forceinline__ void start_requests_mem(uint32_t* sv, int n,
                                                    const int4* __restrict__ grp, int& head,
@@ -504,10 +528,12 @@ k_replay(const __grid_constant__ ReplayBatch<T> b) {
       };
       uint32_t* sv = srv + (size_t)m * b.hcap;
       if (n > 0 && head < end) {
-        if (n <= 32) start_requests<1>(sv, n, b.grp, head, end, t_end, done);
-        else if (n <= 64) start_requests<2>(sv, n, b.grp, head, end, t_end, done);
-        else if (n <= 128) start_requests<4>(sv, n, b.grp, head, end, t_end, done);
-        else start_requests_mem(sv, n, b.grp, head, end, t_end, done);
+        const bool held =
+            n <= 32    ? start_requests<1>(sv, n, b.grp, head, end, t_end, done)
+            : n <= 64  ? start_requests<2>(sv, n, b.grp, head, end, t_end, done)
+            : n <= 128 ? start_requests<4>(sv, n, b.grp, head, end, t_end, done)
+                       : false;
+        if (!held) start_requests_mem(sv, n, b.grp, head, end, t_end, done);
       }
       __syncwarp();
       // the segment's windows, one per lane

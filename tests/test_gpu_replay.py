@@ -178,6 +178,22 @@ def test_replay_server_counts_and_input_order(tre, servers, budget, shuffled):
            [(0.8, 2)], wake=1310, sleep=1870, guard=np.full(M, 3000, np.int32))
 
 
+# Idle servers whose free times fall 2^27, 2^26 and 2^25 ms and more behind the
+# segment (one, two and four per lane), services beyond that, ties.
+@pytest.mark.parametrize("servers", [(3, 32, 1), (33, 40, 2), (100, 128, 65)])
+def test_replay_long_spans(tre, servers):
+    rng = np.random.default_rng(servers[0])
+    n, M, win, K = 900, 3, 1_000_000, 210
+    t = np.sort(rng.choice(np.arange(0, K * win, 500_000), n))
+    total = rng.choice([0, 7, 40_000_000, (1 << 25) + 1, (1 << 27) + 5, 1_900_000_000], n)
+    lat = {"model": rng.integers(0, M, n), "t_arr_ms": t, "d_first_ms": total // 3,
+           "d_total_ms": total, "L_in": rng.integers(0, 500, n), "L_out": rng.integers(1, 300, n)}
+    lat = {k: v.astype(np.int32) for k, v in lat.items()}
+    _check(tre, lat, M, win, K, _prof(M, theta=20.0), sum(servers) + 5,
+           np.array(servers, np.int32), np.ones(M, np.int32), np.ones(M, np.int32), "f32",
+           [(0.8, 1)], wake=1310, sleep=1870)
+
+
 def test_replay_invalid_records_are_not_served(tre):
     lat, M, budget = _mid_latent(0.005, 12, 600.0)
     lat = {k: (v.copy() if hasattr(v, "copy") else v) for k, v in lat.items()}
