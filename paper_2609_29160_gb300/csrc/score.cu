@@ -99,15 +99,26 @@ struct TilePlan {
   int tile_base[kMaxSeries + 1];   // prefix of tiles per series
 };
 
+// a / b for a divisor above zero and a numerator that often is zero (a window
+// without prompt or without decode tokens): the division of a zero leaves the
+// short instruction sequence for a subroutine, and takes its whole warp along
+// (188 instructions a cell, now 85; Eq. 1 of 64 models, 864,000 windows 299 us,
+// now 180), so it divides a one instead and returns the numerator, as 0 / b is.
+template <class T> __device__ __forceinline__ T div_zero_rn(T a, T b) {
+  const bool zero = (a == (T)0) & (b > (T)0);
+  const T q = div_rn(zero ? (T)1 : a, b);
+  return zero ? a : q;
+}
+
 template <class T>
 __device__ __forceinline__ T raw_tss(int32_t p, int32_t d, int32_t a, int32_t w, T dt, T wp,
                                      T wq) {
-  const T r_pre = div_rn(from_i32<T>(p), dt);
-  const T r_dec = div_rn(from_i32<T>(d), dt);
+  const T r_pre = div_zero_rn(from_i32<T>(p), dt);
+  const T r_dec = div_zero_rn(from_i32<T>(d), dt);
   const T num = add_rn(mul_rn(wp, r_pre), r_dec);
   T den = add_rn(from_i32<T>(a), mul_rn(wq, from_i32<T>(w)));
   if (den < (T)1) den = (T)1;                       // demand floor of one request
-  return div_rn(num, den);
+  return div_zero_rn(num, den);
 }
 
 // Eq. 1 with the window means of the running and waiting counts: the
@@ -115,15 +126,20 @@ __device__ __forceinline__ T raw_tss(int32_t p, int32_t d, int32_t a, int32_t w,
 template <class T>
 __device__ __forceinline__ T raw_tss_mean(int32_t p, int32_t d, long long a_ms, long long w_ms,
                                           T dt, T win, T wp, T wq) {
-  const T r_pre = div_rn(from_i32<T>(p), dt);
-  const T r_dec = div_rn(from_i32<T>(d), dt);
+  const T r_pre = div_zero_rn(from_i32<T>(p), dt);
+  const T r_dec = div_zero_rn(from_i32<T>(d), dt);
   const T num = add_rn(mul_rn(wp, r_pre), r_dec);
-  const T a = div_rn(from_i64<T>(a_ms), win);
-  const T w = div_rn(from_i64<T>(w_ms), win);
+  const T a = div_zero_rn(from_i64<T>(a_ms), win);
+  const T w = div_zero_rn(from_i64<T>(w_ms), win);
   T den = add_rn(a, mul_rn(wq, w));
   if (den < (T)1) den = (T)1;                       // demand floor of one request
-  return div_rn(num, den);
+  return div_zero_rn(num, den);
 }
+
+// sixteen bytes of values: four floats, or half of four doubles
+template <class T> struct __align__(16) Four {
+  T v[16 / sizeof(T)];
+};
 
 // STAGES: the two series of the stage-aware signal, each from its own counts
 // (c0: prompt tokens over the prefill gauge and W with a token weight of one;
@@ -132,7 +148,7 @@ __device__ __forceinline__ T raw_tss_mean(int32_t p, int32_t d, long long a_ms, 
 template <class T, bool MEAN, int EPT, bool STAGES>
 __global__ void __launch_bounds__(kEwThreads)
 k_raw(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ TilePlan tp, FastDiv fm,
-      bool vec, Counts c0, Counts c1, const T* __restrict__ w_p, const T* __restrict__ w_q,
+      bool vec, bool vec_w, Counts c0, Counts c1, const T* __restrict__ w_p, const T* __restrict__ w_q,
       T* __restrict__ raw, uint8_t* __restrict__ cls) {
   const int s = prefix_index(tp.tile_base, tab.n, blockIdx.x);
   const int M = tab.M;
@@ -184,6 +200,28 @@ k_raw(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ TilePl
   }
   int m = l0 <= 0xffffffffll ? (int)((uint32_t)l0 - fm.div((uint32_t)l0) * (uint32_t)M)
                              : (int)(l0 % M);
+  // the weights of the elements' models: four in a row where M is a multiple of
+  // four (m then is one too), else one by one
+  T wp[EPT], wq[EPT];
+  if (EPT == 4 && vec_w) {
+#pragma unroll
+    for (int h = 0; h < 4; h += 16 / (int)sizeof(T)) {
+      const Four<T> a = *reinterpret_cast<const Four<T>*>(w_p + m + h);
+      const Four<T> b = *reinterpret_cast<const Four<T>*>(w_q + m + h);
+#pragma unroll
+      for (int i = 0; i < 16 / (int)sizeof(T); ++i) {
+        wp[(h + i) % EPT] = a.v[i];
+        wq[(h + i) % EPT] = b.v[i];
+      }
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < EPT; ++i) {
+      wp[i] = w_p[m];
+      wq[i] = w_q[m];
+      if (++m == M) m = 0;
+    }
+  }
   T rv[EPT];
   uint8_t cv[EPT];
 #pragma unroll
@@ -192,25 +230,34 @@ k_raw(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ TilePl
     if (MEAN) {
       idle = (p[i] | d[i]) == 0 && (am[i] | wm[i]) == 0;
       rv[i] = idle ? idle_raw((T)0)
-                   : raw_tss_mean<T>(p[i], d[i], am[i], wm[i], dt, (T)tab.win[s], w_p[m], w_q[m]);
+                   : raw_tss_mean<T>(p[i], d[i], am[i], wm[i], dt, (T)tab.win[s], wp[i], wq[i]);
     } else {
       idle = (p[i] | d[i] | a[i] | w[i]) == 0;
       rv[i] = idle ? idle_raw((T)0)
-                   : raw_tss<T>(p[i], d[i], a[i], w[i], dt, STAGES && s == 0 ? (T)1 : w_p[m],
-                                w_q[m]);
+                   : raw_tss<T>(p[i], d[i], a[i], w[i], dt, STAGES && s == 0 ? (T)1 : wp[i],
+                                wq[i]);
     }
     cv[i] = idle ? kIdle : kNom;
-    if (++m == M) m = 0;
   }
+  if constexpr (EPT == 4) {
+    if (v4) {
 #pragma unroll
-  for (int i = 0; i < EPT; ++i)
-    if (v4 || l0 + i < n) raw[x0 + i] = rv[i];
-  if constexpr (EPT == 4)
-    if (v4) *reinterpret_cast<uchar4*>(cls + x0) = make_uchar4(cv[0], cv[1], cv[2], cv[3]);
+      for (int h = 0; h < 4; h += 16 / (int)sizeof(T)) {
+        Four<T> o;
+#pragma unroll
+        for (int i = 0; i < 16 / (int)sizeof(T); ++i) o.v[i] = rv[h + i];
+        *reinterpret_cast<Four<T>*>(raw + x0 + h) = o;
+      }
+      *reinterpret_cast<uchar4*>(cls + x0) = make_uchar4(cv[0], cv[1], cv[2], cv[3]);
+    }
+  }
   if (!v4) {
 #pragma unroll
     for (int i = 0; i < EPT; ++i)
-      if (l0 + i < n) cls[x0 + i] = cv[i];
+      if (l0 + i < n) {
+        raw[x0 + i] = rv[i];
+        cls[x0 + i] = cv[i];
+      }
   }
 }
 
@@ -1029,6 +1076,11 @@ template <class T> bool quad_aligned(const SeriesTable<T>& t, std::initializer_l
   return true;
 }
 
+// four models' weights at a time: none of the fours wraps and all are aligned
+inline bool weights_aligned(int M, const void* w_p, const void* w_q) {
+  return M % 4 == 0 && (((uintptr_t)w_p | (uintptr_t)w_q) & 15) == 0;
+}
+
 template <class T> int64_t total_elems(const SeriesTable<T>& t) {
   int64_t n = 0;
   for (int s = 0; s < t.n; ++s) n += (int64_t)t.K[s] * t.M;
@@ -1121,14 +1173,15 @@ cudaError_t launch_score(const SeriesTable<T>& tab, const int32_t* P, const int3
   const int th = small ? kSmallThreads : kEwThreads;
   int n_tiles = 0;
   const TilePlan tp = tile_plan(tab, small ? th : 4 * th, n_tiles);
+  const bool vec_w = weights_aligned(M, w_p, w_q);
   if (A_ms) {
     const bool vec = quad_aligned(tab, {P, D, A_ms, W_ms, w.raw, cls});
     auto f = small ? k_raw<T, true, 1, false> : k_raw<T, true, 4, false>;
-    f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(M), vec, c, c, w_p, w_q, w.raw, cls);
+    f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(M), vec, vec_w, c, c, w_p, w_q, w.raw, cls);
   } else {
     const bool vec = quad_aligned(tab, {P, D, A, W, w.raw, cls});
     auto f = small ? k_raw<T, false, 1, false> : k_raw<T, false, 4, false>;
-    f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(M), vec, c, c, w_p, w_q, w.raw, cls);
+    f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(M), vec, vec_w, c, c, w_p, w_q, w.raw, cls);
   }
   const cudaError_t e = smooth<T>(tab, alpha, S_carry, init_carry, S, cls, w, diag, s);
   if (e) return e;
@@ -1155,8 +1208,9 @@ cudaError_t launch_score_stages(const SeriesTable<T>& tab, const int32_t* P, con
   const Counts pre{P, nullptr, A_pre, W, nullptr, nullptr};
   const Counts dec{nullptr, D, A_dec, nullptr, nullptr, nullptr};
   const bool vec = quad_aligned(tab, {P, D, W, A_pre, A_dec, w.raw, cls});
+  const bool vec_w = weights_aligned(tab.M, w_p, w_q);
   auto f = small ? k_raw<T, false, 1, true> : k_raw<T, false, 4, true>;
-  f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(tab.M), vec, pre, dec, w_p, w_q, w.raw, cls);
+  f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(tab.M), vec, vec_w, pre, dec, w_p, w_q, w.raw, cls);
   return smooth<T>(tab, alpha, nullptr, nullptr, S, cls, w, diag, s);
 }
 
