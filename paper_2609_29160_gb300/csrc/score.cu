@@ -877,6 +877,8 @@ template <> __device__ __forceinline__ void load_quad_z<double>(const double* p,
 // the regions again, one row per thread (64 models, 864,000 windows: 124 us for
 // Z and regions and 120 for the receivers).
 constexpr int kNormCells = 1024;
+template <class T> constexpr int kNormQuadPasses = sizeof(T) == 4 ? 4 : 2;
+constexpr int kNoQuad = 0x7fffffff;
 template <class T>
 __global__ void __launch_bounds__(kEwThreads)
 k_norm_recv(int M, int K, int wt, FastDiv fm, bool vec, const T* __restrict__ S,
@@ -931,6 +933,89 @@ k_norm_recv(int M, int K, int wt, FastDiv fm, bool vec, const T* __restrict__ S,
       }
     }
     recv[k0 + w] = best;
+  }
+}
+
+// The same on large tables whose rows are 1, 2, 4, ... 32 quads of models: a
+// thread keeps its quad of models (their theta and thresholds in registers) and
+// takes one window after another, four in flight; a window's receiver comes from
+// shuffles among the lanes that hold its row. A scan of the row by one thread left
+// 240 of a CTA's 256 threads idle (64 models, 864,000 windows: 173 us, now 138). Bound by
+// memory and by the division's instructions.
+template <class T>
+__global__ void __launch_bounds__(kEwThreads)
+k_norm_quads(int M, int lg_quads, int64_t n_quads, const T* __restrict__ S, const uint8_t* idle_cls,
+             const T* __restrict__ theta, const T* __restrict__ tau_crit,
+             const T* __restrict__ tau_surp, T* __restrict__ Z, uint8_t* cls,
+             int32_t* __restrict__ recv) {
+  constexpr int U = kNormQuadPasses<T>;
+  const unsigned full = 0xffffffffu;
+  const int64_t q0 = (int64_t)blockIdx.x * (kEwThreads * U) + threadIdx.x;
+  const int lanes = 1 << lg_quads, m0 = 4 * (threadIdx.x & (lanes - 1));
+  T th[4], tc[4], ts[4], sv[U][4];
+  uchar4 ic[U];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    th[i] = theta[m0 + i];
+    tc[i] = tau_crit[m0 + i];
+    ts[i] = tau_surp[m0 + i];
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int64_t q = q0 + u * kEwThreads;
+    ic[u] = make_uchar4(kIdle, kIdle, kIdle, kIdle);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) sv[u][i] = (T)1;
+    if (q < n_quads) {
+      load_quad_z<T>(S + 4 * q, sv[u]);
+      ic[u] = *reinterpret_cast<const uchar4*>(idle_cls + 4 * q);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int64_t q = q0 + u * kEwThreads;
+    const uint8_t idle[4] = {ic[u].x, ic[u].y, ic[u].z, ic[u].w};
+    uint8_t cl[4];
+    // the lowest value that is no NaN and its first model; the first model that is
+    // not idle, with a low bit for a NaN (an ascending scan starts from it and
+    // nothing compares below a NaN)
+    int best = kNoQuad, first = kNoQuad;
+    T bz = (T)0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const T z = div_zero_rn(sv[u][i], th[i]);
+      sv[u][i] = z;
+      cl[i] = region_of(idle[i], z, tc[i], ts[i]);
+      const bool on = cl[i] != kIdle, nan = z != z;
+      if (on && first == kNoQuad) first = 2 * (m0 + i) + (nan ? 1 : 0);
+      if (on && !nan && (best == kNoQuad || z < bz)) {
+        best = m0 + i;
+        bz = z;
+      }
+    }
+    if (q < n_quads) {
+#pragma unroll
+      for (int h = 0; h < 4; h += 16 / (int)sizeof(T)) {
+        Four<T> o;
+#pragma unroll
+        for (int i = 0; i < 16 / (int)sizeof(T); ++i) o.v[i] = sv[u][h + i];
+        *reinterpret_cast<Four<T>*>(Z + 4 * q + h) = o;
+      }
+      *reinterpret_cast<uchar4*>(cls + 4 * q) = make_uchar4(cl[0], cl[1], cl[2], cl[3]);
+    }
+    for (int o = 1; o < lanes; o <<= 1) {
+      const int ob = __shfl_xor_sync(full, best, o);
+      const T oz = __shfl_xor_sync(full, bz, o);
+      if (ob != kNoQuad && (best == kNoQuad || oz < bz || (oz == bz && ob < best))) {
+        best = ob;
+        bz = oz;
+      }
+    }
+    if (__any_sync(full, first != kNoQuad && (first & 1))) {
+      for (int o = 1; o < lanes; o <<= 1) first = min(first, __shfl_xor_sync(full, first, o));
+      if (first != kNoQuad && (first & 1)) best = first >> 1;
+    }
+    if (q < n_quads && m0 == 0) recv[q >> lg_quads] = best == kNoQuad ? -1 : best;
   }
 }
 
@@ -1258,6 +1343,15 @@ cudaError_t launch_normalize(const SeriesTable<T>& tab, const T* S, const uint8_
   if (recv) {
     if (tab.n != 1 || !tau_crit || !Z || !cls) return cudaErrorInvalidValue;
     const int M = tab.M, K = tab.K[0], th = small ? kSmallThreads : kEwThreads;
+    int lg_quads = 0;
+    while (lg_quads < 5 && 4 << lg_quads < M) ++lg_quads;
+    if (vec && !small && M == 4 << lg_quads) {
+      constexpr int kPerCta = kEwThreads * kNormQuadPasses<T>;
+      const int64_t n_quads = (int64_t)K << lg_quads;
+      k_norm_quads<T><<<(unsigned)((n_quads + kPerCta - 1) / kPerCta), kEwThreads, 0, s>>>(
+          M, lg_quads, n_quads, S, idle_cls, theta, tau_crit, tau_surp, Z, cls, recv);
+      return cudaGetLastError();
+    }
     const int wt = std::max(1, (small ? th : kNormCells) / M);
     k_norm_recv<T><<<(unsigned)((K + wt - 1) / wt), th, 0, s>>>(
         M, K, wt, FastDiv(M), vec && !small && M % 4 == 0, S, idle_cls, theta, tau_crit, tau_surp,

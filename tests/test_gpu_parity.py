@@ -655,6 +655,34 @@ def test_stage_table_edges(tre, M, win, K):
             np.testing.assert_array_equal(_np(x[k]), o[stage][k], err_msg=stage + " " + k)
 
 
+# one to 32 lanes a row on tables past the small ones, a ragged last CTA, rows with
+# no lanes of their own (24); NaN, infinite and zero values, ties of both zeros
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("M", [4, 8, 16, 24, 32, 64, 128])
+def test_normalize_receiver_rows(tre, dtype, M):
+    rng = np.random.default_rng(M)
+    K = (1 << 18) // M + 37
+    S = rng.standard_normal((K, M)).astype(dtype)
+    S[rng.random((K, M)) < 0.3] = 0.0
+    S[rng.random((K, M)) < 0.1] = -0.0
+    for v in (np.inf, -np.inf, np.nan):
+        S[rng.random((K, M)) < 0.01] = v
+    idle = np.where(rng.random((K, M)) < 0.3, 3, 1).astype(np.uint8)
+    idle[rng.random(K) < 0.05] = 3
+    theta = (rng.random(M) + 0.5).astype(dtype)
+    prof = {"w_p": 0.2, "w_q": 2.0, "alpha": 0.5, "tau_crit": 0.8, "tau_surplus": 1.2,
+            "theta": theta}
+    out = tre.tss_normalize(*_cuda({"S": S, "c": idle}).values(), prof, 100)
+    Z = S / theta
+    np.testing.assert_array_equal(_np(out["Z"]), Z)
+    recv = np.full(K, -1, np.int32)
+    for k in range(K):                       # the first minimum of an ascending scan
+        for m in np.flatnonzero(idle[k] != 3):
+            if recv[k] < 0 or Z[k, m] < Z[k, recv[k]]:
+                recv[k] = m
+    np.testing.assert_array_equal(_np(out["recv"]), recv)
+
+
 def test_calibrate_events(tre):
     w = _events_case(6)
     ev, M, win, K = w["events"], w["M"], w["window_ms"], w["K"]
