@@ -407,6 +407,34 @@ def test_rank_matches_oracle(tre, dtype, seed, K, M):
     np.testing.assert_array_equal(_np(only_d["donors"]), odn)
 
 
+# rows of 16-byte and of odd lengths, at the row and away from its alignment; ties
+# of both zeros, infinities, the types' extremes; regions that are none
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("M,shift", [(1, 0), (3, 0), (4, 0), (4, 1), (7, 0), (8, 0), (8, 4), (9, 0),
+                                     (12, 0), (15, 0), (16, 0), (16, 3)])
+def test_rank_small_edges(tre, dtype, M, shift):
+    import torch
+    rng = np.random.default_rng(100 * M + shift)
+    K = 1500
+    fi = np.finfo(dtype)
+    vals = np.array([0.0, -0.0, 1.0, -1.0, 0.5, 2.0, fi.max, fi.min, fi.tiny, -fi.tiny], dtype)
+    Z = rng.choice(vals, (K, M))
+    Z[::2] = rng.standard_normal((len(Z[::2]), M))
+    odd = rng.random((K, M)) < 0.02
+    Z[odd] = rng.choice(np.array([np.inf, -np.inf], dtype), odd.sum())
+    cls = rng.choice(np.arange(4, dtype=np.uint8), (K, M))
+    cls[5] = 3
+    ref = oracle.rank(Z, cls)
+    dev = []
+    for a in (Z, cls):
+        pad = torch.empty(a.size + shift, dtype=torch.as_tensor(a[:1]).dtype, device="cuda")
+        pad[shift:] = torch.as_tensor(a.reshape(-1)).cuda()
+        dev.append(pad[shift:].view(K, M))
+    g = tre.tss_rank(*dev)
+    np.testing.assert_array_equal(_np(g["recv"]), ref[0])
+    np.testing.assert_array_equal(_np(g["donors"]), ref[1])
+
+
 def test_rank_empty_grid(tre):
     import torch
     g = tre.tss_rank(torch.zeros((0, 4), dtype=torch.float32, device="cuda"),
