@@ -34,9 +34,10 @@
 //   3. scores the windows, one per lane, with the smoothing chain passed from
 //      lane to lane.
 // On a tick one warp runs the controller with the models on its lanes. What
-// bounds a replay is the start chain of its busiest model and the attribution
-// behind it. 160,000 requests of 8 models over 600 windows, 64 instances: 4.9 ms
-// (7.7 when a start took two warp votes and a divergent write); a warp per
+// bounds a replay is the start chain of its busiest model; up to 8 models a second
+// warp takes the attribution off it. 160,000 requests of 8 models over 600 windows,
+// 64 instances: 3.9 ms (4.9 with one warp a model, 7.7 when a start took two warp
+// votes and a divergent write); a warp per
 // instance with a lane per model (heaps of free times, attribution inside the
 // start loop) took 78.3, 2,700 cycles a start.
 #include <algorithm>
@@ -152,6 +153,7 @@ constexpr int kRing = 64;
 enum { kP = 0, kD = 1, kEnd = 2, kLate = 3, kStart = 4, kCounts = 5 };
 constexpr int kFarCounts = 4;        // a start is never beyond its own segment
 constexpr int kMaxWarps = 16;        // models of an instance take turns beyond this
+constexpr int kMaxPairs = 8;         // models with two warps each
 // a server's free time as an unsigned 32-bit millisecond; later ones (wake and
 // sleep delays near 2^31) are kept at kNever, past the end of every grid
 constexpr uint32_t kNever = 0xfffffffeu, kNoServer = 0xffffffffu;
@@ -368,12 +370,26 @@ __device__ __forceinline__ uint32_t warp_scan(uint32_t v) {
   return v;
 }
 
-template <class T>
+// both warps of a pair (barrier 0 is the block's)
+__device__ __forceinline__ void pair_sync(int pair) {
+  asm volatile("bar.sync %0, 64;" :: "r"(pair + 1) : "memory");
+}
+
+// PAIR: two warps per model, one that runs the start chain and one that attributes
+// the batch before and scores. They swap batches of 32 starts through two buffers
+// and meet once a batch, so a batch costs the longer of the two.
+template <class T, bool PAIR>
 __global__ void __launch_bounds__(32 * kMaxWarps)
 k_replay(const __grid_constant__ ReplayBatch<T> b) {
   extern __shared__ __align__(16) unsigned char rsm[];
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_warps = blockDim.x >> 5;
+  __shared__ uint32_t s_batch[PAIR ? kMaxPairs : 1][2][32];   // start times
+  __shared__ int32_t s_more[PAIR ? kMaxPairs : 1][2];         // a batch follows
+  __shared__ int32_t s_head[PAIR ? kMaxPairs : 1];            // next request to start
+  const int lane = threadIdx.x & 31;
+  const int n_warps = (blockDim.x >> 5) / (PAIR ? 2 : 1);
+  const bool starts = PAIR && (int)(threadIdx.x >> 5) >= n_warps;
+  const int wid = (int)(threadIdx.x >> 5) - (starts ? n_warps : 0);
+  int buf = 0;
   const int inst = blockIdx.x;
   const int M = b.M, K = b.K;
   const uint32_t win = (uint32_t)b.win;
@@ -406,6 +422,7 @@ k_replay(const __grid_constant__ ReplayBatch<T> b) {
     s.init = 0;
     s.met = 0;
     s.S = (T)0;
+    if (PAIR) s_head[m] = b.base[m];
     rep[m] = b.r0[m];
     n_srv[m] = max(b.r0[m], 0);
   }
@@ -442,10 +459,35 @@ k_replay(const __grid_constant__ ReplayBatch<T> b) {
     const int k1 = min(min(tick, k0 + 31), K - 1);
     const int n_win = k1 - k0 + 1;
     const uint32_t t_end = (uint32_t)(k1 + 1) * win;
-    for (int m = wid; m < M; m += n_warps) {
+    auto start = [&](int m, int& head, int end, auto&& done) {
+      const int n = n_srv[m];
+      uint32_t* sv = srv + (size_t)m * b.hcap;
+      if (n <= 0 || head >= end) return;
+      const bool held =
+          n <= 32    ? start_requests<1>(sv, n, b.grp, head, end, t_end, done)
+          : n <= 64  ? start_requests<2>(sv, n, b.grp, head, end, t_end, done)
+          : n <= 128 ? start_requests<4>(sv, n, b.grp, head, end, t_end, done)
+                     : false;
+      if (!held) start_requests_mem(sv, n, b.grp, head, end, t_end, done);
+    };
+    if (starts) {
+      auto pass = [&](uint32_t st, bool more) {
+        if (more) s_batch[wid][buf][lane] = st;
+        if (lane == 0) s_more[wid][buf] = more;
+        pair_sync(wid);
+        buf ^= 1;
+      };
+      for (int m = wid; m < M; m += n_warps) {
+        int head = s_head[m];
+        start(m, head, b.base[m + 1],
+              [&](uint32_t st, const int4&, const int4&) { pass(st, true); });
+        pass(kNoServer, false);
+        if (lane == 0) s_head[m] = head;
+        __syncwarp();
+      }
+    } else for (int m = wid; m < M; m += n_warps) {
       ModelState<T>& s = st_m[m];
       uint32_t* my_ring = ring + (size_t)m * kRing;
-      const int n = n_srv[m];
       int head = s.head;
       const int end = s.end, head0 = head;
       int far_hi = -1;
@@ -526,14 +568,29 @@ k_replay(const __grid_constant__ ReplayBatch<T> b) {
         // the running span ends in window te / win (never read past the grid)
         if (te < span && ke >= kp) add(kEnd, ke, 1u);
       };
-      uint32_t* sv = srv + (size_t)m * b.hcap;
-      if (n > 0 && head < end) {
-        const bool held =
-            n <= 32    ? start_requests<1>(sv, n, b.grp, head, end, t_end, done)
-            : n <= 64  ? start_requests<2>(sv, n, b.grp, head, end, t_end, done)
-            : n <= 128 ? start_requests<4>(sv, n, b.grp, head, end, t_end, done)
-                       : false;
-        if (!held) start_requests_mem(sv, n, b.grp, head, end, t_end, done);
+      if (PAIR) {
+        auto fetch = [&](int q, int4& x, int4& y) {
+          if (q < end) {
+            x = __ldg(&b.grp[2 * (size_t)q]);
+            y = __ldg(&b.grp[2 * (size_t)q + 1]);
+          }
+        };
+        int4 c0 = make_int4(0, 0, 0, 0), c1 = c0, x0 = c0, x1 = c0;
+        fetch(head + lane, c0, c1);
+        while (true) {
+          fetch(head + 32 + lane, x0, x1);
+          pair_sync(wid);
+          const bool more = s_more[wid][buf] != 0;
+          const uint32_t st = s_batch[wid][buf][lane];
+          buf ^= 1;
+          if (!more) break;
+          head += __popc(__ballot_sync(kFull, st != kNoServer));
+          done(st, c0, c1);
+          c0 = x0;
+          c1 = x1;
+        }
+      } else {
+        start(m, head, end, done);
       }
       __syncwarp();
       // the segment's windows, one per lane
@@ -619,7 +676,7 @@ k_replay(const __grid_constant__ ReplayBatch<T> b) {
     k0 = k1 + 1;
     if (k != tick) continue;                    // no tick in the segment's last window
     __syncthreads();
-    if (wid == 0) {
+    if (wid == 0 && !starts) {
       const long long Tk = (long long)t_end;
       const bool fast = next_tick(k, win, (uint32_t)b.fast_ms) == k;
       const bool slow = next_tick(k, win, (uint32_t)b.slow_ms) == k;
@@ -859,8 +916,11 @@ template <class T> cudaError_t launch_replay(ReplayBatch<T>& b, ReplayWs& w, cud
         b.lat.n, b.n_inst, (int32_t)(K * b.win), w.vm, b.o_ts, b.o_tf, b.o_te);
     if ((e = cudaGetLastError())) return e;
   }
-  if ((e = func_smem_once((const void*)k_replay<T>, (int)kReplaySmemMax, false))) return e;
-  k_replay<T><<<(unsigned)b.n_inst, 32 * std::min(M, kMaxWarps), (size_t)b.smem_bytes, s>>>(b);
+  // two warps a model while their barriers and the block's warps suffice
+  const bool pair = M <= kMaxPairs;
+  auto f = pair ? k_replay<T, true> : k_replay<T, false>;
+  if ((e = func_smem_once((const void*)f, (int)kReplaySmemMax, false))) return e;
+  f<<<(unsigned)b.n_inst, pair ? 64 * M : 32 * std::min(M, kMaxWarps), (size_t)b.smem_bytes, s>>>(b);
   return cudaGetLastError();
 }
 

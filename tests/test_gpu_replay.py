@@ -194,6 +194,25 @@ def test_replay_long_spans(tre, servers):
            [(0.8, 1)], wake=1310, sleep=1870)
 
 
+# one model, the most that have two warps each, one more; a model without requests,
+# one without replicas, batches of exactly 32 and 64 starts in a segment
+@pytest.mark.parametrize("M", [1, 8, 9])
+def test_replay_model_counts(tre, M):
+    rng = np.random.default_rng(M)
+    n, span = 64 * 40, 200_000
+    t = np.repeat(np.arange(40) * 5000, 64)
+    model = np.where(np.arange(n) % 64 < 32, 0, rng.integers(0, max(M - 1, 1), n))
+    total = rng.integers(0, 9000, n)
+    lat = {"model": model, "t_arr_ms": t, "d_first_ms": total // 3, "d_total_ms": total,
+           "L_in": rng.integers(0, 500, n), "L_out": rng.integers(1, 300, n)}
+    lat = {k: v.astype(np.int32) for k, v in lat.items()}
+    r0 = np.full(M, 30, np.int32)
+    r0[M // 2] = 0 if M > 1 else 30
+    _check(tre, lat, M, 1000, span // 1000, _prof(M, theta=20.0), int(r0.sum()) + 3, r0,
+           np.zeros(M, np.int32), np.ones(M, np.int32), "f64", [(0.8, 2), (0.9, 0)], wake=500,
+           sleep=700, guard=np.full(M, 3000, np.int32))
+
+
 def test_replay_invalid_records_are_not_served(tre):
     lat, M, budget = _mid_latent(0.005, 12, 600.0)
     lat = {k: (v.copy() if hasattr(v, "copy") else v) for k, v in lat.items()}
