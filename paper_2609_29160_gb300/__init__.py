@@ -162,9 +162,15 @@ def load(build_if_missing: bool = True):
 # ---------------------------------------------------------------------------
 # torch plumbing
 # ---------------------------------------------------------------------------
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _ptr(t):
@@ -172,9 +178,14 @@ def _ptr(t):
 
 
 def _stream(stream):
+    if stream is not None:
+        return C.c_void_p(stream.cuda_stream)
     torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    # the current stream's handle, where torch gives it without a Stream object
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return C.c_void_p(raw(torch.cuda.current_device()))
 
 
 def _check(fn, code):
@@ -195,6 +206,14 @@ def new_diag(device="cuda"):
     """Zeroed device-resident tre_diag."""
     torch = _torch()
     return torch.zeros(DIAG_BYTES, dtype=torch.uint8, device=device)
+
+
+def _scratch_diag(diag):
+    """The caller's tre_diag, or for a call that hands none back one that is
+    only added into (never read, so not cleared)."""
+    if diag is not None:
+        return diag
+    return _torch().empty(DIAG_BYTES, dtype=_torch().uint8, device="cuda")
 
 
 def read_diag(diag):
@@ -260,18 +279,30 @@ def _counts(c):
     return Counts(*[c[k].data_ptr() for k in ("P", "D", "A", "W")], *occ)
 
 
+_PROFILE_KEYS = ("w_p", "w_q", "alpha", "theta", "tau_crit", "tau_surplus")
+
+
+def _on_device(v, tdt, dev):
+    """v as a contiguous tensor of type tdt on the current CUDA device (itself
+    when it is one already)."""
+    if v.dtype is tdt and v.get_device() == dev and v.is_contiguous():
+        return v
+    return v.to(device="cuda", dtype=tdt).contiguous()
+
+
 def _profile(prof, M, tdt, code):
     torch = _torch()
+    dev = torch.cuda.current_device()
     out = {}
-    for k in ("w_p", "w_q", "alpha", "theta", "tau_crit", "tau_surplus"):
+    for k in _PROFILE_KEYS:
         v = prof.get(k)
         if v is None:
             out[k] = None
             continue
-        t = v if torch.is_tensor(v) else torch.as_tensor(np.broadcast_to(np.asarray(v), (M,)).copy())
-        out[k] = t.to(device="cuda", dtype=tdt).contiguous()
-    st = Profile(code, *[out[k].data_ptr() if out[k] is not None else None
-                         for k in ("w_p", "w_q", "alpha", "theta", "tau_crit", "tau_surplus")])
+        t = v if isinstance(v, torch.Tensor) else \
+            torch.as_tensor(np.broadcast_to(np.asarray(v), (M,)).copy())
+        out[k] = _on_device(t, tdt, dev)
+    st = Profile(code, *[t.data_ptr() if t is not None else None for t in out.values()])
     return st, out
 
 
@@ -292,7 +323,7 @@ def tss_window_reduce(M, window_ms, K, requests=None, events=None, diag=None, st
         if mean_occupancy:
             for k in ("A_ms", "W_ms"):
                 out[k] = torch.empty((K, M), dtype=torch.int64, device="cuda")
-    diag = new_diag() if diag is None else diag
+    diag = _scratch_diag(diag)
     rq = requests_struct(requests) if requests is not None else None
     ev = events_struct(events) if events is not None else None
     cs = _counts(out)
@@ -316,7 +347,7 @@ def tss_score(counts, profile, window_ms, dtype="f32", carry=None, recv=True, di
     Z = torch.empty((K, M), dtype=tdt, device="cuda")
     cls = torch.empty((K, M), dtype=torch.uint8, device="cuda")
     rv = torch.empty(K, dtype=torch.int32, device="cuda") if recv else None
-    diag = new_diag() if diag is None else diag
+    diag = _scratch_diag(diag)
     cs = _counts(counts)
     s = _stream(stream)
     _workspace("tss_score", lambda ws, n: lib.tss_score(
@@ -373,7 +404,7 @@ def tss_stage_gauges(M, window_ms, K, requests, diag=None, stream=None):
     g = Grid(M, window_ms, K)
     A_p = torch.empty((K, M), dtype=torch.int32, device="cuda")
     A_d = torch.empty((K, M), dtype=torch.int32, device="cuda")
-    diag = new_diag() if diag is None else diag
+    diag = _scratch_diag(diag)
     rq = requests_struct(requests)
     s = _stream(stream)
     _workspace("tss_stage_gauges", lambda ws, n: lib.tss_stage_gauges(
@@ -399,7 +430,7 @@ def tss_stage_calibrate(counts, A_prefill, A_decode, profile, window_ms, slo_ttf
         _need(t, "int32", K * M, what)
     th_p = torch.empty(M, dtype=tdt, device="cuda")
     th_d = torch.empty(M, dtype=tdt, device="cuda")
-    diag = new_diag() if diag is None else diag
+    diag = _scratch_diag(diag)
     rq = requests_struct(requests)
     cs = _counts(counts)
     s = _stream(stream)
@@ -428,7 +459,7 @@ def tss_stage_score(counts, A_prefill, A_decode, profile, window_ms, theta_prefi
     out = [{"S": torch.empty((K, M), dtype=tdt, device="cuda"),
             "Z": torch.empty((K, M), dtype=tdt, device="cuda"),
             "cls": torch.empty((K, M), dtype=torch.uint8, device="cuda")} for _ in range(2)]
-    diag = new_diag() if diag is None else diag
+    diag = _scratch_diag(diag)
     cs = _counts(counts)
     s = _stream(stream)
     _workspace("tss_stage_score", lambda ws, n: lib.tss_stage_score(
@@ -453,7 +484,7 @@ def tss_calibrate(counts, profile, window_ms, slo_ttft_ms, requests=None, events
     slo = torch.as_tensor(np.asarray(slo_ttft_ms, np.int32)).cuda() \
         if not torch.is_tensor(slo_ttft_ms) else slo_ttft_ms
     theta = torch.empty(M, dtype=tdt, device="cuda")
-    diag = new_diag() if diag is None else diag
+    diag = _scratch_diag(diag)
     rq = requests_struct(requests) if requests is not None else None
     ev = events_struct(events) if events is not None else None
     cs = _counts(counts)
@@ -499,15 +530,17 @@ def tre_select_moves(Z, cls, profile, window_ms, budget, r0, r_min, footprint, f
     r = dev(r0).clone()
     rmin, fp = dev(r_min), dev(footprint)
     ctrl = Ctrl(int(budget), rmin.data_ptr(), fp.data_ptr(), fast_ms, slow_ms, pacing_cap)
-    moves = torch.zeros(max(moves_cap, 1) * MOVE_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
-    nmv = torch.zeros(1, dtype=torch.int64, device="cuda")
+    # the number of moves, then the moves: one block, read back once
+    out = torch.zeros(8 + max(moves_cap, 1) * MOVE_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+    moves = C.c_void_p(out.data_ptr() + 8)
     diag = new_diag() if diag is None else diag
     s = _stream(stream)
     _workspace("tre_select_moves", lambda ws, n: lib.tre_select_moves(
-        C.byref(g), _ptr(Z), _ptr(cls), C.byref(pst), C.byref(ctrl), _ptr(r), _ptr(moves),
-        C.c_int64(moves_cap), _ptr(nmv), ws, n, _ptr(diag), s))
-    n = int(nmv.item())
-    mv = np.frombuffer(moves.cpu().numpy().tobytes(), dtype=MOVE_DTYPE)[: min(n, moves_cap)]
+        C.byref(g), _ptr(Z), _ptr(cls), C.byref(pst), C.byref(ctrl), _ptr(r), moves,
+        C.c_int64(moves_cap), _ptr(out), ws, n, _ptr(diag), s))
+    host = out.cpu().numpy()
+    n = int(host[:8].view(np.int64)[0])
+    mv = np.frombuffer(host.tobytes(), dtype=MOVE_DTYPE, offset=8)[: min(n, moves_cap)]
     return mv, r, n, diag
 
 
@@ -680,12 +713,13 @@ class PipelinePlan:
 
     def run(self, stream=None):
         """Enqueue the whole path on `stream` (default: current torch stream)."""
-        torch = _torch()
-        s = stream if stream is not None else torch.cuda.current_stream()
-        with torch.cuda.stream(s):
+        if stream is None:
             self.r.copy_(self.r0, non_blocking=True)
+        else:
+            with _torch().cuda.stream(stream):
+                self.r.copy_(self.r0, non_blocking=True)
         ws = C.c_void_p(self.ws.data_ptr())
-        for name, fn in self._calls(C.c_void_p(s.cuda_stream)):
+        for name, fn in self._calls(_stream(stream)):
             _check(name, fn(ws, C.byref(self._ws_n)))
         return self
 

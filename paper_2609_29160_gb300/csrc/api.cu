@@ -38,26 +38,27 @@ struct Tracer {
 Tracer g_trace;
 
 
-// A column the kernels may read: device memory, or host memory the GPU
-// addresses (pinned and mapped). Plain pageable host memory is refused here,
-// since a kernel reading it would fault. When the runtime cannot tell (no
-// device), the launch decides.
-bool gpu_addressable(const void* p) {
-  cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-    cudaGetLastError();
-    return true;
-  }
-  return a.type != cudaMemoryTypeUnregistered;
-}
-
-bool req_ok(const tre_requests* r) {
+// Columns the kernels may read: device memory, or host memory the GPU addresses
+// (pinned and mapped; *host says whether any column is). Plain pageable host
+// memory is refused here, since a kernel reading it would fault. When the
+// runtime cannot tell (no device), the launch decides.
+bool req_ok(const tre_requests* r, bool* host = nullptr) {
+  if (host) *host = false;
   if (!r || r->n < 0) return false;
   if (r->n == 0) return true;
   const void* cols[7] = {r->model, r->t_arr_ms, r->t_start_ms, r->t_first_ms, r->t_end_ms,
                          r->L_in, r->L_out};
-  for (const void* c : cols)
-    if (!c || !gpu_addressable(c)) return false;
+  for (const void* c : cols) {
+    if (!c) return false;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, c) != cudaSuccess) {
+      cudaGetLastError();
+    } else if (a.type == cudaMemoryTypeUnregistered) {
+      return false;
+    } else if (host && a.type == cudaMemoryTypeHost) {
+      *host = true;
+    }
+  }
   return true;
 }
 
@@ -279,6 +280,7 @@ tre_status select_typed(const tre_grid* g, const void* Z, const uint8_t* cls,
 // ---- tre_sweep --------------------------------------------------------------
 struct SweepPlan {
   int M, n_series, base_win, Kb;
+  bool host;                       // some trace has columns in host memory
   std::vector<int> K, q;           // per window length
   std::vector<int64_t> off;        // per series element offset
   int64_t total;                   // sum over series of K*M
@@ -299,8 +301,12 @@ bool sweep_plan(const tre_sweep_spec* sp, SweepPlan& pl) {
     return false;
   for (int c = 0; c < sp->n_cap; ++c)
     if (sp->pacing_cap[c] < 0 || sp->pacing_cap[c] > 255) return false;
-  for (int t = 0; t < sp->n_traces; ++t)
-    if (!req_ok(&sp->traces[t])) return false;
+  pl.host = false;
+  for (int t = 0; t < sp->n_traces; ++t) {
+    bool host;
+    if (!req_ok(&sp->traces[t], &host)) return false;
+    pl.host = pl.host || host;
+  }
   pl.M = sp->n_models;
   pl.base_win = *std::min_element(sp->window_ms, sp->window_ms + sp->n_win);
   if (pl.base_win < 1 || sp->duration_ms % pl.base_win) return false;
@@ -459,7 +465,7 @@ tre_status sweep_typed(const tre_sweep_spec* sp, const SweepPlan& pl, const tre_
     std::vector<int64_t> red_off(NT);
     for (int t = 0; t < NT; ++t) red_off[t] = in_place ? gp.in_off[t] : (int64_t)t * pl.Kb * M;
     e = launch_reduce_requests(cols.data(), NT, M, pl.base_win, pl.Kb, Pb, Db, rw, slob,
-                               sp->slo_ttft_ms, diag, s, red_off.data());
+                               sp->slo_ttft_ms, pl.host, diag, s, red_off.data());
   }
   if (fused) {
     if (!e) {
@@ -708,7 +714,8 @@ tre_status tss_window_reduce(const tre_grid* grid, const tre_requests* req, cons
                              tre_counts out, void* ws, size_t* ws_bytes, tre_diag* diag,
                              tre_stream stream) {
   if (!grid_ok(grid) || !ws_bytes || (!req) == (!ev)) return TRE_EINVAL;
-  if (req ? !req_ok(req) : !ev_ok(ev)) return TRE_EINVAL;
+  bool host = false;
+  if (req ? !req_ok(req, &host) : !ev_ok(ev)) return TRE_EINVAL;
   if (!counts_ok(&out)) return TRE_EINVAL;
   if (ws && !diag) return TRE_EINVAL;
   const int M = grid->n_models, K = grid->n_windows;
@@ -724,7 +731,7 @@ tre_status tss_window_reduce(const tre_grid* grid, const tre_requests* req, cons
     Scope sc(kReduce, req ? 2 : 4, s);   // clearing + reduction; or clearing and three event passes
     const ReqCols rc = req ? cols_of(req) : ReqCols{};
     e = req ? launch_reduce_requests(&rc, 1, M, grid->window_ms, K, out.P, out.D, w, nullptr,
-                                     nullptr, diag, s)
+                                     nullptr, host, diag, s)
             : launch_reduce_events(cols_of(ev), M, grid->window_ms, K, out.P, out.D, w, diag, s);
   }
   if (!e) {

@@ -119,11 +119,11 @@ void reduce_ws_layout(Arena& a, int M, int K, int n_traces, int64_t n_req, Reduc
 // trace t writes P, D (and the packed SLO counts when slo != null) at element
 // offset out_off[t] (host array; null: t*K*M). slo packs per-(window, model)
 // arrivals (low 32 bits) and the arrivals that met the TTFT bound (high 32
-// bits).
+// bits). host: some column lies in host memory the GPU addresses.
 cudaError_t launch_reduce_requests(const ReqCols* traces, int n_traces, int M, int win, int K,
                                    int32_t* P, int32_t* D, ReduceWs& w, unsigned long long* slo,
-                                   const int32_t* slo_ms, tre_diag* diag, cudaStream_t s,
-                                   const int64_t* out_off = nullptr);
+                                   const int32_t* slo_ms, bool host, tre_diag* diag,
+                                   cudaStream_t s, const int64_t* out_off = nullptr);
 cudaError_t launch_reduce_events(const EvCols& e, int M, int win, int K, int32_t* P, int32_t* D,
                                  ReduceWs& w, tre_diag* diag, cudaStream_t s);
 cudaError_t launch_slo_requests(const ReqCols& r, int M, int win, int K,

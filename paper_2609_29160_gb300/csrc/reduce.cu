@@ -1243,8 +1243,8 @@ void reduce_ws_layout(Arena& a, int M, int K, int n_traces, int64_t n_req, Reduc
 
 cudaError_t launch_reduce_requests(const ReqCols* traces, int n_traces, int M, int win, int K,
                                    int32_t* P, int32_t* D, ReduceWs& w, unsigned long long* slo,
-                                   const int32_t* slo_ms, tre_diag* diag, cudaStream_t s,
-                                   const int64_t* out_off) {
+                                   const int32_t* slo_ms, bool host, tre_diag* diag,
+                                   cudaStream_t s, const int64_t* out_off) {
   if (n_traces < 1 || n_traces > kMaxTraces || n_traces > w.n_traces)
     return cudaErrorInvalidValue;
   const size_t cells = (size_t)K * M * n_traces;
@@ -1268,20 +1268,7 @@ cudaError_t launch_reduce_requests(const ReqCols* traces, int n_traces, int M, i
   // records that live in host memory (pinned, mapped) are copied into shared
   // memory once per CTA rather than read twice over the host link; any column
   // in host memory selects the copying variant (it reads device columns too)
-  bool copy_records = false;
-  for (int t = 0; t < n_traces; ++t) {
-    const ReqCols& c = traces[t];
-    if (c.n == 0) continue;
-    const void* cols[7] = {c.model, c.t_arr, c.t_start, c.t_first, c.t_end, c.L_in, c.L_out};
-    for (const void* p : cols) {
-      cudaPointerAttributes pa;
-      if (cudaPointerGetAttributes(&pa, p) != cudaSuccess) {
-        cudaGetLastError();
-        continue;
-      }
-      if (pa.type == cudaMemoryTypeHost) copy_records = true;
-    }
-  }
+  const bool copy_records = host;
   const int64_t mean_n = std::max<int64_t>(total_n / n_traces, 1);
   // model rows padded to a power of two on the arrival side; start side runs
   // of F (power of two) windows per model
