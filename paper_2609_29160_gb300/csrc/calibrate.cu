@@ -340,13 +340,14 @@ template <class T> size_t search_smem_bytes() {
   return fast > descent ? fast : descent;
 }
 
-// One CTA per (series, model), or a cluster of CL of them. DIRECT: the keys are made here, from the
-// model's column of S, classes and counts, and stay in registers (series of up
+// One CTA per (series, model), or a cluster of CL of them. DIRECT: the keys are made
+// here, from the model's column of S, classes and counts, and stay in registers (series of up
 // to kDirectK windows): one launch where packing, its threshold table and the
 // search were three. Otherwise they come from the packing pass, and are read
 // again for the gather. What bounds a search is its chain of block-wide steps.
-// 8 models, 3,600 windows: 15.4 us in one launch (25.3 in three, with a bitonic
-// sort of the gathered keys and every test in double); 16 models, 43,200
+// 8 models, 3,600 windows: 12.0 us in one launch (25.3 in three, with a bitonic
+// sort of the gathered keys and every test in double; 14.0 with 4,096 buckets, four
+// a thread, where a short series fills a bucket a thread as well); 16 models, 43,200
 // windows: 21.6 us (30.5); the sweep's 224 searches: 24.5 us (33.3).
 //
 // With CL CTAs each reads its part of the keys: they count into their own
@@ -363,6 +364,7 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
   begin_after_previous();
   using U = typename KeyOf<T>::U;
   constexpr int NL = KeyOf<T>::kLevels;
+  constexpr int kFineHere = DIRECT ? kNB : kFine;   // a bucket a thread on short series
   constexpr int kThrDirect = 256;
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ U lo_s[NL], hi_s[NL];
@@ -387,12 +389,12 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
   T* const th_out = theta1 && s == 1 ? theta1 + m : theta + out;
   const float rel_f = (float)reliability;
   int32_t* fcnt = reinterpret_cast<int32_t*>(dyn);
-  int32_t* fhl = fcnt + kFine;
-  int32_t* fst = fhl + kFine;                   // where a selected bucket's keys start, -1 if not
-  int32_t* fca = fst + kFine;                   // windows in buckets above
-  int32_t* fha = fca + kFine;                   // healthy windows in buckets above
-  U* list = reinterpret_cast<U*>(fha + kFine);
-  for (int b = tid; b < kFine; b += kNB) {
+  int32_t* fhl = fcnt + kFineHere;
+  int32_t* fst = fhl + kFineHere;                   // where a selected bucket's keys start, -1 if not
+  int32_t* fca = fst + kFineHere;                   // windows in buckets above
+  int32_t* fha = fca + kFineHere;                   // healthy windows in buckets above
+  U* list = reinterpret_cast<U*>(fha + kFineHere);
+  for (int b = tid; b < kFineHere; b += kNB) {
     fcnt[b] = 0;
     fhl[b] = 0;
   }
@@ -471,7 +473,7 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
   // not below it in its own bucket: no order within a bucket is needed.
   {
     int sh = 0;
-    while (sh < 63 && ((kmax - kmin) >> sh) >= (U)kFine) ++sh;
+    while (sh < 63 && ((kmax - kmin) >> sh) >= (U)kFineHere) ++sh;
     __syncthreads();
     // with fewer than 2^16 candidates, a bucket's count and healthy count
     // share one 32-bit word (one atomic per key)
@@ -505,7 +507,7 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
     });
     __syncthreads();
     if constexpr (CL > 1) cg::this_cluster().sync();
-    constexpr int PER = kFine / kNB;            // consecutive buckets per thread
+    constexpr int PER = kFineHere / kNB;            // consecutive buckets per thread
     int bf = 0x7fffffff, nsel = 0;
     if (rank == 0) {
     const int b0 = tid * PER;
@@ -588,7 +590,7 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
       cl.sync();
       if (rank > 0) {
         const int32_t* src = cl.map_shared_rank(fst, 0);
-        for (int q = tid; q < kFine; q += kNB) fst[q] = src[q];
+        for (int q = tid; q < kFineHere; q += kNB) fst[q] = src[q];
         nsel = cl.map_shared_rank(plan_s, 0)[0];
         bf = cl.map_shared_rank(plan_s, 0)[1];
         place = cl.map_shared_rank(fhl, 0);
