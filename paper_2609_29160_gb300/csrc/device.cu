@@ -1,10 +1,9 @@
-// Per-device launch state: SM counts, raised shared-memory limits and the kernels
-// launched so far, kept for each GPU separately (a function attribute set on one device does not apply
+// Per-device launch state: SM counts and raised shared-memory limits, kept for
+// each GPU separately (a function attribute set on one device does not apply
 // on another) and guarded for concurrent host threads.
 #include <mutex>
 #include <set>
 #include <tuple>
-#include <utility>
 
 #include "internal.h"
 
@@ -15,7 +14,6 @@ constexpr int kMaxDevices = 64;
 int g_sms[kMaxDevices];                     // 0 = not looked up yet
 std::mutex g_mu;
 std::set<std::tuple<int, const void*, int, bool>> g_attr;   // (device, fn, bytes, carveout)
-std::set<std::pair<int, const void*>> g_launched;            // (device, fn)
 
 int current_device() {
   int dev = 0;
@@ -54,12 +52,6 @@ cudaError_t func_smem_once(const void* fn, int bytes, bool max_carveout) {
   if (e) return e;
   g_attr.insert(key);
   return cudaSuccess;
-}
-
-bool launched_before(const void* fn) {
-  const int dev = current_device();
-  std::lock_guard<std::mutex> lk(g_mu);
-  return !g_launched.insert(std::make_pair(dev, fn)).second;
 }
 
 }  // namespace tre

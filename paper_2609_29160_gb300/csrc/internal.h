@@ -14,9 +14,7 @@ namespace tre {
 // before it (begin_after_previous() in common.cuh keeps the order): a pass over
 // a short trace is a dozen kernels of a few microseconds, with 1.5 to 2 us
 // between them otherwise (3 models, 600 windows: 109 us, now 78).
-// A kernel's first launch on a device, which loads its code, is a plain one.
 // Errors stay with the runtime (cudaGetLastError).
-bool launched_before(const void* fn);
 template <class... P, class... A>
 inline void launch_clusters(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, int cluster,
                             cudaStream_t s, A&&... args) {
@@ -26,20 +24,13 @@ inline void launch_clusters(void (*kernel)(P...), dim3 grid, dim3 block, size_t 
   c.dynamicSmemBytes = smem;
   c.stream = s;
   cudaLaunchAttribute at[2];
-  int n = 0;
-  if (cluster > 1) {
-    at[n].id = cudaLaunchAttributeClusterDimension;
-    at[n].val.clusterDim.x = (unsigned)cluster;
-    at[n].val.clusterDim.y = at[n].val.clusterDim.z = 1;
-    ++n;
-  }
-  if (launched_before(reinterpret_cast<const void*>(kernel))) {
-    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[n].val.programmaticStreamSerializationAllowed = 1;
-    ++n;
-  }
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cluster;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
   c.attrs = at;
-  c.numAttrs = (unsigned)n;
+  c.numAttrs = cluster > 1 ? 2 : 1;
   cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
 template <class... P, class... A>
