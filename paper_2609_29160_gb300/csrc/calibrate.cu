@@ -70,7 +70,6 @@ __device__ __forceinline__ int32_t healthy_from(double ok_frac, int a) {
 // resets the per-(series, model) candidate key ranges filled by k_pack
 template <class U>
 __global__ void k_thr(double ok_frac, int32_t* thr, int n_sm, U* kmin, U* kmax, uint32_t* ncand) {
-  begin_after_previous();
   const int a = blockIdx.x * blockDim.x + threadIdx.x;
   if (a < n_sm) {
     kmin[a] = ~(U)0;
@@ -138,7 +137,6 @@ k_pack_vec(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ P
            const unsigned long long* __restrict__ slo, const int32_t* __restrict__ thr,
            double ok_frac, typename KeyOf<T>::U* __restrict__ keys,
            typename KeyOf<T>::U* kmin_g, typename KeyOf<T>::U* kmax_g, uint32_t* ncand_g) {
-  begin_after_previous();
   using U = typename KeyOf<T>::U;
   static_assert(kPackTile == 4 * kPackThreads, "four elements per thread");
   __shared__ U tile[kPackTile + 32];
@@ -217,7 +215,6 @@ k_pack(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ PackP
        const unsigned long long* __restrict__ slo, const int32_t* __restrict__ thr,
        double ok_frac, typename KeyOf<T>::U* __restrict__ keys, typename KeyOf<T>::U* kmin_g,
        typename KeyOf<T>::U* kmax_g, uint32_t* ncand_g) {
-  begin_after_previous();
   using U = typename KeyOf<T>::U;
   __shared__ U tile[kPackTile + 32];
   __shared__ U smin[32], smax[32];
@@ -361,7 +358,6 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
          const uint32_t* ncand_g, const T* __restrict__ S, const uint8_t* __restrict__ cls,
          const unsigned long long* __restrict__ slo, double ok_frac, double reliability, T* theta,
          T* theta1, tre_diag* diag) {
-  begin_after_previous();
   using U = typename KeyOf<T>::U;
   constexpr int NL = KeyOf<T>::kLevels;
   constexpr int kFineHere = DIRECT ? kNB : kFine;   // a bucket a thread on short series
@@ -777,12 +773,12 @@ cudaError_t launch_calibrate(const SeriesTable<T>& tab, const T* S, const uint8_
   if (direct && cells <= kDirectCells) {
     cudaError_t e = func_smem_once((const void*)k_search<T, true, 1>, (int)smem, true);
     if (e) return e;
-    launch(k_search<T, true, 1>, n_sm, kNB, smem, s, tab, static_cast<U*>(w.keys), kmin, kmax,
-           w.ncand, S, cls, slo, ok_frac, reliability, theta, theta1, diag);
+    k_search<T, true, 1><<<n_sm, kNB, smem, s>>>(tab, static_cast<U*>(w.keys), kmin, kmax, w.ncand, S,
+                                              cls, slo, ok_frac, reliability, theta, theta1, diag);
     return cudaGetLastError();
   }
   const int thr_n = std::max(kThrTable, n_sm);
-  launch(k_thr<U>, (thr_n + 255) / 256, 256, 0, s, ok_frac, w.thr, n_sm, kmin, kmax, w.ncand);
+  k_thr<U><<<(thr_n + 255) / 256, 256, 0, s>>>(ok_frac, w.thr, n_sm, kmin, kmax, w.ncand);
   PackPlan pp;
   pp.lg_tm = 0;
   while ((1 << pp.lg_tm) < tab.M && pp.lg_tm < 5) ++pp.lg_tm;
@@ -800,11 +796,11 @@ cudaError_t launch_calibrate(const SeriesTable<T>& tab, const T* S, const uint8_
   const bool vec = tab.M % pp.tm == 0 && tab.M % 4 == 0 &&
                    (((uintptr_t)S | (uintptr_t)cls | (uintptr_t)slo) & 15) == 0;
   if (tiles > 0 && vec)
-    launch(k_pack_vec<T>, tiles, kPackThreads, 0, s, tab, pp, S, cls, slo, w.thr, ok_frac,
-           static_cast<U*>(w.keys), kmin, kmax, w.ncand);
+    k_pack_vec<T><<<tiles, kPackThreads, 0, s>>>(tab, pp, S, cls, slo, w.thr, ok_frac,
+                                                 static_cast<U*>(w.keys), kmin, kmax, w.ncand);
   else if (tiles > 0)
-    launch(k_pack<T>, tiles, kPackThreads, 0, s, tab, pp, S, cls, slo, w.thr, ok_frac,
-           static_cast<U*>(w.keys), kmin, kmax, w.ncand);
+    k_pack<T><<<tiles, kPackThreads, 0, s>>>(tab, pp, S, cls, slo, w.thr, ok_frac,
+                                             static_cast<U*>(w.keys), kmin, kmax, w.ncand);
   // clusters while the searches leave SMs idle (two share an SM where their
   // tables fit) and a CTA's part still has eight windows a thread
   int cl = 1;
@@ -816,8 +812,21 @@ cudaError_t launch_calibrate(const SeriesTable<T>& tab, const T* S, const uint8_
                                                           : k_search<T, false, 1>;
   cudaError_t e = func_smem_once((const void*)search, (int)smem, true);
   if (e) return e;
-  launch_clusters(search, n_sm * cl, kNB, smem, cl, s, tab, static_cast<U*>(w.keys), kmin, kmax,
-                  w.ncand, S, cls, slo, ok_frac, reliability, theta, theta1, diag);
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3((unsigned)(n_sm * cl));
+  c.blockDim = dim3(kNB);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)cl;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  c.attrs = &at;
+  c.numAttrs = cl > 1 ? 1 : 0;
+  e = cudaLaunchKernelEx(&c, search, tab, static_cast<U*>(w.keys), static_cast<const U*>(kmin),
+                         static_cast<const U*>(kmax), static_cast<const uint32_t*>(w.ncand), S,
+                         cls, slo, ok_frac, reliability, theta, theta1, diag);
+  if (e) return e;
   return cudaGetLastError();
 }
 

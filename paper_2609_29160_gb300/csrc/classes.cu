@@ -6,7 +6,6 @@
 // n_models * n_classes models.
 #include <algorithm>
 
-#include "common.cuh"
 #include "internal.h"
 
 namespace tre {
@@ -15,7 +14,6 @@ namespace {
 __global__ void __launch_bounds__(256)
 k_class_models(int64_t n, const int32_t* model, const int32_t* __restrict__ cls, int32_t M,
                int32_t C, int32_t* out) {
-  begin_after_previous();
   for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * 256) {
     const int32_t m = model[i], c = cls[i];
@@ -36,7 +34,7 @@ extern "C" tre_status tss_class_models(int64_t n, const int32_t* model, const in
   if (!model || !cls || !model_out) return TRE_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int64_t blocks = std::min<int64_t>((n + 255) / 256, 152 * 32);
-  tre::launch(tre::k_class_models, (unsigned)blocks, 256, 0, s, n, model, cls, n_models, n_classes,
-              model_out);
+  tre::k_class_models<<<(unsigned)blocks, 256, 0, s>>>(n, model, cls, n_models, n_classes,
+                                                      model_out);
   return cudaGetLastError() == cudaSuccess ? TRE_OK : TRE_ECUDA;
 }

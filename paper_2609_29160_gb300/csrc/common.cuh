@@ -8,17 +8,6 @@
 
 namespace tre {
 
-// Every kernel of the library is launched with programmatic stream serialisation
-// (launch() in internal.h): its launch overlaps the end of the kernel before it on
-// the stream, and it starts with this. The wait returns when that kernel has ended
-// and its writes are visible (which it cannot before the ones before it have, as it
-// waited for them in turn). No kernel lets the next one in early: with
-// griddepcontrol.launch_dependents here the next kernel's CTAs piled onto the SMs
-// that were free first (seven traces of 1M records: 361 us a sweep for 305).
-__device__ __forceinline__ void begin_after_previous() {
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");
-}
-
 // ---------------------------------------------------------------------------
 // IEEE arithmetic with explicit rounding, one operation at a time. The library
 // is compiled with -fmad=false as well, but the intrinsics make the intent

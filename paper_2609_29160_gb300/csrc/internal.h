@@ -9,36 +9,6 @@
 
 namespace tre {
 
-// Launches a kernel of the library behind the work already on the stream. With
-// programmatic stream serialisation the launch overlaps the end of the kernel
-// before it (begin_after_previous() in common.cuh keeps the order): a pass over
-// a short trace is a dozen kernels of a few microseconds, with 1.5 to 2 us
-// between them otherwise (3 models, 600 windows: 109 us, now 78).
-// Errors stay with the runtime (cudaGetLastError).
-template <class... P, class... A>
-inline void launch_clusters(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, int cluster,
-                            cudaStream_t s, A&&... args) {
-  cudaLaunchConfig_t c = {};
-  c.gridDim = grid;
-  c.blockDim = block;
-  c.dynamicSmemBytes = smem;
-  c.stream = s;
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  at[1].id = cudaLaunchAttributeClusterDimension;
-  at[1].val.clusterDim.x = (unsigned)cluster;
-  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
-  c.attrs = at;
-  c.numAttrs = cluster > 1 ? 2 : 1;
-  cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
-}
-template <class... P, class... A>
-inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                   A&&... args) {
-  launch_clusters(kernel, grid, block, smem, 1, s, static_cast<A&&>(args)...);
-}
-
 // Bump allocator over the caller's workspace. With base == nullptr it only
 // measures (the query pass of every entry point).
 struct Arena {

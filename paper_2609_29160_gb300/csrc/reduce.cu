@@ -95,7 +95,6 @@ k_reduce_requests(const __grid_constant__ ReqBatch bt, int M, int lgMp, int win,
                   int32_t* __restrict__ D0, int32_t* __restrict__ dA0, int32_t* __restrict__ dW0,
                   unsigned long long* __restrict__ slo0, const int32_t* __restrict__ slo_ms,
                   tre_diag* diag) {
-  begin_after_previous();
   extern __shared__ unsigned long long smem[];
   uint32_t n_range = 0, n_model = 0, n_order = 0;
   // a CTA takes slices blockIdx.x, blockIdx.x + gridDim.x, ...: one slice when
@@ -444,7 +443,6 @@ constexpr int kSloPer = 4096;
 __global__ void __launch_bounds__(kThreads)
 k_slo_requests(ReqCols r, int M, int win, FastDiv fd, int K, int rows, bool vec,
                unsigned long long* __restrict__ slo, const int32_t* __restrict__ slo_ms) {
-  begin_after_previous();
   extern __shared__ uint32_t s_slo[];   // [rows][M]
   const int64_t i0 = (int64_t)blockIdx.x * kSloPer;
   const int n_loc = (int)min64(r.n - i0, (int64_t)kSloPer);
@@ -594,7 +592,6 @@ __global__ void __launch_bounds__(kThreads)
 k_reduce_events(EvCols e, int M, uint32_t span, FastDiv31 fd, int K, int per_cta, int rows,
                 bool vec, int32_t* __restrict__ P, int32_t* __restrict__ D,
                 int32_t* __restrict__ first, int32_t* __restrict__ last, tre_diag* diag) {
-  begin_after_previous();
   extern __shared__ __align__(16) unsigned char ev_smem[];
   const int64_t i0 = (int64_t)blockIdx.x * per_cta;
   const int n_loc = (int)min64(e.n - i0, (int64_t)per_cta);
@@ -789,7 +786,6 @@ k_reduce_events(EvCols e, int M, uint32_t span, FastDiv31 fd, int K, int per_cta
 }
 
 __global__ void k_fill_first_last(int32_t* first, int32_t* last, int64_t n) {
-  begin_after_previous();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     first[i] = 0x7fffffff;
@@ -807,7 +803,6 @@ k_event_gauges(EvCols e, int M, FastDiv fd, FastDiv fchunk, int K,
                const int32_t* __restrict__ first, const int32_t* __restrict__ last,
                int32_t* __restrict__ dA, int32_t* __restrict__ dW, int32_t* __restrict__ pA,
                int32_t* __restrict__ pW, tre_diag* diag) {
-  begin_after_previous();
   unsigned long long n_order = 0;
   auto add = [&](int32_t* d, int32_t* p, int64_t k, int m, int v) {
     atomicAdd(&d[k * M + m], v);
@@ -837,7 +832,6 @@ k_event_gauges(EvCols e, int M, FastDiv fd, FastDiv fchunk, int K,
 __global__ void __launch_bounds__(kThreads)
 k_slo_events(EvCols e, int M, int win, int K, unsigned long long* __restrict__ slo,
              const int32_t* __restrict__ slo_ms) {
-  begin_after_previous();
   const int64_t span = (int64_t)K * win;
   for (int64_t r = (int64_t)blockIdx.x * kThreads + threadIdx.x; r < e.n_req;
        r += (int64_t)gridDim.x * kThreads) {
@@ -860,7 +854,6 @@ __global__ void __launch_bounds__(kThreads)
 k_scan_partials(int M, int K, int L, int n_chunks, const int32_t* __restrict__ dA,
                 const int32_t* __restrict__ dW, int32_t* __restrict__ pA,
                 int32_t* __restrict__ pW) {
-  begin_after_previous();
   const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   if (t >= (int64_t)n_chunks * M) return;
   dA += (size_t)blockIdx.y * (K + 1) * M;
@@ -898,7 +891,6 @@ k_scan_partials(int M, int K, int L, int n_chunks, const int32_t* __restrict__ d
 template <int PT>
 __global__ void __launch_bounds__(1024)
 k_scan_chunks(int M, int n_chunks, int32_t* __restrict__ pA, int32_t* __restrict__ pW) {
-  begin_after_previous();
   __shared__ int2 sums[32];
   const unsigned full = 0xffffffffu;
   const int m = blockIdx.x;
@@ -940,7 +932,6 @@ __global__ void __launch_bounds__(kThreads)
 k_scan_apply(int M, int K, int L, int n_chunks, const int32_t* __restrict__ dA,
              const int32_t* __restrict__ dW, const int32_t* __restrict__ pA,
              const int32_t* __restrict__ pW, int32_t* __restrict__ A, int32_t* __restrict__ W) {
-  begin_after_previous();
   const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   if (t >= (int64_t)n_chunks * M) return;
   dA += (size_t)blockIdx.y * (K + 1) * M;
@@ -986,7 +977,6 @@ k_aggregate(const __grid_constant__ AggPlan pl, const int32_t* __restrict__ P,
             const int32_t* __restrict__ W, const unsigned long long* __restrict__ slo,
             int32_t* __restrict__ Pq, int32_t* __restrict__ Dq, int32_t* __restrict__ Aq,
             int32_t* __restrict__ Wq, unsigned long long* __restrict__ sloq) {
-  begin_after_previous();
   const int w = blockIdx.y, tr = blockIdx.z;
   const int M = pl.M, q = pl.q[w];
   const int64_t n = (int64_t)pl.Kq[w] * M;
@@ -1031,7 +1021,6 @@ void zero_add(ZeroList& zl, void* p, int64_t words) {
 }
 
 __global__ void __launch_bounds__(kThreads) k_zero(const __grid_constant__ ZeroList zl) {
-  begin_after_previous();
   const int r = prefix_index(zl.cta_base, zl.n, blockIdx.x);
   uint32_t* p = zl.ptr[r];
   const int64_t n = zl.words[r];
@@ -1054,7 +1043,7 @@ void zero_launch(ZeroList& zl, cudaStream_t s) {
     ctas += (int)((zl.words[r] + kZeroChunk - 1) / kZeroChunk);
   }
   zl.cta_base[zl.n] = ctas;
-  if (ctas > 0) launch(k_zero, ctas, kThreads, 0, s, zl);
+  if (ctas > 0) k_zero<<<ctas, kThreads, 0, s>>>(zl);
 }
 
 // ---- gauge scan fused with the exact coarsening (sweeps) --------------------
@@ -1068,7 +1057,6 @@ __global__ void __launch_bounds__(kThreads)
 k_gauge_blocks(const __grid_constant__ GaugePlan gp, const int32_t* __restrict__ dA,
                const int32_t* __restrict__ dW, int32_t* __restrict__ pA,
                int32_t* __restrict__ pW) {
-  begin_after_previous();
   const int M = gp.M, Kb = gp.Kb;
   const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   if (t >= (int64_t)gp.n_traces * gp.nblk * M) return;
@@ -1091,7 +1079,6 @@ k_gauge_blocks(const __grid_constant__ GaugePlan gp, const int32_t* __restrict__
 __global__ void __launch_bounds__(kThreads)
 k_gauge_block_scan(const __grid_constant__ GaugePlan gp, int32_t* __restrict__ pA,
                    int32_t* __restrict__ pW) {
-  begin_after_previous();
   __shared__ int32_t wa[kThreads / 32], ww[kThreads / 32];
   const int M = gp.M, nb = gp.nblk;
   const int tr = blockIdx.x / M, m = blockIdx.x % M;
@@ -1134,7 +1121,6 @@ k_gauge_apply(const __grid_constant__ GaugePlan gp, const int32_t* __restrict__ 
               const int32_t* __restrict__ Din, const unsigned long long* __restrict__ sloin,
               int32_t* __restrict__ P, int32_t* __restrict__ D, int32_t* __restrict__ A,
               int32_t* __restrict__ W, unsigned long long* __restrict__ slo) {
-  begin_after_previous();
   constexpr int RB = 4;   // rows whose loads are issued together
   const int M = gp.M, Kb = gp.Kb;
   const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
@@ -1359,17 +1345,21 @@ cudaError_t launch_reduce_requests(const ReqCols* traces, int n_traces, int M, i
                             ? (unsigned)std::min(ctas, 2 * std::max(1, device_sm_count() * 2 / 3))
                             : (unsigned)ctas;
   if (slo && copy_records)
-    launch(k_reduce_requests<true, true>, grid, kThreads, smem, s, bt, M, lgMp, win, fd, K,
-           near_rows, lgF, P, D, w.dA, w.dW, slo, slo_ms, diag);
+    k_reduce_requests<true, true><<<grid, kThreads, smem, s>>>(bt, M, lgMp, win, fd, K,
+                                                               near_rows, lgF, P, D, w.dA, w.dW,
+                                                               slo, slo_ms, diag);
   else if (slo)
-    launch(k_reduce_requests<true, false>, grid, kThreads, smem, s, bt, M, lgMp, win, fd, K,
-           near_rows, lgF, P, D, w.dA, w.dW, slo, slo_ms, diag);
+    k_reduce_requests<true, false><<<grid, kThreads, smem, s>>>(bt, M, lgMp, win, fd, K,
+                                                                near_rows, lgF, P, D, w.dA, w.dW,
+                                                                slo, slo_ms, diag);
   else if (copy_records)
-    launch(k_reduce_requests<false, true>, grid, kThreads, smem, s, bt, M, lgMp, win, fd, K,
-           near_rows, lgF, P, D, w.dA, w.dW, nullptr, nullptr, diag);
+    k_reduce_requests<false, true><<<grid, kThreads, smem, s>>>(bt, M, lgMp, win, fd, K,
+                                                                near_rows, lgF, P, D, w.dA, w.dW,
+                                                                nullptr, nullptr, diag);
   else
-    launch(k_reduce_requests<false, false>, grid, kThreads, smem, s, bt, M, lgMp, win, fd, K,
-           near_rows, lgF, P, D, w.dA, w.dW, nullptr, nullptr, diag);
+    k_reduce_requests<false, false><<<grid, kThreads, smem, s>>>(bt, M, lgMp, win, fd, K,
+                                                                 near_rows, lgF, P, D, w.dA, w.dW,
+                                                                 nullptr, nullptr, diag);
   return cudaGetLastError();
 }
 
@@ -1386,8 +1376,8 @@ cudaError_t launch_slo_requests(const ReqCols& r, int M, int win, int K,
   const bool vec = (((uintptr_t)r.model | (uintptr_t)r.t_arr | (uintptr_t)r.t_start |
                      (uintptr_t)r.t_first | (uintptr_t)r.t_end | (uintptr_t)r.L_in |
                      (uintptr_t)r.L_out) & 15) == 0;
-  launch(k_slo_requests, grid, kThreads, (size_t)rows * M * 4, s, r, M, win, FastDiv(win), K, rows,
-         vec, slo, slo_ms);
+  k_slo_requests<<<grid, kThreads, (size_t)rows * M * 4, s>>>(r, M, win, FastDiv(win), K, rows,
+                                                              vec, slo, slo_ms);
   return cudaGetLastError();
 }
 
@@ -1411,7 +1401,7 @@ cudaError_t launch_reduce_events(const EvCols& ev, int M, int win, int K, int32_
   zero_launch(zl, s);
   if ((e = cudaGetLastError())) return e;
   if (ev.n_req > 0) {
-    launch(k_fill_first_last, grid_for(ev.n_req, 4), kThreads, 0, s, w.first, w.last, ev.n_req);
+    k_fill_first_last<<<grid_for(ev.n_req, 4), kThreads, 0, s>>>(w.first, w.last, ev.n_req);
     if ((e = cudaGetLastError())) return e;
   }
   if (ev.n > 0) {
@@ -1431,17 +1421,17 @@ cudaError_t launch_reduce_events(const EvCols& ev, int M, int win, int K, int32_
       if ((e = func_smem_once(f, kEventSmem + kStageBytes, true))) return e;
     const uint32_t span = (uint32_t)((int64_t)K * win);
     if (pair)
-      launch(k_reduce_events<true>, grid, kThreads, smem, s, ev, M, span, FastDiv31(win), K,
-             (int)per, rows, vec, P, D, w.first, w.last, diag);
+      k_reduce_events<true><<<grid, kThreads, smem, s>>>(ev, M, span, FastDiv31(win), K, (int)per,
+                                                         rows, vec, P, D, w.first, w.last, diag);
     else
-      launch(k_reduce_events<false>, grid, kThreads, smem, s, ev, M, span, FastDiv31(win), K,
-             (int)per, rows, vec, P, D, w.first, w.last, diag);
+      k_reduce_events<false><<<grid, kThreads, smem, s>>>(ev, M, span, FastDiv31(win), K, (int)per,
+                                                          rows, vec, P, D, w.first, w.last, diag);
     if ((e = cudaGetLastError())) return e;
   }
   if (ev.n_req > 0) {
-    launch(k_event_gauges, grid_for(ev.n_req, 4), kThreads, 0, s, ev, M, FastDiv(win), FastDiv(L),
-           K, w.first, w.last, w.dA, w.dW, w.chunks_summed ? w.partA : nullptr,
-           w.chunks_summed ? w.partW : nullptr, diag);
+    k_event_gauges<<<grid_for(ev.n_req, 4), kThreads, 0, s>>>(
+        ev, M, FastDiv(win), FastDiv(L), K, w.first, w.last, w.dA, w.dW,
+        w.chunks_summed ? w.partA : nullptr, w.chunks_summed ? w.partW : nullptr, diag);
     if ((e = cudaGetLastError())) return e;
   }
   return cudaSuccess;
@@ -1451,7 +1441,7 @@ cudaError_t launch_slo_events(const EvCols& ev, int M, int win, int K, unsigned 
                               const int32_t* slo_ms, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(slo, 0, (size_t)K * M * sizeof(unsigned long long), s);
   if (e || ev.n_req == 0) return e;
-  launch(k_slo_events, grid_for(ev.n_req, 4), kThreads, 0, s, ev, M, win, K, slo, slo_ms);
+  k_slo_events<<<grid_for(ev.n_req, 4), kThreads, 0, s>>>(ev, M, win, K, slo, slo_ms);
   return cudaGetLastError();
 }
 
@@ -1465,10 +1455,10 @@ cudaError_t launch_gauge_scan(int M, int K, ReduceWs& w, int32_t* A, int32_t* W,
   const int64_t segs = (int64_t)n_chunks * M;
   dim3 g((unsigned)((segs + kThreads - 1) / kThreads), w.n_traces);
   if (!w.chunks_summed)
-    launch(k_scan_partials, g, kThreads, 0, s, M, K, L, n_chunks, w.dA, w.dW, w.partA, w.partW);
+    k_scan_partials<<<g, kThreads, 0, s>>>(M, K, L, n_chunks, w.dA, w.dW, w.partA, w.partW);
   auto scan = n_chunks <= 1024 ? k_scan_chunks<1> : k_scan_chunks<kMaxChunksPerThread>;
-  launch(scan, dim3(M, w.n_traces), 1024, 0, s, M, n_chunks, w.partA, w.partW);
-  launch(k_scan_apply, g, kThreads, 0, s, M, K, L, n_chunks, w.dA, w.dW, w.partA, w.partW, A, W);
+  scan<<<dim3(M, w.n_traces), 1024, 0, s>>>(M, n_chunks, w.partA, w.partW);
+  k_scan_apply<<<g, kThreads, 0, s>>>(M, K, L, n_chunks, w.dA, w.dW, w.partA, w.partW, A, W);
   return cudaGetLastError();
 }
 
@@ -1495,7 +1485,6 @@ k_occ_staged(ReqCols r, bool vec, bool stage, int M, int lgMp, int win, FastDiv 
              int near_rows, int lgF, unsigned long long* __restrict__ pA,
              unsigned long long* __restrict__ pW, int32_t* __restrict__ fA,
              int32_t* __restrict__ fW) {
-  begin_after_previous();
   extern __shared__ uint32_t osm32[];
   const int64_t i0 = (int64_t)blockIdx.x * kOccPerCta;
   const int n_loc = (int)min64(r.n - i0, kOccPerCta);
@@ -1658,7 +1647,6 @@ k_occ_apply(int M, int K, int L, int n_chunks, int win, const int32_t* __restric
             const int32_t* __restrict__ fW, const int32_t* __restrict__ pA,
             const int32_t* __restrict__ pW, long long* __restrict__ A_ms,
             long long* __restrict__ W_ms) {
-  begin_after_previous();
   const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   if (t >= (int64_t)n_chunks * M) return;
   const int m = (int)(t % M);
@@ -1702,7 +1690,6 @@ k_occ_events(EvCols ev, int M, int win, FastDiv fd, int K, const int32_t* __rest
              const int32_t* __restrict__ last, unsigned long long* __restrict__ pA,
              unsigned long long* __restrict__ pW, int32_t* __restrict__ fA,
              int32_t* __restrict__ fW) {
-  begin_after_previous();
   const uint32_t span = (uint32_t)K * (uint32_t)win, uw = (uint32_t)win;
   for (int64_t r = (int64_t)blockIdx.x * kThreads + threadIdx.x; r < ev.n_req;
        r += (int64_t)gridDim.x * kThreads) {
@@ -1740,12 +1727,13 @@ cudaError_t occ_finish(int M, int win, int K, ReduceWs& w, int64_t* A_ms, int64_
   const int n_chunks = (K + L - 1) / L;
   const int64_t segs = (int64_t)n_chunks * M;
   const unsigned g = (unsigned)((segs + kThreads - 1) / kThreads);
-  launch(k_scan_partials, dim3(g, 1), kThreads, 0, s, M, K, L, n_chunks, w.dA, w.dW, w.partA,
-         w.partW);
+  k_scan_partials<<<dim3(g, 1), kThreads, 0, s>>>(M, K, L, n_chunks, w.dA, w.dW, w.partA,
+                                                  w.partW);
   auto scan = n_chunks <= 1024 ? k_scan_chunks<1> : k_scan_chunks<kMaxChunksPerThread>;
-  launch(scan, dim3(M, 1), 1024, 0, s, M, n_chunks, w.partA, w.partW);
-  launch(k_occ_apply, g, kThreads, 0, s, M, K, L, n_chunks, win, w.dA, w.dW, w.partA, w.partW,
-         reinterpret_cast<long long*>(A_ms), reinterpret_cast<long long*>(W_ms));
+  scan<<<dim3(M, 1), 1024, 0, s>>>(M, n_chunks, w.partA, w.partW);
+  k_occ_apply<<<g, kThreads, 0, s>>>(M, K, L, n_chunks, win, w.dA, w.dW, w.partA, w.partW,
+                                     reinterpret_cast<long long*>(A_ms),
+                                     reinterpret_cast<long long*>(W_ms));
   return cudaGetLastError();
 }
 
@@ -1779,9 +1767,11 @@ cudaError_t launch_occupancy_mean(const ReqCols& r, int M, int win, int K, Reduc
     if (e) return e;
     if (smem > 96 * 1024) return cudaErrorInvalidValue;
     const unsigned ctas = (unsigned)((r.n + kOccPerCta - 1) / kOccPerCta);
-    launch(k_occ_staged, ctas, kThreads, smem, s, r, vec, stage, M, lgMp, win, FastDiv(win), K,
-           near_rows, lgF, reinterpret_cast<unsigned long long*>(A_ms),
-           reinterpret_cast<unsigned long long*>(W_ms), w.dA, w.dW);
+    k_occ_staged<<<ctas, kThreads, smem, s>>>(r, vec, stage, M, lgMp, win, FastDiv(win), K,
+                                              near_rows, lgF,
+                                              reinterpret_cast<unsigned long long*>(A_ms),
+                                              reinterpret_cast<unsigned long long*>(W_ms), w.dA,
+                                              w.dW);
   }
   return occ_finish(M, win, K, w, A_ms, W_ms, s);
 }
@@ -1796,9 +1786,10 @@ cudaError_t launch_occupancy_mean_events(const EvCols& ev, int M, int win, int K
   if (!e) e = cudaMemsetAsync(w.dW, 0, cells1 * sizeof(int32_t), s);
   if (e) return e;
   if (ev.n_req > 0) {
-    launch(k_occ_events, grid_for(ev.n_req, 4), kThreads, 0, s, ev, M, win, FastDiv(win), K,
-           w.first, w.last, reinterpret_cast<unsigned long long*>(A_ms),
-           reinterpret_cast<unsigned long long*>(W_ms), w.dA, w.dW);
+    k_occ_events<<<grid_for(ev.n_req, 4), kThreads, 0, s>>>(
+        ev, M, win, FastDiv(win), K, w.first, w.last,
+        reinterpret_cast<unsigned long long*>(A_ms), reinterpret_cast<unsigned long long*>(W_ms),
+        w.dA, w.dW);
     if ((e = cudaGetLastError())) return e;
   }
   return occ_finish(M, win, K, w, A_ms, W_ms, s);
@@ -1808,9 +1799,9 @@ cudaError_t launch_gauge_prefix(const GaugePlan& gp, ReduceWs& w, cudaStream_t s
   if (gp.n_traces > w.n_traces || (int64_t)gp.nblk * gp.M > w.part_cap) return cudaErrorInvalidValue;
   const int64_t n = (int64_t)gp.n_traces * gp.nblk * gp.M;
   if (n == 0) return cudaSuccess;
-  launch(k_gauge_blocks, (unsigned)((n + kThreads - 1) / kThreads), kThreads, 0, s, gp, w.dA, w.dW,
-         w.partA, w.partW);
-  launch(k_gauge_block_scan, gp.n_traces * gp.M, kThreads, 0, s, gp, w.partA, w.partW);
+  k_gauge_blocks<<<(unsigned)((n + kThreads - 1) / kThreads), kThreads, 0, s>>>(gp, w.dA, w.dW,
+                                                                                w.partA, w.partW);
+  k_gauge_block_scan<<<gp.n_traces * gp.M, kThreads, 0, s>>>(gp, w.partA, w.partW);
   return cudaGetLastError();
 }
 
@@ -1822,11 +1813,11 @@ cudaError_t launch_gauge_apply(const GaugePlan& gp, ReduceWs& w, const int32_t* 
   if (n == 0) return cudaSuccess;
   const unsigned g = (unsigned)((n + kThreads - 1) / kThreads);
   if (gp.n_win <= 4)
-    launch(k_gauge_apply<4>, g, kThreads, 0, s, gp, w.dA, w.dW, w.partA, w.partW, Pin, Din, sloin,
-           P, D, A, W, slo);
+    k_gauge_apply<4><<<g, kThreads, 0, s>>>(gp, w.dA, w.dW, w.partA, w.partW, Pin, Din, sloin,
+                                            P, D, A, W, slo);
   else
-    launch(k_gauge_apply<kGaugeMaxWin>, g, kThreads, 0, s, gp, w.dA, w.dW, w.partA, w.partW, Pin,
-           Din, sloin, P, D, A, W, slo);
+    k_gauge_apply<kGaugeMaxWin><<<g, kThreads, 0, s>>>(gp, w.dA, w.dW, w.partA, w.partW, Pin, Din,
+                                                       sloin, P, D, A, W, slo);
   return cudaGetLastError();
 }
 
@@ -1838,7 +1829,7 @@ cudaError_t launch_aggregate(const AggPlan& pl, const int32_t* P, const int32_t*
   for (int w = 0; w < pl.n_win; ++w) mx = std::max<int64_t>(mx, (int64_t)pl.Kq[w] * pl.M);
   if (mx == 0) return cudaSuccess;
   dim3 g(grid_for(mx), pl.n_win, pl.n_traces);
-  launch(k_aggregate, g, kThreads, 0, s, pl, P, D, A, W, slo, Pq, Dq, Aq, Wq, sloq);
+  k_aggregate<<<g, kThreads, 0, s>>>(pl, P, D, A, W, slo, Pq, Dq, Aq, Wq, sloq);
   return cudaGetLastError();
 }
 

@@ -57,7 +57,6 @@ constexpr int kGroupBlock = 1024;
 __global__ void __launch_bounds__(kGroupBlock)
 k_rp_valid(ReplayLatent lat, int M, FastDiv fwin, int64_t span, int8_t* __restrict__ vm,
            int32_t* __restrict__ arr_cnt, int32_t* __restrict__ blk_cnt) {
-  begin_after_previous();
   __shared__ int32_t cnt[64];
   if (threadIdx.x < M) cnt[threadIdx.x] = 0;
   __syncthreads();
@@ -81,7 +80,6 @@ k_rp_valid(ReplayLatent lat, int M, FastDiv fwin, int64_t span, int8_t* __restri
 // its block counts, then the models' offsets in the grouped order
 __global__ void __launch_bounds__(1024)
 k_rp_offsets(int M, int n_blk, int32_t* __restrict__ blk_cnt, int32_t* __restrict__ base) {
-  begin_after_previous();
   __shared__ int32_t total[64];
   const int lane = threadIdx.x & 31;
   for (int m = threadIdx.x >> 5; m < M; m += 32) {
@@ -117,7 +115,6 @@ __global__ void __launch_bounds__(kGroupBlock)
 k_rp_group(ReplayLatent lat, int M, const int8_t* __restrict__ vm,
            const int32_t* __restrict__ blk_off, const int32_t* __restrict__ base,
            int4* __restrict__ g) {
-  begin_after_previous();
   __shared__ int32_t wcnt[kGroupBlock / 32][64];
   const int64_t i = (int64_t)blockIdx.x * kGroupBlock + threadIdx.x;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -138,7 +135,6 @@ k_rp_group(ReplayLatent lat, int M, const int8_t* __restrict__ vm,
 // served records start as "not started" (K*win) or "not served" (-1)
 __global__ void k_rp_init_records(int64_t n, int n_inst, int32_t span, const int8_t* __restrict__ vm,
                                   int32_t* ts, int32_t* tf, int32_t* te) {
-  begin_after_previous();
   const int64_t total = n * n_inst;
   for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total;
        x += (int64_t)gridDim.x * blockDim.x) {
@@ -385,7 +381,6 @@ __device__ __forceinline__ void pair_sync(int pair) {
 template <class T, bool PAIR>
 __global__ void __launch_bounds__(32 * kMaxWarps)
 k_replay(const __grid_constant__ ReplayBatch<T> b) {
-  begin_after_previous();
   extern __shared__ __align__(16) unsigned char rsm[];
   __shared__ uint32_t s_batch[PAIR ? kMaxPairs : 1][2][32];   // start times
   __shared__ int32_t s_more[PAIR ? kMaxPairs : 1][2];         // a batch follows
@@ -910,23 +905,22 @@ template <class T> cudaError_t launch_replay(ReplayBatch<T>& b, ReplayWs& w, cud
   if (e) return e;
   const FastDiv fwin((uint32_t)b.win);
   if (w.n_blk > 0)
-    launch(k_rp_valid, w.n_blk, kGroupBlock, 0, s, b.lat, M, fwin, (int64_t)K * b.win, w.vm,
-           w.arr_cnt, w.blk_cnt);
-  launch(k_rp_offsets, 1, 1024, 0, s, M, w.n_blk, w.blk_cnt, w.base);
+    k_rp_valid<<<w.n_blk, kGroupBlock, 0, s>>>(b.lat, M, fwin, (int64_t)K * b.win, w.vm, w.arr_cnt,
+                                               w.blk_cnt);
+  k_rp_offsets<<<1, 1024, 0, s>>>(M, w.n_blk, w.blk_cnt, w.base);
   if (w.n_blk > 0)
-    launch(k_rp_group, w.n_blk, kGroupBlock, 0, s, b.lat, M, w.vm, w.blk_cnt, w.base, w.grp);
+    k_rp_group<<<w.n_blk, kGroupBlock, 0, s>>>(b.lat, M, w.vm, w.blk_cnt, w.base, w.grp);
   if ((e = cudaGetLastError())) return e;
   if (b.o_ts && b.lat.n > 0) {
-    launch(k_rp_init_records, (unsigned)device_sm_count() * 8, 256, 0, s, b.lat.n, b.n_inst,
-           (int32_t)(K * b.win), w.vm, b.o_ts, b.o_tf, b.o_te);
+    k_rp_init_records<<<(unsigned)device_sm_count() * 8, 256, 0, s>>>(
+        b.lat.n, b.n_inst, (int32_t)(K * b.win), w.vm, b.o_ts, b.o_tf, b.o_te);
     if ((e = cudaGetLastError())) return e;
   }
   // two warps a model while their barriers and the block's warps suffice
   const bool pair = M <= kMaxPairs;
   auto f = pair ? k_replay<T, true> : k_replay<T, false>;
   if ((e = func_smem_once((const void*)f, (int)kReplaySmemMax, false))) return e;
-  launch(f, (unsigned)b.n_inst, pair ? 64 * M : 32 * std::min(M, kMaxWarps), (size_t)b.smem_bytes,
-         s, b);
+  f<<<(unsigned)b.n_inst, pair ? 64 * M : 32 * std::min(M, kMaxWarps), (size_t)b.smem_bytes, s>>>(b);
   return cudaGetLastError();
 }
 

@@ -150,7 +150,6 @@ __global__ void __launch_bounds__(kEwThreads)
 k_raw(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ TilePlan tp, FastDiv fm,
       bool vec, bool vec_w, Counts c0, Counts c1, const T* __restrict__ w_p, const T* __restrict__ w_q,
       T* __restrict__ raw, uint8_t* __restrict__ cls) {
-  begin_after_previous();
   const int s = prefix_index(tp.tile_base, tab.n, blockIdx.x);
   const int M = tab.M;
   const int64_t n = (int64_t)tab.K[s] * M;
@@ -341,7 +340,6 @@ template <class T>
 __global__ void __launch_bounds__(256)
 k_active(const __grid_constant__ SeriesTable<T> tab, FastDiv fm, const uint8_t* __restrict__ cls,
          int32_t* __restrict__ active) {
-  begin_after_previous();
   extern __shared__ int32_t s_idle[];
   const int seg = blockIdx.x;
   const int s = series_of_seg(tab, seg);
@@ -471,7 +469,6 @@ k_ema(const __grid_constant__ SeriesTable<T> tab, const T* __restrict__ raw, con
       const T* S_carry, const uint8_t* init_carry, const int32_t* __restrict__ active,
       T* __restrict__ b_S, int32_t* __restrict__ b_init, T* __restrict__ e_S,
       int32_t* __restrict__ e_init, T* __restrict__ S_out) {
-  begin_after_previous();
   extern __shared__ __align__(16) unsigned char ema_smem[];
   constexpr int V = Windows<T>::V, kStage = kGroup / V * kChains;
   Windows<T>* inb = reinterpret_cast<Windows<T>*>(ema_smem);    // [kLoaders] stages of inputs
@@ -696,7 +693,6 @@ __global__ void __launch_bounds__(kResolveThreads)
 k_resolve(const __grid_constant__ SeriesTable<T> tab, const T* __restrict__ raw, const T* alpha,
           const T* start_S, const int32_t* start_init, T* end_S, int32_t* end_init, T* S_out,
           const uint8_t* __restrict__ cls, T* S_carry, uint8_t* init_carry, tre_diag* diag) {
-  begin_after_previous();
   const int M = tab.M;
   const int lane = threadIdx.x & 31;
   const int s = blockIdx.x / M, m = blockIdx.x % M;
@@ -822,7 +818,6 @@ __global__ void __launch_bounds__(kEwThreads)
 k_normalize(const __grid_constant__ SeriesTable<T> tab, const __grid_constant__ TilePlan tp,
             FastDiv fm, bool vec, const T* S, const uint8_t* idle_cls, const T* theta,
             const T* tau_crit, T tau_crit_v, const T* tau_surp, T* Z, uint8_t* cls) {
-  begin_after_previous();
   const int s = prefix_index(tp.tile_base, tab.n, blockIdx.x);
   const int M = tab.M;
   const int64_t n = (int64_t)tab.K[s] * M;
@@ -890,7 +885,6 @@ k_norm_recv(int M, int K, int wt, FastDiv fm, bool vec, const T* __restrict__ S,
             const uint8_t* idle_cls, const T* __restrict__ theta, const T* __restrict__ tau_crit,
             const T* __restrict__ tau_surp, T* __restrict__ Z, uint8_t* cls,
             int32_t* __restrict__ recv) {
-  begin_after_previous();
   __shared__ T zs[2 * kNormCells];                     // [wt][M + 1]
   __shared__ uint8_t on[2 * kNormCells];               // not idle
   const int k0 = (int)min64((int64_t)blockIdx.x * wt, K);
@@ -954,7 +948,6 @@ k_norm_quads(int M, int lg_quads, int64_t n_quads, const T* __restrict__ S, cons
              const T* __restrict__ theta, const T* __restrict__ tau_crit,
              const T* __restrict__ tau_surp, T* __restrict__ Z, uint8_t* cls,
              int32_t* __restrict__ recv) {
-  begin_after_previous();
   constexpr int U = kNormQuadPasses<T>;
   const unsigned full = 0xffffffffu;
   const int64_t q0 = (int64_t)blockIdx.x * (kEwThreads * U) + threadIdx.x;
@@ -1041,7 +1034,6 @@ __device__ __forceinline__ bool donor_key_less(int ga, T za, int ia, int gb, T z
 template <class T>
 __global__ void k_rank(int M, int K, const T* Z, const uint8_t* cls, int32_t* recv,
                        int32_t* donors) {
-  begin_after_previous();
   const int64_t k = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   if (k >= K) return;
   const int lane = threadIdx.x & 31;
@@ -1168,7 +1160,6 @@ template <class T, int MMAX, bool QUAD>
 __global__ void __launch_bounds__(256)
 k_rank_small(int M, int K, const T* __restrict__ Z, const uint8_t* __restrict__ cls,
              int32_t* __restrict__ recv, int32_t* __restrict__ donors, bool store4) {
-  begin_after_previous();
   static_assert(MMAX <= 16 && kRankDonors <= 8, "four bits a place, places in one word");
   static_assert(kCrit < 4 && kNom < 4 && kSurp < 4 && kIdle < 4, "two bits a region");
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1358,15 +1349,17 @@ static cudaError_t smooth(const SeriesTable<T>& tab, const T* alpha, T* S_carry,
   // extra pass over the classes is small beside the smoothing
   const int32_t* active = nullptr;
   if (total_elems(tab) >= kActiveMinCells) {
-    launch(k_active<T>, n_seg, 256, (size_t)M * sizeof(int32_t), s, tab, FastDiv(M), cls, w.active);
+    k_active<T><<<n_seg, 256, (size_t)M * sizeof(int32_t), s>>>(tab, FastDiv(M), cls, w.active);
     active = w.active;
   }
   cudaError_t e = func_smem_once((const void*)k_ema<T>, ema_smem_bytes<T>(), false);
   if (e) return e;
-  launch(k_ema<T>, g, kEmaThreads, ema_smem_bytes<T>(), s, tab, w.raw, alpha, S_carry, init_carry,
-         active, w.start_S, w.start_init, w.end_S, w.end_init, S);
-  launch(k_resolve<T>, tab.n * M, kResolveThreads, 0, s, tab, w.raw, alpha, w.start_S, w.start_init,
-         w.end_S, w.end_init, S, cls, S_carry, init_carry, diag);
+  k_ema<T><<<g, kEmaThreads, ema_smem_bytes<T>(), s>>>(tab, w.raw, alpha, S_carry, init_carry,
+                                                       active, w.start_S, w.start_init, w.end_S,
+                                                       w.end_init, S);
+  k_resolve<T><<<tab.n * M, kResolveThreads, 0, s>>>(tab, w.raw, alpha, w.start_S, w.start_init,
+                                                     w.end_S, w.end_init, S, cls, S_carry,
+                                                     init_carry, diag);
   return cudaGetLastError();
 }
 
@@ -1390,11 +1383,11 @@ cudaError_t launch_score(const SeriesTable<T>& tab, const int32_t* P, const int3
   if (A_ms) {
     const bool vec = quad_aligned(tab, {P, D, A_ms, W_ms, w.raw, cls});
     auto f = small ? k_raw<T, true, 1, false> : k_raw<T, true, 4, false>;
-    launch(f, n_tiles, th, 0, s, tab, tp, FastDiv(M), vec, vec_w, c, c, w_p, w_q, w.raw, cls);
+    f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(M), vec, vec_w, c, c, w_p, w_q, w.raw, cls);
   } else {
     const bool vec = quad_aligned(tab, {P, D, A, W, w.raw, cls});
     auto f = small ? k_raw<T, false, 1, false> : k_raw<T, false, 4, false>;
-    launch(f, n_tiles, th, 0, s, tab, tp, FastDiv(M), vec, vec_w, c, c, w_p, w_q, w.raw, cls);
+    f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(M), vec, vec_w, c, c, w_p, w_q, w.raw, cls);
   }
   const cudaError_t e = smooth<T>(tab, alpha, S_carry, init_carry, S, cls, w, diag, s);
   if (e) return e;
@@ -1423,7 +1416,7 @@ cudaError_t launch_score_stages(const SeriesTable<T>& tab, const int32_t* P, con
   const bool vec = quad_aligned(tab, {P, D, W, A_pre, A_dec, w.raw, cls});
   const bool vec_w = weights_aligned(tab.M, w_p, w_q);
   auto f = small ? k_raw<T, false, 1, true> : k_raw<T, false, 4, true>;
-  launch(f, n_tiles, th, 0, s, tab, tp, FastDiv(tab.M), vec, vec_w, pre, dec, w_p, w_q, w.raw, cls);
+  f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(tab.M), vec, vec_w, pre, dec, w_p, w_q, w.raw, cls);
   return smooth<T>(tab, alpha, nullptr, nullptr, S, cls, w, diag, s);
 }
 
@@ -1433,7 +1426,6 @@ __global__ void __launch_bounds__(kSmallThreads)
 k_norm_stages(const __grid_constant__ SeriesTable<T> tab, FastDiv fm, const T* __restrict__ S,
               const uint8_t* __restrict__ idle_cls, const T* __restrict__ tau_crit,
               const T* __restrict__ tau_surp, StageOut<T> o0, StageOut<T> o1) {
-  begin_after_previous();
   const StageOut<T> o = blockIdx.y ? o1 : o0;
   const int M = tab.M;
   const int64_t n = (int64_t)tab.K[0] * M, off = tab.off[blockIdx.y];
@@ -1456,8 +1448,8 @@ cudaError_t launch_norm_stages(const SeriesTable<T>& tab, const T* S, const uint
   if (n == 0) return cudaSuccess;
   const int64_t b = std::min<int64_t>((n + kSmallThreads - 1) / kSmallThreads,
                                       (int64_t)device_sm_count() * 16);
-  launch(k_norm_stages<T>, dim3((unsigned)b, 2), kSmallThreads, 0, s, tab, FastDiv(tab.M), S,
-         idle_cls, tau_crit, tau_surp, pre, dec);
+  k_norm_stages<T><<<dim3((unsigned)b, 2), kSmallThreads, 0, s>>>(
+      tab, FastDiv(tab.M), S, idle_cls, tau_crit, tau_surp, pre, dec);
   return cudaGetLastError();
 }
 
@@ -1477,21 +1469,22 @@ cudaError_t launch_normalize(const SeriesTable<T>& tab, const T* S, const uint8_
     if (vec && !small && M == 4 << lg_quads) {
       constexpr int kPerCta = kEwThreads * kNormQuadPasses<T>;
       const int64_t n_quads = (int64_t)K << lg_quads;
-      launch(k_norm_quads<T>, (unsigned)((n_quads + kPerCta - 1) / kPerCta), kEwThreads, 0, s, M,
-             lg_quads, n_quads, S, idle_cls, theta, tau_crit, tau_surp, Z, cls, recv);
+      k_norm_quads<T><<<(unsigned)((n_quads + kPerCta - 1) / kPerCta), kEwThreads, 0, s>>>(
+          M, lg_quads, n_quads, S, idle_cls, theta, tau_crit, tau_surp, Z, cls, recv);
       return cudaGetLastError();
     }
     const int wt = std::max(1, (small ? th : kNormCells) / M);
-    launch(k_norm_recv<T>, (unsigned)((K + wt - 1) / wt), th, 0, s, M, K, wt, FastDiv(M),
-           vec && !small && M % 4 == 0, S, idle_cls, theta, tau_crit, tau_surp, Z, cls, recv);
+    k_norm_recv<T><<<(unsigned)((K + wt - 1) / wt), th, 0, s>>>(
+        M, K, wt, FastDiv(M), vec && !small && M % 4 == 0, S, idle_cls, theta, tau_crit, tau_surp,
+        Z, cls, recv);
     return cudaGetLastError();
   }
   int n_tiles = 0;
   const int th = small ? kSmallThreads : kEwThreads;
   const TilePlan tp = tile_plan(tab, small ? th : 4 * th, n_tiles);
   auto f = small ? k_normalize<T, 1> : k_normalize<T, 4>;
-  launch(f, n_tiles, th, 0, s, tab, tp, FastDiv(tab.M), vec, S, idle_cls, theta, tau_crit,
-         tau_crit_v, tau_surp, Z, cls);
+  f<<<n_tiles, th, 0, s>>>(tab, tp, FastDiv(tab.M), vec, S, idle_cls, theta, tau_crit, tau_crit_v,
+                           tau_surp, Z, cls);
   return cudaGetLastError();
 }
 
@@ -1505,10 +1498,10 @@ cudaError_t launch_rank(int M, int K, const T* Z, const uint8_t* cls, int32_t* r
   if (M <= 16) {
     auto f = M <= 8 ? (quad ? k_rank_small<T, 8, true> : k_rank_small<T, 8, false>)
                     : (quad ? k_rank_small<T, 16, true> : k_rank_small<T, 16, false>);
-    launch(f, thread_blocks, 256, 0, s, M, K, Z, cls, recv, donors, store4);
+    f<<<thread_blocks, 256, 0, s>>>(M, K, Z, cls, recv, donors, store4);
   }
   else
-    launch(k_rank<T>, (unsigned)((K + 7) / 8), 256, 0, s, M, K, Z, cls, recv, donors);
+    k_rank<T><<<(unsigned)((K + 7) / 8), 256, 0, s>>>(M, K, Z, cls, recv, donors);
   return cudaGetLastError();
 }
 

@@ -65,7 +65,6 @@ template <class T>
 __global__ void __launch_bounds__(256)
 k_tick_rank(const __grid_constant__ WalkBatch<T> b, int16_t* recv_out, int16_t* ndon_out,
             uint16_t* rank, uint16_t* order, unsigned long long* dm64) {
-  begin_after_previous();
   const int M = b.M;
   const int64_t gid = (int64_t)blockIdx.x * 256 + threadIdx.x;
   const int64_t total_ent = (int64_t)b.ent_base[b.n_series] * b.n_tau;
@@ -265,7 +264,6 @@ __global__ void __launch_bounds__(128)
 k_tick_rank_small(const __grid_constant__ WalkBatch<T> b, int16_t* recv_out, int16_t* ndon_out,
                   uint16_t* rank, uint16_t* order, unsigned long long* packed, uint32_t* dmask,
                   bool need_rank, unsigned long long* dm64) {
-  begin_after_previous();
   const int M = b.M;
   const int64_t e = (int64_t)blockIdx.x * 128 + threadIdx.x;
   if (e >= (int64_t)b.ent_base[b.n_series] * b.n_tau) return;
@@ -335,7 +333,6 @@ template <class T, int MPL, bool STAGED>
 __global__ void __launch_bounds__(kCapWarps * 32)
 k_walk(const __grid_constant__ WalkBatch<T> b, const int16_t* recv_tab, const int16_t* ndon_tab,
        const uint16_t* rank, const uint16_t* order, const unsigned long long* dm64) {
-  begin_after_previous();
   extern __shared__ __align__(16) unsigned char dyn[];
   const int grp = blockIdx.x;                       // (series, tau)
   const int ti = grp % b.n_tau;
@@ -608,7 +605,6 @@ template <class T, int MMAX>
 __global__ void __launch_bounds__(32)
 k_walk_thread(const __grid_constant__ WalkBatch<T> b, const int16_t* recv_tab,
               const unsigned long long* packed, const uint32_t* dmask) {
-  begin_after_previous();
   extern __shared__ __align__(16) unsigned char dyn[];
   const int grp = blockIdx.x;
   const int ti = grp % b.n_tau;
@@ -937,7 +933,6 @@ template <class T, int MP, bool QUAD>
 __global__ void __launch_bounds__(kChunk)
 k_tick_rows(const __grid_constant__ WalkBatch<T> b, void* __restrict__ rows,
             uint8_t* __restrict__ recs, uint8_t* __restrict__ nexts) {
-  begin_after_previous();
   __shared__ uint8_t s_rank[kChunk][MP];
   __shared__ uint8_t s_rec[kChunk];
   const int M = b.M;
@@ -1031,7 +1026,6 @@ template <class T, int MP>
 __global__ void __launch_bounds__(kWideThreads)
 k_tick_rows_wide(const __grid_constant__ WalkBatch<T> b, void* __restrict__ rows,
                  uint8_t* __restrict__ recs, uint8_t* __restrict__ nexts) {
-  begin_after_previous();
   constexpr int MPL = MP / 32;
   __shared__ uint8_t s_rank[kChunk][MP];
   __shared__ uint8_t s_rec[kChunk];
@@ -1176,7 +1170,6 @@ __device__ __forceinline__ void copy16(void* smem, const void* gmem) {
 template <int MP>
 __global__ void __launch_bounds__(kLaneThreads)
 k_walk_lane(const __grid_constant__ LaneWalk w) {
-  begin_after_previous();
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ uint32_t s_log[kLaneThreads / 32][kLaneLog];
   __shared__ int s_foot[64];
@@ -1487,9 +1480,9 @@ cudaError_t walk_launch(const WalkBatch<T>& b, WalkWs& w, cudaStream_t s) {
   if (smem <= kStageMax) {
     cudaError_t e = func_smem_once((const void*)k_walk<T, MPL, true>, (int)kStageMax, false);
     if (e) return e;
-    launch(k_walk<T, MPL, true>, grid, th, smem, s, b, w.recv, w.n_donor, w.rank, w.order, w.dm64);
+    k_walk<T, MPL, true><<<grid, th, smem, s>>>(b, w.recv, w.n_donor, w.rank, w.order, w.dm64);
   } else {
-    launch(k_walk<T, MPL, false>, grid, th, 0, s, b, w.recv, w.n_donor, w.rank, w.order, w.dm64);
+    k_walk<T, MPL, false><<<grid, th, 0, s>>>(b, w.recv, w.n_donor, w.rank, w.order, w.dm64);
   }
   return cudaGetLastError();
 }
@@ -1515,14 +1508,12 @@ cudaError_t lane_launch(const WalkBatch<T>& b, const WalkWs& w, cudaStream_t s, 
       // rows start on 16-byte boundaries when M is a multiple of 4 (series
       // offsets are multiples of M) and both arrays are 16-byte aligned
       if (b.M % 4 == 0 && (((uintptr_t)b.Z | (uintptr_t)b.cls) & 15) == 0)
-        launch(k_tick_rows<T, MP, true>, (unsigned)chunks, kChunk, 0, s, b, w.rows, w.recs,
-               w.nexts);
+        k_tick_rows<T, MP, true><<<(unsigned)chunks, kChunk, 0, s>>>(b, w.rows, w.recs, w.nexts);
       else
-        launch(k_tick_rows<T, MP, false>, (unsigned)chunks, kChunk, 0, s, b, w.rows, w.recs,
-               w.nexts);
+        k_tick_rows<T, MP, false><<<(unsigned)chunks, kChunk, 0, s>>>(b, w.rows, w.recs, w.nexts);
     } else {
-      launch(k_tick_rows_wide<T, MP>, (unsigned)chunks, kWideThreads, 0, s, b, w.rows, w.recs,
-             w.nexts);
+      k_tick_rows_wide<T, MP><<<(unsigned)chunks, kWideThreads, 0, s>>>(b, w.rows, w.recs,
+                                                                        w.nexts);
     }
     if (launches) ++*launches;
   }
@@ -1563,7 +1554,7 @@ cudaError_t lane_launch(const WalkBatch<T>& b, const WalkWs& w, cudaStream_t s, 
   if (e) return e;
   const dim3 grid((unsigned)(b.n_series * b.n_tau),
                   (unsigned)((b.n_cap + kLaneThreads / 32 - 1) / (kLaneThreads / 32)));
-  launch(k_walk_lane<MP>, grid, kLaneThreads, (size_t)slab_bytes<MP>(v.slab) * v.n_buf, s, v);
+  k_walk_lane<MP><<<grid, kLaneThreads, (size_t)slab_bytes<MP>(v.slab) * v.n_buf, s>>>(v);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
@@ -1572,7 +1563,7 @@ template <class T, int MMAX>
 cudaError_t walk_thread_launch(const WalkBatch<T>& b, WalkWs& w, size_t smem, cudaStream_t s) {
   cudaError_t e = func_smem_once((const void*)k_walk_thread<T, MMAX>, (int)kStageMax, false);
   if (e) return e;
-  launch(k_walk_thread<T, MMAX>, b.n_series * b.n_tau, 32, smem, s, b, w.recv, w.packed, w.dmask);
+  k_walk_thread<T, MMAX><<<b.n_series * b.n_tau, 32, smem, s>>>(b, w.recv, w.packed, w.dmask);
   return cudaGetLastError();
 }
 
@@ -1632,18 +1623,18 @@ cudaError_t launch_walk(const WalkBatch<T>& b, WalkWs& w, cudaStream_t s, int* l
   if (ents > 0) {
     const unsigned g = (unsigned)((ents + 127) / 128);
     if (b.M <= 8) {
-      launch(k_tick_rank_small<T, 8>, g, 128, 0, s, b, w.recv, w.n_donor, w.rank, w.order, w.packed,
-             w.dmask, !thread_walk, w.dm64);
+      k_tick_rank_small<T, 8><<<g, 128, 0, s>>>(b, w.recv, w.n_donor, w.rank, w.order, w.packed,
+                                                w.dmask, !thread_walk, w.dm64);
     } else if (b.M <= 16) {
-      launch(k_tick_rank_small<T, 16>, g, 128, 0, s, b, w.recv, w.n_donor, w.rank, w.order,
-             w.packed, w.dmask, !thread_walk, w.dm64);
+      k_tick_rank_small<T, 16><<<g, 128, 0, s>>>(b, w.recv, w.n_donor, w.rank, w.order,
+                                                 w.packed, w.dmask, !thread_walk, w.dm64);
     } else if (b.M <= 32) {
-      launch(k_tick_rank_small<T, 32>, g, 128, 0, s, b, w.recv, w.n_donor, w.rank, w.order,
-             w.packed, w.dmask, true, w.dm64);
+      k_tick_rank_small<T, 32><<<g, 128, 0, s>>>(b, w.recv, w.n_donor, w.rank, w.order,
+                                                 w.packed, w.dmask, true, w.dm64);
     } else {
       const int64_t th = ents * b.M;
-      launch(k_tick_rank<T>, (unsigned)((th + 255) / 256), 256, 0, s, b, w.recv, w.n_donor, w.rank,
-             w.order, w.dm64);
+      k_tick_rank<T><<<(unsigned)((th + 255) / 256), 256, 0, s>>>(b, w.recv, w.n_donor, w.rank,
+                                                                   w.order, w.dm64);
     }
   }
   if (thread_walk)

@@ -31,7 +31,6 @@ k_stage_requests(ReqCols r, int M, int win, FastDiv fd, int K, int32_t* __restri
                  int32_t* __restrict__ dDec, unsigned long long* __restrict__ ttft,
                  unsigned long long* __restrict__ tpot, const int32_t* __restrict__ ttft_ms,
                  const int32_t* __restrict__ tpot_ms) {
-  begin_after_previous();
   const int64_t span = (int64_t)K * win;
   for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < r.n;
        i += (int64_t)gridDim.x * kThreads) {
@@ -88,8 +87,8 @@ cudaError_t launch_stage_requests(const ReqCols& r, int M, int win, int K, int32
     if (e) return e;
   }
   if (r.n == 0) return cudaSuccess;
-  launch(k_stage_requests, grid_of(r.n), kThreads, 0, s, r, M, win, FastDiv(win), K, dPre, dDec,
-         ttft, tpot, ttft_ms, tpot_ms);
+  k_stage_requests<<<grid_of(r.n), kThreads, 0, s>>>(r, M, win, FastDiv(win), K, dPre, dDec,
+                                                      ttft, tpot, ttft_ms, tpot_ms);
   return cudaGetLastError();
 }
 
