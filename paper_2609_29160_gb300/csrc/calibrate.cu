@@ -580,7 +580,6 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
     // where the buckets' keys go: this CTA's copy of the table, the first one's list
     int32_t* place = fhl;
     U* keep = list;
-    U* low = &bfmin_s;
     if constexpr (CL > 1) {
       const cg::cluster_group cl = cg::this_cluster();
       cl.sync();
@@ -591,7 +590,6 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
         bf = cl.map_shared_rank(plan_s, 0)[1];
         place = cl.map_shared_rank(fhl, 0);
         keep = cl.map_shared_rank(list, 0);
-        low = cl.map_shared_rank(&bfmin_s, 0);
       }
       cl.sync();                    // the first CTA may end from here on unless keys are listed
     }
@@ -604,9 +602,18 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
           if (st >= 0) keep[st + atomicAdd(&place[b], 1)] = p;
           if (b == bf && (p >> 1) < lmin) lmin = p >> 1;
         });
-        if (lmin != ~(U)0) atomicMin(low, lmin);
+        if (lmin != ~(U)0) atomicMin(&bfmin_s, lmin);
         if constexpr (CL > 1) {
-          cg::this_cluster().sync();
+          // each CTA's smallest is its own until all have it: a 64-bit minimum in
+          // another CTA's memory is not atomic with those of that CTA
+          const cg::cluster_group cl = cg::this_cluster();
+          cl.sync();
+          if (rank == 0 && tid == 0)
+            for (int r = 1; r < CL; ++r) {
+              const U v = *cl.map_shared_rank(&bfmin_s, r);
+              if (v < bfmin_s) bfmin_s = v;
+            }
+          cl.sync();
           if (rank > 0) return;
         }
         __syncthreads();
