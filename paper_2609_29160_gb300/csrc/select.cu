@@ -1268,12 +1268,14 @@ k_walk_lane(const __grid_constant__ LaneWalk w) {
       n_out += n_log;
       n_log = 0;
     };
+    // between two appends the log is never full: either one flushes it before or as
+    // it fills (a run is at most 255 moves, so an empty log takes any)
     auto log_one = [&](bool here, uint32_t a, int seq, int donor) {
       if (here) log[n_log] = a | (uint32_t)seq << 11 | (uint32_t)donor << 19;
       if (++n_log == kLaneLog) flush();
     };
     auto log_run = [&](uint32_t a, int seq, int donor, int take) {   // take <= 255
-      if (n_log + take > kLaneLog) flush();
+      if (n_log + take >= kLaneLog) flush();
       for (int q = lane; q < take; q += 32)
         log[n_log + q] = a | (uint32_t)(seq + q) << 11 | (uint32_t)donor << 19;
       n_log += take;

@@ -197,3 +197,38 @@ def test_lane_walk_chunk_and_slab_edges(tre, M, ticks, hetero, cap):
         Z[rng.random(Z.shape) < 0.04] = v
     budget += 2
     _check(tre, Z, cls, g, r0, budget, r_min, 1000, cap, 1000, 2000)
+
+
+# A warp logs 256 moves before it writes them out. Idle pools of whole multiples
+# of that, and one fewer and more, are drawn on one a tick within the first slab of
+# staged ticks (1024 for 8 models, 384 for 40), with donors' moves behind them;
+# the caps' warps lie side by side, cap 1 in the first or in the last of a block.
+@pytest.mark.parametrize("caps", [[1, 2, 3, 4, 5, 6, 7, 8], [2, 3, 4, 5, 6, 7, 8, 1]])
+@pytest.mark.parametrize("M,pool", [(8, 255), (8, 256), (8, 257), (8, 512), (40, 255), (40, 256)])
+def test_lane_walk_full_log(tre, M, pool, caps):
+    import torch
+    import tracegen
+    sw = tracegen.sweep_workload(scale=0.02, n_traces=1, duration_s=200.0)
+    t = sw["traces"][0]
+    more = np.random.default_rng(8).integers(0, M // 8, len(t["model"]))
+    t["model"] = (t["model"] + 8 * more).astype(np.int32)
+    r0, r_min, foot, slo = (np.resize(sw[k], M).astype(np.int32)
+                            for k in ("r0", "r_min", "footprint", "slo_ttft_ms"))
+    args = (M, sw["duration_ms"])
+    rest = (sw["w_p"], sw["w_q"], sw["tau_surplus"])
+    ctrl = (int(r0.sum()) + pool, r0, r_min, foot)
+    ref = oracle.sweep(sw["traces"], *args, [100], [0.8], caps, *rest, [0.02], slo, *ctrl,
+                       fast_ms=100, slow_ms=100)["instances"]
+    first = ref[caps.index(1)]["moves"]
+    drawn = first["donor"] < 0
+    slab = 1024 if M <= 16 else 384
+    assert drawn.sum() == pool and ((first["window"] < slab) & ~drawn).sum() > 100
+    out = tre.tre_sweep([{k: torch.as_tensor(v).cuda() for k, v in t.items()}], *args, [100],
+                        [0.02], [0.8], caps, *rest, slo, *ctrl, fast_ms=100, slow_ms=100,
+                        moves_cap=4096)
+    moves = tre.sweep_moves(out, len(ref), 4096)
+    for i, inst in enumerate(ref):
+        assert int(_np(out["n_moves"])[i]) == len(inst["moves"]) <= 4096
+        for f in ("window", "recv", "donor", "kind", "seq"):
+            np.testing.assert_array_equal(moves[i][f], inst["moves"][f], err_msg=f"{i} {f}")
+        np.testing.assert_array_equal(_np(out["r_final"])[i], inst["r_final"])
