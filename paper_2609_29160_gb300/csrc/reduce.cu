@@ -586,7 +586,9 @@ __device__ __forceinline__ int4 load_slot(const int4* p) {
 
 // PAIR: two neighbouring cells' counts flushed with one 64-bit addition (an
 // even model count, 8-byte aligned outputs, and fewer than 2^31 events, so that
-// no 32-bit count carries into its neighbour)
+// no 32-bit count carries into its neighbour). Events outside the staged windows
+// are added to the same aligned pairs in 64 bits: other CTAs flush into those
+// words, and additions of two widths to one word are not promised to be atomic.
 template <bool PAIR>
 __global__ void __launch_bounds__(kThreads)
 k_reduce_events(EvCols e, int M, uint32_t span, FastDiv31 fd, int K, int per_cta, int rows,
@@ -654,8 +656,15 @@ k_reduce_events(EvCols e, int M, uint32_t span, FastDiv31 fd, int K, int per_cta
       ++n_order;
     } else {
       const uint32_t k = fd.div(tick), rel = k - (uint32_t)k_lo;
-      if (rel < (uint32_t)used) atomicAdd(&cells[rel * M + m], ph == 0 ? 1u : 65536u);
-      else atomicAdd(&(ph == 0 ? P : D)[(size_t)k * M + m], 1);
+      int32_t* const out = ph == 0 ? P : D;
+      const size_t x = (size_t)k * M + m;
+      if (rel < (uint32_t)used)
+        atomicAdd(&cells[rel * M + m], ph == 0 ? 1u : 65536u);
+      else if (PAIR)
+        atomicAdd(reinterpret_cast<unsigned long long*>(out + (x & ~(size_t)1)),
+                  x & 1 ? 1ull << 32 : 1ull);
+      else
+        atomicAdd(&out[x], 1);
       const int tk = (int)tick;
       if (slot >= 0) {
         if (tk < sl.y) atomicMin(&slots[slot].y, tk);

@@ -246,6 +246,30 @@ def test_reduce_events_edges(tre, M, n, n_req, win, K, shift):
     assert [d["dropped_range"], d["dropped_model"], d["dropped_order"]] == drops.tolist()
 
 
+# Out of time order, most events of a slice fall outside its staged windows: with
+# an even model count they are added to pairs of cells that other CTAs flush
+# into; with an odd one, or outputs that are not 8-byte aligned, to single cells.
+@pytest.mark.parametrize("M,shift", [(2, 0), (64, 0), (64, 1), (5, 0)])
+def test_reduce_events_pairs_of_cells(tre, M, shift):
+    import torch
+    rng = np.random.default_rng(M)
+    n, n_req, win, K = 60000, 4000, 100, 300
+    req_model = rng.integers(0, M, n_req).astype(np.int32)
+    req = rng.integers(0, n_req, n).astype(np.int32)
+    t = np.sort(rng.random(n) * K * win / 1000.0).astype(np.float32)
+    t[n // 2:] = rng.permutation(t[n // 2:])            # half in order, half not
+    ev = {"model": req_model[req], "req": req, "t_s": t,
+          "phase": rng.integers(0, 2, n).astype(np.uint8), "req_model": req_model,
+          "req_t_arr_ms": np.zeros(n_req, np.int32), "req_ttft_ms": np.zeros(n_req, np.int32)}
+    P, D, A, W, drops = oracle.reduce_events(ev, M, win, K)
+    out = {k: torch.empty(K * M + shift, dtype=torch.int32, device="cuda")[shift:].view(K, M)
+           for k in "PDAW"}
+    c = tre.tss_window_reduce(M, win, K, events=_cuda(ev), out=out)
+    for k, ref in zip("PDAW", (P, D, A, W)):
+        np.testing.assert_array_equal(_np(c[k]), ref, err_msg=k)
+    assert drops.sum() == 0
+
+
 def _score_inputs(rng, K, M, idle_frac=0.2):
     cnt = {}
     for k, hi in (("P", 5000), ("D", 800), ("A", 30), ("W", 60)):
