@@ -588,9 +588,11 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
         for (int q = tid; q < kFineHere; q += kNB) fst[q] = src[q];
         nsel = cl.map_shared_rank(plan_s, 0)[0];
         bf = cl.map_shared_rank(plan_s, 0)[1];
-        place = cl.map_shared_rank(fhl, 0);
-        keep = cl.map_shared_rank(list, 0);
       }
+      // every CTA, the first one too, adds to the places by cluster addresses: the
+      // same 32-bit addition from all of them
+      place = cl.map_shared_rank(fhl, 0);
+      keep = cl.map_shared_rank(list, 0);
       cl.sync();                    // the first CTA may end from here on unless keys are listed
     }
     __syncthreads();
@@ -604,8 +606,10 @@ k_search(const __grid_constant__ SeriesTable<T> tab, typename KeyOf<T>::U* __res
         });
         if (lmin != ~(U)0) atomicMin(&bfmin_s, lmin);
         if constexpr (CL > 1) {
-          // each CTA's smallest is its own until all have it: a 64-bit minimum in
-          // another CTA's memory is not atomic with those of that CTA
+          // each CTA's smallest is its own until all have it. (With one minimum in the
+          // first CTA's memory, its own by shared and the others' by cluster addresses,
+          // boundaries in double were one value off now and then; that the two do not
+          // exclude each other in 64 bits is inferred from this, not documented.)
           const cg::cluster_group cl = cg::this_cluster();
           cl.sync();
           if (rank == 0 && tid == 0)

@@ -1007,7 +1007,8 @@ def test_reduce_requests_1024_models(tre, where):
 @pytest.mark.parametrize("dtype", ["f32", "f64"])
 @pytest.mark.parametrize("levels", [0, 40])
 @pytest.mark.parametrize("K,M", [(1, 1), (63, 3), (1024, 2), (8192, 2), (8193, 2), (7000, 37),
-                                 (7100, 37), (16384, 4), (33001, 9)])
+                                 (7100, 37), (16383, 2), (16384, 4), (32767, 2), (32768, 3),
+                                 (33001, 9)])
 def test_calibrate_search_edges(tre, dtype, levels, K, M):
     rng = np.random.default_rng(K + M + levels)
     npdt = np.float32 if dtype == "f32" else np.float64
