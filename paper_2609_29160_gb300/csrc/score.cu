@@ -104,8 +104,18 @@ struct TilePlan {
 // short instruction sequence for a subroutine, and takes its whole warp along
 // (188 instructions a cell, now 85; Eq. 1 of 64 models, 864,000 windows 299 us,
 // now 180), so it divides a one instead and returns the numerator, as 0 / b is.
+// The tests on doubles are made on their bits: comparisons of doubles go through
+// the pipe that the division itself waits for.
+__device__ __forceinline__ bool zero_by_positive(float a, float b) {
+  return (a == 0.f) & (b > 0.f);
+}
+__device__ __forceinline__ bool zero_by_positive(double a, double b) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(a);
+  const unsigned long long v = (unsigned long long)__double_as_longlong(b);
+  return (u << 1 == 0) & (v - 1 < 0x7ff0000000000000ull);      // 0 < b <= infinity
+}
 template <class T> __device__ __forceinline__ T div_zero_rn(T a, T b) {
-  const bool zero = (a == (T)0) & (b > (T)0);
+  const bool zero = zero_by_positive(a, b);
   const T q = div_rn(zero ? (T)1 : a, b);
   return zero ? a : q;
 }
@@ -870,14 +880,43 @@ template <> __device__ __forceinline__ void load_quad_z<double>(const double* p,
   v[0] = a.x; v[1] = a.y; v[2] = c.x; v[3] = c.y;
 }
 
+// Z as an unsigned key in the order of the values (-0 as 0); any NaN comes after
+// every value, and all ones, for an idle model, after that. Comparisons of
+// doubles would take the pipe that their divisions wait for.
+__device__ __forceinline__ uint32_t z_key(float z) {
+  const uint32_t u = __float_as_uint(z);
+  if ((u << 1) > 0xff000000u) return ~0u - 1u;
+  return u == 0x80000000u ? u : u ^ ((u >> 31) ? ~0u : 0x80000000u);
+}
+__device__ __forceinline__ unsigned long long z_key(double z) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(z);
+  if ((u << 1) > 0xffe0000000000000ull) return ~0ull - 1ull;
+  return u == 0x8000000000000000ull ? u : u ^ ((u >> 63) ? ~0ull : 0x8000000000000000ull);
+}
+template <class T> struct ZKey;
+template <> struct ZKey<float> { using U = uint32_t; };
+template <> struct ZKey<double> { using U = unsigned long long; };
+__device__ __forceinline__ uint32_t lowest_key(uint32_t k) {
+  return __reduce_min_sync(0xffffffffu, k);
+}
+__device__ __forceinline__ unsigned long long lowest_key(unsigned long long k) {
+  const uint32_t hi = (uint32_t)(k >> 32), h = __reduce_min_sync(0xffffffffu, hi);
+  const uint32_t l = __reduce_min_sync(0xffffffffu, hi == h ? (uint32_t)k : ~0u);
+  return (unsigned long long)h << 32 | l;
+}
+
 // One series with the Eq. 3 receiver per window: argmin Z over non-idle models,
-// lowest index on ties (the first minimum in index order), -1 when every model
-// is idle. A CTA takes wt whole windows; their Z stay in shared memory (padded
-// rows) for one thread per window to scan, where a kernel of its own read Z and
-// the regions again, one row per thread (64 models, 864,000 windows: 124 us for
-// Z and regions and 120 for the receivers).
+// lowest index on ties (the first minimum in index order; a NaN only where it is
+// the first model that is not idle), -1 when every model is idle. A CTA takes wt
+// whole windows, the keys of their Z in shared memory (padded rows). Up to
+// kRowThread models one thread per window scans its row, above that a warp: 48
+// models, 130,000 windows in float 25.0 us by threads, 29.7 by warps; 72 models
+// 26.7 and 28.3; 96 models 27.0 and 25.1; 1,000 models, 10,000 windows 128 and 40
+// (double 327 and 189; 1,137 when the threads compared doubles). Bound in double
+// by the divisions.
 constexpr int kNormCells = 1024;
-template <class T> constexpr int kNormQuadPasses = sizeof(T) == 4 ? 4 : 2;
+constexpr int kRowThread = 80;
+constexpr int kNormQuadPasses = 4;
 constexpr int kNoQuad = 0x7fffffff;
 template <class T>
 __global__ void __launch_bounds__(kEwThreads)
@@ -885,8 +924,9 @@ k_norm_recv(int M, int K, int wt, FastDiv fm, bool vec, const T* __restrict__ S,
             const uint8_t* idle_cls, const T* __restrict__ theta, const T* __restrict__ tau_crit,
             const T* __restrict__ tau_surp, T* __restrict__ Z, uint8_t* cls,
             int32_t* __restrict__ recv) {
-  __shared__ T zs[2 * kNormCells];                     // [wt][M + 1]
-  __shared__ uint8_t on[2 * kNormCells];               // not idle
+  using U = typename ZKey<T>::U;
+  constexpr U kIdleKey = ~(U)0, kNanKey = ~(U)0 - 1;
+  __shared__ U zs[2 * kNormCells];                     // [wt][M + 1]
   const int k0 = (int)min64((int64_t)blockIdx.x * wt, K);
   const int nw = min(wt, K - k0), n = nw * M;
   const size_t x0 = (size_t)k0 * M;
@@ -894,8 +934,7 @@ k_norm_recv(int M, int K, int wt, FastDiv fm, bool vec, const T* __restrict__ S,
     const int w = (int)fm.div((uint32_t)c), m = c - w * M;
     z = div_rn(sv, theta[m]);
     cl = region_of(ic, z, tau_crit[m], tau_surp[m]);
-    zs[w * (M + 1) + m] = z;
-    on[w * (M + 1) + m] = cl != kIdle;
+    zs[w * (M + 1) + m] = cl != kIdle ? z_key(z) : kIdleKey;
   };
   if (vec) {                                           // wt * M is a multiple of 4
     for (int c = 4 * threadIdx.x; c < n; c += 4 * blockDim.x) {
@@ -921,18 +960,39 @@ k_norm_recv(int M, int K, int wt, FastDiv fm, bool vec, const T* __restrict__ S,
     }
   }
   __syncthreads();
-  for (int w = threadIdx.x; w < nw; w += blockDim.x) {
-    int best = -1;
-    T bz = (T)0;
+  if (M <= kRowThread) {
+    for (int w = threadIdx.x; w < nw; w += blockDim.x) {
+      int best = -1;
+      U low = kIdleKey;
 #pragma unroll 8
-    for (int m = 0; m < M; ++m) {
-      const T z = zs[w * (M + 1) + m];
-      if (on[w * (M + 1) + m] && (best < 0 || z < bz)) {
+      for (int m = 0; m < M; ++m) {
+        const U k = zs[w * (M + 1) + m];
+        if (k < low) {
+          best = m;
+          low = k == kNanKey ? (U)0 : k;               // nothing is lower than a first NaN
+        }
+      }
+      recv[k0 + w] = best;
+    }
+    return;
+  }
+  const int lane = threadIdx.x & 31;
+  for (int w = threadIdx.x >> 5; w < nw; w += blockDim.x >> 5) {
+    int best = kNoQuad, first = kNoQuad;               // first: low bit for a NaN
+    U low = kIdleKey;
+#pragma unroll 4
+    for (int m = lane; m < M; m += 32) {
+      const U k = zs[w * (M + 1) + m];
+      if (k != kIdleKey && first == kNoQuad) first = 2 * m + (k == kNanKey ? 1 : 0);
+      if (k < low) {
         best = m;
-        bz = z;
+        low = k;
       }
     }
-    recv[k0 + w] = best;
+    const U l = lowest_key(low);
+    best = __reduce_min_sync(0xffffffffu, low == l ? best : kNoQuad);
+    first = __reduce_min_sync(0xffffffffu, first);
+    if (lane == 0) recv[k0 + w] = first == kNoQuad ? -1 : first & 1 ? first >> 1 : best;
   }
 }
 
@@ -941,18 +1001,18 @@ k_norm_recv(int M, int K, int wt, FastDiv fm, bool vec, const T* __restrict__ S,
 // takes one window after another, four in flight; a window's receiver comes from
 // shuffles among the lanes that hold its row. A scan of the row by one thread left
 // 240 of a CTA's 256 threads idle (64 models, 864,000 windows: 173 us, now 138). Bound by
-// memory and by the division's instructions.
-template <class T>
+// memory and by the division's instructions. Float only: in double k_norm_recv is
+// faster (6.4 M cells: 122 us for 148, whatever the row's length).
 __global__ void __launch_bounds__(kEwThreads)
-k_norm_quads(int M, int lg_quads, int64_t n_quads, const T* __restrict__ S, const uint8_t* idle_cls,
-             const T* __restrict__ theta, const T* __restrict__ tau_crit,
-             const T* __restrict__ tau_surp, T* __restrict__ Z, uint8_t* cls,
+k_norm_quads(int lg_quads, int64_t n_quads, const float* __restrict__ S, const uint8_t* idle_cls,
+             const float* __restrict__ theta, const float* __restrict__ tau_crit,
+             const float* __restrict__ tau_surp, float* __restrict__ Z, uint8_t* cls,
              int32_t* __restrict__ recv) {
-  constexpr int U = kNormQuadPasses<T>;
+  constexpr int U = kNormQuadPasses;
   const unsigned full = 0xffffffffu;
   const int64_t q0 = (int64_t)blockIdx.x * (kEwThreads * U) + threadIdx.x;
   const int lanes = 1 << lg_quads, m0 = 4 * (threadIdx.x & (lanes - 1));
-  T th[4], tc[4], ts[4], sv[U][4];
+  float th[4], tc[4], ts[4], sv[U][4];
   uchar4 ic[U];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -965,9 +1025,9 @@ k_norm_quads(int M, int lg_quads, int64_t n_quads, const T* __restrict__ S, cons
     const int64_t q = q0 + u * kEwThreads;
     ic[u] = make_uchar4(kIdle, kIdle, kIdle, kIdle);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) sv[u][i] = (T)1;
+    for (int i = 0; i < 4; ++i) sv[u][i] = 1.f;
     if (q < n_quads) {
-      load_quad_z<T>(S + 4 * q, sv[u]);
+      load_quad_z<float>(S + 4 * q, sv[u]);
       ic[u] = *reinterpret_cast<const uchar4*>(idle_cls + 4 * q);
     }
   }
@@ -980,10 +1040,10 @@ k_norm_quads(int M, int lg_quads, int64_t n_quads, const T* __restrict__ S, cons
     // not idle, with a low bit for a NaN (an ascending scan starts from it and
     // nothing compares below a NaN)
     int best = kNoQuad, first = kNoQuad;
-    T bz = (T)0;
+    float bz = 0.f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const T z = div_zero_rn(sv[u][i], th[i]);
+      const float z = div_zero_rn(sv[u][i], th[i]);
       sv[u][i] = z;
       cl[i] = region_of(idle[i], z, tc[i], ts[i]);
       const bool on = cl[i] != kIdle, nan = z != z;
@@ -994,18 +1054,12 @@ k_norm_quads(int M, int lg_quads, int64_t n_quads, const T* __restrict__ S, cons
       }
     }
     if (q < n_quads) {
-#pragma unroll
-      for (int h = 0; h < 4; h += 16 / (int)sizeof(T)) {
-        Four<T> o;
-#pragma unroll
-        for (int i = 0; i < 16 / (int)sizeof(T); ++i) o.v[i] = sv[u][h + i];
-        *reinterpret_cast<Four<T>*>(Z + 4 * q + h) = o;
-      }
+      *reinterpret_cast<float4*>(Z + 4 * q) = make_float4(sv[u][0], sv[u][1], sv[u][2], sv[u][3]);
       *reinterpret_cast<uchar4*>(cls + 4 * q) = make_uchar4(cl[0], cl[1], cl[2], cl[3]);
     }
     for (int o = 1; o < lanes; o <<= 1) {
       const int ob = __shfl_xor_sync(full, best, o);
-      const T oz = __shfl_xor_sync(full, bz, o);
+      const float oz = __shfl_xor_sync(full, bz, o);
       if (ob != kNoQuad && (best == kNoQuad || oz < bz || (oz == bz && ob < best))) {
         best = ob;
         bz = oz;
@@ -1466,12 +1520,14 @@ cudaError_t launch_normalize(const SeriesTable<T>& tab, const T* S, const uint8_
     const int M = tab.M, K = tab.K[0], th = small ? kSmallThreads : kEwThreads;
     int lg_quads = 0;
     while (lg_quads < 5 && 4 << lg_quads < M) ++lg_quads;
-    if (vec && !small && M == 4 << lg_quads) {
-      constexpr int kPerCta = kEwThreads * kNormQuadPasses<T>;
-      const int64_t n_quads = (int64_t)K << lg_quads;
-      k_norm_quads<T><<<(unsigned)((n_quads + kPerCta - 1) / kPerCta), kEwThreads, 0, s>>>(
-          M, lg_quads, n_quads, S, idle_cls, theta, tau_crit, tau_surp, Z, cls, recv);
-      return cudaGetLastError();
+    if constexpr (sizeof(T) == 4) {
+      if (vec && !small && M == 4 << lg_quads) {
+        constexpr int kPerCta = kEwThreads * kNormQuadPasses;
+        const int64_t n_quads = (int64_t)K << lg_quads;
+        k_norm_quads<<<(unsigned)((n_quads + kPerCta - 1) / kPerCta), kEwThreads, 0, s>>>(
+            lg_quads, n_quads, S, idle_cls, theta, tau_crit, tau_surp, Z, cls, recv);
+        return cudaGetLastError();
+      }
     }
     const int wt = std::max(1, (small ? th : kNormCells) / M);
     k_norm_recv<T><<<(unsigned)((K + wt - 1) / wt), th, 0, s>>>(

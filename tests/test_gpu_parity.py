@@ -708,9 +708,10 @@ def test_stage_table_edges(tre, M, win, K):
 
 
 # one to 32 lanes a row on tables past the small ones, a ragged last CTA, rows with
-# no lanes of their own (24); NaN, infinite and zero values, ties of both zeros
+# no lanes of their own (24) and rows scanned by a warp (81 and more, one window a
+# CTA from 513); NaN, infinite and zero values, ties of both zeros
 @pytest.mark.parametrize("dtype", [np.float32, np.float64])
-@pytest.mark.parametrize("M", [4, 8, 16, 24, 32, 64, 128])
+@pytest.mark.parametrize("M", [4, 8, 16, 24, 32, 33, 64, 80, 81, 128, 513, 1024])
 def test_normalize_receiver_rows(tre, dtype, M):
     rng = np.random.default_rng(M)
     K = (1 << 18) // M + 37
@@ -733,6 +734,24 @@ def test_normalize_receiver_rows(tre, dtype, M):
             if recv[k] < 0 or Z[k, m] < Z[k, recv[k]]:
                 recv[k] = m
     np.testing.assert_array_equal(_np(out["recv"]), recv)
+
+
+# theta that no calibration gives: a zero series over it is what IEEE division says
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_normalize_zero_over_odd_theta(tre, dtype):
+    tiny = np.finfo(dtype).smallest_subnormal
+    theta = np.array([0.0, -0.0, 1.0, -1.0, np.inf, -np.inf, np.nan, tiny], dtype)
+    S = np.tile(np.array([[0.0], [-0.0], [1.0], [np.nan]], dtype), (1 << 14, len(theta)))
+    idle = np.ones(S.shape, np.uint8)
+    prof = {"w_p": 0.2, "w_q": 2.0, "alpha": 0.5, "tau_crit": 0.8, "tau_surplus": 1.2,
+            "theta": theta}
+    for n in (60, len(S)):
+        out = tre.tss_normalize(*_cuda({"S": S[:n], "c": idle[:n]}).values(), prof, 100)
+        with np.errstate(all="ignore"):
+            Z = S[:n] / theta
+        got = _np(out["Z"])
+        np.testing.assert_array_equal(got, Z)
+        np.testing.assert_array_equal(np.signbit(got)[~np.isnan(Z)], np.signbit(Z)[~np.isnan(Z)])
 
 
 def test_calibrate_events(tre):
