@@ -301,7 +301,7 @@ __device__ __forceinline__ void load_batch(const T* __restrict__ raw, const uint
 // `verify`, stop at the first window whose new S equals the stored one with the
 // same init state: from there the stored trajectory is the one this start
 // produces. Returns true if it stopped early.
-template <class T, bool WRITE = true>
+template <class T>
 __device__ __forceinline__ bool run_segment(size_t base, int M, int64_t k0, int64_t k1,
                                             const T* __restrict__ raw, const ModelParams<T>& q,
                                             T& S, int& init, bool verify, int stored_init,
@@ -331,7 +331,6 @@ __device__ __forceinline__ bool run_segment(size_t base, int M, int64_t k0, int6
         stored_init = 1;
       }
       if (verify && init == stored_init && same_bits(S, old[j])) return true;
-      if (!WRITE) continue;
       S_out[base + (size_t)(k + j) * M] = init ? S : (T)0;
     }
 #pragma unroll
@@ -414,6 +413,22 @@ constexpr int64_t kShortChains = 16384;       // most chains a table is cut into
 // group in double, two in float, where a chain's start costs as much as a group
 template <class T> constexpr int short_chunk() { return sizeof(T) == 8 ? kGroup : 2 * kGroup; }
 
+// Burn-in length, in updates (non-idle windows): (1 - alpha)^B <= e^-c, in
+// whole groups, with c well past the point where a start error falls
+// below the type's last bit, so that the rounded trajectories have met
+// (c = 28 for float's 6e-8 = e^-16.6, 45 for double's 1.1e-16 = e^-36.7)
+template <class T> __device__ __forceinline__ int burn_in(T alpha) {
+  const float a = (float)alpha;
+  const float c = sizeof(T) == 4 ? 28.f : 45.f;
+  int B = kMaxBurn;
+  if (a >= 1.f) B = kGroup;
+  else if (a > 0.f) {
+    const float x = c / -log1pf(-a);
+    if (x < (float)kMaxBurn) B = (int)x + 1;
+  }
+  return (B + kGroup - 1) / kGroup * kGroup;
+}
+
 // The chain's input for one window: raw, or in double alpha * raw
 template <class T> constexpr bool kPremul = sizeof(T) == 8;
 
@@ -494,21 +509,7 @@ k_ema(const __grid_constant__ SeriesTable<T> tab, const T* __restrict__ raw, con
   const ModelParams<T> q = load_params(tab, s, m, alpha);
   const int L = tab.seg_len[s];
   const int64_t k0 = (int64_t)(seg - tab.seg_base[s]) * L, k1 = min64(k0 + L, tab.K[s]);
-  // burn-in length, in updates (non-idle windows): (1 - alpha)^B <= e^-c, in
-  // whole groups, with c well past the point where a start error falls
-  // below the type's last bit, so that the rounded trajectories have met
-  // (c = 28 for float's 6e-8 = e^-16.6, 45 for double's 1.1e-16 = e^-36.7)
-  int B = kMaxBurn;
-  {
-    const float a = (float)q.a;
-    const float c = sizeof(T) == 4 ? 28.f : 45.f;
-    if (a >= 1.f) B = kGroup;
-    else if (a > 0.f) {
-      const float x = c / -log1pf(-a);
-      if (x < (float)kMaxBurn) B = (int)x + 1;
-    }
-    B = (B + kGroup - 1) / kGroup * kGroup;
-  }
+  const int B = burn_in(q.a);
   // The burn-in runs over spans of windows [sp_lo, sp_hi), ascending. Without
   // activity counts it is the one span [k0 - B, k0). With them (non-idle
   // windows per chunk) it walks back over the preceding chunks until they hold
@@ -690,31 +691,51 @@ k_ema(const __grid_constant__ SeriesTable<T> tab, const T* __restrict__ raw, con
 // ---- pass 2: boundary check and repair, one CTA per (series, model) ---------
 // The CTA compares every chunk's burn-in state with its predecessor's end state
 // (one round of loads; a warp that took 32 boundaries at a time waited on
-// memory once per 32). Where none differs, as almost always, that is all. Else
-// one warp repairs: a chunk whose burn-in state differs is run again from its
-// predecessor's end until its new trajectory meets the stored one; first as a
-// dry run, so that a chunk is rewritten only when every chunk before it keeps
-// its end state. A chunk whose re-run never meets its stored trajectory changes
-// its end state, and from the next chunk on the boundaries are walked in order
-// by one lane.
+// memory once per 32). Where none differs, as almost always, that is all. Else it
+// repairs in passes: each chunk whose start differs is run again from its
+// predecessor's end, a chunk a thread, until its new trajectory meets the stored
+// one. A pass carries the states one chunk further, and a start error shrinks with
+// every non-idle window on the way, so where burn-ins fell short because windows
+// were idle here and there some passes make all starts equal the ends before them,
+// which is the sequential result. From the share of idle windows that the first
+// pass sees, the CTA reckons how many that takes; where they would cost more than
+// half of a walk in order (long idle stretches, a tiny alpha), one lane walks. 8
+// models, 36,000 windows, every other one idle, alpha 0.2: 128 us a call in float,
+// 651 in double; 1,813 and 8,254 with one dry run before the walk in order,
+// in which chunks had to meet within their own 64 or 32 windows.
 constexpr int kResolveThreads = 128;
+constexpr int kRerun = 2;          // start_init: the chunk has been run again
 template <class T>
 __global__ void __launch_bounds__(kResolveThreads)
 k_resolve(const __grid_constant__ SeriesTable<T> tab, const T* __restrict__ raw, const T* alpha,
-          const T* start_S, const int32_t* start_init, T* end_S, int32_t* end_init, T* S_out,
+          T* start_S, int32_t* start_init, T* end_S, int32_t* end_init, T* S_out,
           const uint8_t* __restrict__ cls, T* S_carry, uint8_t* init_carry, tre_diag* diag) {
+  __shared__ int first_s, seen_s[2];
   const int M = tab.M;
-  const int lane = threadIdx.x & 31;
   const int s = blockIdx.x / M, m = blockIdx.x % M;
   const int n_seg = tab.seg_base[s + 1] - tab.seg_base[s];
   if (n_seg == 0) return;
   const size_t g0 = (size_t)tab.seg_base[s] * M + m;
+  const int L = tab.seg_len[s];
+  const size_t base = (size_t)tab.off[s] + m;
+  // chunk c's state before it (its predecessor's end) and at its own start
+  struct Edge {
+    T pS;
+    int pI, sI;
+    bool bad;
+  };
+  auto edge = [&](int c) {
+    const size_t x = g0 + (size_t)c * M;
+    Edge e;
+    e.pS = end_S[x - M];
+    e.pI = end_init[x - M];
+    e.sI = start_init[x];
+    e.bad = (e.sI & 1) != e.pI || !same_bits(start_S[x], e.pS);
+    return e;
+  };
   bool differs = false;
 #pragma unroll 4
-  for (int c = 1 + threadIdx.x; c < n_seg; c += kResolveThreads) {
-    const size_t x = g0 + (size_t)c * M;
-    differs |= start_init[x] != end_init[x - M] || !same_bits(start_S[x], end_S[x - M]);
-  }
+  for (int c = 1 + threadIdx.x; c < n_seg; c += kResolveThreads) differs |= edge(c).bad;
   if (!__syncthreads_or(differs)) {
     if (S_carry && threadIdx.x == 0) {
       const size_t last = g0 + (size_t)(n_seg - 1) * M;
@@ -723,60 +744,73 @@ k_resolve(const __grid_constant__ SeriesTable<T> tab, const T* __restrict__ raw,
     }
     return;
   }
-  if (threadIdx.x >= 32) return;
   const ModelParams<T> q = load_params(tab, s, m, alpha);
-  const int L = tab.seg_len[s];
-  const size_t base = (size_t)tab.off[s] + m;
-  int first_bad = n_seg;   // the in-order walk starts here
-  for (int c0 = 1; c0 < n_seg; c0 += 32) {
-    const int c = c0 + lane;
-    bool bad = false, moved = false;
-    T pS = (T)0;
-    int pI = 0, sI = 0;
-    int64_t k0 = 0, k1 = 0;
-    if (c < n_seg) {
-      const size_t x = g0 + (size_t)c * M;
-      pS = end_S[x - M];
-      pI = end_init[x - M];
-      sI = start_init[x];
-      bad = sI != pI || !same_bits(start_S[x], pS);
-      k0 = (int64_t)c * L;
-      k1 = min64(k0 + L, tab.K[s]);
-    }
-    if (bad) {
-      T S = pS;
-      int init = pI;
-      moved = !run_segment<T, false>(base, M, k0, k1, raw, q, S, init, true, sI, S_out, cls);
-    }
-    const unsigned mv = __ballot_sync(0xffffffffu, moved);
-    const int lim = mv ? c0 + __ffs(mv) - 1 : n_seg;   // predecessors final up to here
-    if (bad && c <= lim) {
-      T S = pS;
-      int init = pI;
-      const bool met = run_segment<T>(base, M, k0, k1, raw, q, S, init, true, sI, S_out, cls);
-      if (!met) {
-        end_S[g0 + (size_t)c * M] = S;
-        end_init[g0 + (size_t)c * M] = init;
+  unsigned n_rerun = 0;
+  bool some = true;
+  const int rounds = (n_seg - 2) / kResolveThreads + 1;   // of a pass
+  if (threadIdx.x < 2) seen_s[threadIdx.x] = 0;
+  for (int pass = 0, n_pass = 1; pass < n_pass && some; ++pass) {
+    some = false;
+    int windows = 0, on = 0;       // of the chunks that met nothing stored
+    for (int c0 = 1; c0 < n_seg; c0 += kResolveThreads) {
+      const int c = c0 + (int)threadIdx.x;
+      Edge e = {};
+      if (c < n_seg) e = edge(c);
+      // every thread has its predecessor's end before any of them changes
+      if (!__syncthreads_or(e.bad)) continue;
+      some = true;
+      if (e.bad) {
+        const size_t x = g0 + (size_t)c * M;
+        const int64_t k0 = (int64_t)c * L, k1 = min64(k0 + L, tab.K[s]);
+        T S = e.pS;
+        int init = e.pI;
+        const bool met =
+            run_segment<T>(base, M, k0, k1, raw, q, S, init, true, e.sI & 1, S_out, cls);
+        start_S[x] = e.pS;
+        start_init[x] = e.pI | kRerun;
+        if (!met) {
+          end_S[x] = S;
+          end_init[x] = init;
+          if (pass == 0) {
+            windows += (int)(k1 - k0);
+#pragma unroll 8
+            for (int64_t k = k0; k < k1; ++k) on += cls[base + (size_t)k * M] != kIdle;
+          }
+        }
+        n_rerun += !(e.sI & kRerun);
       }
-      atomicAdd(&diag->ema_resolved, 1ull);
+      __syncthreads();
     }
-    if (mv) {
-      first_bad = lim + 1;
-      break;
+    if (pass == 0 && some) {
+      if (windows) atomicAdd(&seen_s[0], windows);
+      if (on) atomicAdd(&seen_s[1], on);
+      __syncthreads();
+      // updates that the burn-ins lacked, over those of a chunk; and two passes for
+      // chunks with fewer than the mean
+      const float w = (float)seen_s[0], u = (float)seen_s[1];
+      const float passes = 2.f + (float)burn_in(q.a) * (w - u) / (u * (float)L);
+      if (!(u < w)) n_pass = 2;
+      else if (passes * (float)(2 * rounds) <= (float)n_seg) n_pass = 2 + (int)passes;
     }
   }
-  __syncwarp();
-  if (lane != 0) return;
-  const size_t last = g0 + (size_t)(min(first_bad, n_seg) - 1) * M;
+  if (n_rerun) atomicAdd(&diag->ema_resolved, (unsigned long long)n_rerun);
+  int first_bad = n_seg;   // the in-order walk starts here
+  if (some) {
+    if (threadIdx.x == 0) first_s = n_seg;
+    __syncthreads();
+    for (int c = 1 + (int)threadIdx.x; c < n_seg; c += kResolveThreads)
+      if (edge(c).bad) {
+        atomicMin(&first_s, c);
+        break;
+      }
+    __syncthreads();
+    first_bad = first_s;
+  }
+  if (threadIdx.x != 0) return;
+  const size_t last = g0 + (size_t)(first_bad - 1) * M;
   T S = end_S[last];
   int init = end_init[last];
-  if (first_bad >= n_seg) {
-    if (S_carry) {
-      S_carry[m] = S;
-      init_carry[m] = (uint8_t)init;
-    }
-    return;
-  }
+  n_rerun = 0;
   for (int q0 = first_bad; q0 < n_seg; q0 += kBatch) {
     // load the boundary states of a batch of segments ahead of the checks
     T bS[kBatch], bE[kBatch];
@@ -795,20 +829,22 @@ k_resolve(const __grid_constant__ SeriesTable<T> tab, const T* __restrict__ raw,
     for (int j = 0; j < kBatch; ++j) {
       const int qq = q0 + j;
       if (qq >= n_seg) break;
-      if (init == bI[j] && same_bits(S, bS[j])) {
+      if (init == (bI[j] & 1) && same_bits(S, bS[j])) {
         S = bE[j];
         init = bEI[j];
         continue;
       }
       const int64_t k0 = (int64_t)qq * L, k1 = min64(k0 + L, tab.K[s]);
-      const bool met = run_segment<T>(base, M, k0, k1, raw, q, S, init, true, bI[j], S_out, cls);
+      const bool met =
+          run_segment<T>(base, M, k0, k1, raw, q, S, init, true, bI[j] & 1, S_out, cls);
       if (met) {
         S = bE[j];
         init = bEI[j];
       }
-      atomicAdd(&diag->ema_resolved, 1ull);
+      n_rerun += !(bI[j] & kRerun);
     }
   }
+  if (n_rerun) atomicAdd(&diag->ema_resolved, (unsigned long long)n_rerun);
   if (S_carry) {
     S_carry[m] = S;
     init_carry[m] = (uint8_t)init;

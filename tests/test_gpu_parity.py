@@ -1192,6 +1192,41 @@ def test_score_when_burn_ins_cannot_converge(tre, dtype):
     assert tre.read_diag(diag)["ema_resolved"] > 0
 
 
+# Windows idle here and there: burn-ins see too few updates and the chunks (64 windows
+# in float, 32 in double) are run again, in a few passes (every other window
+# idle) or in order after ten (nine of ten idle; an alpha of 0.001); one chunk,
+# one round of 128 chunks and one more, the state carried across two calls.
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("alpha,idle", [(0.2, 0.5), (0.2, 0.9), (0.02, 0.5), (0.001, 0.3)])
+@pytest.mark.parametrize("K", [65, 4129, 8192, 8300, 20001])
+def test_score_scattered_idle_windows(tre, dtype, alpha, idle, K):
+    import torch
+    rng = np.random.default_rng(K)
+    M, win = 2, 100
+    cnt = {k: rng.integers(0, 900, (K, M)).astype(np.int32) for k in "PDAW"}
+    off = rng.random((K, M)) < idle
+    for k in cnt:
+        cnt[k][off] = 0
+    prof = {"w_p": 0.2, "w_q": 2.0, "alpha": alpha, "theta": 3.0, "tau_crit": 0.8,
+            "tau_surplus": 1.2}
+    npdt = np.float32 if dtype == "f32" else np.float64
+    S, Z, cls, recv = oracle.score(cnt["P"], cnt["D"], cnt["A"], cnt["W"], prof, win, npdt)
+    tdt = torch.float32 if dtype == "f32" else torch.float64
+    diag = tre.new_diag()
+    carry = {"S": torch.zeros(M, dtype=tdt, device="cuda"),
+             "init": torch.zeros(M, dtype=torch.uint8, device="cuda")}
+    cut = K // 7
+    parts = [tre.tss_score(_cuda({k: np.ascontiguousarray(v[a:b]) for k, v in cnt.items()}), prof,
+                           win, dtype=dtype, carry=carry, diag=diag)
+             for a, b in ((0, cut), (cut, K))]
+    for k, ref in (("S", S), ("Z", Z), ("cls", cls), ("recv", recv)):
+        np.testing.assert_array_equal(np.concatenate([_np(p[k]) for p in parts]), ref, err_msg=k)
+    np.testing.assert_array_equal(_np(carry["S"]), S[-1])
+    chunks = M * sum(-(-n // (64 if dtype == "f32" else 32)) for n in (cut, K - cut))
+    resolved = tre.read_diag(diag)["ema_resolved"]
+    assert resolved <= chunks and (resolved > 0 or K < 8000 or alpha < 0.2)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "f64"])
 def test_score_long_table_idle_stretches(tre, dtype):
     """A table long enough for the burn-ins that skip wholly idle chunks (at
