@@ -328,13 +328,36 @@ __device__ __forceinline__ bool start_requests(uint32_t* sv, int n, const int4* 
 }
 
 // the same with the free times left in memory, for more servers than four per
-// lane and for longer stretches of time
-template <class F>
+// lane and for longer stretches of time. A start reads all free times up to
+// kScanServers; above (BLOCKS) the earliest one of each of up to 256 blocks of
+// servers is kept eight per lane, and a start reads one block. 20,000 requests of 2
+// models in 60 windows: 200 servers a model 2.62 ms by reading all, 3.23 by blocks;
+// 600 servers 3.21 and 3.21; 1,000 servers 5.13 and 3.22; 32,768 servers 112 and 4.0.
+constexpr int kScanServers = 600;
+template <bool BLOCKS, class F>
 __device__ __forceinline__ void start_requests_mem(uint32_t* sv, int n,
                                                    const int4* __restrict__ grp, int& head,
                                                    int end, uint32_t t_end, F&& done) {
+  constexpr int R = BLOCKS ? 8 : 1;
   const int lane = threadIdx.x & 31;
   bool more = head < end;
+  if (!more || (uint32_t)__ldg(&grp[2 * (size_t)head]).x >= t_end) return;
+  const int len = ((n + 32 * R - 1) / (32 * R) + 31) / 32 * 32;   // of a block
+  uint32_t low[R];                       // of block r * 32 + lane
+  if constexpr (BLOCKS) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      low[r] = kNoServer;
+#pragma unroll 4
+      for (int i = 0; i < 32; ++i) {
+        const int q0 = (r * 32 + i) * len, q1 = min(q0 + len, n);
+        uint32_t v = kNoServer;
+        for (int q = q0 + lane; q < q1; q += 32) v = min(v, sv[q]);
+        v = __reduce_min_sync(kFull, v);
+        if (i == lane) low[r] = v;
+      }
+    }
+  }
   while (more) {
     int4 c0 = make_int4(0, 0, 0, 0), c1 = c0;
     if (head + lane < end) {
@@ -347,12 +370,50 @@ __device__ __forceinline__ void start_requests_mem(uint32_t* sv, int n,
     for (; j < cnt; ++j) {
       const uint32_t ta = (uint32_t)__shfl_sync(kFull, c0.x, j);
       const uint32_t dt = (uint32_t)__shfl_sync(kFull, c0.z, j);
-      int at;
-      const uint32_t st = max(ta, Servers{sv, n}.first(at));
-      if (st >= t_end) break;
-      __syncwarp();
-      if (lane == 0) sv[at] = min(st + dt, kNever);
-      __syncwarp();
+      uint32_t st;
+      if constexpr (BLOCKS) {
+        uint32_t l = low[0];
+        int lr = 0;
+#pragma unroll
+        for (int r = 1; r < R; ++r)
+          if (low[r] < l) {
+            l = low[r];
+            lr = r;
+          }
+        const uint32_t first = __reduce_min_sync(kFull, l);
+        st = max(ta, first);
+        if (st >= t_end) break;
+        const int owner = __ffs(__ballot_sync(kFull, l == first)) - 1;
+        const int blk = __shfl_sync(kFull, lr, owner) * 32 + owner;
+        // the block's first server, and the block's minimum with its new free time
+        uint32_t best = kNoServer, next = kNoServer;
+        int at = -1;
+        for (int q = blk * len + lane; q < min((blk + 1) * len, n); q += 32) {
+          const uint32_t v = sv[q];
+          next = min(next, max(v, best));
+          if (v < best) {
+            best = v;
+            at = q;
+          }
+        }
+        const uint32_t te = min(st + dt, kNever);
+        if (lane == __ffs(__ballot_sync(kFull, best == first)) - 1) {
+          sv[at] = te;
+          best = min(next, te);
+        }
+        __syncwarp();
+        const uint32_t left = __reduce_min_sync(kFull, best);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          if (blk == r * 32 + lane) low[r] = left;
+      } else {
+        int at;
+        st = max(ta, Servers{sv, n}.first(at));
+        if (st >= t_end) break;
+        __syncwarp();
+        if (lane == 0) sv[at] = min(st + dt, kNever);
+        __syncwarp();
+      }
       if (lane == j) mine = st;
     }
     head += j;
@@ -468,7 +529,10 @@ k_replay(const __grid_constant__ ReplayBatch<T> b) {
           : n <= 64  ? start_requests<2>(sv, n, b.grp, head, end, t_end, done)
           : n <= 128 ? start_requests<4>(sv, n, b.grp, head, end, t_end, done)
                      : false;
-      if (!held) start_requests_mem(sv, n, b.grp, head, end, t_end, done);
+      if (!held) {
+        if (n <= kScanServers) start_requests_mem<false>(sv, n, b.grp, head, end, t_end, done);
+        else start_requests_mem<true>(sv, n, b.grp, head, end, t_end, done);
+      }
     };
     if (starts) {
       auto pass = [&](uint32_t st, bool more) {

@@ -157,12 +157,15 @@ def test_replay_sixty_four_models(tre):
 
 
 # A model's free times sit one, two or four to a lane, in shared memory above
-# 128 servers, in the workspace when a budget's do not fit there. Arrivals out of
-# order: a request waits for the one before it in the input, and what it would
-# add to windows already scored is not seen.
+# 128 servers (read by blocks of 32 above 600, of more above 8,192), in the
+# workspace when a budget's do not fit there. Arrivals out of order: a request
+# waits for the one before it in the input, and what it would add to windows
+# already scored is not seen.
 @pytest.mark.parametrize("shuffled", [False, True])
 @pytest.mark.parametrize("servers,budget", [((33, 5, 64), 120), ((65, 128, 1), 200),
-                                            ((129, 2, 300), 440), ((20, 30, 40), 30000)])
+                                            ((129, 2, 300), 440), ((20, 30, 40), 30000),
+                                            ((600, 601, 250), 1460), ((8192, 700, 4001), 12900),
+                                            ((8193, 17000, 1), 25200)])
 def test_replay_server_counts_and_input_order(tre, servers, budget, shuffled):
     rng = np.random.default_rng(budget + shuffled)
     n, M, span = 3000, 3, 300000
