@@ -1182,7 +1182,7 @@ template <> struct RankKey<float> {
   float v;
   RankKey() = default;
   __device__ __forceinline__ explicit RankKey(float z) : v(z) {}
-  __device__ __forceinline__ bool finite() const { return fabsf(v) < __int_as_float(0x7f800000); }
+  __device__ __forceinline__ bool nan() const { return v != v; }
   static __device__ __forceinline__ RankKey most() { return RankKey(__int_as_float(0x7f800000)); }
 };
 template <> struct RankKey<double> {
@@ -1192,8 +1192,8 @@ template <> struct RankKey<double> {
     const unsigned long long u = (unsigned long long)__double_as_longlong(z);
     v = u == 0x8000000000000000ull ? u : u ^ ((u >> 63) ? ~0ull : 0x8000000000000000ull);
   }
-  __device__ __forceinline__ bool finite() const {
-    return v - 0x0010000000000000ull < 0xffe0000000000000ull;
+  __device__ __forceinline__ bool nan() const {    // outside the keys of both infinities
+    return v - 0x000fffffffffffffull > 0xffe0000000000001ull;
   }
   static __device__ __forceinline__ RankKey most() {
     RankKey k;
@@ -1210,7 +1210,7 @@ __device__ __forceinline__ uint32_t shift_left(uint32_t x, uint32_t n) {
 }
 
 // One window by comparisons of its values, as an ascending scan orders them: for
-// rows with infinities or NaN.
+// rows with a NaN among the models that are not idle.
 template <class T>
 __device__ __noinline__ void rank_window(int M, const T* z, const uint8_t* c, int32_t* recv,
                                          int32_t* out) {
@@ -1301,12 +1301,13 @@ k_rank_small(int M, int K, const T* __restrict__ Z, const uint8_t* __restrict__ 
 #pragma unroll
   for (int m = 0; m < MMAX; ++m) {
     const bool on = busy >> m & 1u;
-    odd |= on & !zv[m].finite();
+    odd |= on & zv[m].nan();
     if (on & (zv[m].v < bz.v)) {
       best = m;
       bz = zv[m];
     }
   }
+  if (best < 0 && busy) best = __ffs(busy) - 1;      // nothing below infinity: the first
   int32_t* out = donors ? donors + (size_t)k * kRankDonors : nullptr;
   if (odd) {
     rank_window<T>(M, z, c, recv ? recv + k : nullptr, out);

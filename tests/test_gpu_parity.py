@@ -459,6 +459,24 @@ def test_rank_small_edges(tre, dtype, M, shift):
     np.testing.assert_array_equal(_np(g["donors"]), ref[1])
 
 
+# Windows whose models are infinite, all of them or all but a few, in any region;
+# NaN only where a model is idle
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("M", [1, 2, 8, 11, 16])
+def test_rank_infinite_rows(tre, dtype, M):
+    rng = np.random.default_rng(M)
+    K = 2000
+    Z = rng.choice(np.array([np.inf, np.inf, np.inf, -np.inf], dtype), (K, M))
+    Z[::3] = np.inf
+    Z[rng.random((K, M)) < 0.2] = 1.0
+    cls = rng.choice(np.arange(4, dtype=np.uint8), (K, M))
+    ref = oracle.rank(Z, cls)
+    Z[(cls == 3) & (rng.random((K, M)) < 0.5)] = np.nan
+    g = tre.tss_rank(*_cuda({"Z": Z, "cls": cls}).values())
+    np.testing.assert_array_equal(_np(g["recv"]), ref[0])
+    np.testing.assert_array_equal(_np(g["donors"]), ref[1])
+
+
 def test_rank_empty_grid(tre):
     import torch
     g = tre.tss_rank(torch.zeros((0, 4), dtype=torch.float32, device="cuda"),
