@@ -226,7 +226,7 @@ tre_status calibrate_typed(const tre_grid* g, const tre_requests* req, const tre
                         in->A_ms, in->W_ms);
   }
   if (!e) {
-    Scope sc(kCalibrate, 3, s);
+    Scope sc(kCalibrate, calibrate_launches(tab), s);
     e = launch_calibrate<T>(tab, S, cls, slo, ok_frac, rel, static_cast<T*>(theta), cw, diag, s);
   }
   return cuda_status(e);
@@ -493,7 +493,7 @@ tre_status sweep_typed(const tre_sweep_spec* sp, const SweepPlan& pl, const tre_
                         nullptr, nullptr, S, nullptr, idle, nullptr, sw, diag, s);
   }
   if (!e) {
-    Scope sc(kCalibrate, 3, s);
+    Scope sc(kCalibrate, calibrate_launches(tab), s);
     e = launch_calibrate<T>(tab, S, idle, slo, sp->ok_frac, sp->reliability, theta, cw, diag, s);
   }
   if (!e) {
@@ -566,7 +566,7 @@ tre_status stage_calibrate_typed(const tre_grid* g, const tre_requests* req, con
                                static_cast<const T*>(p->alpha), S, cls, sw, diag, s);
   }
   if (!e) {
-    Scope sc(kCalibrate, 3, s);
+    Scope sc(kCalibrate, calibrate_launches(tab), s);
     e = launch_calibrate<T>(tab, S, cls, ttft, ok_frac, rel, static_cast<T*>(th_pre), cw, diag, s,
                             static_cast<T*>(th_dec));
   }

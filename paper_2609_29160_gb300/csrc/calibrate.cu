@@ -765,6 +765,21 @@ template <class T> void calib_ws_layout(Arena& a, int64_t elems, int n_sm, Calib
   w.n_sm = n_sm;
 }
 
+// series short enough, and a table small enough, to be searched without packing
+template <class T> static bool direct_search(const SeriesTable<T>& tab) {
+  int64_t cells = 0;
+  for (int i = 0; i < tab.n; ++i) {
+    if (tab.K[i] > kDirectK) return false;
+    cells += (int64_t)tab.K[i] * tab.M;
+  }
+  return cells <= kDirectCells;
+}
+
+// thresholds, packing and search, or the search alone
+template <class T> int calibrate_launches(const SeriesTable<T>& tab) {
+  return direct_search(tab) ? 1 : 3;
+}
+
 template <class T>
 cudaError_t launch_calibrate(const SeriesTable<T>& tab, const T* S, const uint8_t* cls,
                              const unsigned long long* slo, double ok_frac, double reliability,
@@ -775,13 +790,7 @@ cudaError_t launch_calibrate(const SeriesTable<T>& tab, const T* S, const uint8_
   U* kmin = static_cast<U*>(w.kmin);
   U* kmax = static_cast<U*>(w.kmax);
   const size_t smem = search_smem_bytes<T>();
-  bool direct = true;
-  int64_t cells = 0;
-  for (int i = 0; i < tab.n; ++i) {
-    direct = direct && tab.K[i] <= kDirectK;
-    cells += (int64_t)tab.K[i] * tab.M;
-  }
-  if (direct && cells <= kDirectCells) {
+  if (direct_search(tab)) {
     cudaError_t e = func_smem_once((const void*)k_search<T, true, 1>, (int)smem, true);
     if (e) return e;
     k_search<T, true, 1><<<n_sm, kNB, smem, s>>>(tab, static_cast<U*>(w.keys), kmin, kmax, w.ncand, S,
@@ -841,6 +850,8 @@ cudaError_t launch_calibrate(const SeriesTable<T>& tab, const T* S, const uint8_
   return cudaGetLastError();
 }
 
+template int calibrate_launches<float>(const SeriesTable<float>&);
+template int calibrate_launches<double>(const SeriesTable<double>&);
 template void calib_ws_layout<float>(Arena&, int64_t, int, CalibWs<float>&);
 template void calib_ws_layout<double>(Arena&, int64_t, int, CalibWs<double>&);
 template cudaError_t launch_calibrate<float>(const SeriesTable<float>&, const float*,

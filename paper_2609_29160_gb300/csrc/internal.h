@@ -233,6 +233,8 @@ template <class T> struct CalibWs {
   int n_sm;                    // (series, model) pairs the range arrays hold
 };
 template <class T> void calib_ws_layout(Arena& a, int64_t elems, int n_sm, CalibWs<T>& w);
+// kernels one launch_calibrate call issues (for the phase trace)
+template <class T> int calibrate_launches(const SeriesTable<T>& tab);
 // theta[s*M + m] for every series of the table (theta1: where the second series'
 // boundaries go when not there)
 template <class T>

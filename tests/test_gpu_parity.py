@@ -1085,6 +1085,34 @@ def test_calibrate_search_edges(tre, dtype, levels, K, M):
             assert tre.read_diag(diag)["degenerate_calib"] == deg
 
 
+def test_trace_counts_calibration_launches(tre):
+    """The phase trace counts one launch for series searched without packing
+    their keys (up to 8192 windows) and three for longer ones."""
+    import ctypes as C
+    import torch
+
+    class Trace(C.Structure):
+        _fields_ = [("n_phases", C.c_int32), ("name", C.c_char_p * 11), ("ms", C.c_double * 11),
+                    ("calls", C.c_int64 * 11), ("launches", C.c_int64 * 11)]
+
+    lib = tre.load()
+    slo = np.full(2, 1000, np.int32)
+    req = _cuda({k: np.ones(8, np.int32) for k in REQ_KEYS})
+    prof = {"w_p": 0.25, "w_q": 2.0, "alpha": 0.5}
+    for K, launches in ((8192, 1), (8193, 3)):
+        c = tre.tss_window_reduce(2, 1000, K, requests=req)
+        lib.tre_trace_enable(C.c_int(1))
+        try:
+            tre.tss_calibrate(c, prof, 1000, slo, requests=req, dtype="f32")
+            torch.cuda.synchronize()
+            tr = Trace()
+            assert lib.tre_trace_collect(C.byref(tr)) == 0
+        finally:
+            lib.tre_trace_enable(C.c_int(0))
+        got = {tr.name[i].decode(): (tr.calls[i], tr.launches[i]) for i in range(tr.n_phases)}
+        assert got["calibrate"] == (1, launches)
+
+
 def test_calibrate_1024_models(tre):
     import torch
     rng = np.random.default_rng(4)
