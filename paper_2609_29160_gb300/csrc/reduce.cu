@@ -95,7 +95,7 @@ k_reduce_requests(const __grid_constant__ ReqBatch bt, int M, int lgMp, int win,
                   int32_t* __restrict__ D0, int32_t* __restrict__ dA0, int32_t* __restrict__ dW0,
                   unsigned long long* __restrict__ slo0, const int32_t* __restrict__ slo_ms,
                   tre_diag* diag) {
-  extern __shared__ unsigned long long smem[];
+  extern __shared__ __align__(16) unsigned long long smem[];   // cleared 16 bytes a store
   uint32_t n_range = 0, n_model = 0, n_order = 0;
   // a CTA takes slices blockIdx.x, blockIdx.x + gridDim.x, ...: one slice when
   // the grid holds them all; a smaller grid leaves SMs to other streams' work
