@@ -1210,11 +1210,17 @@ unsigned grid_for(int64_t work, int per_thread = 1) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)num_sms() * 16));
 }
 
-int scan_chunk_rows(int K) {
-  // up to 1024 chunks of at least 16 rows; four times as many for long series, so
-  // that there are (chunk, model) threads enough to keep memory busy (64 models,
-  // 864,000 windows: the pass that applies the prefixes 211 -> 150 us)
-  const int chunks = K > 256 * 1024 ? 1024 * kMaxChunksPerThread : 1024;
+// Rows per chunk of the gauge scan: up to 1024 chunks of at least 16 rows, or four
+// times as many on long series, whose threads would each walk a long chain of
+// rows. The line lies where 4096 chunks begin to win (three passes of the scan,
+// 1024 chunks and 4096): 8 models, 70,000 windows 23.1 and 23.8 us, 130,000 windows
+// 31.7 and 26.4, 864,000 windows 179 and 72; 64 models 27.5 and 31.5, 55.7 and
+// 43.8, 324 and 245. With four models or fewer, whose 1024 chunks are few threads,
+// it lies lower: 10,000 windows 16.9 and 16.9, 40,000 windows 23.1 and 20.0 (one
+// model 30.3 and 18.9).
+int scan_chunk_rows(int M, int K) {
+  const bool many = K > 96 * 1024 || (M <= 4 && K > 16 * 1024);
+  const int chunks = many ? 1024 * kMaxChunksPerThread : 1024;
   const int L = (K + chunks - 1) / chunks;
   return L < 16 ? 16 : L;
 }
@@ -1229,7 +1235,7 @@ void reduce_ws_layout(Arena& a, int M, int K, int n_traces, int64_t n_req, Reduc
   w.dW = a.take<int32_t>(cells);
   w.first = n_req > 0 ? a.take<int32_t>((size_t)n_req) : nullptr;
   w.last = n_req > 0 ? a.take<int32_t>((size_t)n_req) : nullptr;
-  const int L = scan_chunk_rows(K);
+  const int L = scan_chunk_rows(M, K);
   const int n_chunks = std::max((K + L - 1) / L, (K + kGaugeMinBlk - 1) / kGaugeMinBlk);
   w.part_cap = (int64_t)std::max(n_chunks, 1) * M;
   w.partA = a.take<int32_t>((size_t)w.part_cap * n_traces);
@@ -1395,7 +1401,7 @@ cudaError_t launch_reduce_events(const EvCols& ev, int M, int win, int K, int32_
   const size_t cells = (size_t)K * M;
   cudaError_t e;
   // every array the passes add into, in one launch
-  const int L = scan_chunk_rows(K);
+  const int L = scan_chunk_rows(M, K);
   w.chunks_summed = true;
   ZeroList zl;
   zl.n = 0;
@@ -1459,7 +1465,7 @@ int gauge_scan_launches(const ReduceWs& w) { return w.chunks_summed ? 2 : 3; }
 cudaError_t launch_gauge_scan(int M, int K, ReduceWs& w, int32_t* A, int32_t* W,
                               cudaStream_t s) {
   if (K == 0) return cudaSuccess;
-  const int L = scan_chunk_rows(K);
+  const int L = scan_chunk_rows(M, K);
   const int n_chunks = (K + L - 1) / L;
   const int64_t segs = (int64_t)n_chunks * M;
   dim3 g((unsigned)((segs + kThreads - 1) / kThreads), w.n_traces);
@@ -1732,7 +1738,7 @@ k_occ_events(EvCols ev, int M, int win, FastDiv fd, int K, const int32_t* __rest
 // partial sums
 cudaError_t occ_finish(int M, int win, int K, ReduceWs& w, int64_t* A_ms, int64_t* W_ms,
                        cudaStream_t s) {
-  const int L = scan_chunk_rows(K);
+  const int L = scan_chunk_rows(M, K);
   const int n_chunks = (K + L - 1) / L;
   const int64_t segs = (int64_t)n_chunks * M;
   const unsigned g = (unsigned)((segs + kThreads - 1) / kThreads);

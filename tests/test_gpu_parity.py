@@ -130,6 +130,13 @@ def test_reduce_requests_unaligned_columns(tre):
         np.testing.assert_array_equal(_np(c[k]), ref, err_msg=k)
 
 
+# The gauge scan takes more and shorter chunks of windows from a line that depends
+# on the model count; more chunks than one scan thread each from 1,024 on
+@pytest.mark.parametrize("M,K", [(4, 16384), (4, 16385), (1, 17000), (5, 98304), (5, 98305)])
+def test_reduce_scan_chunk_edges(tre, M, K):
+    _check_reduce(tre, _adversarial(np.random.default_rng(K), 20000, M, 10, K), M, 10, K)
+
+
 def test_reduce_empty_and_zero_windows(tre):
     req = {k: np.zeros(0, np.int32) for k in REQ_KEYS}
     _check_reduce(tre, req, 4, 1000, 10)
