@@ -805,7 +805,7 @@ __global__ void k_fill_first_last(int32_t* first, int32_t* last, int64_t n) {
 // per request with at least one valid event: waiting on [t_arr, first),
 // running on [first, last). A request changes four cells of a long, mostly empty
 // difference array, so its chunk sums for the gauge scan (rows of fchunk
-// windows; pA, pW null: not wanted) are added here, where summing the array
+// windows, in pA and pW) are added here, where summing the array
 // afterwards read all of it (864,000 windows of 64 models: 110 us).
 __global__ void __launch_bounds__(kThreads)
 k_event_gauges(EvCols e, int M, FastDiv fd, FastDiv fchunk, int K,
@@ -815,7 +815,7 @@ k_event_gauges(EvCols e, int M, FastDiv fd, FastDiv fchunk, int K,
   unsigned long long n_order = 0;
   auto add = [&](int32_t* d, int32_t* p, int64_t k, int m, int v) {
     atomicAdd(&d[k * M + m], v);
-    if (p && k < K) atomicAdd(&p[(size_t)fchunk.div((uint32_t)k) * M + m], v);
+    if (k < K) atomicAdd(&p[(size_t)fchunk.div((uint32_t)k) * M + m], v);
   };
   for (int64_t r = (int64_t)blockIdx.x * kThreads + threadIdx.x; r < e.n_req;
        r += (int64_t)gridDim.x * kThreads) {
@@ -1402,17 +1402,15 @@ cudaError_t launch_reduce_events(const EvCols& ev, int M, int win, int K, int32_
   cudaError_t e;
   // every array the passes add into, in one launch
   const int L = scan_chunk_rows(M, K);
-  w.chunks_summed = true;
   ZeroList zl;
   zl.n = 0;
   zero_add(zl, P, (int64_t)cells);
   zero_add(zl, D, (int64_t)cells);
   zero_add(zl, w.dA, (int64_t)(cells + M));
   zero_add(zl, w.dW, (int64_t)(cells + M));
-  if (w.chunks_summed) {
-    zero_add(zl, w.partA, (int64_t)((K + L - 1) / L) * M);
-    zero_add(zl, w.partW, (int64_t)((K + L - 1) / L) * M);
-  }
+  zero_add(zl, w.partA, (int64_t)((K + L - 1) / L) * M);
+  zero_add(zl, w.partW, (int64_t)((K + L - 1) / L) * M);
+  w.chunks_summed = true;                      // by the gauge pass below
   zero_launch(zl, s);
   if ((e = cudaGetLastError())) return e;
   if (ev.n_req > 0) {
@@ -1445,8 +1443,7 @@ cudaError_t launch_reduce_events(const EvCols& ev, int M, int win, int K, int32_
   }
   if (ev.n_req > 0) {
     k_event_gauges<<<grid_for(ev.n_req, 4), kThreads, 0, s>>>(
-        ev, M, FastDiv(win), FastDiv(L), K, w.first, w.last, w.dA, w.dW,
-        w.chunks_summed ? w.partA : nullptr, w.chunks_summed ? w.partW : nullptr, diag);
+        ev, M, FastDiv(win), FastDiv(L), K, w.first, w.last, w.dA, w.dW, w.partA, w.partW, diag);
     if ((e = cudaGetLastError())) return e;
   }
   return cudaSuccess;
