@@ -484,6 +484,29 @@ def test_rank_infinite_rows(tre, dtype, M):
     np.testing.assert_array_equal(_np(g["donors"]), ref[1])
 
 
+# A NaN where a model is not idle is outside what tss_rank promises an order for; its
+# receiver is still that of an ascending scan, and windows beside it are not touched
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("M", [2, 8, 16])
+def test_rank_nan_rows(tre, dtype, M):
+    rng = np.random.default_rng(M)
+    Z, cls = _rank_case(rng, 1200, M, dtype)
+    ref_r, ref_d = oracle.rank(Z, cls)
+    rows = rng.random(len(Z)) < 0.3
+    hit = rows[:, None] & (rng.random(Z.shape) < 0.4)
+    Z[hit] = np.nan
+    rows = (hit & (cls != 3)).any(1)
+    for k in np.flatnonzero(rows):
+        ref_r[k] = -1
+        for m in np.flatnonzero(cls[k] != 3):
+            if ref_r[k] < 0 or Z[k, m] < Z[k, ref_r[k]]:
+                ref_r[k] = m
+    g = tre.tss_rank(*_cuda({"Z": Z, "cls": cls}).values())
+    np.testing.assert_array_equal(_np(g["recv"]), ref_r)
+    np.testing.assert_array_equal(_np(g["donors"])[~rows], ref_d[~rows])
+    assert ((_np(g["donors"]) >= -1) & (_np(g["donors"]) < M)).all()
+
+
 def test_rank_empty_grid(tre):
     import torch
     g = tre.tss_rank(torch.zeros((0, 4), dtype=torch.float32, device="cuda"),
@@ -994,8 +1017,7 @@ def test_sweep_small(tre):
 @pytest.mark.parametrize("dtype", ["f32", "f64"])
 def test_sweep_many_series_rank_in_walk(tre, dtype):
     """Five traces x 4 window lengths x 8 rescue thresholds: at least one
-    (series, threshold) block per SM, so the jump walk ranks its own ticks
-    from the Z and class rows (one launch) instead of reading tick tables."""
+    (series, threshold) block per SM in one launch of the lane walk."""
     sw, alpha = _sweep_case(0.02, 5, 600.0)
     sw["pacing_cap"] = sw["pacing_cap"][::4]
     ref, out = _run_sweep_both(tre, sw, alpha, moves_cap=512, dtype=dtype)

@@ -162,8 +162,7 @@ def test_sweep_twenty_four_models(tre, caps):
 
 def test_jump_walk_long_series_sixteen_models(tre):
     """Sixteen models over 43,200 windows of 500 ms (the code/chat workload's
-    shape): the jump walk's tables fill nearly all of a block's shared memory,
-    and the tick windows are recomputed at each visit instead of staged."""
+    shape): 4,320 ticks, five slabs of the lane walk in two buffers."""
     Z, cls, g, r0, budget, r_min = _case(16, 43200, 16, idle=0.05)
     for cap in (1, 2):
         _check(tre, Z, cls, g, r0, budget, r_min, 500, cap)
@@ -173,22 +172,23 @@ def test_jump_walk_long_series_sixteen_models(tre):
 @pytest.mark.parametrize("fast_ms,slow_ms,win", [(3000, 10000, 1000), (500, 10000, 1000),
                                                  (700, 2100, 100)])
 def test_warp_walk_cadences(tre, M, fast_ms, slow_ms, win):
-    """The warp walk for more than 16 models on cadences that are not nested
-    or a fast tick shorter than a window (every tick visited in order), and on
-    nested ones (32 ticks tested against the state at once)."""
+    """More than 16 models on cadences that are not nested or with a fast tick
+    shorter than a window (the warp walk, every tick visited in order), and on
+    nested ones (the lane walk)."""
     Z, cls, g, r0, budget, r_min = _case(900 + M + fast_ms, 3000, M)
     for cap in (1, 3):
         _check(tre, Z, cls, g, r0, budget, r_min, win, cap, fast_ms, slow_ms)
 
 
-# One tick per window. Ticks are ranked in chunks of 128 and staged 1024 (768
-# for more than 32 models) at a time; row words hold 3 to 6 rank bits for 8,
-# 16, 32 and 64 models. Infinite Z and zeros of both signs (equal, so the lower
+# One tick per window. Ticks are ranked in chunks of 128 and staged 1024 at a time
+# (768 for more than 16 models, 384 for more than 32), series of one slab in one
+# buffer; row words hold 3 to 6 rank bits for 8, 16, 32 and 64 models. Infinite Z and zeros of both signs (equal, so the lower
 # index goes first) sit among the ties.
 @pytest.mark.parametrize("hetero,cap", [(False, 1), (False, 5), (True, 3)])
 @pytest.mark.parametrize("M,ticks", [(2, 129), (8, 127), (8, 128), (8, 1025), (9, 2200),
-                                     (16, 1024), (17, 129), (32, 1153), (33, 769), (64, 768),
-                                     (64, 1700)])
+                                     (16, 1024), (16, 1025), (17, 129), (32, 768), (32, 769),
+                                     (32, 1153), (33, 384), (33, 769), (64, 384), (64, 385),
+                                     (64, 768), (64, 1700)])
 def test_lane_walk_chunk_and_slab_edges(tre, M, ticks, hetero, cap):
     dtype = np.float64 if ticks % 2 else np.float32
     Z, cls, g, r0, budget, r_min = _case(40 + M + ticks, ticks, M, hetero=hetero, dtype=dtype)
@@ -197,6 +197,36 @@ def test_lane_walk_chunk_and_slab_edges(tre, M, ticks, hetero, cap):
         Z[rng.random(Z.shape) < 0.04] = v
     budget += 2
     _check(tre, Z, cls, g, r0, budget, r_min, 1000, cap, 1000, 2000)
+
+
+# A Z that is no number (a zero theta under a zero series) has a place of its own in
+# every order: the walk ends, and its moves, final replicas, floors and budget agree
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("M,hetero,cap", [(8, False, 1), (16, False, 4), (16, True, 2),
+                                          (33, False, 2), (64, True, 1)])
+def test_lane_walk_nan_values(tre, dtype, M, hetero, cap):
+    import torch
+    K = 1500
+    Z, cls, g, r0, budget, r_min = _case(M + cap, K, M, hetero=hetero, dtype=dtype)
+    Z[np.random.default_rng(M).random(Z.shape) < 0.1] = np.nan
+    prof = {"w_p": 0.2, "w_q": 2.0, "alpha": 0.2, "theta": 1.0, "tau_crit": 0.8,
+            "tau_surplus": 1.2}
+    mv, rf, n, diag = tre.tre_select_moves(torch.as_tensor(Z).cuda(), torch.as_tensor(cls).cuda(),
+                                           prof, 1000, budget, r0, r_min, g, fast_ms=1000,
+                                           slow_ms=2000, pacing_cap=cap, moves_cap=1 << 15)
+    assert 0 < n == len(mv) and tre.read_diag(diag)["err"] == 0
+    r, floor = r0.astype(int), np.minimum(r_min, r0)
+    same = lambda a, b: (a["window"], a["seq"], a["recv"]) == (b["window"], b["seq"], b["recv"])
+    for i, x in enumerate(mv):
+        assert x["window"] >= mv[max(i - 1, 0)]["window"] and x["donor"] != x["recv"]
+        assert cls[x["window"], x["recv"]] != 3
+        if x["donor"] >= 0:
+            r[x["donor"]] -= 1
+            assert r[x["donor"]] >= floor[x["donor"]]
+        if i + 1 == n or not same(x, mv[i + 1]):
+            r[x["recv"]] += 1
+            assert (g * r).sum() <= budget
+    np.testing.assert_array_equal(_np(rf), r)
 
 
 # A warp logs 256 moves before it writes them out. Idle pools of whole multiples
