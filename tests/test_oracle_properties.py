@@ -181,5 +181,20 @@ def test_closed_loop_against_batch_rescoring(case):
     np.testing.assert_array_equal(cls, o["cls"])
     mv, rf, _ = oracle.select_moves(Z, cls, 0.8, 1.2, 1000, budget, r0, np.zeros(M),
                                     np.ones(M), pacing_cap=Kp)
-    np.testing.assert_array_equal(mv, o["moves"])
-    np.testing.assert_array_equal(rf, o["r_final"])
+    # the open-loop walk does not see waiting requests: the two agree up to the first
+    # fast tick at which a model has some and no replica (it is rescued for that)
+    lost = K
+    for k in range(4, K, 5):
+        r = np.array(r0)
+        for x in o["moves"]:
+            if x["window"] < k:
+                r[x["recv"]] += 1
+                if x["donor"] >= 0:
+                    r[x["donor"]] -= 1
+        if ((r == 0) & (W[k] > 0)).any():
+            lost = k
+            break
+    np.testing.assert_array_equal(mv[mv["window"] < lost],
+                                  o["moves"][o["moves"]["window"] < lost])
+    if lost == K:
+        np.testing.assert_array_equal(rf, o["r_final"])
