@@ -956,10 +956,9 @@ constexpr int kNormQuadPasses = 4;
 constexpr int kNoQuad = 0x7fffffff;
 template <class T>
 __global__ void __launch_bounds__(kEwThreads)
-k_norm_recv(int M, int K, int wt, FastDiv fm, bool vec, const T* __restrict__ S,
+k_norm_recv(int M, int K, int wt, FastDiv fm, bool vec, const T* S,
             const uint8_t* idle_cls, const T* __restrict__ theta, const T* __restrict__ tau_crit,
-            const T* __restrict__ tau_surp, T* __restrict__ Z, uint8_t* cls,
-            int32_t* __restrict__ recv) {
+            const T* __restrict__ tau_surp, T* Z, uint8_t* cls, int32_t* __restrict__ recv) {
   using U = typename ZKey<T>::U;
   constexpr U kIdleKey = ~(U)0, kNanKey = ~(U)0 - 1;
   __shared__ U zs[2 * kNormCells];                     // [wt][M + 1]
@@ -1040,9 +1039,9 @@ k_norm_recv(int M, int K, int wt, FastDiv fm, bool vec, const T* __restrict__ S,
 // memory and by the division's instructions. Float only: in double k_norm_recv is
 // faster (6.4 M cells: 122 us for 148, whatever the row's length).
 __global__ void __launch_bounds__(kEwThreads)
-k_norm_quads(int lg_quads, int64_t n_quads, const float* __restrict__ S, const uint8_t* idle_cls,
+k_norm_quads(int lg_quads, int64_t n_quads, const float* S, const uint8_t* idle_cls,
              const float* __restrict__ theta, const float* __restrict__ tau_crit,
-             const float* __restrict__ tau_surp, float* __restrict__ Z, uint8_t* cls,
+             const float* __restrict__ tau_surp, float* Z, uint8_t* cls,
              int32_t* __restrict__ recv) {
   constexpr int U = kNormQuadPasses;
   const unsigned full = 0xffffffffu;

@@ -782,6 +782,11 @@ def test_normalize_receiver_rows(tre, dtype, M):
             if recv[k] < 0 or Z[k, m] < Z[k, recv[k]]:
                 recv[k] = m
     np.testing.assert_array_equal(_np(out["recv"]), recv)
+    # Z over S and the regions over the idle classes
+    s, c = _cuda({"S": S, "c": idle}).values()
+    over = tre.tss_normalize(s, c, prof, 100, Z_out=s, cls_out=c)
+    for k in ("Z", "cls", "recv"):
+        np.testing.assert_array_equal(_np(over[k]), _np(out[k]), err_msg=k)
 
 
 # theta that no calibration gives: a zero series over it is what IEEE division says
