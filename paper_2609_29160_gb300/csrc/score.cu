@@ -12,15 +12,16 @@
 //      for double), records the state
 //      it reached, then runs its chunk from that state and stores the result;
 //   2. one CTA per (series, model) checks the chunk boundaries: a chunk whose
-//      recorded burn-in state equals its predecessor's exact end state (bit
-//      for bit, with the same started/not-started flag) is exact, because
-//      every step depends only on the previous state; any other chunk is run
-//      again from the exact state until its new trajectory meets the stored
-//      one. A chunk whose burn-in reaches window 0 starts from the true initial
-//      state and is exact by construction.
-// The result is therefore the sequential one in every case; the in-order pass
-// only re-runs chunks when a burn-in did not converge (long idle stretches, a
-// tiny alpha), counted in tre_diag.ema_resolved.
+//      recorded burn-in state equals its predecessor's end state (bit for bit,
+//      with the same started/not-started flag) goes on where the one before it
+//      ends, because every step depends only on the previous state; any other
+//      chunk is run again from that end until its new trajectory meets the stored
+//      one, in passes over all chunks and in order where passes would be many. A
+//      chunk whose burn-in reaches window 0 starts from the true initial state
+//      and is exact by construction.
+// Where every boundary agrees, the result is the sequential one; chunks are re-run
+// only when a burn-in did not converge (idle windows, a tiny alpha), counted in
+// tre_diag.ema_resolved.
 #include <algorithm>
 #include <initializer_list>
 
