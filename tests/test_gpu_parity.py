@@ -905,7 +905,7 @@ def test_select_heterogeneous_footprints_and_overflow(tre):
 @pytest.mark.parametrize("M,r_each,extra", [(8, 20, 3), (8, 40, 5), (5, 60, 0), (7, 1, 1)])
 @pytest.mark.parametrize("cap", [1, 2])
 def test_select_unit_footprints_small_and_large_budgets(tre, M, r_each, extra, cap):
-    # budgets up to 255 keep every model's replicas in one byte; larger ones not
+    # donors one, many or no replicas above their floors, with and without an idle pool
     import torch
     rng = np.random.default_rng(M * 100 + r_each)
     K, win = 4000, 500
