@@ -945,14 +945,13 @@ __device__ __forceinline__ unsigned long long lowest_key(unsigned long long k) {
 // One series with the Eq. 3 receiver per window: argmin Z over non-idle models,
 // lowest index on ties (the first minimum in index order; a NaN only where it is
 // the first model that is not idle), -1 when every model is idle. A CTA takes wt
-// whole windows, the keys of their Z in shared memory (padded rows). Up to
-// kRowThread models one thread per window scans its row, above that a warp: 48
-// models, 130,000 windows in float 25.0 us by threads, 29.7 by warps; 72 models
-// 26.7 and 28.3; 96 models 27.0 and 25.1; 1,000 models, 10,000 windows 128 and 40
-// (double 327 and 189; 1,137 when the threads compared doubles). Bound in double
-// by the divisions.
+// whole windows, their Z in shared memory (padded rows). Up to kRowThread models
+// one thread per window scans its row, above that a warp: 48 models, 130,000
+// windows in float 24.3 us by threads, 29.7 by warps; 72 models 30.6 and 28.3; 96
+// models 29.4 and 25.1; 1,000 models, 10,000 windows 140 and 40 (double 327 and 189;
+// 1,137 when the threads compared doubles). Bound in double by the divisions.
 constexpr int kNormCells = 1024;
-constexpr int kRowThread = 80;
+constexpr int kRowThread = 64;
 constexpr int kNormQuadPasses = 4;
 constexpr int kNoQuad = 0x7fffffff;
 template <class T>
@@ -962,7 +961,11 @@ k_norm_recv(int M, int K, int wt, FastDiv fm, bool vec, const T* S,
             const T* __restrict__ tau_surp, T* Z, uint8_t* cls, int32_t* __restrict__ recv) {
   using U = typename ZKey<T>::U;
   constexpr U kIdleKey = ~(U)0, kNanKey = ~(U)0 - 1;
+  // values of a float row that one thread scans, else keys: a comparison of floats
+  // costs no more, and making keys does
+  const bool values = sizeof(T) == 4 && M <= kRowThread;
   __shared__ U zs[2 * kNormCells];                     // [wt][M + 1]
+  __shared__ uint8_t on[sizeof(T) == 4 ? 2 * kNormCells : 1];   // values: not idle
   const int k0 = (int)min64((int64_t)blockIdx.x * wt, K);
   const int nw = min(wt, K - k0), n = nw * M;
   const size_t x0 = (size_t)k0 * M;
@@ -970,7 +973,14 @@ k_norm_recv(int M, int K, int wt, FastDiv fm, bool vec, const T* S,
     const int w = (int)fm.div((uint32_t)c), m = c - w * M;
     z = div_rn(sv, theta[m]);
     cl = region_of(ic, z, tau_crit[m], tau_surp[m]);
-    zs[w * (M + 1) + m] = cl != kIdle ? z_key(z) : kIdleKey;
+    const int at = w * (M + 1) + m;
+    if constexpr (sizeof(T) == 4)
+      if (values) {
+        zs[at] = __float_as_uint(z);
+        on[at] = cl != kIdle;
+        return;
+      }
+    zs[at] = cl != kIdle ? z_key(z) : kIdleKey;
   };
   if (vec) {                                           // wt * M is a multiple of 4
     for (int c = 4 * threadIdx.x; c < n; c += 4 * blockDim.x) {
@@ -999,13 +1009,25 @@ k_norm_recv(int M, int K, int wt, FastDiv fm, bool vec, const T* S,
   if (M <= kRowThread) {
     for (int w = threadIdx.x; w < nw; w += blockDim.x) {
       int best = -1;
-      U low = kIdleKey;
+      if constexpr (sizeof(T) == 4) {
+        float low = 0.f;
 #pragma unroll 8
-      for (int m = 0; m < M; ++m) {
-        const U k = zs[w * (M + 1) + m];
-        if (k < low) {
-          best = m;
-          low = k == kNanKey ? (U)0 : k;               // nothing is lower than a first NaN
+        for (int m = 0; m < M; ++m) {
+          const float z = __uint_as_float(zs[w * (M + 1) + m]);
+          if (on[w * (M + 1) + m] && (best < 0 || z < low)) {
+            best = m;
+            low = z;
+          }
+        }
+      } else {
+        U low = kIdleKey;
+#pragma unroll 8
+        for (int m = 0; m < M; ++m) {
+          const U k = zs[w * (M + 1) + m];
+          if (k < low) {
+            best = m;
+            low = k == kNanKey ? (U)0 : k;             // nothing is lower than a first NaN
+          }
         }
       }
       recv[k0 + w] = best;

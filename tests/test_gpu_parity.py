@@ -756,10 +756,10 @@ def test_stage_table_edges(tre, M, win, K):
 
 
 # one to 32 lanes a row on tables past the small ones, a ragged last CTA, rows with
-# no lanes of their own (24) and rows scanned by a warp (81 and more, one window a
+# no lanes of their own (24) and rows scanned by a warp (65 and more, one window a
 # CTA from 513); NaN, infinite and zero values, ties of both zeros
 @pytest.mark.parametrize("dtype", [np.float32, np.float64])
-@pytest.mark.parametrize("M", [4, 8, 16, 24, 32, 33, 64, 80, 81, 128, 513, 1024])
+@pytest.mark.parametrize("M", [4, 8, 16, 24, 32, 33, 63, 64, 65, 80, 81, 128, 513, 1024])
 def test_normalize_receiver_rows(tre, dtype, M):
     rng = np.random.default_rng(M)
     K = (1 << 18) // M + 37
